@@ -34,8 +34,9 @@ struct Grad {
 };
 
 // What the adjoint reads for one env: the loaded parameters (transposes), the coefficients the
-// forward step used (re-running it bit for bit) and, on the general path, the env's off-diagonal
-// hydrodynamic coefficients (a row of MG_NXPARAM floats in shared memory).
+// re-run steps with (the forward's, with the dense thruster allocation: equal to the forward's
+// states within the rounding of the allocation's sums) and, on the general path, the env's
+// off-diagonal hydrodynamic coefficients (a row of MG_NXPARAM floats in shared memory).
 template <bool GEN>
 struct AdjEnv {
   Par<!GEN> P;
@@ -588,7 +589,7 @@ template <bool GEN>
 __device__ __forceinline__ void load_env(const FleetView &fv, int64_t e, bool ca,
                                          const float *sxh_row, AdjEnv<GEN> &A) {
   load_par<!GEN>(fv.pa, e, A.P);
-  A.F = make_coef<!GEN>(A.P);
+  A.F = make_coef<!GEN>(A.P, nullptr, nullptr);
   A.xh = GEN ? sxh_row : nullptr;
 }
 
@@ -918,11 +919,11 @@ __global__ void __maxnreg__(XH ? kRegsXH : DIAG ? kRegsWide : kRegsGeneral)
 
   St<MT> s;
   load_state<MT>(fv.st, e, s);
-  Coef<DIAG> P;
+  Coef<DIAG, NH> P;
   {
     Par<DIAG> raw;
     load_par<DIAG>(fv.pa, e, raw);
-    P = make_coef<DIAG>(raw);
+    P = make_coef<DIAG, NH>(raw, sdir, sarm);
   }
   const int64_t step0 = s_cursor + fv.cursor_off;
   int64_t seg = step0 / fv.hold;
@@ -963,13 +964,16 @@ cudaError_t rollout_fwd_t(const FleetView &fv, const BlockDesc *blocks, int n_bl
 
 template <int NTV>
 cudaError_t rollout_fwd_d(const FleetView &fv, const BlockDesc *blocks, int n_blocks,
-                          int threads, bool diag, bool structured, int32_t T, int32_t C,
+                          int threads, bool diag, int layout, int32_t T, int32_t C,
                           float *traj, float *ckpt, cudaStream_t stream) {
   if (fv.xh)
     return rollout_fwd_t<NTV, false, 0, true>(fv, blocks, n_blocks, threads, T, C, traj, ckpt,
                                               stream);
-  if (diag && structured)
-    return rollout_fwd_t<NTV, true, 4, false>(fv, blocks, n_blocks, threads, T, C, traj, ckpt,
+  if (diag && layout == MG_LAYOUT_MIRRORED)
+    return rollout_fwd_t<NTV, true, MG_LAYOUT_MIRRORED, false>(fv, blocks, n_blocks, threads, T, C,
+                                                               traj, ckpt, stream);
+  if (diag && layout == MG_LAYOUT_VECTORED)
+    return rollout_fwd_t<NTV, true, MG_LAYOUT_VECTORED, false>(fv, blocks, n_blocks, threads, T, C, traj, ckpt,
                                               stream);
   if (diag)
     return rollout_fwd_t<NTV, true, 0, false>(fv, blocks, n_blocks, threads, T, C, traj, ckpt,
@@ -986,7 +990,7 @@ cudaError_t launch_checkpoint(const StatePlanes &st, int64_t n, float *ck, cudaS
 }
 
 cudaError_t launch_rollout_forward(const FleetView &fv, const BlockDesc *blocks, int n_blocks,
-                                   int threads, NtVariant ntv, bool diag, bool structured,
+                                   int threads, NtVariant ntv, bool diag, int layout,
                                    int32_t T, int32_t C, float *traj, float *ckpt,
                                    cudaStream_t stream) {
   if (threads < 32 || threads > 256 || threads % 32 || n_blocks < 1 || T < 1 || C < 1 ||
@@ -994,13 +998,13 @@ cudaError_t launch_rollout_forward(const FleetView &fv, const BlockDesc *blocks,
     return cudaErrorInvalidValue;
   switch (ntv) {
     case NT_6:
-      return rollout_fwd_d<NT_6>(fv, blocks, n_blocks, threads, diag, structured, T, C, traj,
+      return rollout_fwd_d<NT_6>(fv, blocks, n_blocks, threads, diag, layout, T, C, traj,
                                  ckpt, stream);
     case NT_8:
-      return rollout_fwd_d<NT_8>(fv, blocks, n_blocks, threads, diag, structured, T, C, traj,
+      return rollout_fwd_d<NT_8>(fv, blocks, n_blocks, threads, diag, layout, T, C, traj,
                                  ckpt, stream);
     default:
-      return rollout_fwd_d<NT_MIXED>(fv, blocks, n_blocks, threads, diag, structured, T, C,
+      return rollout_fwd_d<NT_MIXED>(fv, blocks, n_blocks, threads, diag, layout, T, C,
                                      traj, ckpt, stream);
   }
 }

@@ -146,11 +146,11 @@ __device__ __forceinline__ void advance_env(const FleetView &fv, int64_t e, int 
   const float h = fv.dt;
 
   load_state<MT, L2>(fv.st, e, s);
-  Coef<DIAG> P;
+  Coef<DIAG, NH> P;
   {
     Par<DIAG> raw;
     load_par<DIAG>(fv.pa, e, raw);
-    P = make_coef<DIAG>(raw);
+    P = make_coef<DIAG, NH>(raw, gdir, garm);
   }
 
   // Action cursor: sub-step j uses segment j / hold (clamped to the last buffered segment).

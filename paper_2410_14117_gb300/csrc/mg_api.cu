@@ -12,7 +12,7 @@
 #include <string>
 #include <vector>
 
-#include "mg_internal.h"
+#include "mg_device.cuh"
 
 using namespace mg;
 
@@ -36,6 +36,36 @@ bool mg::vectored_layout(const Geo &g) {
     if (i >= 4 && (g.dir[i].x != 0.f || g.dir[i].y != 0.f || g.arm[i].z != 0.f)) return false;
   }
   return true;
+}
+
+namespace {
+
+// Mirror images (MG_LAYOUT_MIRRORED): six or eight thrusters whose rows repeat one magnitude each
+// with the signs given there.
+bool mirrored_layout(const Geo &g) {
+  if ((g.n_thr != 6 && g.n_thr != 8) || !vectored_layout(g)) return false;
+  const float4 *d = g.dir, *a = g.arm;
+  auto rows = [](float x0, float x1, float x2, float x3, int s1, int s2, int s3) {
+    return x1 == s1 * x0 && x2 == s2 * x0 && x3 == s3 * x0;
+  };
+  if (!rows(d[0].x, d[1].x, d[2].x, d[3].x, 1, -1, -1) ||
+      !rows(d[0].y, d[1].y, d[2].y, d[3].y, -1, 1, -1) ||
+      !rows(a[0].x, a[1].x, a[2].x, a[3].x, -1, 1, -1) ||
+      !rows(a[0].y, a[1].y, a[2].y, a[3].y, 1, -1, -1) ||
+      !rows(a[0].z, a[1].z, a[2].z, a[3].z, -1, -1, 1))
+    return false;
+  if (g.n_thr == 6)
+    return d[5].z == d[4].z && a[5].x == -a[4].x && a[4].y == 0.f && a[5].y == 0.f;
+  return rows(d[4].z, d[5].z, d[6].z, d[7].z, 1, 1, 1) &&
+         rows(a[4].x, a[5].x, a[6].x, a[7].x, -1, 1, -1) &&
+         rows(a[4].y, a[5].y, a[6].y, a[7].y, 1, -1, -1);
+}
+
+}  // namespace
+
+int mg::thruster_layout(const Geo &g, const mg_vehicle_params &v) {
+  if (mirrored_layout(g) && v.rb[0] == 0.f && v.rb[1] == 0.f) return MG_LAYOUT_MIRRORED;
+  return vectored_layout(g) ? MG_LAYOUT_VECTORED : MG_LAYOUT_DENSE;
 }
 
 namespace {
@@ -96,7 +126,13 @@ struct mg_sim {
   // current-acceleration term, so a sim that switches that term off takes the general path.
   bool mass_diag = true;
   bool diag = true;
-  bool structured = false;  // every type present has the vectored thruster layout
+  // Thruster allocation of the diagonal-mass step (MG_LAYOUT_*): by the geometry and nominal r_b of
+  // the types present, and the one in use, which is the vectored one at most while some env's r_b is
+  // off the z axis (mg_set_params).
+  int type_layout = MG_LAYOUT_DENSE;
+  int layout = MG_LAYOUT_DENSE;
+  bool on_axis = true;          // every env's r_b lies on the body's z axis
+  bool nominal_on_axis = true;  // so do the types' present (randomised r_b stays there)
   bool nominal_diag = true;  // every type has r_g = 0 (randomised M_RB + M_A stays diagonal)
   cudaStream_t stream = nullptr;
   cudaStream_t cap_stream = nullptr;
@@ -350,7 +386,7 @@ mg_status launch_chunks(mg_sim *s, int32_t k, float *traj, cudaStream_t stream) 
   FleetView v = s->view();
   if (s->queue && !traj) {
     v.cursor_adv = k;
-    MG_CK(launch_fleet_queue(v, s->slices_d, s->n_slices, s->ntv, s->diag, s->structured,
+    MG_CK(launch_fleet_queue(v, s->slices_d, s->n_slices, s->ntv, s->diag, s->layout,
                              s->wide, s->queue_warps_per_sm, k, s->spl, s->sched, s->n_sm,
                              stream));
     return MG_OK;
@@ -360,7 +396,7 @@ mg_status launch_chunks(mg_sim *s, int32_t k, float *traj, cudaStream_t stream) 
     float *t = traj ? traj + (int64_t)done * MG_NTRAJ * s->n : nullptr;
     v.cursor_off = done;
     v.cursor_adv = (done + kk == k) ? k : 0;
-    MG_CK(launch_fleet(v, s->blocks_d, s->n_blocks, s->threads, s->ntv, s->diag, s->structured,
+    MG_CK(launch_fleet(v, s->blocks_d, s->n_blocks, s->threads, s->ntv, s->diag, s->layout,
                        s->wide, kk, t, stream));
     done += kk;
   }
@@ -405,12 +441,17 @@ mg_status read_counter(mg_sim *s, int idx, unsigned long long *out) {
   return MG_OK;
 }
 
-// Record the fleet's mass structure and pick the kernel path (see mg_sim::diag).
-void set_mass_diag(mg_sim *s, bool mass_diag) {
+// Record the fleet's mass structure and whether every r_b lies on the z axis, and pick the kernel
+// path (see mg_sim::diag, mg_sim::layout).
+void set_mass_diag(mg_sim *s, bool mass_diag, bool on_axis) {
   s->mass_diag = mass_diag;
+  s->on_axis = on_axis;
   const bool diag = mass_diag && !(s->model_flags & MG_MODEL_NO_CURRENT_ACCEL);
-  if (diag != s->diag) s->drop_graphs();
+  const int layout =
+      on_axis ? s->type_layout : std::min<int>(s->type_layout, MG_LAYOUT_VECTORED);
+  if (diag != s->diag || layout != s->layout) s->drop_graphs();
   s->diag = diag;
+  s->layout = layout;
 }
 
 // After a parameter change: count non-SPD envs and pick the diagonal or general kernel.
@@ -420,7 +461,8 @@ mg_status finish_params(mg_sim *s) {
   MG_CK(cudaMemcpyAsync(&off, s->offdiag, sizeof off, cudaMemcpyDeviceToHost, s->stream));
   mg_status st = read_counter(s, 1, &bad);
   if (st != MG_OK) return st;
-  set_mass_diag(s, (off == 0) && !s->has_xh);  // the extension always takes the general path
+  // the extension always takes the general path
+  set_mass_diag(s, !(off & 1u) && !s->has_xh, !(off & 2u));
   if (bad) {
     char buf[160];
     snprintf(buf, sizeof buf, "%llu envs have a mass matrix that is not positive definite", bad);
@@ -500,7 +542,7 @@ mg_status mg_step_noalloc(mg_sim *s, int32_t k) {
   if (st != MG_OK) return st;
   FleetView v = s->view();
   v.cursor_adv = k;
-  MG_CK(launch_fleet_queue(v, s->slices_d, s->n_slices, s->ntv, s->diag, s->structured,
+  MG_CK(launch_fleet_queue(v, s->slices_d, s->n_slices, s->ntv, s->diag, s->layout,
                            s->wide, s->queue_warps_per_sm, k, s->spl, sched, s->n_sm,
                            s->stream));
   s->cursor += k;
@@ -609,7 +651,7 @@ mg_status mg_create(int64_t n_envs, const int32_t *vehicle_types,
 
   // Per-type geometry and nominal records.
   std::vector<Geo> geo(n_types);
-  s->structured = true;
+  s->type_layout = MG_LAYOUT_MIRRORED;
   std::vector<float> nom((size_t)n_types * MG_NPARAM, 0.f);
   for (int32_t t = 0; t < n_types; ++t) {
     const mg_vehicle_params &v = params[t];
@@ -622,7 +664,8 @@ mg_status mg_create(int64_t n_envs, const int32_t *vehicle_types,
       g.arm[i] = make_float4(r[1] * d[2] - r[2] * d[1], r[2] * d[0] - r[0] * d[2],
                              r[0] * d[1] - r[1] * d[0], 0.f);
     }
-    if (seen[t] && !vectored_layout(g)) s->structured = false;
+    if (seen[t]) s->type_layout = std::min(s->type_layout, thruster_layout(g, v));
+    if (seen[t] && (v.rb[0] != 0.f || v.rb[1] != 0.f)) s->nominal_on_axis = false;
     if (v.rg[0] != 0.f || v.rg[1] != 0.f || v.rg[2] != 0.f) s->nominal_diag = false;
     float *p = &nom[(size_t)t * MG_NPARAM];
     p[MG_P_M] = v.m;
@@ -736,7 +779,7 @@ mg_status mg_set_model_flags(mg_sim *s, uint32_t flags) {
   if (flags & ~MG_MODEL_NO_CURRENT_ACCEL) return fail(MG_EINVAL, "unknown model flag");
   s->model_flags = flags;
   s->drop_graphs();
-  set_mass_diag(s, s->mass_diag);
+  set_mass_diag(s, s->mass_diag, s->on_axis);
   return MG_OK;
 }
 
@@ -878,7 +921,7 @@ mg_status mg_randomize(mg_sim *s, uint64_t seed, const mg_ranges *r) {
   s->reset_seed = seed;
   s->nu0_sigma = (double)r->nu0_sigma;
   if (async) {  // diagonal by construction; a pivot <= 0 is left to mg_sync
-    set_mass_diag(s, true);
+    set_mass_diag(s, true, s->nominal_on_axis);
     return MG_OK;
   }
   return finish_params(s);
@@ -1168,7 +1211,7 @@ mg_status mg_rollout_forward(mg_sim *s, int32_t T, int32_t C, float *traj, float
   v.cursor_off = 0;
   v.cursor_adv = T;
   MG_CK(launch_rollout_forward(v, s->blocks_d, s->n_blocks, s->threads, s->ntv, s->diag,
-                               s->structured, T, C, traj, ckpt, s->stream));
+                               s->layout, T, C, traj, ckpt, s->stream));
   s->cursor += T;
   if (step0_out) *step0_out = step0;
   return MG_OK;
@@ -1283,7 +1326,7 @@ mg_status task_step_outputs(mg_sim *s, int32_t k, float *obs, float *err, float 
   FleetView v = s->view();
   v.cursor_adv = k_last;
   MG_CK(launch_fleet_task(v, s->blocks_d, s->n_blocks, s->threads, s->ntv, s->diag,
-                          s->structured, k_last, k, s->task_view(), to, s->stream));
+                          s->layout, k_last, k, s->task_view(), to, s->stream));
   s->cursor += k_last;
   return MG_OK;
 }
@@ -1482,10 +1525,10 @@ mg_status mg_kernel_info(mg_sim *s, int32_t *regs, int32_t *max_threads, int32_t
   cudaFuncAttributes a;
   int per_sm = 0;
   if (s->queue)
-    MG_CK(queue_kernel_attributes(s->ntv, s->diag, s->wide, s->structured, s->has_xh, &a,
+    MG_CK(queue_kernel_attributes(s->ntv, s->diag, s->wide, s->layout, s->has_xh, &a,
                                   &per_sm));
   else
-    MG_CK(fleet_kernel_attributes(s->ntv, s->diag, s->structured, false, s->wide, &a));
+    MG_CK(fleet_kernel_attributes(s->ntv, s->diag, s->layout, false, s->wide, &a));
   if (regs) *regs = a.numRegs;
   if (max_threads) *max_threads = a.maxThreadsPerBlock;
   if (local_bytes) *local_bytes = (int32_t)a.localSizeBytes;

@@ -200,14 +200,77 @@ __device__ __forceinline__ StepDiag step_diag(const ParDiag &P) {
   return C;
 }
 
+// The same coefficients for a mirrored frame (MG_LAYOUT_MIRRORED below).  The thrusters enter a row
+// only through sums and differences of their forces n|n| in which every member has the same
+// weight, so the weight (a direction or moment arm of the type) is folded into the row's
+// coefficient and the sub-step reads no geometry at all; G lies along z, so four of the six
+// products of G x k_e are gone.
+//   At: mi kT {d_x, d_y of the horizontals, d_z of the verticals};  roll: Kh (horizontals),
+//   Kv (verticals);  pitch: Mh, Mv;  yaw: Nh;  Gr, Gp: mi G_z of the roll and pitch rows.
+struct StepMirrored {
+  float At[3], Wt[3], bp[3], bm[3], dlt[3], dqt[3];
+  float Kh, Kv, Mh, Mv, Nh, B[3], C[3], dlr[3], dqr[3], Gr, Gp;
+  float vc0, vc1, vc2, itau;
+};
+
+// Thruster allocations of the diagonal-mass step (the NH parameter of the kernels).
+//   MG_LAYOUT_DENSE     any geometry: all six rows of every thruster.
+//   MG_LAYOUT_VECTORED  thrusters [0, 4) horizontal (d_z = 0), the rest vertical (d_x = d_y = 0).
+//   MG_LAYOUT_MIRRORED  vectored with 6 or 8 thrusters placed by mirror images (see
+//                       mirrored_layout), and r_b on the body's z axis in every env: the
+//                       horizontals' force and moment rows are d_x (+ + - -), d_y (+ - + -),
+//                       arm_x (+ - + -), arm_y (+ + - -), arm_z (+ - - +) times one magnitude each,
+//                       the verticals' d_z (+ +), arm_x (- + [- +]), arm_y (- - [+ +]; zero with
+//                       two verticals).  Every such frame with the centres on the z axis, which is
+//                       what the vehicles of the experiments are.
+// Vectored against mirrored, CUDA events: 65,536 six-thruster envs x 1,000 sub-steps on the work
+// queue 1.69 -> 1.40 ms; 262,144 mixed envs x 500 on the static grid 3.38 -> 2.85 ms; no spills at
+// 128 registers (vectored: about 100 bytes with six thrusters, 200 with eight), so 65,536-env
+// environment steps of 10 sub-steps 40.7 -> 28.7 us and 30,000 recorded 8-thruster envs x 200
+// 413 -> 283 us.
+enum : int { MG_LAYOUT_DENSE = 0, MG_LAYOUT_VECTORED = 4, MG_LAYOUT_MIRRORED = 5 };
+
+__device__ __forceinline__ StepMirrored step_mirrored(const ParDiag &P, const float4 *gdir,
+                                                      const float4 *garm) {
+  const StepDiag D = step_diag(P);
+  StepMirrored C;
+  const float d[3] = {gdir[0].x, gdir[0].y, gdir[4].z};
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    C.At[i] = D.At[i] * d[i];
+    C.Wt[i] = D.Wt[i];
+    C.bp[i] = D.bp[i];
+    C.bm[i] = D.bm[i];
+    C.dlt[i] = D.dlt[i];
+    C.dqt[i] = D.dqt[i];
+    C.B[i] = D.B[i];
+    C.C[i] = D.C[i];
+    C.dlr[i] = D.dlr[i];
+    C.dqr[i] = D.dqr[i];
+  }
+  C.Kh = D.Ar[0] * garm[0].x;
+  C.Kv = D.Ar[0] * garm[5].x;
+  C.Mh = D.Ar[1] * garm[0].y;
+  C.Mv = -(D.Ar[1] * garm[4].y);
+  C.Nh = D.Ar[2] * garm[0].z;
+  C.Gr = D.Gm[0];
+  C.Gp = D.Gp[1];
+  C.vc0 = D.vc0; C.vc1 = D.vc1; C.vc2 = D.vc2; C.itau = D.itau;
+  return C;
+}
+
 // What the step's right-hand side reads: the diagonal-mass coefficients above, or the general
 // parameters as loaded.
-template <bool DIAG>
-using Coef = typename std::conditional<DIAG, StepDiag, ParGen>::type;
+template <bool DIAG, int NH = MG_LAYOUT_DENSE>
+using Coef = typename std::conditional<
+    DIAG, typename std::conditional<NH == MG_LAYOUT_MIRRORED, StepMirrored, StepDiag>::type,
+    ParGen>::type;
 
-template <bool DIAG>
-__device__ __forceinline__ Coef<DIAG> make_coef(const Par<DIAG> &P) {
-  if constexpr (DIAG) return step_diag(P);
+template <bool DIAG, int NH = MG_LAYOUT_DENSE>
+__device__ __forceinline__ Coef<DIAG, NH> make_coef(const Par<DIAG> &P, const float4 *gdir,
+                                                    const float4 *garm) {
+  if constexpr (DIAG && NH == MG_LAYOUT_MIRRORED) return step_mirrored(P, gdir, garm);
+  else if constexpr (DIAG) return step_diag(P);
   else return P;
 }
 
@@ -286,7 +349,10 @@ __device__ __forceinline__ void store_state(const StatePlanes &sp, int64_t e, co
 // their lag state stays 0), so no warp branches on the count.  NH > 0 selects the vectored layout's
 // allocation: thrusters [0, NH) horizontal (d_z = 0: no heave force), the rest vertical
 // (d_x = d_y = 0, so r x d has no yaw component); the skipped products are exact zeros, so the
-// result is bit-identical to the dense 6 x N allocation (NH = 0).
+// result is bit-identical to the dense 6 x N allocation (NH = 0).  NH = MG_LAYOUT_MIRRORED forms
+// the mirrored frame's sums instead (no geometry read: 13 operations in place of 32 with six
+// thrusters, most of them with two register operands instead of three, and the issue rate of this
+// step is bound by register operand reads).
 //
 // XH (general path only): the env's off-diagonal hydrodynamic coefficients xh[MG_NXPARAM]
 // (M_A above its diagonal, then D_l's off-diagonal entries, both row-major; mg.h) enter the
@@ -294,13 +360,35 @@ __device__ __forceinline__ void store_state(const StatePlanes &sp, int64_t e, co
 // LAGD = false leaves d.n unset (the caller integrates the linear throttle lag in closed form).
 // The diagonal-mass path always includes the current-acceleration term (current_accel unused).
 template <int MT, bool DIAG, bool MIXED, int NH = 0, bool XH = false, bool LAGD = true>
-__device__ __forceinline__ void rhs(const St<MT> &s, const float (&cs)[MT], const Coef<DIAG> &P,
+__device__ __forceinline__ void rhs(const St<MT> &s, const float (&cs)[MT], const Coef<DIAG, NH> &P,
                                     const float4 *gdir, const float4 *garm, int nt,
                                     bool current_accel, St<MT> &d,
                                     const float *__restrict__ xh = nullptr) {
   static_assert(!(XH && DIAG), "the off-diagonal hydrodynamics use the general path");
   // Thrusters (Eq. 3 actions): F_i = kT n_i|n_i| along d_i at r_i; n_i' = (c_i - n_i) / tau_m.
+  constexpr bool MIRRORED = DIAG && NH == MG_LAYOUT_MIRRORED;
   float t0 = 0.f, t1 = 0.f, t2 = 0.f, t3 = 0.f, t4 = 0.f, t5 = 0.f;
+  if constexpr (MIRRORED) {
+    auto f = [&](int i) { return s.n[i] * fabsf(s.n[i]); };
+    auto add = [&](int i, float x) { return fmaf(s.n[i], fabsf(s.n[i]), x); };
+    const float f3 = f(3), f2 = f(2), f4 = f(4);
+    const float s03 = add(0, f3), d03 = add(0, -f3), s12 = add(1, f2), d12 = add(1, -f2);
+    t0 = d03 + d12;   // surge
+    t1 = d03 - d12;   // sway, and the horizontals' roll and pitch by t1 and t0
+    t5 = s03 - s12;   // yaw
+    t2 = add(5, f4);  // heave
+    t3 = add(5, -f4);  // the verticals' roll
+    if constexpr (MT > 6) {
+      const float f6 = f(6), s67 = add(7, f6);
+      t4 = s67 - t2;  // the verticals' pitch
+      t2 += s67;
+      t3 += add(7, -f6);
+    }
+    if constexpr (LAGD) {
+#pragma unroll
+      for (int i = 0; i < MT; ++i) d.n[i] = fmaf(-s.n[i], P.itau, cs[i]);
+    }
+  } else
 #pragma unroll
   for (int i = 0; i < MT; ++i) {
     {
@@ -358,9 +446,18 @@ __device__ __forceinline__ void rhs(const St<MT> &s, const float (&cs)[MT], cons
     }
     // Rotational rows: thrust moment, G x k_e, Munk and gyroscopic products, damping.
     {
-      float b0 = fmaf(-P.Gm[0], R21, fmaf(P.Gp[0], R22, P.Ar[0] * t3));
-      float b1 = fmaf(-P.Gm[1], R22, fmaf(P.Gp[1], R20, P.Ar[1] * t4));
-      float b2 = fmaf(-P.Gm[2], R20, fmaf(P.Gp[2], R21, P.Ar[2] * t5));
+      float b0, b1, b2;
+      if constexpr (MIRRORED) {
+        b0 = fmaf(-P.Gr, R21, fmaf(P.Kv, t3, P.Kh * t1));
+        b1 = P.Mh * t0;
+        if constexpr (MT > 6) b1 = fmaf(P.Mv, t4, b1);
+        b1 = fmaf(P.Gp, R20, b1);
+        b2 = P.Nh * t5;
+      } else {
+        b0 = fmaf(-P.Gm[0], R21, fmaf(P.Gp[0], R22, P.Ar[0] * t3));
+        b1 = fmaf(-P.Gm[1], R22, fmaf(P.Gp[1], R20, P.Ar[1] * t4));
+        b2 = fmaf(-P.Gm[2], R20, fmaf(P.Gp[2], R21, P.Ar[2] * t5));
+      }
       b0 = fmaf(P.C[0] * w1, w2, fmaf(P.B[0] * r1, r2, b0));
       b1 = fmaf(P.C[1] * w2, w0, fmaf(P.B[1] * r2, r0, b1));
       b2 = fmaf(P.C[2] * w0, w1, fmaf(P.B[2] * r0, r1, b2));
@@ -533,7 +630,7 @@ __device__ __forceinline__ void lag_segment(const float (&cs)[MT], const LagEnv 
 // One sub-step (§METHOD): classical RK4 of size h, command held (cs = c / tau_m), then
 // q <- q / |q|.
 template <int MT, bool DIAG, bool MIXED, int NH = 0, bool XH = false>
-__device__ __forceinline__ void rk4_step(St<MT> &s, const float (&cs)[MT], const Coef<DIAG> &P,
+__device__ __forceinline__ void rk4_step(St<MT> &s, const float (&cs)[MT], const Coef<DIAG, NH> &P,
                                          const float4 *gdir, const float4 *garm, int nt,
                                          bool current_accel, float h,
                                          const float *__restrict__ xh = nullptr) {
@@ -561,7 +658,7 @@ __device__ __forceinline__ void rk4_step(St<MT> &s, const float (&cs)[MT], const
 // the lag state.
 template <int MT, bool DIAG, bool MIXED, int NH = 0, bool XH = false>
 __device__ __forceinline__ void rk4_step_lag(St<MT> &s, const float (&b)[MT], const LagEnv &L,
-                                             const Coef<DIAG> &P, const float4 *gdir,
+                                             const Coef<DIAG, NH> &P, const float4 *gdir,
                                              const float4 *garm, int nt, bool current_accel,
                                              float h, const float *__restrict__ xh = nullptr) {
   const float hh = 0.5f * h, h3 = h * (1.0f / 3.0f), h6 = h * (1.0f / 6.0f);

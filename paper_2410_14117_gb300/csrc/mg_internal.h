@@ -112,13 +112,13 @@ enum NtVariant { NT_6 = 0, NT_8 = 1, NT_MIXED = 2 };
 
 // ---------------------------------------------------------------- launchers (mg_step.cu)
 // Static schedule: one block per BlockDesc, k sub-steps per launch.
-// structured: every vehicle type present has the vectored layout (thrusters 0..3 with d_z = 0,
-// the rest with d_x = d_y = 0), so the allocation skips its exact zeros (diagonal mass only).
+// layout: MG_LAYOUT_* (mg_device.cuh), the thruster allocation of the diagonal-mass step: the
+// fastest one that every vehicle type present has.
 // wide: the diagonal-mass kernel without recording gets 200 registers instead of 128.
 cudaError_t launch_fleet(const FleetView &fv, const BlockDesc *blocks, int n_blocks, int threads,
-                         NtVariant ntv, bool diag, bool structured, bool wide, int32_t k,
+                         NtVariant ntv, bool diag, int layout, bool wide, int32_t k,
                          float *traj, cudaStream_t stream);
-cudaError_t fleet_kernel_attributes(NtVariant ntv, bool diag, bool structured, bool record,
+cudaError_t fleet_kernel_attributes(NtVariant ntv, bool diag, int layout, bool record,
                                     bool wide, cudaFuncAttributes *attr);
 
 // Work-queue schedule: warps claim (32-env slice, chunk of sub-steps) units in chunk-major
@@ -130,15 +130,18 @@ size_t queue_sched_bytes(int n_slices);
 // wide: 200-register variant of the diagonal-mass step (fewer resident warps, more registers
 // each); warps_per_sm > 0 caps the resident warps per SM.
 cudaError_t launch_fleet_queue(const FleetView &fv, const BlockDesc *slices, int n_slices,
-                               NtVariant ntv, bool diag, bool structured, bool wide,
+                               NtVariant ntv, bool diag, int layout, bool wide,
                                int warps_per_sm, int32_t k, int32_t chunk, uint32_t *sched,
                                int n_sm, cudaStream_t stream);
 // xh: the general path's off-diagonal-hydrodynamics variant.
-cudaError_t queue_kernel_attributes(NtVariant ntv, bool diag, bool wide, bool structured,
+cudaError_t queue_kernel_attributes(NtVariant ntv, bool diag, bool wide, int layout,
                                     bool xh, cudaFuncAttributes *attr, int *blocks_per_sm);
 
 // True when thrusters [0, 4) of the geometry have d_z = 0 and the rest d_x = d_y = 0.
 bool vectored_layout(const Geo &g);
+// The fastest MG_LAYOUT_* that vehicle type v with geometry g has (mirrored asks for r_b on the
+// z axis too).
+int thruster_layout(const Geo &g, const mg_vehicle_params &v);
 
 // ---------------------------------------------------------------- launchers (mg_setup.cu)
 struct SetupView {
@@ -148,7 +151,7 @@ struct SetupView {
   float *raw;                // device [n][MG_NPARAM] (the record layout of mg.h)
   ParamPlanes pa;
   unsigned long long *n_not_spd;
-  unsigned int *any_offdiag;
+  unsigned int *any_offdiag;  // bit 0: some mass matrix is full; bit 1: some r_b is off the z axis
   const float *xh;           // device [MG_NXPARAM][xh_stride] off-diagonal hydrodynamics, or null
   int64_t xh_stride;         // floats between xh's component planes (0: n)
 };
@@ -188,7 +191,7 @@ cudaError_t launch_checkpoint(const StatePlanes &st, int64_t n, float *ck, cudaS
 // The rollout's forward in one launch on the static grid (mg_adjoint.cu): T sub-steps, ckpt
 // [ceil(T / C)][MG_NSTATE][n] before sub-steps 0, C, ..., traj [T][MG_NTRAJ][n] after each.
 cudaError_t launch_rollout_forward(const FleetView &fv, const BlockDesc *blocks, int n_blocks,
-                                   int threads, NtVariant ntv, bool diag, bool structured,
+                                   int threads, NtVariant ntv, bool diag, int layout,
                                    int32_t T, int32_t C, float *traj, float *ckpt,
                                    cudaStream_t stream);
 // Backward kernel: mode 1 one warp per 32 envs, 2 the two-warp form (producer and consumer warps
@@ -236,7 +239,7 @@ struct TaskOut {
 // Final launch of a task step: k_launch sub-steps (static grid), then the task epilogue for a
 // task step of k_task sub-steps in total.
 cudaError_t launch_fleet_task(const FleetView &fv, const BlockDesc *blocks, int n_blocks,
-                              int threads, NtVariant ntv, bool diag, bool structured,
+                              int threads, NtVariant ntv, bool diag, int layout,
                               int32_t k_launch, int32_t k_task, const TaskView &tv, TaskOut to,
                               cudaStream_t stream);
 

@@ -80,11 +80,11 @@ __global__ void __maxnreg__(XH ? kRegsXH : !DIAG ? kRegsGeneral : WIDE ? kRegsWi
 
   St<MT> s;
   load_state<MT>(fv.st, e, s);
-  Coef<DIAG> P;
+  Coef<DIAG, NH> P;
   {
     Par<DIAG> raw;
     load_par<DIAG>(fv.pa, e, raw);
-    P = make_coef<DIAG>(raw);
+    P = make_coef<DIAG, NH>(raw, sdir, sarm);
   }
   int64_t seg = jd.step0 / jd.hold;
   int32_t left = jd.hold - (int32_t)(jd.step0 - seg * jd.hold);
@@ -117,6 +117,25 @@ __global__ void __maxnreg__(XH ? kRegsXH : !DIAG ? kRegsGeneral : WIDE ? kRegsWi
     }
   }
   store_state<MT>(fv.st, e, s);
+}
+
+template <int NH>
+void launch_serve(bool wide, int grid, const FleetView &v, const JobDesc *jobs,
+                  const ServeBlock *blocks, cudaStream_t stream) {
+  if (wide)
+    k_serve<true, NH, true><<<grid, kServeThreads, 0, stream>>>(v, jobs, blocks);
+  else
+    k_serve<true, NH><<<grid, kServeThreads, 0, stream>>>(v, jobs, blocks);
+}
+
+void launch_serve_diag(int layout, bool wide, int grid, const FleetView &v, const JobDesc *jobs,
+                       const ServeBlock *blocks, cudaStream_t stream) {
+  if (layout == MG_LAYOUT_MIRRORED)
+    launch_serve<MG_LAYOUT_MIRRORED>(wide, grid, v, jobs, blocks, stream);
+  else if (layout == MG_LAYOUT_VECTORED)
+    launch_serve<MG_LAYOUT_VECTORED>(wide, grid, v, jobs, blocks, stream);
+  else
+    launch_serve<MG_LAYOUT_DENSE>(wide, grid, v, jobs, blocks, stream);
 }
 
 __global__ void k_fill_i32(int32_t *p, int64_t n, int32_t v) {
@@ -180,7 +199,7 @@ struct mg_pool {
   int32_t n_types = 0;
   std::vector<mg_vehicle_params> vp;
   bool diag = true;
-  bool structured = true;  // every vehicle type has the vectored thruster layout
+  int layout = MG_LAYOUT_MIRRORED;  // the fastest one that every vehicle type has
   cudaStream_t stream = nullptr;
   void *arena = nullptr;
   StatePlanes st{};
@@ -350,7 +369,7 @@ mg_status mg_pool_create(int64_t capacity_envs, const mg_vehicle_params *params,
       g.arm[i] = make_float4(r[1] * d[2] - r[2] * d[1], r[2] * d[0] - r[0] * d[2],
                              r[0] * d[1] - r[1] * d[0], 0.f);
     }
-    if (!vectored_layout(g)) p->structured = false;
+    p->layout = std::min(p->layout, thruster_layout(g, v));
     float *q = &nom[(size_t)t * MG_NPARAM];
     q[MG_P_M] = v.m;
     q[MG_P_IG] = v.Ixx;
@@ -591,14 +610,8 @@ mg_status mg_pool_tick(mg_pool *p, int32_t k, int32_t *n_running) {
   const bool wide = g <= 2 * p->n_sm;
   if (g == 0)
     ;
-  else if (p->diag && p->structured && wide)
-    k_serve<true, 4, true><<<g, kServeThreads, 0, p->stream>>>(v, jt, bl);
-  else if (p->diag && p->structured)
-    k_serve<true, 4><<<g, kServeThreads, 0, p->stream>>>(v, jt, bl);
-  else if (p->diag && wide)
-    k_serve<true, 0, true><<<g, kServeThreads, 0, p->stream>>>(v, jt, bl);
   else if (p->diag)
-    k_serve<true, 0><<<g, kServeThreads, 0, p->stream>>>(v, jt, bl);
+    launch_serve_diag(p->layout, wide, g, v, jt, bl, p->stream);
   else
     k_serve<false, 0><<<g, kServeThreads, 0, p->stream>>>(v, jt, bl);
   PK(cudaGetLastError());

@@ -35,6 +35,11 @@ constexpr int kRandThreads = 128;
 // that one block fits beside a step kernel's resident blocks on every SM.
 constexpr int kRandBgThreads = 64;
 
+// Tell the host of an r_b off the body's z axis (the mirrored thruster allocation needs it on it).
+__device__ __forceinline__ void note_off_axis(const SetupView &v, const double *p) {
+  if (p[MG_P_RB] != 0.0 || p[MG_P_RB + 1] != 0.0) atomicOr(v.any_offdiag, 2u);
+}
+
 // derive() for an env whose mass matrix is diagonal (r_g = 0, no off-diagonal added mass): the
 // same values derive() stores, without building the 6 x 6 matrices (FP64 runs at a 64th of the
 // FP32 rate on this GPU).  I_o = I_g exactly and every off-diagonal entry is +0 when r_g = 0.
@@ -53,6 +58,7 @@ __device__ void derive_diag(const SetupView &v, int64_t e, const double *p) {
     mi[j] = Mjj[j] > 0.0 ? 1.0 / Mjj[j] : 0.0;
   }
   if (!spd) atomicAdd(v.n_not_spd, 1ull);
+  note_off_axis(v, p);
   const double W = p[MG_P_W], B = p[MG_P_B];
   const double G[3] = {W * rg[0] - B * p[MG_P_RB], W * rg[1] - B * p[MG_P_RB + 1],
                        W * rg[2] - B * p[MG_P_RB + 2]};
@@ -166,6 +172,7 @@ __device__ void derive(const SetupView &v, int64_t e, const double *p) {
     }
   if (!spd) atomicAdd(v.n_not_spd, 1ull);
   if (!diagonal) atomicOr(v.any_offdiag, 1u);
+  note_off_axis(v, p);
 
   const double W = p[MG_P_W], B = p[MG_P_B];
   const double G[3] = {W * rg[0] - B * p[MG_P_RB], W * rg[1] - B * p[MG_P_RB + 1],

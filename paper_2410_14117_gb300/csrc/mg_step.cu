@@ -163,76 +163,93 @@ cudaError_t launch_pdl(Kernel kernel, int n_blocks, int threads, size_t smem, cu
   return cudaLaunchKernelEx(&cfg, kernel, fv, blocks, k, traj);
 }
 
-// Structured allocation (NH = 4) is only instantiated for the diagonal-mass step, the
+// The vectored and mirrored allocations are only instantiated for the diagonal-mass step, the
 // off-diagonal hydrodynamics (XH) only for the general one, the wide register budget only for
 // the diagonal-mass step without recording.
 template <int NTV, bool DIAG, bool REC, bool WIDE>
 cudaError_t launch_t(const FleetView &fv, const BlockDesc *blocks, int n_blocks, int threads,
-                     bool structured, int32_t k, float *traj, cudaStream_t stream) {
+                     int layout, int32_t k, float *traj, cudaStream_t stream) {
   if constexpr (!DIAG) if (fv.xh)
     return launch_pdl(k_fleet<NTV, false, REC, 0, true>, n_blocks, threads,
                       sizeof(float) * MG_NXPARAM * threads, stream, fv, blocks, k, traj);
-  if (DIAG && structured)
-    return launch_pdl(k_fleet<NTV, DIAG, REC, (DIAG ? 4 : 0), false, WIDE>, n_blocks, threads,
-                      0, stream, fv, blocks, k, traj);
+  if constexpr (DIAG) {
+    if (layout == MG_LAYOUT_MIRRORED)
+      return launch_pdl(k_fleet<NTV, true, REC, MG_LAYOUT_MIRRORED, false, WIDE>, n_blocks, threads,
+                        0, stream, fv, blocks, k, traj);
+    if (layout == MG_LAYOUT_VECTORED)
+      return launch_pdl(k_fleet<NTV, true, REC, MG_LAYOUT_VECTORED, false, WIDE>, n_blocks, threads,
+                        0, stream, fv, blocks, k, traj);
+  }
   return launch_pdl(k_fleet<NTV, DIAG, REC, 0, false, WIDE>, n_blocks, threads, 0, stream, fv,
                     blocks, k, traj);
 }
 
 template <int NTV, bool DIAG>
 cudaError_t launch_r(const FleetView &fv, const BlockDesc *blocks, int n_blocks, int threads,
-                     bool structured, bool wide, int32_t k, float *traj, cudaStream_t stream) {
+                     int layout, bool wide, int32_t k, float *traj, cudaStream_t stream) {
   if (traj)
-    return launch_t<NTV, DIAG, true, false>(fv, blocks, n_blocks, threads, structured, k, traj,
+    return launch_t<NTV, DIAG, true, false>(fv, blocks, n_blocks, threads, layout, k, traj,
                                             stream);
   if constexpr (DIAG)
     if (wide)
-      return launch_t<NTV, true, false, true>(fv, blocks, n_blocks, threads, structured, k,
+      return launch_t<NTV, true, false, true>(fv, blocks, n_blocks, threads, layout, k,
                                               traj, stream);
-  return launch_t<NTV, DIAG, false, false>(fv, blocks, n_blocks, threads, structured, k, traj,
+  return launch_t<NTV, DIAG, false, false>(fv, blocks, n_blocks, threads, layout, k, traj,
                                            stream);
 }
 
 template <int NTV>
 cudaError_t launch_d(const FleetView &fv, const BlockDesc *blocks, int n_blocks, int threads,
-                     bool diag, bool structured, bool wide, int32_t k, float *traj,
+                     bool diag, int layout, bool wide, int32_t k, float *traj,
                      cudaStream_t stream) {
-  return diag ? launch_r<NTV, true>(fv, blocks, n_blocks, threads, structured, wide, k, traj,
+  return diag ? launch_r<NTV, true>(fv, blocks, n_blocks, threads, layout, wide, k, traj,
                                     stream)
-              : launch_r<NTV, false>(fv, blocks, n_blocks, threads, structured, wide, k, traj,
+              : launch_r<NTV, false>(fv, blocks, n_blocks, threads, layout, wide, k, traj,
                                      stream);
 }
 
 template <int NTV, bool DIAG, bool REC, bool WIDE = false>
-const void *kernel_ptr(bool structured) {
-  if (DIAG && structured)
-    return reinterpret_cast<const void *>(&k_fleet<NTV, DIAG, REC, (DIAG ? 4 : 0), false, WIDE>);
+const void *kernel_ptr(int layout) {
+  if constexpr (DIAG) {
+    if (layout == MG_LAYOUT_MIRRORED)
+      return reinterpret_cast<const void *>(
+          &k_fleet<NTV, true, REC, MG_LAYOUT_MIRRORED, false, WIDE>);
+    if (layout == MG_LAYOUT_VECTORED)
+      return reinterpret_cast<const void *>(
+          &k_fleet<NTV, true, REC, MG_LAYOUT_VECTORED, false, WIDE>);
+  }
   return reinterpret_cast<const void *>(&k_fleet<NTV, DIAG, REC, 0, false, WIDE>);
 }
 
 template <int NTV, bool DIAG>
-const void *queue_ptr(bool wide, bool structured, bool xh) {
+const void *queue_ptr(bool wide, int layout, bool xh) {
   constexpr int S = DIAG ? 4 : 0;
   if constexpr (!DIAG)
     if (xh) return reinterpret_cast<const void *>(&k_fleet_queue<NTV, false, false, 0, true>);
-  if (DIAG && structured)
-    return wide ? reinterpret_cast<const void *>(&k_fleet_queue<NTV, DIAG, true, S>)
-                : reinterpret_cast<const void *>(&k_fleet_queue<NTV, DIAG, false, S>);
+  if constexpr (DIAG) {
+    constexpr int M = MG_LAYOUT_MIRRORED, V = MG_LAYOUT_VECTORED;
+    if (layout == M)
+      return wide ? reinterpret_cast<const void *>(&k_fleet_queue<NTV, true, true, M>)
+                  : reinterpret_cast<const void *>(&k_fleet_queue<NTV, true, false, M>);
+    if (layout == V)
+      return wide ? reinterpret_cast<const void *>(&k_fleet_queue<NTV, true, true, V>)
+                  : reinterpret_cast<const void *>(&k_fleet_queue<NTV, true, false, V>);
+  }
   return wide ? reinterpret_cast<const void *>(&k_fleet_queue<NTV, DIAG, true, 0>)
               : reinterpret_cast<const void *>(&k_fleet_queue<NTV, DIAG, false, 0>);
 }
 
-const void *queue_kernel(NtVariant ntv, bool diag, bool wide, bool structured, bool xh) {
+const void *queue_kernel(NtVariant ntv, bool diag, bool wide, int layout, bool xh) {
   switch (ntv) {
     case NT_6:
-      return diag ? queue_ptr<NT_6, true>(wide, structured, false)
-                  : queue_ptr<NT_6, false>(wide, false, xh);
+      return diag ? queue_ptr<NT_6, true>(wide, layout, false)
+                  : queue_ptr<NT_6, false>(wide, MG_LAYOUT_DENSE, xh);
     case NT_8:
-      return diag ? queue_ptr<NT_8, true>(wide, structured, false)
-                  : queue_ptr<NT_8, false>(wide, false, xh);
+      return diag ? queue_ptr<NT_8, true>(wide, layout, false)
+                  : queue_ptr<NT_8, false>(wide, MG_LAYOUT_DENSE, xh);
     default:
-      return diag ? queue_ptr<NT_MIXED, true>(wide, structured, false)
-                  : queue_ptr<NT_MIXED, false>(wide, false, xh);
+      return diag ? queue_ptr<NT_MIXED, true>(wide, layout, false)
+                  : queue_ptr<NT_MIXED, false>(wide, MG_LAYOUT_DENSE, xh);
   }
 }
 
@@ -240,64 +257,100 @@ const void *queue_kernel(NtVariant ntv, bool diag, bool wide, bool structured, b
 constexpr size_t kQueueXhBytes = sizeof(float) * kQueueWarps * 32 * MG_NXPARAM;
 
 template <int NTV, bool DIAG, int NH>
-void queue_launch_w(bool wide, int grid, const FleetView &fv, const BlockDesc *slices,
+void queue_launch_w(bool wide, int grid, size_t smem, const FleetView &fv, const BlockDesc *slices,
                     int32_t n_slices, int32_t k, int32_t chunk, uint32_t *sched,
                     cudaStream_t stream) {
   if constexpr (!DIAG)
     if (fv.xh) {
-      k_fleet_queue<NTV, false, false, 0, true><<<grid, kQueueWarps * 32, kQueueXhBytes, stream>>>(
+      k_fleet_queue<NTV, false, false, 0, true><<<grid, kQueueWarps * 32, smem, stream>>>(
           fv, slices, n_slices, k, chunk, sched);
       return;
     }
   if (wide)
-    k_fleet_queue<NTV, DIAG, true, NH><<<grid, kQueueWarps * 32, 0, stream>>>(
+    k_fleet_queue<NTV, DIAG, true, NH><<<grid, kQueueWarps * 32, smem, stream>>>(
         fv, slices, n_slices, k, chunk, sched);
   else
-    k_fleet_queue<NTV, DIAG, false, NH><<<grid, kQueueWarps * 32, 0, stream>>>(
+    k_fleet_queue<NTV, DIAG, false, NH><<<grid, kQueueWarps * 32, smem, stream>>>(
         fv, slices, n_slices, k, chunk, sched);
 }
 
+// Dynamic shared memory (at least `need`) that lets per_sm blocks of kernel f onto an SM and no
+// more: the warps_per_sm cap would otherwise only size the grid, and where more blocks fit, a
+// kernel on another stream (the background draw of mg_randomize_prefetch) makes the hardware
+// place three of them on some SMs and one on others.  65,536 six-thruster envs x 1,000 sub-steps
+// with the next episode's draw beside them, 8 warps per SM: 1,840 us without, 1,510 with
+// (1,400 for the steps alone).
+cudaError_t queue_even_smem(const void *f, const cudaFuncAttributes &attr, int per_sm,
+                            size_t need, size_t *smem) {
+  *smem = need;
+  int dev = 0, per_sm_bytes = 0, per_block = 0, reserved = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess)
+    e = cudaDeviceGetAttribute(&per_sm_bytes, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
+  if (e == cudaSuccess)
+    e = cudaDeviceGetAttribute(&per_block, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  if (e == cudaSuccess)
+    e = cudaDeviceGetAttribute(&reserved, cudaDevAttrReservedSharedMemoryPerBlock, dev);
+  if (e != cudaSuccess) return e;
+  const size_t fixed = attr.sharedSizeBytes + (size_t)reserved;
+  // a block's share when per_sm + 1 of them would just not fit
+  const size_t share = (size_t)per_sm_bytes / (per_sm + 1) + 1024;
+  if (share < fixed + need || share * per_sm > (size_t)per_sm_bytes ||
+      share - reserved > (size_t)per_block)
+    return cudaSuccess;
+  *smem = share - fixed;
+  // the same limit whatever the cap: it belongs to the function, which other sims launch too
+  return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              per_block - (int)attr.sharedSizeBytes);
+}
+
 template <int NTV>
-void queue_launch(bool diag, bool wide, bool structured, int grid, const FleetView &fv,
+void queue_launch(bool diag, bool wide, int layout, int grid, size_t smem, const FleetView &fv,
                   const BlockDesc *slices, int32_t n_slices, int32_t k, int32_t chunk,
                   uint32_t *sched, cudaStream_t stream) {
-  if (diag && structured)
-    queue_launch_w<NTV, true, 4>(wide, grid, fv, slices, n_slices, k, chunk, sched, stream);
+  if (diag && layout == MG_LAYOUT_MIRRORED)
+    queue_launch_w<NTV, true, MG_LAYOUT_MIRRORED>(wide, grid, smem, fv, slices, n_slices, k, chunk,
+                                                  sched, stream);
+  else if (diag && layout == MG_LAYOUT_VECTORED)
+    queue_launch_w<NTV, true, MG_LAYOUT_VECTORED>(wide, grid, smem, fv, slices, n_slices, k, chunk,
+                                                  sched, stream);
   else if (diag)
-    queue_launch_w<NTV, true, 0>(wide, grid, fv, slices, n_slices, k, chunk, sched, stream);
+    queue_launch_w<NTV, true, MG_LAYOUT_DENSE>(wide, grid, smem, fv, slices, n_slices, k, chunk, sched,
+                                               stream);
   else
-    queue_launch_w<NTV, false, 0>(wide, grid, fv, slices, n_slices, k, chunk, sched, stream);
+    queue_launch_w<NTV, false, 0>(wide, grid, smem, fv, slices, n_slices, k, chunk, sched,
+                                               stream);
 }
 
 }  // namespace
 
 cudaError_t launch_fleet(const FleetView &fv, const BlockDesc *blocks, int n_blocks, int threads,
-                         NtVariant ntv, bool diag, bool structured, bool wide, int32_t k,
+                         NtVariant ntv, bool diag, int layout, bool wide, int32_t k,
                          float *traj, cudaStream_t stream) {
   if (threads < 32 || threads > kMaxThreads || threads % 32 || n_blocks < 1 || k < 1 ||
       (fv.xh && diag))
     return cudaErrorInvalidValue;
   switch (ntv) {
     case NT_6:
-      return launch_d<NT_6>(fv, blocks, n_blocks, threads, diag, structured, wide, k, traj,
+      return launch_d<NT_6>(fv, blocks, n_blocks, threads, diag, layout, wide, k, traj,
                             stream);
     case NT_8:
-      return launch_d<NT_8>(fv, blocks, n_blocks, threads, diag, structured, wide, k, traj,
+      return launch_d<NT_8>(fv, blocks, n_blocks, threads, diag, layout, wide, k, traj,
                             stream);
     default:
-      return launch_d<NT_MIXED>(fv, blocks, n_blocks, threads, diag, structured, wide, k, traj,
+      return launch_d<NT_MIXED>(fv, blocks, n_blocks, threads, diag, layout, wide, k, traj,
                                 stream);
   }
 }
 
-cudaError_t fleet_kernel_attributes(NtVariant ntv, bool diag, bool structured, bool rec,
+cudaError_t fleet_kernel_attributes(NtVariant ntv, bool diag, int layout, bool rec,
                                     bool wide, cudaFuncAttributes *attr) {
   const void *f = nullptr;
 #define MG_PICK(N)                                                                      \
-  f = diag ? (rec ? kernel_ptr<N, true, true>(structured)                               \
-                  : wide ? kernel_ptr<N, true, false, true>(structured)                 \
-                         : kernel_ptr<N, true, false>(structured))                      \
-           : (rec ? kernel_ptr<N, false, true>(false) : kernel_ptr<N, false, false>(false));
+  f = diag ? (rec ? kernel_ptr<N, true, true>(layout)                               \
+                  : wide ? kernel_ptr<N, true, false, true>(layout)                 \
+                         : kernel_ptr<N, true, false>(layout))                      \
+           : (rec ? kernel_ptr<N, false, true>(0) : kernel_ptr<N, false, false>(0));
   switch (ntv) {
     case NT_6: MG_PICK(NT_6) break;
     case NT_8: MG_PICK(NT_8) break;
@@ -309,10 +362,10 @@ cudaError_t fleet_kernel_attributes(NtVariant ntv, bool diag, bool structured, b
 
 size_t queue_sched_bytes(int n_slices) { return 16 + 4 * (size_t)n_slices; }
 
-cudaError_t queue_kernel_attributes(NtVariant ntv, bool diag, bool wide, bool structured,
+cudaError_t queue_kernel_attributes(NtVariant ntv, bool diag, bool wide, int layout,
                                     bool xh, cudaFuncAttributes *attr, int *blocks_per_sm) {
   xh = xh && !diag;
-  const void *f = queue_kernel(ntv, diag, wide, structured, xh);
+  const void *f = queue_kernel(ntv, diag, wide, layout, xh);
   cudaError_t e = cudaFuncGetAttributes(attr, f);
   if (e != cudaSuccess) return e;
   return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, f, kQueueWarps * 32,
@@ -320,20 +373,27 @@ cudaError_t queue_kernel_attributes(NtVariant ntv, bool diag, bool wide, bool st
 }
 
 cudaError_t launch_fleet_queue(const FleetView &fv, const BlockDesc *slices, int n_slices,
-                               NtVariant ntv, bool diag, bool structured, bool wide,
+                               NtVariant ntv, bool diag, int layout, bool wide,
                                int warps_per_sm, int32_t k, int32_t chunk, uint32_t *sched,
                                int n_sm, cudaStream_t stream) {
   if (n_slices < 1 || k < 1 || chunk < 1 || n_sm < 1 || (fv.xh && diag))
     return cudaErrorInvalidValue;
   cudaFuncAttributes attr;
   int per_sm = 0;
-  cudaError_t e = queue_kernel_attributes(ntv, diag, wide, structured, fv.xh != nullptr, &attr,
+  cudaError_t e = queue_kernel_attributes(ntv, diag, wide, layout, fv.xh != nullptr, &attr,
                                           &per_sm);
   if (e != cudaSuccess) return e;
   if (per_sm < 1) per_sm = 1;
   // Resident warps: at most what fits (and at most warps_per_sm per SM when that is > 0), and no
   // more than there are slices in a chunk.
-  if (warps_per_sm > 0) per_sm = std::max(1, std::min(per_sm, warps_per_sm / kQueueWarps));
+  size_t smem = fv.xh ? kQueueXhBytes : 0;
+  const int cap = std::max(1, warps_per_sm / kQueueWarps);
+  if (warps_per_sm > 0 && cap < per_sm) {
+    per_sm = cap;
+    e = queue_even_smem(queue_kernel(ntv, diag, wide, layout, fv.xh != nullptr), attr, per_sm, smem,
+                        &smem);
+    if (e != cudaSuccess) return e;
+  }
   int grid = per_sm * n_sm;
   const int need = (n_slices + kQueueWarps - 1) / kQueueWarps;
   if (grid > need) grid = need;
@@ -350,15 +410,15 @@ cudaError_t launch_fleet_queue(const FleetView &fv, const BlockDesc *slices, int
     piece.cursor_adv = (done + kk == k) ? fv.cursor_adv : 0;
     switch (ntv) {
       case NT_6:
-        queue_launch<NT_6>(diag, wide, structured, grid, piece, slices, n_slices, kk, chunk,
+        queue_launch<NT_6>(diag, wide, layout, grid, smem, piece, slices, n_slices, kk, chunk,
                            sched, stream);
         break;
       case NT_8:
-        queue_launch<NT_8>(diag, wide, structured, grid, piece, slices, n_slices, kk, chunk,
+        queue_launch<NT_8>(diag, wide, layout, grid, smem, piece, slices, n_slices, kk, chunk,
                            sched, stream);
         break;
       default:
-        queue_launch<NT_MIXED>(diag, wide, structured, grid, piece, slices, n_slices, kk, chunk,
+        queue_launch<NT_MIXED>(diag, wide, layout, grid, smem, piece, slices, n_slices, kk, chunk,
                                sched, stream);
         break;
     }

@@ -323,15 +323,18 @@ cudaError_t fleet_task_t(const FleetView &fv, const BlockDesc *blocks, int n_blo
 
 template <int NTV>
 cudaError_t fleet_task_d(const FleetView &fv, const BlockDesc *blocks, int n_blocks, int threads,
-                         bool diag, bool structured, int32_t k_launch, int32_t k_task,
+                         bool diag, int layout, int32_t k_launch, int32_t k_task,
                          const TaskView &tv, const TaskOut &to, size_t smem,
                          cudaStream_t stream) {
   if (fv.xh)
     return fleet_task_t<NTV, false, 0, true>(fv, blocks, n_blocks, threads, k_launch, k_task, tv,
                                              to, smem, stream);
-  if (diag && structured)
-    return fleet_task_t<NTV, true, 4>(fv, blocks, n_blocks, threads, k_launch, k_task, tv, to,
-                                      smem, stream);
+  if (diag && layout == MG_LAYOUT_MIRRORED)
+    return fleet_task_t<NTV, true, MG_LAYOUT_MIRRORED>(fv, blocks, n_blocks, threads, k_launch,
+                                                       k_task, tv, to, smem, stream);
+  if (diag && layout == MG_LAYOUT_VECTORED)
+    return fleet_task_t<NTV, true, MG_LAYOUT_VECTORED>(fv, blocks, n_blocks, threads, k_launch,
+                                                       k_task, tv, to, smem, stream);
   if (diag)
     return fleet_task_t<NTV, true, 0>(fv, blocks, n_blocks, threads, k_launch, k_task, tv, to,
                                       smem, stream);
@@ -379,7 +382,7 @@ cudaError_t launch_task(const StatePlanes &st, const TaskView &tv, int64_t n, in
 }
 
 cudaError_t launch_fleet_task(const FleetView &fv, const BlockDesc *blocks, int n_blocks,
-                              int threads, NtVariant ntv, bool diag, bool structured,
+                              int threads, NtVariant ntv, bool diag, int layout,
                               int32_t k_launch, int32_t k_task, const TaskView &tv, TaskOut to,
                               cudaStream_t stream) {
   if (threads < 32 || threads > 256 || threads % 32 || n_blocks < 1 || k_launch < 1 ||
@@ -393,13 +396,13 @@ cudaError_t launch_fleet_task(const FleetView &fv, const BlockDesc *blocks, int 
   const size_t dyn = xh_bytes + (to.stage ? smem : 0);
   switch (ntv) {
     case NT_6:
-      return fleet_task_d<NT_6>(fv, blocks, n_blocks, threads, diag, structured, k_launch,
+      return fleet_task_d<NT_6>(fv, blocks, n_blocks, threads, diag, layout, k_launch,
                                 k_task, tv, to, dyn, stream);
     case NT_8:
-      return fleet_task_d<NT_8>(fv, blocks, n_blocks, threads, diag, structured, k_launch,
+      return fleet_task_d<NT_8>(fv, blocks, n_blocks, threads, diag, layout, k_launch,
                                 k_task, tv, to, dyn, stream);
     default:
-      return fleet_task_d<NT_MIXED>(fv, blocks, n_blocks, threads, diag, structured, k_launch,
+      return fleet_task_d<NT_MIXED>(fv, blocks, n_blocks, threads, diag, layout, k_launch,
                                     k_task, tv, to, dyn, stream);
   }
 }

@@ -1,0 +1,101 @@
+"""Thruster allocations of the diagonal-mass step (dense, vectored, mirrored frame) against the
+FP64 oracle: vehicles on each side of every condition that picks one, one sub-step from random
+states and a rollout, with the same bits from every kernel that steps them."""
+import copy
+
+import numpy as np
+import pytest
+import torch
+
+from _helpers import TOL_ROLLOUT, TOL_STEP, oracle_nominal, rel_err, vehicles
+from oracle import oracle as O
+from paper_2410_14117_gb300 import inputs as I
+from test_gpu_parity import H, gpu_state, make_sim, oracle_types_geo
+
+pytestmark = pytest.mark.gpu
+
+
+def _swapped(v, i, j):  # the same vehicle, two thrusters numbered the other way round
+    w = copy.deepcopy(v)
+    w.r[[i, j]], w.d[[i, j]] = v.r[[j, i]], v.d[[j, i]]
+    return w
+
+
+def _moved(v, i, axis, by, what="r"):
+    w = copy.deepcopy(v)
+    getattr(w, what)[i, axis] += by
+    return w
+
+
+def _without(v, n):  # the vehicle's first n thrusters
+    w = copy.deepcopy(v)
+    w.n_thr = n
+    w.r[n:], w.d[n:] = 0.0, 0.0
+    return w
+
+
+def _rb(v, x):  # centre of buoyancy off the z axis
+    w = copy.deepcopy(v)
+    w.params[I.P_RB] = x
+    return w
+
+
+ROV, HEAVY = vehicles()
+FLEETS = {
+    "six": ([ROV], 0), "eight": ([HEAVY], 0), "both": ([ROV, HEAVY], None),
+    "literal frame": (vehicles("literal"), None),
+    "swapped horizontals": ([_swapped(ROV, 0, 1), HEAVY], None),
+    "swapped verticals": ([_swapped(HEAVY, 5, 6)], 0),
+    "one arm longer": ([_moved(ROV, 4, 1, 0.05)], 0),
+    "verticals ahead": ([_moved(_moved(ROV, 4, 0, 0.1), 5, 0, 0.1)], 0),
+    "tilted horizontal": ([_moved(ROV, 2, 2, 0.3, "d")], 0),
+    "four thrusters": ([_without(ROV, 4)], 0), "seven": ([_without(HEAVY, 7), ROV], None),
+    "type off axis": ([_rb(ROV, 0.01), HEAVY], None),
+    "record off axis": ([ROV, HEAVY], None),
+}
+
+
+@pytest.mark.parametrize("name", FLEETS)
+def test_allocation_matches_oracle_on_every_kernel(name):
+    vs, only = FLEETS[name]
+    n = 700
+    types = np.full(n, 0, np.int32) if only == 0 else I.mixed_fleet(4, n, max_group=90)
+    nt = np.array([vs[t].n_thr for t in types])
+    params = I.perturbed_params(5, oracle_nominal(vs)[types], n)
+    if name == "record off axis":
+        params[n // 2, I.P_RB + 1] = 0.0078125
+    states = I.random_states(6, n, nt)
+    cmds = I.commands(7, 4, n, nt).astype(np.float64)
+    t, geo = oracle_types_geo(types, vs)
+    for k, tol in ((1, TOL_STEP), (40, TOL_ROLLOUT)):
+        ref = O.rollout(params, geo, t, states, cmds, 10, k, h=H)
+        out = []
+        for queue, wide, spl in ((False, True, 50), (False, False, 7), (True, True, 9),
+                                 (True, False, 50)):
+            sim = make_sim(types, vs, epb=64, spl=spl, queue=queue, wide=wide)
+            # the path follows the parameters: mirrored (if the types allow it) before this call
+            sim.randomize(3, 0.8, 1.2, 0.2, 0.3)
+            sim.set_params(torch.tensor(params, dtype=torch.float32, device="cuda"))
+            sim.set_state(torch.tensor(states, dtype=torch.float32, device="cuda"))
+            sim.set_actions(torch.tensor(cmds, dtype=torch.float32, device="cuda"), 10)
+            sim.step(k)
+            assert sim.sync() == 0
+            out.append(gpu_state(sim))
+            sim.close()
+        assert rel_err(out[0], ref).max() <= tol
+        for o in out[1:]:
+            np.testing.assert_array_equal(o, out[0])
+
+
+def test_recorded_and_rolled_out_states_equal_the_step():
+    types = I.mixed_fleet(4, 500, max_group=90)
+    got = []
+    for record in (False, True):
+        sim = make_sim(types, [ROV, HEAVY])
+        sim.randomize(3, 0.8, 1.2, 0.2, 0.3)
+        sim.reset()
+        sim.set_procedural_actions(5, 10)
+        sim.step_record(25) if record else sim.step(25)
+        got.append(gpu_state(sim))
+        sim.close()
+    np.testing.assert_array_equal(got[0], got[1])
