@@ -289,6 +289,7 @@ struct mg_sim {
     v.n_not_spd = counters + 1;
     v.any_offdiag = offdiag;
     v.xh = has_xh ? xh : nullptr;
+    v.diag_only = nominal_diag && !has_xh;
     return v;
   }
 

@@ -70,19 +70,10 @@ __device__ __forceinline__ void procedural_commands(uint64_t seed, uint64_t gid,
   }
 }
 
-// Box-Muller pair from two open-interval uniforms (FP64).
-__device__ __forceinline__ void box_muller(double u1, double u2, double &z0, double &z1) {
-  const double r = sqrt(-2.0 * log(u1));
-  double s, c;
-  sincospi(2.0 * u2, &s, &c);
-  z0 = r * c;
-  z1 = r * s;
-}
-
-// Box-Muller in FP32, for the episode-start draws: the same uniforms (exact in FP32) and the
-// same formula, each result within a few ulp of the FP64 form.  Resets run inside step-time
-// kernels (auto-reset), where a warp with one resetting env would otherwise pay GB300's
-// reduced-rate FP64 transcendentals for all 32 lanes.
+// Box-Muller pair from two open-interval uniforms in FP32, for the episode-start draws: each result
+// within a few ulp of the FP64 form.  Resets run inside step-time kernels (auto-reset), where a
+// warp with one resetting env would otherwise pay GB300's reduced-rate FP64 transcendentals for
+// all 32 lanes.
 __device__ __forceinline__ void box_muller_f(float u1, float u2, float &z0, float &z1) {
   const float r = sqrtf(-2.f * logf(u1));
   float s, c;

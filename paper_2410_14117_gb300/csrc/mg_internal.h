@@ -154,6 +154,8 @@ struct SetupView {
   unsigned int *any_offdiag;  // bit 0: some mass matrix is full; bit 1: some r_b is off the z axis
   const float *xh;           // device [MG_NXPARAM][xh_stride] off-diagonal hydrodynamics, or null
   int64_t xh_stride;         // floats between xh's component planes (0: n)
+  bool diag_only;            // nominal mass matrices are diagonal and xh is null: a draw without r_g
+                             // keeps them so
 };
 
 // background_blocks > 0: at most that many 64-thread blocks striding over the fleet (leaves room

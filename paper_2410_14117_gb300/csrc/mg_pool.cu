@@ -454,6 +454,7 @@ cudaError_t init_job(mg_pool *p, const mg_job_spec &s, int64_t env0, const float
   v.pa = sub_params(p->pa, env0);
   v.n_not_spd = p->counters + 1;
   v.any_offdiag = p->offdiag;
+  v.diag_only = p->diag && !xh;
   if (xh) {
     // stride of the planes: the capacity
     const size_t bytes = (size_t)n * MG_NXPARAM * 4;

@@ -1,14 +1,17 @@
 // Set-up kernels, run when parameters or episodes change (not per sub-step):
-//   - domain randomisation (§METHOD) from Philox4x32-10 draws, in FP64, stored FP32;
+//   - domain randomisation (§METHOD) from Philox4x32-10 draws, each value rounded once to FP32
+//     from two-float arithmetic (mg_df32.cuh);
 //   - derivation of what the step reads, including M^-1 of the 6x6 mass matrix M_RB + M_A of
-//     Eq. 1 by an FP64 Cholesky factorisation (M is symmetric positive definite for any
-//     physical vehicle; a non-positive pivot is counted and reported);
+//     Eq. 1: its reciprocals where it is diagonal, else by an FP64 Cholesky factorisation (M is
+//     symmetric positive definite for any physical vehicle; a non-positive pivot is counted and
+//     reported);
 //   - episode reset, and conversions between the SoA planes and the record layouts of mg.h.
 #include <algorithm>
 #include <cstdint>
 #include <type_traits>
 
 #include "mg_device.cuh"
+#include "mg_df32.cuh"
 
 namespace mg {
 
@@ -28,57 +31,67 @@ static_assert(MG_P_M == 0 && MG_P_IG == 1 && MG_P_MA == 4 && MG_P_DL == 10 && MG
 __host__ __device__ constexpr int rand_idx(int j) {
   return j < 24 ? j : j == 24 ? MG_P_RB + 2 : j == 25 ? MG_P_KT : MG_P_TAU;
 }
-// Block size of the randomisation kernel: at ~150 registers two or three 128-thread blocks fit
-// per SM, where one 256-thread block leaves 65,536 envs 1.7 waves.
+// Block size of the randomisation kernel and of the record copies.
 constexpr int kRandThreads = 128;
-// Background form: 64-thread blocks (two warps, ~10 K registers) striding over the fleet, so
-// that one block fits beside a step kernel's resident blocks on every SM.
+// Background form: 64-thread blocks (two warps) striding over the fleet, so that one block fits
+// beside a step kernel's resident blocks on every SM.
 constexpr int kRandBgThreads = 64;
 
-// Tell the host of an r_b off the body's z axis (the mirrored thruster allocation needs it on it).
-__device__ __forceinline__ void note_off_axis(const SetupView &v, const double *p) {
-  if (p[MG_P_RB] != 0.0 || p[MG_P_RB + 1] != 0.0) atomicOr(v.any_offdiag, 2u);
+__device__ __forceinline__ bool aligned16(const void *p) {
+  return (reinterpret_cast<uintptr_t>(p) & 15u) == 0;
 }
 
-// derive() for an env whose mass matrix is diagonal (r_g = 0, no off-diagonal added mass): the
-// same values derive() stores, without building the 6 x 6 matrices (FP64 runs at a 64th of the
-// FP32 rate on this GPU).  I_o = I_g exactly and every off-diagonal entry is +0 when r_g = 0.
-__device__ void derive_diag(const SetupView &v, int64_t e, const double *p) {
-  const double m = p[MG_P_M];
-  const double *ma = p + MG_P_MA;
-  const double rg[3] = {p[MG_P_RG], p[MG_P_RG + 1], p[MG_P_RG + 2]};
-  double Mjj[6], mi[6];
-  bool spd = true;
-  for (int i = 0; i < 3; ++i) {
-    Mjj[i] = m + ma[i];
-    Mjj[3 + i] = p[MG_P_IG + i] + ma[3 + i];
+// Copy count floats, all threads of the block taking part; 16-byte vectors when both ends allow.
+__device__ __forceinline__ void block_copy(float *dst, const float *src, int count) {
+  int done = 0;
+  if (aligned16(dst) && aligned16(src)) {
+    done = count & ~3;
+    for (int i = threadIdx.x; i < done / 4; i += blockDim.x)
+      reinterpret_cast<float4 *>(dst)[i] = reinterpret_cast<const float4 *>(src)[i];
   }
+  for (int i = done + threadIdx.x; i < count; i += blockDim.x) dst[i] = src[i];
+}
+
+// Tell the host of an r_b off the body's z axis (the mirrored thruster allocation needs it on it).
+__device__ __forceinline__ void note_off_axis(const SetupView &v, const float *p) {
+  if (p[MG_P_RB] != 0.f || p[MG_P_RB + 1] != 0.f) atomicOr(v.any_offdiag, 2u);
+}
+
+// The step's parameter planes of an env whose mass matrix is diagonal (r_g = 0, no off-diagonal
+// added mass) from its record p[MG_NPARAM]: I_o = I_g exactly, M^-1 = diag(1 / M_jj) and every
+// off-diagonal entry is +0.  Each stored value is the FP64 expression's, rounded once: a sum,
+// difference or product of two FP32 numbers is one FP32 operation, and 1 / (a + b) takes the sum
+// in two floats.
+__device__ __forceinline__ void derive_diag(const SetupView &v, int64_t e, const float *p) {
+  const float m = p[MG_P_M];
+  const float *ma = p + MG_P_MA, *rg = p + MG_P_RG, *rb = p + MG_P_RB;
+  float J[3], mi[6];
+  bool spd = true;
+#pragma unroll
   for (int j = 0; j < 6; ++j) {
-    if (!(Mjj[j] > 0.0)) spd = false;
-    mi[j] = Mjj[j] > 0.0 ? 1.0 / Mjj[j] : 0.0;
+    const df32 M = two_sum(j < 3 ? m : p[MG_P_IG + j - 3], ma[j]);
+    if (j >= 3) J[j - 3] = M.h;
+    if (!(M.h > 0.f)) spd = false;
+    mi[j] = M.h > 0.f ? df_rcp(M) : 0.f;
   }
   if (!spd) atomicAdd(v.n_not_spd, 1ull);
   note_off_axis(v, p);
-  const double W = p[MG_P_W], B = p[MG_P_B];
-  const double G[3] = {W * rg[0] - B * p[MG_P_RB], W * rg[1] - B * p[MG_P_RB + 1],
-                       W * rg[2] - B * p[MG_P_RB + 2]};
+  const float W = p[MG_P_W], B = p[MG_P_B];
+  float G[3];
+#pragma unroll
+  for (int i = 0; i < 3; ++i) G[i] = __fsub_rn(__fmul_rn(W, rg[i]), __fmul_rn(B, rb[i]));
   const ParamPlanes &pa = v.pa;
-  auto f = [](double x) { return (float)x; };
-  pa.d0[e] = make_float4(f(m), f(ma[0]), f(ma[1]), f(ma[2]));
-  pa.d1[e] = make_float4(f(Mjj[3]), f(Mjj[4]), f(Mjj[5]), f(W - B));
-  pa.d2[e] = make_float4(f(p[MG_P_DL]), f(p[MG_P_DL + 1]), f(p[MG_P_DL + 2]),
-                         f(p[MG_P_DL + 3]));
-  pa.d3[e] = make_float4(f(p[MG_P_DL + 4]), f(p[MG_P_DL + 5]), f(p[MG_P_DQ]),
-                         f(p[MG_P_DQ + 1]));
-  pa.d4[e] = make_float4(f(p[MG_P_DQ + 2]), f(p[MG_P_DQ + 3]), f(p[MG_P_DQ + 4]),
-                         f(p[MG_P_DQ + 5]));
-  pa.d5[e] = make_float4(f(G[0]), f(G[1]), f(G[2]), f(p[MG_P_KT]));
-  pa.d6[e] = make_float4(f(p[MG_P_VC]), f(p[MG_P_VC + 1]), f(p[MG_P_VC + 2]),
-                         f(1.0 / p[MG_P_TAU]));
-  pa.d7[e] = make_float4(f(mi[0]), f(mi[1]), f(mi[2]), f(mi[3]));
-  pa.d8[e] = make_float2(f(mi[4]), f(mi[5]));
-  pa.g0[e] = make_float4(f(m * rg[0]), f(m * rg[1]), f(m * rg[2]), 0.f);
+  pa.d0[e] = make_float4(m, ma[0], ma[1], ma[2]);
+  pa.d1[e] = make_float4(J[0], J[1], J[2], __fsub_rn(W, B));
+  pa.d2[e] = make_float4(p[MG_P_DL], p[MG_P_DL + 1], p[MG_P_DL + 2], p[MG_P_DL + 3]);
+  pa.d3[e] = make_float4(p[MG_P_DL + 4], p[MG_P_DL + 5], p[MG_P_DQ], p[MG_P_DQ + 1]);
+  pa.d4[e] = make_float4(p[MG_P_DQ + 2], p[MG_P_DQ + 3], p[MG_P_DQ + 4], p[MG_P_DQ + 5]);
+  pa.d5[e] = make_float4(G[0], G[1], G[2], p[MG_P_KT]);
+  pa.d6[e] = make_float4(p[MG_P_VC], p[MG_P_VC + 1], p[MG_P_VC + 2], __frcp_rn(p[MG_P_TAU]));
+  pa.d7[e] = make_float4(mi[0], mi[1], mi[2], mi[3]);
+  pa.d8[e] = make_float2(mi[4], mi[5]);
   const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+  pa.g0[e] = make_float4(__fmul_rn(m, rg[0]), __fmul_rn(m, rg[1]), __fmul_rn(m, rg[2]), 0.f);
   pa.g1[e] = z;
   pa.g2[e] = z;
   pa.g3[e] = z;
@@ -86,22 +99,25 @@ __device__ void derive_diag(const SetupView &v, int64_t e, const double *p) {
   pa.g5[e] = 0.f;
 }
 
-// Derive the step's parameter planes for env e from its FP64 record p[MG_NPARAM].
-__device__ void derive(const SetupView &v, int64_t e, const double *p) {
-  const double m = p[MG_P_M];
-  const double rg[3] = {p[MG_P_RG], p[MG_P_RG + 1], p[MG_P_RG + 2]};
-  const double *ma = p + MG_P_MA;
-  const double r2 = rg[0] * rg[0] + rg[1] * rg[1] + rg[2] * rg[2];
+// Derive the step's parameter planes for env e from its record f[MG_NPARAM]; a full mass matrix
+// is inverted in FP64.
+__device__ void derive(const SetupView &v, int64_t e, const float *f32) {
   const int64_t xs = v.xh_stride ? v.xh_stride : v.n;
-  if (r2 == 0.0) {
+  if (f32[MG_P_RG] == 0.f && f32[MG_P_RG + 1] == 0.f && f32[MG_P_RG + 2] == 0.f) {
     bool xh_zero = true;
     if (v.xh)
       for (int t = 0; t < 15; ++t) xh_zero = xh_zero && v.xh[(int64_t)t * xs + e] == 0.f;
     if (xh_zero) {
-      derive_diag(v, e, p);
+      derive_diag(v, e, f32);
       return;
     }
   }
+  double p[MG_NPARAM];
+  for (int j = 0; j < MG_NPARAM; ++j) p[j] = (double)f32[j];
+  const double m = p[MG_P_M];
+  const double rg[3] = {p[MG_P_RG], p[MG_P_RG + 1], p[MG_P_RG + 2]};
+  const double *ma = p + MG_P_MA;
+  const double r2 = rg[0] * rg[0] + rg[1] * rg[1] + rg[2] * rg[2];
   // I_o = I_g - m S(r_g)^2 = I_g + m (|r_g|^2 I - r_g r_g^T)  (inertia about the body origin)
   double Io[3][3];
   for (int i = 0; i < 3; ++i)
@@ -119,7 +135,6 @@ __device__ void derive(const SetupView &v, int64_t e, const double *p) {
       M[3 + i][j] = m * S[i][j];
       M[3 + i][3 + j] = Io[i][j] + ((i == j) ? ma[3 + i] : 0.0);
     }
-  bool ma_off = false;
   if (v.xh) {
     int t = 0;
     for (int i = 0; i < 6; ++i)
@@ -127,22 +142,13 @@ __device__ void derive(const SetupView &v, int64_t e, const double *p) {
         const double a = (double)v.xh[(int64_t)t * xs + e];
         M[i][j] += a;
         M[j][i] += a;
-        ma_off = ma_off || a != 0.0;
       }
   }
 
-  // Cholesky M = L L^T; L^-1 by forward substitution; M^-1 = L^-T L^-1.  With r_g = 0 the
-  // matrix is diagonal (diagonal M_A), its factor is diag(sqrt(M_jj)) and the inverse 1 / M_jj.
+  // Cholesky M = L L^T; L^-1 by forward substitution; M^-1 = L^-T L^-1.
   double L[6][6] = {}, Li[6][6] = {}, Mi[6][6] = {};
   bool spd = true;
-  const bool diagonal = (r2 == 0.0) && !ma_off;
-  if (diagonal) {
-    for (int j = 0; j < 6; ++j) {
-      if (!(M[j][j] > 0.0)) spd = false;
-      Mi[j][j] = M[j][j] > 0.0 ? 1.0 / M[j][j] : 0.0;
-    }
-  }
-  for (int j = 0; j < 6 && !diagonal; ++j) {
+  for (int j = 0; j < 6; ++j) {
     double d = M[j][j];
     for (int k = 0; k < j; ++k) d -= L[j][k] * L[j][k];
     if (!(d > 0.0)) {
@@ -156,7 +162,7 @@ __device__ void derive(const SetupView &v, int64_t e, const double *p) {
       L[i][j] = s / L[j][j];
     }
   }
-  for (int j = 0; j < 6 && !diagonal; ++j) {
+  for (int j = 0; j < 6; ++j) {
     Li[j][j] = 1.0 / L[j][j];
     for (int i = j + 1; i < 6; ++i) {
       double s = 0.0;
@@ -164,15 +170,15 @@ __device__ void derive(const SetupView &v, int64_t e, const double *p) {
       Li[i][j] = -s / L[i][i];
     }
   }
-  for (int i = 0; i < 6 && !diagonal; ++i)
+  for (int i = 0; i < 6; ++i)
     for (int j = 0; j < 6; ++j) {
       double s = 0.0;
       for (int k = (i > j ? i : j); k < 6; ++k) s += Li[k][i] * Li[k][j];
       Mi[i][j] = s;
     }
   if (!spd) atomicAdd(v.n_not_spd, 1ull);
-  if (!diagonal) atomicOr(v.any_offdiag, 1u);
-  note_off_axis(v, p);
+  atomicOr(v.any_offdiag, 1u);
+  note_off_axis(v, f32);
 
   const double W = p[MG_P_W], B = p[MG_P_B];
   const double G[3] = {W * rg[0] - B * p[MG_P_RB], W * rg[1] - B * p[MG_P_RB + 1],
@@ -201,73 +207,129 @@ __device__ void derive(const SetupView &v, int64_t e, const double *p) {
   pa.g5[e] = f(Mi[4][5]);
 }
 
-__device__ __forceinline__ void randomize_env(const SetupView &v, const float *__restrict__ nominal,
-                                              uint64_t seed, double lo, double hi,
-                                              double current_sigma, double rg_halfwidth,
-                                              int64_t e) {
-  const uint64_t gid = (uint64_t)(v.gid0 + e);
-  const float *nom = nominal + (int64_t)v.types[e] * MG_NPARAM;
-  double p[MG_NPARAM];
-  for (int j = 0; j < MG_NPARAM; ++j) p[j] = (double)nom[j];
-  uint4 x = make_uint4(0, 0, 0, 0);
+// What a randomisation draws: each of the 27 scalars times lo + (hi - lo) u with hi - lo in two
+// floats, the current's sigma and the half-width of r_g.
+struct Draw {
+  uint64_t seed;
+  float lo;
+  df32 width;
+  float sigma;
+  double rg_halfwidth;
+};
+
+// nominal x (lo + (hi - lo) u), rounded once.
+__device__ __forceinline__ float scaled(const Draw &d, float nominal, float u) {
+  df32 p = two_prod(d.width.h, u);
+  p.l = __fmaf_rn(d.width.l, u, p.l);
+  df32 s = two_sum(d.lo, p.h);
+  s.l = __fadd_rn(s.l, p.l);
+  const float q = __fmul_rn(s.h, nominal);
+  const float r = __fmaf_rn(s.l, nominal, __fmaf_rn(s.h, nominal, -q));
+  return isfinite(q) ? __fadd_rn(q, r) : q;
+}
+
+// c + sigma r x, rounded once.
+__device__ __forceinline__ float current(const Draw &d, float c, df32 r, df32 x) {
+  const df32 z = df_mul(r, x);
+  df32 p = two_prod(d.sigma, z.h);
+  p.l = __fmaf_rn(d.sigma, z.l, p.l);
+  const df32 s = two_sum(c, p.h);
+  return __fadd_rn(s.h, __fadd_rn(s.l, p.l));
+}
+
+// Draw one tile of blockDim.x envs from e0 on: each thread draws and derives its env, the records
+// are staged in rows [blockDim.x][MG_NPARAM] and leave as one contiguous run (a thread's own row is
+// 140 bytes, so direct stores would touch 32 sectors each).  Everything is FP32 pairs: the FP64
+// form of the same draws took 840 us for 1,048,576 envs, FP64-pipe bound, against 55 us for the
+// 360 bytes per env it stores; this takes 63 us.
+// DIAG: every mass matrix is diagonal (no r_g, no extension), so the FP64 Cholesky is not compiled
+// in (it doubles the registers).
+template <bool DIAG>
+__device__ __forceinline__ void randomize_tile(const SetupView &v,
+                                               const float *__restrict__ nominal, const Draw &d,
+                                               int64_t e0, float *rows) {
+  const int64_t e = e0 + threadIdx.x;
+  if (e < v.n) {
+    const uint64_t gid = (uint64_t)(v.gid0 + e);
+    const float *nom = nominal + (int64_t)v.types[e] * MG_NPARAM;
+    float p[MG_NPARAM];
 #pragma unroll
-  for (int j = 0; j < 27; ++j) {
-    if (j % 4 == 0) x = draw4(seed, gid, STREAM_PARAMS, (uint32_t)(j / 4));
-    const uint32_t w = (j % 4 == 0) ? x.x : (j % 4 == 1) ? x.y : (j % 4 == 2) ? x.z : x.w;
-    const int idx = rand_idx(j);
-    p[idx] = (double)nom[idx] * (lo + (hi - lo) * u01d(w));
+    for (int j = 0; j < MG_NPARAM; ++j) p[j] = nom[j];
+    uint4 x = make_uint4(0, 0, 0, 0);
+#pragma unroll
+    for (int j = 0; j < 27; ++j) {
+      if (j % 4 == 0) x = draw4(d.seed, gid, STREAM_PARAMS, (uint32_t)(j / 4));
+      const uint32_t w = (j % 4 == 0) ? x.x : (j % 4 == 1) ? x.y : (j % 4 == 2) ? x.z : x.w;
+      p[rand_idx(j)] = scaled(d, p[rand_idx(j)], u01f(w));
+    }
+    // Box-Muller normals of the current: two of the first pair, the cosine of the second
+    const uint4 c = draw4(d.seed, gid, STREAM_CURRENT, 0u);
+    df32 cs, sn;
+    df32 r = df_normal_radius(u01f(c.x));
+    df_cos_sin_turn(u01f(c.y), cs, sn);
+    p[MG_P_VC] = current(d, p[MG_P_VC], r, cs);
+    p[MG_P_VC + 1] = current(d, p[MG_P_VC + 1], r, sn);
+    r = df_normal_radius(u01f(c.z));
+    df_cos_sin_turn(u01f(c.w), cs, sn);
+    p[MG_P_VC + 2] = current(d, p[MG_P_VC + 2], r, cs);
+    if constexpr (!DIAG) {
+      if (d.rg_halfwidth > 0.0) {  // off-centre gravity: nominal + U[-w, w] per axis
+        const uint4 g = draw4(d.seed, gid, STREAM_PARAMS, 7u);
+        const uint32_t w[3] = {g.x, g.y, g.z};
+#pragma unroll
+        for (int i = 0; i < 3; ++i)
+          p[MG_P_RG + i] =
+              (float)((double)p[MG_P_RG + i] + d.rg_halfwidth * (2.0 * u01d(w[i]) - 1.0));
+      }
+    }
+    // Everything the step reads is derived from the stored FP32 values, so that it is consistent
+    // with what mg_get_params reports.
+#pragma unroll
+    for (int j = 0; j < MG_NPARAM; ++j) rows[threadIdx.x * MG_NPARAM + j] = p[j];
+    if constexpr (DIAG) derive_diag(v, e, p);
+    else derive(v, e, p);
   }
-  const uint4 c = draw4(seed, gid, STREAM_CURRENT, 0u);
-  double z0, z1, z2, z3;
-  box_muller(u01d(c.x), u01d(c.y), z0, z1);
-  box_muller(u01d(c.z), u01d(c.w), z2, z3);
-  p[MG_P_VC] += current_sigma * z0;
-  p[MG_P_VC + 1] += current_sigma * z1;
-  p[MG_P_VC + 2] += current_sigma * z2;
-  if (rg_halfwidth > 0.0) {  // off-centre gravity: nominal + U[-w, w] per axis
-    const uint4 r = draw4(seed, gid, STREAM_PARAMS, 7u);
-    p[MG_P_RG] += rg_halfwidth * (2.0 * u01d(r.x) - 1.0);
-    p[MG_P_RG + 1] += rg_halfwidth * (2.0 * u01d(r.y) - 1.0);
-    p[MG_P_RG + 2] += rg_halfwidth * (2.0 * u01d(r.z) - 1.0);
-  }
-  // Store FP32; derive from the stored values so that everything the step reads is consistent
-  // with what mg_get_params reports.
-  for (int j = 0; j < MG_NPARAM; ++j) {
-    const float f = (float)p[j];
-    v.raw[e * MG_NPARAM + j] = f;
-    p[j] = (double)f;
-  }
-  derive(v, e, p);
+  __syncthreads();
+  const int64_t left = v.n - e0;
+  block_copy(v.raw + e0 * MG_NPARAM, rows,
+             (int)(left < blockDim.x ? left : blockDim.x) * MG_NPARAM);
 }
 
 // One env per thread.
+template <bool DIAG>
 __global__ void __launch_bounds__(kRandThreads)
-    k_randomize(const SetupView v, const float *__restrict__ nominal, uint64_t seed,
-                            double lo, double hi, double current_sigma, double rg_halfwidth) {
-  const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (e < v.n) randomize_env(v, nominal, seed, lo, hi, current_sigma, rg_halfwidth, e);
+    k_randomize(const SetupView v, const float *__restrict__ nominal, const Draw d) {
+  __shared__ __align__(16) float rows[kRandThreads * MG_NPARAM];
+  randomize_tile<DIAG>(v, nominal, d, (int64_t)blockIdx.x * kRandThreads, rows);
 }
 
 // Background form: a grid smaller than the fleet strides over it, leaving room on every SM for
 // a step kernel running concurrently on another stream.  Same per-env arithmetic.
 __global__ void __launch_bounds__(kRandBgThreads)
-    k_randomize_bg(const SetupView v, const float *__restrict__ nominal, uint64_t seed,
-                   double lo, double hi, double current_sigma, double rg_halfwidth) {
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < v.n; e += stride)
-    randomize_env(v, nominal, seed, lo, hi, current_sigma, rg_halfwidth, e);
+    k_randomize_bg(const SetupView v, const float *__restrict__ nominal, const Draw d) {
+  __shared__ __align__(16) float rows[kRandBgThreads * MG_NPARAM];
+  const int64_t stride = (int64_t)gridDim.x * kRandBgThreads;
+  for (int64_t e0 = (int64_t)blockIdx.x * kRandBgThreads; e0 < v.n; e0 += stride) {
+    randomize_tile<true>(v, nominal, d, e0, rows);
+    __syncthreads();
+  }
 }
 
-__global__ void k_import_params(const SetupView v, const float *__restrict__ in) {
-  const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= v.n) return;
-  double p[MG_NPARAM];
-  for (int j = 0; j < MG_NPARAM; ++j) {
-    const float f = in[e * MG_NPARAM + j];
-    v.raw[e * MG_NPARAM + j] = f;
-    p[j] = (double)f;
-  }
-  derive(v, e, p);
+// in may be the stored records themselves (re-derived in place).
+__global__ void __launch_bounds__(kRandThreads)
+    k_import_params(const SetupView v, const float *in) {
+  __shared__ __align__(16) float rows[kRandThreads * MG_NPARAM];
+  const int64_t e0 = (int64_t)blockIdx.x * kRandThreads;
+  const int64_t left = v.n - e0;
+  const int total = (int)(left < kRandThreads ? left : kRandThreads) * MG_NPARAM;
+  block_copy(rows, in + e0 * MG_NPARAM, total);
+  __syncthreads();
+  if (in != v.raw) block_copy(v.raw + e0 * MG_NPARAM, rows, total);
+  if ((int64_t)threadIdx.x >= left) return;
+  float p[MG_NPARAM];
+#pragma unroll
+  for (int j = 0; j < MG_NPARAM; ++j) p[j] = rows[threadIdx.x * MG_NPARAM + j];
+  derive(v, e0 + threadIdx.x, p);
 }
 
 // Off-diagonal hydrodynamics between the record layout [n][MG_NXPARAM] and the planes
@@ -284,10 +346,12 @@ __global__ void k_xh_transpose(const float *__restrict__ in, float *__restrict__
   }
 }
 
-__global__ void k_export_params(const SetupView v, float *__restrict__ out) {
-  const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= v.n) return;
-  for (int j = 0; j < MG_NPARAM; ++j) out[e * MG_NPARAM + j] = v.raw[e * MG_NPARAM + j];
+// The records as they are, a contiguous run per block.
+__global__ void __launch_bounds__(kThreads)
+    k_export_params(const SetupView v, float *__restrict__ out) {
+  constexpr int kRun = kThreads * 16;
+  const int64_t i0 = (int64_t)blockIdx.x * kRun, left = v.n * MG_NPARAM - i0;
+  block_copy(out + i0, v.raw + i0, (int)(left < kRun ? left : kRun));
 }
 
 __global__ void k_reset(const StatePlanes st, int64_t n, int64_t gid0,
@@ -303,10 +367,6 @@ __global__ void k_reset(const StatePlanes st, int64_t n, int64_t gid0,
 // block's rows move as one contiguous span (16-byte vectors when the row buffer is 16-byte
 // aligned: a block's span starts at a multiple of kRowThreads x 84 B = 10,752 B).
 constexpr int kRowThreads = 128;
-
-__device__ __forceinline__ bool aligned16(const void *p) {
-  return (reinterpret_cast<uintptr_t>(p) & 15u) == 0;
-}
 
 __global__ void __launch_bounds__(kRowThreads)
     k_export_state(const StatePlanes st, int64_t n, float *__restrict__ out) {
@@ -385,15 +445,26 @@ __global__ void k_philox(const uint32_t *__restrict__ ctr, const uint32_t *__res
 cudaError_t launch_randomize(const SetupView &v, const float *nominal, uint64_t seed, double lo,
                              double hi, double current_sigma, double rg_halfwidth,
                              cudaStream_t stream, int background_blocks) {
+  Draw d{};
+  d.seed = seed;
+  d.lo = (float)lo;  // the bounds are FP32 numbers
+  const double width = hi - lo;
+  d.width.h = (float)width;
+  d.width.l = (float)(width - (double)d.width.h);
+  d.sigma = (float)current_sigma;
+  d.rg_halfwidth = rg_halfwidth;
   if (background_blocks > 0) {
+    if (!v.diag_only || rg_halfwidth != 0.0) return cudaErrorInvalidValue;
     const int64_t full = (v.n + kRandBgThreads - 1) / kRandBgThreads;
     const int blocks = (int)std::min<int64_t>(full, background_blocks);
-    k_randomize_bg<<<blocks, kRandBgThreads, 0, stream>>>(v, nominal, seed, lo, hi,
-                                                          current_sigma, rg_halfwidth);
-  } else {
-    k_randomize<<<(int)((v.n + kRandThreads - 1) / kRandThreads), kRandThreads, 0, stream>>>(
-        v, nominal, seed, lo, hi, current_sigma, rg_halfwidth);
+    k_randomize_bg<<<blocks, kRandBgThreads, 0, stream>>>(v, nominal, d);
+    return cudaGetLastError();
   }
+  const int blocks = (int)((v.n + kRandThreads - 1) / kRandThreads);
+  if (v.diag_only && rg_halfwidth == 0.0)
+    k_randomize<true><<<blocks, kRandThreads, 0, stream>>>(v, nominal, d);
+  else
+    k_randomize<false><<<blocks, kRandThreads, 0, stream>>>(v, nominal, d);
   return cudaGetLastError();
 }
 
@@ -405,12 +476,14 @@ cudaError_t launch_xh_transpose(const float *in, float *out, int64_t n, bool to_
 }
 
 cudaError_t launch_import_params(const SetupView &v, const float *in, cudaStream_t stream) {
-  k_import_params<<<blocks_for(v.n), kThreads, 0, stream>>>(v, in);
+  k_import_params<<<(int)((v.n + kRandThreads - 1) / kRandThreads), kRandThreads, 0, stream>>>(v,
+                                                                                            in);
   return cudaGetLastError();
 }
 
 cudaError_t launch_export_params(const SetupView &v, float *out, cudaStream_t stream) {
-  k_export_params<<<blocks_for(v.n), kThreads, 0, stream>>>(v, out);
+  constexpr int64_t kRun = (int64_t)kThreads * 16;
+  k_export_params<<<(int)((v.n * MG_NPARAM + kRun - 1) / kRun), kThreads, 0, stream>>>(v, out);
   return cudaGetLastError();
 }
 

@@ -1,0 +1,61 @@
+"""The domain randomisation in two-float arithmetic against the FP64 oracle over its ranges, and the
+parameter records through every alignment and ragged tail."""
+import numpy as np
+import pytest
+import torch
+
+from _helpers import f32, oracle_nominal, vehicles
+from oracle import oracle as O
+from paper_2410_14117_gb300 import inputs as I
+from paper_2410_14117_gb300.sim import Sim
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("n,lo,hi,sigma", [
+    (1, 0.8, 1.2, 0.2), (127, 1.0, 1.0, 0.0), (129, 0.003, 7.5, 5.0), (20011, 0.8, 1.2, 0.2),
+    (4096, 1e-3, 1e3, 1e-4)])
+@pytest.mark.parametrize("background", [False, True])
+def test_draws_are_the_fp64_values_rounded_once(n, lo, hi, sigma, background):
+    vs = vehicles()
+    types = I.mixed_fleet(3, n, max_group=max(1, n // 7))
+    sim = Sim(n, types, vs)
+    if background:
+        sim.randomize_prefetch(77, lo, hi, sigma)
+    sim.randomize(77, lo, hi, sigma, 0.3)
+    got = sim.get_params().double().cpu().numpy()
+    sim.close()
+    ref = O.randomize(77, oracle_nominal(vs), types, f32(lo), f32(hi), f32(sigma))
+    # half an FP32 ulp of the FP64 value; the two-float value is within 2^-35 of it before it is
+    # rounded (2^-24 is half an ulp relative to the smallest mantissa)
+    np.testing.assert_allclose(got, ref, rtol=2.0 ** -24 + 2.0 ** -34, atol=1e-30)
+
+
+@pytest.mark.parametrize("n", [1, 33, 128, 257, 1000])
+@pytest.mark.parametrize("off", [0, 1, 2])
+def test_records_round_trip_any_alignment(n, off):
+    vs = vehicles()
+    sim = Sim(n, np.zeros(n, np.int32), vs)
+    p = np.ascontiguousarray(I.perturbed_params(5, oracle_nominal(vs)[np.zeros(n, int)], n))
+    buf = torch.zeros(n * I.NPARAM + off + 1, device="cuda")
+    rec = buf[off:off + n * I.NPARAM].view(n, I.NPARAM)
+    rec.copy_(torch.tensor(p, dtype=torch.float32))
+    sim.set_params(rec)
+    out = torch.full_like(buf, -1.0)
+    sim.get_params(out[off:off + n * I.NPARAM].view(n, I.NPARAM))
+    assert torch.equal(out[off:off + n * I.NPARAM], buf[off:off + n * I.NPARAM])
+    assert (out[:off] == -1).all() and out[-1] == -1
+    sim.close()
+
+
+def test_not_spd_and_off_axis_records_are_seen():
+    vs = vehicles()
+    n = 300
+    p = np.ascontiguousarray(I.perturbed_params(5, oracle_nominal(vs)[np.zeros(n, int)], n))
+    p[17, I.P_MA + 2] = -p[17, I.P_M]  # M_33 = 0
+    sim = Sim(n, np.zeros(n, np.int32), vs)
+    from paper_2410_14117_gb300.sim import MGError
+    with pytest.raises(MGError):
+        sim.set_params(torch.tensor(p, dtype=torch.float32, device="cuda"))
+    assert np.array_equal(sim.get_params().double().cpu().numpy(), p)
+    sim.close()
