@@ -369,10 +369,10 @@ __device__ __forceinline__ void fwd_rhs(const St<MT> &y, const float (&cs)[MT],
 }
 
 template <int MT, bool GEN>
-__device__ __forceinline__ void fwd_step(St<MT> &S, const float (&b)[MT], const LagEnv &L,
+__device__ __forceinline__ void fwd_step(St<MT> &S, const float (&c)[MT], const LagEnv &L,
                                          const AdjEnv<GEN> &A, const float4 *gdir,
-                                         const float4 *garm, int nt, bool ca, float h) {
-  rk4_step_lag<MT, !GEN, true, 0, GEN>(S, b, L, A.F, gdir, garm, nt, ca, h, A.xh);
+                                         const float4 *garm, int nt, bool ca, const RkStep &rk) {
+  rk4_step<MT, !GEN, true, 0, GEN>(S, c, L, A.F, gdir, garm, nt, ca, rk, A.xh);
 }
 
 // The RK4 stage states of one sub-step from its start state s (y1 = s):
@@ -387,16 +387,16 @@ __device__ __forceinline__ void stage_states(const St<MT> &s, const float (&cs)[
   const float hh = 0.5f * h, h3 = h * (1.0f / 3.0f), h6 = h * (1.0f / 6.0f);
   St<MT> k;
   fwd_rhs<MT, GEN>(s, cs, A, gdir, garm, nt, current_accel, k);
-  axpy(z, s, h6, k);
-  axpy(y2, s, hh, k);
+  axpy(z, s, h6, 0.5f * h6, k);
+  axpy(y2, s, hh, 0.5f * hh, k);
   fwd_rhs<MT, GEN>(y2, cs, A, gdir, garm, nt, current_accel, k);
-  axpy(z, z, h3, k);
-  axpy(y3, s, hh, k);
+  axpy(z, z, h3, 0.5f * h3, k);
+  axpy(y3, s, hh, 0.5f * hh, k);
   fwd_rhs<MT, GEN>(y3, cs, A, gdir, garm, nt, current_accel, k);
-  axpy(z, z, h3, k);
-  axpy(y4, s, h, k);
+  axpy(z, z, h3, 0.5f * h3, k);
+  axpy(y4, s, h, hh, k);
   fwd_rhs<MT, GEN>(y4, cs, A, gdir, garm, nt, current_accel, k);
-  axpy(z, z, h6, k);
+  axpy(z, z, h6, 0.5f * h6, k);
 }
 
 template <int MT>
@@ -476,10 +476,11 @@ __device__ void step_vjp(const St<MT> &s, const float (&cs)[MT], const AdjEnv<GE
 
 constexpr int kMaxSeg = 32;  // largest checkpoint interval
 
-// The buffered command of sub-step j (cursor position), pre-divided by tau_m as the step reads it.
+// The buffered command of sub-step j (cursor position) times scale: 1 for the forward's step, 1 /
+// tau_m for the right-hand side.
 template <int MT>
 __device__ __forceinline__ void commands_at(const FleetView &fv, int64_t e, int64_t j, int nt,
-                                            float itau, float (&c)[MT]) {
+                                            float scale, float (&c)[MT]) {
   int64_t seg = j / fv.hold;
   if (seg > fv.n_seg - 1) seg = fv.n_seg - 1;
   for (int i = 0; i < MT; ++i) c[i] = 0.f;
@@ -487,7 +488,7 @@ __device__ __forceinline__ void commands_at(const FleetView &fv, int64_t e, int6
     const float *a = fv.act + (seg * fv.n + e) * fv.act_w;
     #pragma unroll
     for (int i = 0; i < MT; ++i)
-      if (i < nt) c[i] = a[i] * itau;
+      if (i < nt) c[i] = a[i] * scale;
   }
 }
 
@@ -635,10 +636,8 @@ __global__ void __launch_bounds__(kAdjThreads)
     load_checkpoint<MT>(ckpt, sg, n, e, S[0]);
     for (int32_t j = 1; j < len; ++j) {
       S[j] = S[j - 1];
-      commands_at<MT>(fv, e, step0 + t0 + j - 1, nt, A.P.itau, c);
-      float b[MT];
-      lag_segment<MT>(c, L, b);
-      fwd_step<MT, GEN>(S[j], b, L, A, gdir, garm, nt, ca, h);
+      commands_at<MT>(fv, e, step0 + t0 + j - 1, nt, 1.f, c);
+      fwd_step<MT, GEN>(S[j], c, L, A, gdir, garm, nt, ca, fv.rk);
     }
     // walk it backwards
     for (int32_t j = len - 1; j >= 0; --j) {
@@ -691,9 +690,11 @@ __device__ __forceinline__ void produce_segment(const FleetView &fv, int64_t e,
   load_checkpoint<MT>(ckpt, sg, n, e, S);
   float c[MT];
   for (int32_t j = 0; j < len; ++j) {
-    commands_at<MT>(fv, e, step0 + t0 + j, nt, A.P.itau, c);
+    commands_at<MT>(fv, e, step0 + t0 + j, nt, 1.f, c);
+    float cs[MT];
+    for (int i = 0; i < MT; ++i) cs[i] = c[i] * A.P.itau;
     St<MT> y2, y3, y4, z;
-    stage_states<MT, GEN>(S, c, A, gdir, garm, nt, ca, h, y2, y3, y4, z);
+    stage_states<MT, GEN>(S, cs, A, gdir, garm, nt, ca, h, y2, y3, y4, z);
     float *r = rec + (int64_t)j * W * n;
     put_stage<MT>(r, n, 0, S);
     put_stage<MT>(r, n, Y, y2);
@@ -701,9 +702,7 @@ __device__ __forceinline__ void produce_segment(const FleetView &fv, int64_t e,
     put_stage<MT>(r, n, 3 * Y, y4);
     for (int i = 0; i < 4; ++i) r[(int64_t)(4 * Y + i) * n] = z.q[i];
     if (j + 1 < len) {  // the next start state, as the forward computed it
-      float b[MT];
-      lag_segment<MT>(c, L, b);
-      fwd_step<MT, GEN>(S, b, L, A, gdir, garm, nt, ca, h);
+      fwd_step<MT, GEN>(S, c, L, A, gdir, garm, nt, ca, fv.rk);
     }
   }
 }
@@ -914,7 +913,6 @@ __global__ void __maxnreg__(XH ? kRegsXH : DIAG ? kRegsWide : kRegsGeneral)
   const int64_t n = fv.n;
   const int nt = MIXED ? bd.n_thr : MT;
   const bool current_accel = !(fv.model_flags & MG_MODEL_NO_CURRENT_ACCEL);
-  const float h = fv.dt;
   const float *xh = XH ? sxh + threadIdx.x * MG_NXPARAM : nullptr;
 
   St<MT> s;
@@ -928,23 +926,17 @@ __global__ void __maxnreg__(XH ? kRegsXH : DIAG ? kRegsWide : kRegsGeneral)
   const int64_t step0 = s_cursor + fv.cursor_off;
   int64_t seg = step0 / fv.hold;
   int32_t left = fv.hold - (int32_t)(step0 - seg * fv.hold);
-  const LagEnv L = lag_env(P.itau, h);
-  float b[MT];
-  {
-    float c[MT];
-    load_commands<MT>(fv, e, seg, nt, P.itau, c);
-    lag_segment<MT>(c, L, b);
-  }
+  const LagEnv L = lag_env(P.itau, fv.dt);
+  float c[MT];
+  load_commands<MT>(fv, e, seg, nt, c);
   for (int32_t it = 0; it < T; ++it) {
     if (it % C == 0) write_checkpoint<MT>(ckpt + (int64_t)(it / C) * MG_NSTATE * n, n, e, s);
     if (left == 0) {
       ++seg;
       left = fv.hold;
-      float c[MT];
-      load_commands<MT>(fv, e, seg, nt, P.itau, c);
-      lag_segment<MT>(c, L, b);
+      load_commands<MT>(fv, e, seg, nt, c);
     }
-    rk4_step_lag<MT, DIAG, MIXED, NH, XH>(s, b, L, P, sdir, sarm, nt, current_accel, h, xh);
+    rk4_step<MT, DIAG, MIXED, NH, XH>(s, c, L, P, sdir, sarm, nt, current_accel, fv.rk, xh);
     --left;
     record<MT>(traj + (int64_t)it * MG_NTRAJ * n, n, e, s);
   }

@@ -270,6 +270,7 @@ struct mg_sim {
     v.proc = proc;
     v.model_flags = model_flags;
     v.dt = dt;
+    v.rk = rk_step(dt);
     v.flags = flags;
     v.counters = counters;
     v.xh = has_xh ? xh : nullptr;

@@ -327,8 +327,8 @@ __device__ __forceinline__ void store_state(const StatePlanes &sp, int64_t e, co
 
 // ---------------------------------------------------------------- right-hand side of Eq. 1
 // d = f(s; c) with two storage conventions that save multiplies in the hot loop:
-//   - cs[i] = c_i / tau_m (the command pre-divided by the lag constant once per segment), so
-//     n_i' = cs_i - n_i / tau_m is a single FMA;
+//   - cs[i] = c_i / tau_m (the command divided by the lag constant by the caller), so
+//     n_i' = cs_i - n_i / tau_m is a single FMA (LAGD only);
 //   - d.q holds 2 q' (the 1/2 of q' = 1/2 q (x) (0, w) is folded into the RK4 weights).
 // Every sum is written as a chain of FMAs (same terms as Eq. 1; only the rounding order differs
 // from a term-by-term evaluation).  The diagonal-mass path reads the StepDiag coefficients (each
@@ -570,11 +570,11 @@ __device__ __forceinline__ void rhs(const St<MT> &s, const float (&cs)[MT], cons
   d.q[3] = fmaf(qw, w2, fmaf(qx, w1, -qy * w0));
 }
 
-// y = x + a k, with the quaternion taking a / 2 (its derivative is stored doubled).  WN = false
-// leaves the throttle states alone.
+// y = x + a k, with the quaternion taking aq = a / 2 (its derivative is stored doubled).  WN =
+// false leaves the throttle states alone.
 template <int MT, bool WN = true>
-__device__ __forceinline__ void axpy(St<MT> &y, const St<MT> &x, float a, const St<MT> &k) {
-  const float aq = 0.5f * a;
+__device__ __forceinline__ void axpy(St<MT> &y, const St<MT> &x, float a, float aq,
+                                     const St<MT> &k) {
 #pragma unroll
   for (int i = 0; i < 3; ++i) {
     y.p[i] = fmaf(a, k.p[i], x.p[i]);
@@ -590,89 +590,58 @@ __device__ __forceinline__ void axpy(St<MT> &y, const St<MT> &x, float a, const 
 }
 
 // The throttle lag n' = (c - n) / tau_m is linear with the command held, so RK4 applied to it has
-// closed forms: with g2 = -h / (2 tau_m), g3 = -h / tau_m and b = (h/2) c / tau_m the stage
-// values are y2 = n + g2 n + b, y3 = n + g2 y2 + b, y4 = n + g3 y3 + 2 b, and the step gives
-// n+ = P n + (1 - P) c with P = 1 + z + z^2/2 + z^3/6 + z^4/24, z = g3 (RK4's stability
-// polynomial) — the same numbers as RK4's stage updates and weighted sum, in 6 operations per
-// thruster instead of 11.
+// closed forms in the deviation d = n - c: with z = -h / tau_m the stage values are c + f2 d, c +
+// f3 d and c + f4 d, f2 = 1 + z/2, f3 = 1 + z/2 + z^2/4, f4 = 1 + z + z^2/2 + z^3/4, and the step
+// gives c + P d, P = 1 + z + z^2/2 + z^3/6 + z^4/24 (RK4's stability polynomial) — the same numbers
+// as RK4's stage updates and weighted sum, in 5 operations per thruster instead of 11 (a form in n
+// and h c / tau_m takes 7).  With the RK4 weights as kernel parameters (RkStep), against that form
+// and weights in registers: 65,536 envs x 1,000 sub-steps, whole episodes, 1,459 -> 1,326 us;
+// 1,048,576 x 100 2,194 -> 2,027; 262,144 mixed x 500 2,888 -> 2,649.
 struct LagEnv {
-  float g2, g3, P, lambda, hh;  // lambda = (1 - P) / (g2 tau_m): (1 - P) c = lambda b; hh = h/2
+  float f2, f3, f4, P;
 };
 
 __device__ __forceinline__ LagEnv lag_env(float itau, float h) {
   LagEnv L;
-  L.hh = 0.5f * h;
-  L.g3 = -h * itau;
-  L.g2 = 0.5f * L.g3;
-  const float z = L.g3;
+  const float z = -h * itau;
+  L.f2 = fmaf(0.5f, z, 1.f);
+  L.f3 = fmaf(fmaf(0.25f, z, 0.5f), z, 1.f);
+  L.f4 = fmaf(fmaf(fmaf(0.25f, z, 0.5f), z, 1.f), z, 1.f);
   L.P = fmaf(fmaf(fmaf(fmaf(z, 1.f / 24.f, 1.f / 6.f), z, 0.5f), z, 1.f), z, 1.f);
-  L.lambda = (1.f - L.P) / (L.hh * itau);
   return L;
 }
 
-// Per command segment: b_i = (h/2) c_i / tau_m from cs_i = c_i / tau_m.
-template <int MT>
-__device__ __forceinline__ void lag_segment(const float (&cs)[MT], const LagEnv &L,
-                                            float (&b)[MT]) {
-#pragma unroll
-  for (int i = 0; i < MT; ++i) b[i] = L.hh * cs[i];
-}
-
-// One sub-step (§METHOD): classical RK4 of size h, command held (cs = c / tau_m), then
-// q <- q / |q|.
+// One sub-step (§METHOD): classical RK4 of size rk.h with the command c held, the throttle lag in
+// its closed forms, then q <- q / |q|.
 template <int MT, bool DIAG, bool MIXED, int NH = 0, bool XH = false>
-__device__ __forceinline__ void rk4_step(St<MT> &s, const float (&cs)[MT], const Coef<DIAG, NH> &P,
-                                         const float4 *gdir, const float4 *garm, int nt,
-                                         bool current_accel, float h,
+__device__ __forceinline__ void rk4_step(St<MT> &s, const float (&c)[MT], const LagEnv &L,
+                                         const Coef<DIAG, NH> &P, const float4 *gdir,
+                                         const float4 *garm, int nt, bool current_accel,
+                                         const RkStep &rk,
                                          const float *__restrict__ xh = nullptr) {
-  const float hh = 0.5f * h, h3 = h * (1.0f / 3.0f), h6 = h * (1.0f / 6.0f);
   St<MT> k, y, acc;
-  rhs<MT, DIAG, MIXED, NH, XH>(s, cs, P, gdir, garm, nt, current_accel, k, xh);
-  axpy(acc, s, h6, k);
-  axpy(y, s, hh, k);
-  rhs<MT, DIAG, MIXED, NH, XH>(y, cs, P, gdir, garm, nt, current_accel, k, xh);
-  axpy(acc, acc, h3, k);
-  axpy(y, s, hh, k);
-  rhs<MT, DIAG, MIXED, NH, XH>(y, cs, P, gdir, garm, nt, current_accel, k, xh);
-  axpy(acc, acc, h3, k);
-  axpy(y, s, h, k);
-  rhs<MT, DIAG, MIXED, NH, XH>(y, cs, P, gdir, garm, nt, current_accel, k, xh);
-  axpy(s, acc, h6, k);
-  const float inv = rsqrtf(fmaf(s.q[0], s.q[0], fmaf(s.q[1], s.q[1],
-                                fmaf(s.q[2], s.q[2], s.q[3] * s.q[3]))));
+  float d[MT];
 #pragma unroll
-  for (int i = 0; i < 4; ++i) s.q[i] *= inv;
-}
-
-// One sub-step as rk4_step, with the throttle lag in the closed forms above (b from lag_segment
-// for the held command; e = (1 - P) c recovered as lambda b).  Same RK4, different rounding of
-// the lag state.
-template <int MT, bool DIAG, bool MIXED, int NH = 0, bool XH = false>
-__device__ __forceinline__ void rk4_step_lag(St<MT> &s, const float (&b)[MT], const LagEnv &L,
-                                             const Coef<DIAG, NH> &P, const float4 *gdir,
-                                             const float4 *garm, int nt, bool current_accel,
-                                             float h, const float *__restrict__ xh = nullptr) {
-  const float hh = 0.5f * h, h3 = h * (1.0f / 3.0f), h6 = h * (1.0f / 6.0f);
-  St<MT> k, y, acc;
-  rhs<MT, DIAG, MIXED, NH, XH, false>(s, b, P, gdir, garm, nt, current_accel, k, xh);
-  axpy<MT, false>(acc, s, h6, k);
-  axpy<MT, false>(y, s, hh, k);
+  for (int i = 0; i < MT; ++i) d[i] = s.n[i] - c[i];
+  rhs<MT, DIAG, MIXED, NH, XH, false>(s, c, P, gdir, garm, nt, current_accel, k, xh);
+  axpy<MT, false>(acc, s, rk.h6, rk.q12, k);
+  axpy<MT, false>(y, s, rk.hh, rk.qh, k);
 #pragma unroll
-  for (int i = 0; i < MT; ++i) y.n[i] = fmaf(L.g2, s.n[i], s.n[i] + b[i]);
-  rhs<MT, DIAG, MIXED, NH, XH, false>(y, b, P, gdir, garm, nt, current_accel, k, xh);
-  axpy<MT, false>(acc, acc, h3, k);
-  axpy<MT, false>(y, s, hh, k);
+  for (int i = 0; i < MT; ++i) y.n[i] = fmaf(L.f2, d[i], c[i]);
+  rhs<MT, DIAG, MIXED, NH, XH, false>(y, c, P, gdir, garm, nt, current_accel, k, xh);
+  axpy<MT, false>(acc, acc, rk.h3, rk.h6, k);
+  axpy<MT, false>(y, s, rk.hh, rk.qh, k);
 #pragma unroll
-  for (int i = 0; i < MT; ++i) y.n[i] = fmaf(L.g2, y.n[i], s.n[i] + b[i]);
-  rhs<MT, DIAG, MIXED, NH, XH, false>(y, b, P, gdir, garm, nt, current_accel, k, xh);
-  axpy<MT, false>(acc, acc, h3, k);
-  axpy<MT, false>(y, s, h, k);
+  for (int i = 0; i < MT; ++i) y.n[i] = fmaf(L.f3, d[i], c[i]);
+  rhs<MT, DIAG, MIXED, NH, XH, false>(y, c, P, gdir, garm, nt, current_accel, k, xh);
+  axpy<MT, false>(acc, acc, rk.h3, rk.h6, k);
+  axpy<MT, false>(y, s, rk.h, rk.hh, k);
 #pragma unroll
-  for (int i = 0; i < MT; ++i) y.n[i] = fmaf(L.g3, y.n[i], fmaf(2.f, b[i], s.n[i]));
-  rhs<MT, DIAG, MIXED, NH, XH, false>(y, b, P, gdir, garm, nt, current_accel, k, xh);
-  axpy<MT, false>(s, acc, h6, k);
+  for (int i = 0; i < MT; ++i) y.n[i] = fmaf(L.f4, d[i], c[i]);
+  rhs<MT, DIAG, MIXED, NH, XH, false>(y, c, P, gdir, garm, nt, current_accel, k, xh);
+  axpy<MT, false>(s, acc, rk.h6, rk.q12, k);
 #pragma unroll
-  for (int i = 0; i < MT; ++i) s.n[i] = fmaf(L.P, s.n[i], L.lambda * b[i]);
+  for (int i = 0; i < MT; ++i) s.n[i] = fmaf(L.P, d[i], c[i]);
   const float inv = rsqrtf(fmaf(s.q[0], s.q[0], fmaf(s.q[1], s.q[1],
                                 fmaf(s.q[2], s.q[2], s.q[3] * s.q[3]))));
 #pragma unroll

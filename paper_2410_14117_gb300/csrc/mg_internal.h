@@ -70,6 +70,24 @@ struct BlockDesc {
   int32_t n_thr;
 };
 
+// RK4's weights for sub-step size h.  They travel with the kernel parameters so that the stage
+// updates can take them as constant-bank operands: the step's issue rate is bound by register
+// operand reads, and a multiply-add with one constant reads two registers instead of three.
+struct RkStep {
+  float h, hh, h3, h6;  // h, h/2, h/3, h/6
+  float qh, q12;        // h/4 and h/12: the quaternion's halves of hh and h6 (its rate is doubled)
+};
+inline RkStep rk_step(float h) {
+  RkStep r;
+  r.h = h;
+  r.hh = 0.5f * h;
+  r.h3 = h * (1.0f / 3.0f);
+  r.h6 = h * (1.0f / 6.0f);
+  r.qh = 0.5f * r.hh;
+  r.q12 = 0.5f * r.h6;
+  return r;
+}
+
 // Everything a step kernel reads besides its block list; passed by value.
 struct FleetView {
   StatePlanes st;
@@ -86,6 +104,7 @@ struct FleetView {
   int32_t proc;
   uint32_t model_flags;
   float dt;
+  RkStep rk;                 // rk_step(dt)
   uint32_t *flags;           // [n] bit 0 = non-finite
   unsigned long long *counters;  // [0] envs flagged non-finite, [2] work-queue wait time-outs
   // Action cursor (sub-steps since the actions were set) in device memory: every step launch

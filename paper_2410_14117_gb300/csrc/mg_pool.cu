@@ -89,13 +89,11 @@ __global__ void __maxnreg__(XH ? kRegsXH : !DIAG ? kRegsGeneral : WIDE ? kRegsWi
   int64_t seg = jd.step0 / jd.hold;
   int32_t left = jd.hold - (int32_t)(jd.step0 - seg * jd.hold);
   const LagEnv L = lag_env(P.itau, fv.dt);
-  float lb[MT];
+  float c[MT];
   auto load = [&](int64_t sg) {
-    float c[MT];
     procedural_commands<MT>(jd.cmd_seed, (uint64_t)el, sg, c);
 #pragma unroll
-    for (int i = 0; i < MT; ++i) c[i] = (i < nt) ? c[i] * P.itau : 0.f;
-    lag_segment<MT>(c, L, lb);
+    for (int i = 0; i < MT; ++i) c[i] = (i < nt) ? c[i] : 0.f;
   };
   load(seg);
   for (int32_t it = 0; it < jd.steps; ++it) {
@@ -104,8 +102,8 @@ __global__ void __maxnreg__(XH ? kRegsXH : !DIAG ? kRegsGeneral : WIDE ? kRegsWi
       left = jd.hold;
       load(seg);
     }
-    rk4_step_lag<MT, DIAG, true, NH, XH>(s, lb, L, P, sdir, sarm, nt, current_accel, fv.dt,
-                                         XH ? sxh + threadIdx.x * MG_NXPARAM : nullptr);
+    rk4_step<MT, DIAG, true, NH, XH>(s, c, L, P, sdir, sarm, nt, current_accel, fv.rk,
+                                     XH ? sxh + threadIdx.x * MG_NXPARAM : nullptr);
     --left;
     if (jd.traj) {
       float *t = jd.traj + ((int64_t)(jd.step0 + it) * MG_NTRAJ) * jd.n + el;
@@ -234,6 +232,7 @@ FleetView pool_view(const mg_pool *p) {
   v.n_types = p->n_types;
   v.n = p->cap;
   v.dt = p->dt;
+  v.rk = rk_step(p->dt);
   v.flags = p->flags;
   v.counters = p->counters;
   v.hold = 1;

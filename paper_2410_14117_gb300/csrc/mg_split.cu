@@ -71,7 +71,7 @@ __device__ __forceinline__ void sym6_apply(const float d[6], const float *__rest
 }
 
 // One split sub-step of env state s with acceleration memory a (updated in place).  cs: the
-// held command divided by tau_m (as load_commands returns it).  GEN: xh is the env's extension
+// held command divided by tau_m.  GEN: xh is the env's extension
 // record (MG_NXPARAM floats; zeros for an env without one).
 template <int MT, bool GEN>
 __device__ __forceinline__ void split_substep(St<MT> &s, float (&a)[6], const float (&cs)[MT],
@@ -284,13 +284,18 @@ __global__ void __launch_bounds__(256)
   const int64_t step0 = s_cursor + fv.cursor_off;
   int64_t seg = step0 / fv.hold;
   int32_t left = fv.hold - (int32_t)(step0 - seg * fv.hold);
-  float c[MT];
-  load_commands<MT>(fv, e, seg, nt, P.itau, c);
+  float c[MT];  // the held command divided by tau_m
+  auto load = [&](int64_t sg) {
+    load_commands<MT>(fv, e, sg, nt, c);
+#pragma unroll
+    for (int i = 0; i < MT; ++i) c[i] *= P.itau;
+  };
+  load(seg);
   for (int32_t it = 0; it < k; ++it) {
     if (left == 0) {
       ++seg;
       left = fv.hold;
-      load_commands<MT>(fv, e, seg, nt, P.itau, c);
+      load(seg);
     }
     split_substep<MT, GEN>(s, a, c, P, sdir, sarm, nt, current_accel, fv.dt,
                            GEN ? sxh + threadIdx.x * MG_NXPARAM : nullptr);
