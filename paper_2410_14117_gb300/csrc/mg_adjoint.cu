@@ -2,23 +2,30 @@
 // respect to each env's hydrodynamic coefficients (added mass, linear and quadratic damping
 // diagonals of Eq. 1) and to the buffered throttle actions (Eq. 3).
 //
-// The forward pass (k_fleet with recording) writes the state after every sub-step; the
-// checkpoint kernel below saves the full state every C sub-steps.  The backward kernel runs one
-// thread per env: for each checkpoint segment, last first, it re-runs the segment's sub-steps
-// from the checkpoint (keeping the C step-start states in local memory), then walks them in
-// reverse, applying the transpose Jacobian of one sub-step
+// The forward pass (k_rollout_fwd) writes the state after every sub-step and the full state every
+// C sub-steps.  The backward kernels, one env per lane: for each checkpoint segment, last first,
+// the segment's sub-steps are re-run from the checkpoint, then walked in reverse, applying the
+// transpose Jacobian of one sub-step
 //     s+ = N(s + h/6 (k1 + 2 k2 + 2 k3 + k4)),  N = quaternion renormalisation,
 // through N, the RK4 combination and the four right-hand-side evaluations (reverse mode of
 // rhs(), written out below).  It is the adjoint of the discrete map the forward computes, so it
 // matches finite differences of the rollout itself, not of the continuous equations.
 //
-// Two parameter paths, as the forward has:
-//   - diagonal mass (r_g = 0, no off-diagonal extension): M^-1 = diag(1 / M_jj);
-//   - general (GEN): off-centre gravity (the m r_g coupling of M_RB and C_RB, off-diagonal
-//     I_o) and the off-diagonal added mass and linear damping of the extension record (zeros
-//     when the fleet has none), with the full M^-1.  A diagonal coefficient theta = M_A,jj enters
-//     M = M_RB + M_A, so nu' = M^-1 f gets d nu'/d theta = -M^-1 e_j nu'_j, whose contribution to
-//     the gradient is -(M^-1 g)_j nu'_j for the loss adjoint g of nu' (M^-1 is symmetric).
+// The throttle lag is linear with the command held (LagEnv): the stage throttles are c + f_i d
+// with d = n - c and the step gives c + P d.  So with e_i the adjoint of stage i's throttle
+// through the thrust, the throttle's own adjoint goes lambda_n <- P lambda_n + sum f_i e_i and the
+// command's gains (1 - P) lambda_n + sum (1 - f_i) e_i (f_1 = 1); the throttles stay out of the
+// stage combinations.
+//
+// Parameter paths, as the forward has:
+//   - diagonal mass (r_g = 0, no off-diagonal extension): rhs_vjp_diag, the transpose of the step's
+//     own coefficient form (StepDiag, or StepMirrored with its thrust sums);
+//   - general (GEN): rhs_vjp_gen, off-centre gravity (the m r_g coupling of M_RB and C_RB,
+//     off-diagonal I_o) and the off-diagonal added mass and linear damping of the extension record
+//     (zeros when the fleet has none), with the full M^-1.
+// A diagonal coefficient theta = M_A,jj enters M = M_RB + M_A, so nu' = M^-1 f gets d nu'/d theta =
+// -M^-1 e_j nu'_j, whose contribution to the gradient is -(M^-1 g)_j nu'_j for the loss adjoint g of
+// nu' (M^-1 is symmetric).  nu' itself comes recorded with the stage states.
 #include <type_traits>
 
 #include "mg_advance.cuh"
@@ -29,18 +36,45 @@ namespace {
 
 constexpr int kAdjThreads = 128;
 
-struct Grad {
-  float ma[3], J[3], mv[6], dl[6], dq[6];  // mv: the M_A,jj gradient through M^-1
-};
+// Which transpose a kernel is compiled for.
+enum AdjPath { ADJ_GEN = 0, ADJ_DENSE = 1, ADJ_MIRRORED = 2 };
 
-// What the adjoint reads for one env: the loaded parameters (transposes), the coefficients the
-// re-run steps with (the forward's, with the dense thruster allocation: equal to the forward's
-// states within the rounding of the allocation's sums) and, on the general path, the env's
-// off-diagonal hydrodynamic coefficients (a row of MG_NXPARAM floats in shared memory).
-template <bool GEN>
+// The thruster allocation of the re-run: the forward's (the vectored one only skips exact zeros of
+// the dense one, so the states are the forward's bit for bit either way).
+__host__ __device__ constexpr int adj_layout(int path) {
+  return path == ADJ_MIRRORED ? MG_LAYOUT_MIRRORED : MG_LAYOUT_DENSE;
+}
+
+// Sums over stages and sub-steps that the coefficient gradients are formed from at the end.
+// General path: the gradients themselves (mv: M_A,jj through M^-1).
+struct GradGen {
+  float ma[3], J[3], mv[6], dl[6], dq[6];
+};
+// Diagonal mass, with g the loss adjoint of nu' (trans/rotational rows i, i1 = i+1, i2 = i+2 mod 3):
+//   dl, dq   sum g_j x_j, sum g_j |x_j| x_j         (x = r, w)
+//   own      sum g_i (w_i2 c_i1 - w_i1 c_i2), c = v - r the current seen from the body
+//   up, dn   sum g_i w_i2 r_i1, sum g_i w_i1 r_i2
+//   munk     sum g_3+i r_i1 r_i2;  gyro  sum g_3+i w_i1 w_i2;  mv  sum g_j nu'_j
+struct GradDiag {
+  float dl[6], dq[6], own[3], up[3], dn[3], munk[3], gyro[3], mv[6];
+};
+template <int PATH>
+using Grad = typename std::conditional<PATH == ADJ_GEN, GradGen, GradDiag>::type;
+
+template <typename G>
+__device__ __forceinline__ void zero_grad(G &g) {
+  float *f = reinterpret_cast<float *>(&g);
+#pragma unroll
+  for (int i = 0; i < (int)(sizeof(G) / sizeof(float)); ++i) f[i] = 0.f;
+}
+
+// What the adjoint reads for one env: the coefficients the forward step used and, on the general
+// path, the env's off-diagonal hydrodynamic coefficients (a row of MG_NXPARAM floats in shared
+// memory).
+template <int PATH>
 struct AdjEnv {
-  Par<!GEN> P;
-  Coef<!GEN> F;
+  Coef<PATH != ADJ_GEN, adj_layout(PATH)> F;
+  LagEnv L;
   const float *xh;
 };
 
@@ -87,26 +121,23 @@ __device__ __forceinline__ void minv_apply(const ParGen &P, const float x[6], fl
          fmaf(o[14], x[4], P.mi[5] * x[5])))));
 }
 
-// gs += (d rhs / d s)^T gd; parameter and command adjoints accumulated into G and gcs.  The
-// forward quantities are recomputed from Eq. 1 in the general path's Kirchhoff form (the
-// diagonal-mass path drops the terms that vanish with r_g = 0 and diagonal M_A, D_l); gd.q is
-// the adjoint of d.q = q (x) (0, w) (the doubled quaternion rate rhs() stores).
-template <int MT, bool GEN>
-__device__ void rhs_vjp(const St<MT> &s, const float (&cs)[MT], const AdjEnv<GEN> &A,
-                        const float4 *gdir, const float4 *garm, int nt, bool current_accel,
-                        const St<MT> &gd, St<MT> &gs, Grad &G, float (&gcs)[MT]) {
-  const auto &P = A.P;
+// A rigid-body quantity of the transposes: the pose's and velocity's parts of a state adjoint.
+struct Body {
+  float p[3], q[4], v[3], w[3];
+};
+
+// gs = (d rhs / d s)^T gd for the pose and velocity of stage state s, with en[i] the adjoint of the
+// stage throttle n_i through the thrust and the coefficient sums accumulated into G; nud is the
+// stage's recorded nu'.  The forward quantities are recomputed from Eq. 1 in the general path's
+// Kirchhoff form; gd.q is the adjoint of d.q = q (x) (0, w) (the doubled quaternion rate rhs()
+// stores).
+template <int MT>
+__device__ void rhs_vjp_gen(const St<MT> &s, const float (&nud)[6], const AdjEnv<ADJ_GEN> &A,
+                            const float4 *gdir, const float4 *garm, int nt, bool current_accel,
+                            const Body &gd, Body &gs, GradGen &G, float (&en)[MT]) {
+  const auto &P = A.F;
   const float *xh = A.xh;
   // ---------------- forward recomputation
-  float t[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-  for (int i = 0; i < MT; ++i) {
-    if (i >= nt) continue;  // compile-time indices keep the arrays in registers
-    const float f = s.n[i] * fabsf(s.n[i]);
-    const float4 dd = gdir[i], aa = garm[i];
-    t[0] = fmaf(f, dd.x, t[0]); t[1] = fmaf(f, dd.y, t[1]); t[2] = fmaf(f, dd.z, t[2]);
-    t[3] = fmaf(f, aa.x, t[3]); t[4] = fmaf(f, aa.y, t[4]); t[5] = fmaf(f, aa.z, t[5]);
-  }
   const float qw = s.q[0], qx = s.q[1], qy = s.q[2], qz = s.q[3];
   float R[3][3];
   R[0][0] = fmaf(-2.f, fmaf(qy, qy, qz * qz), 1.f);
@@ -122,10 +153,7 @@ __device__ void rhs_vjp(const St<MT> &s, const float (&cs)[MT], const AdjEnv<GEN
   const float vc[3] = {P.vc0, P.vc1, P.vc2}, ma[3] = {P.ma0, P.ma1, P.ma2};
   const float J[3] = {P.J0, P.J1, P.J2}, G3[3] = {P.G0, P.G1, P.G2};
   float cb[3], r[3], qm[3], h[3], k[3], c[3] = {0.f, 0.f, 0.f}, am[3] = {0.f, 0.f, 0.f};
-  float mrg[3] = {0.f, 0.f, 0.f};
-  if constexpr (GEN) {
-    mrg[0] = P.mrg0; mrg[1] = P.mrg1; mrg[2] = P.mrg2;
-  }
+  const float mrg[3] = {P.mrg0, P.mrg1, P.mrg2};
   for (int i = 0; i < 3; ++i)
     cb[i] = fmaf(R[2][i], vc[2], fmaf(R[1][i], vc[1], R[0][i] * vc[0]));
   for (int i = 0; i < 3; ++i) {
@@ -134,22 +162,20 @@ __device__ void rhs_vjp(const St<MT> &s, const float (&cs)[MT], const AdjEnv<GEN
     k[i] = J[i] * w[i];
   }
   const float nur[6] = {r[0], r[1], r[2], w[0], w[1], w[2]};
-  if constexpr (GEN) {
-    // off-diagonal added mass in the momenta; w x m r_g; off-diagonal I_o w + m r_g x v
+  // off-diagonal added mass in the momenta; w x m r_g; off-diagonal I_o w + m r_g x v
 #pragma unroll
-    for (int i = 0; i < 3; ++i)
+  for (int i = 0; i < 3; ++i)
 #pragma unroll
-      for (int j = 0; j < 6; ++j) {
-        if (j != i) qm[i] = fmaf(xa(xh, i, j), nur[j], qm[i]);
-        if (j != 3 + i) k[i] = fmaf(xa(xh, 3 + i, j), nur[j], k[i]);
-      }
-    am[0] = fmaf(w[1], mrg[2], -w[2] * mrg[1]);
-    am[1] = fmaf(w[2], mrg[0], -w[0] * mrg[2]);
-    am[2] = fmaf(w[0], mrg[1], -w[1] * mrg[0]);
-    k[0] = fmaf(P.Ixy, w[1], fmaf(P.Ixz, w[2], fmaf(mrg[1], v[2], fmaf(-mrg[2], v[1], k[0]))));
-    k[1] = fmaf(P.Ixy, w[0], fmaf(P.Iyz, w[2], fmaf(mrg[2], v[0], fmaf(-mrg[0], v[2], k[1]))));
-    k[2] = fmaf(P.Ixz, w[0], fmaf(P.Iyz, w[1], fmaf(mrg[0], v[1], fmaf(-mrg[1], v[0], k[2]))));
-  }
+    for (int j = 0; j < 6; ++j) {
+      if (j != i) qm[i] = fmaf(xa(xh, i, j), nur[j], qm[i]);
+      if (j != 3 + i) k[i] = fmaf(xa(xh, 3 + i, j), nur[j], k[i]);
+    }
+  am[0] = fmaf(w[1], mrg[2], -w[2] * mrg[1]);
+  am[1] = fmaf(w[2], mrg[0], -w[0] * mrg[2]);
+  am[2] = fmaf(w[0], mrg[1], -w[1] * mrg[0]);
+  k[0] = fmaf(P.Ixy, w[1], fmaf(P.Ixz, w[2], fmaf(mrg[1], v[2], fmaf(-mrg[2], v[1], k[0]))));
+  k[1] = fmaf(P.Ixy, w[0], fmaf(P.Iyz, w[2], fmaf(mrg[2], v[0], fmaf(-mrg[0], v[2], k[1]))));
+  k[2] = fmaf(P.Ixz, w[0], fmaf(P.Iyz, w[1], fmaf(mrg[0], v[1], fmaf(-mrg[1], v[0], k[2]))));
   for (int i = 0; i < 3; ++i) h[i] = fmaf(P.m, v[i], qm[i]) + am[i];
   if (current_accel) {
     c[0] = fmaf(w[1], cb[2], -w[2] * cb[1]);
@@ -157,54 +183,12 @@ __device__ void rhs_vjp(const St<MT> &s, const float (&cs)[MT], const AdjEnv<GEN
     c[2] = fmaf(w[0], cb[1], -w[1] * cb[0]);
   }
   const float e[3] = {R[2][0], R[2][1], R[2][2]};
-  // translational: kT t + (W - B) e - w x h - (Dl + Dq |r|) r [- M_A [w x v_c^b; 0]]
-  //                [- off-diagonal D_l nu_r]
-  float f[6];
-  for (int i = 0; i < 3; ++i) {
-    const int i1 = (i + 1) % 3, i2 = (i + 2) % 3;
-    float x = fmaf(P.kT, t[i], P.wb * e[i]);
-    x = fmaf(-w[i1], h[i2], fmaf(w[i2], h[i1], x));
-    x = fmaf(-fmaf(P.dq[i], fabsf(r[i]), P.dl[i]), r[i], x);
-    f[i] = fmaf(-ma[i], c[i], x);
-  }
-  // rotational: kT t' - r x Q1 - w x k [- v x (w x m r_g)] - (Dl + Dq |w|) w + G x e
-  //             [- M_A [w x v_c^b; 0]] [- off-diagonal D_l nu_r]
-  for (int i = 0; i < 3; ++i) {
-    const int i1 = (i + 1) % 3, i2 = (i + 2) % 3;
-    float x = fmaf(P.kT, t[3 + i], fmaf(-r[i1], qm[i2], r[i2] * qm[i1]));
-    x = fmaf(-w[i1], k[i2], fmaf(w[i2], k[i1], x));
-    if constexpr (GEN) x = fmaf(-v[i1], am[i2], fmaf(v[i2], am[i1], x));
-    x = fmaf(-fmaf(P.dq[3 + i], fabsf(w[i]), P.dl[3 + i]), w[i], x);
-    f[3 + i] = fmaf(G3[i1], e[i2], fmaf(-G3[i2], e[i1], x));
-  }
-  if constexpr (GEN) {
-#pragma unroll
-    for (int i = 0; i < 6; ++i)
-#pragma unroll
-      for (int j = 0; j < 6; ++j) {
-        if (j < 3 && j != i) f[i] = fmaf(-xa(xh, i, j), c[j], f[i]);
-        if (j != i) f[i] = fmaf(-xd(xh, i, j), nur[j], f[i]);
-      }
-  }
-  float nud[6];  // nu' = M^-1 f
-  if constexpr (GEN) minv_apply(P, f, nud);
-  else
-    for (int j = 0; j < 6; ++j) nud[j] = P.mi[j] * f[j];
 
   // ---------------- reverse
-  // lag: d.n_i = cs_i - n_i / tau_m
-#pragma unroll
-  for (int i = 0; i < MT; ++i) {
-    if (i >= nt) continue;
-    gcs[i] += gd.n[i];
-    gs.n[i] = fmaf(-P.itau, gd.n[i], gs.n[i]);
-  }
   // nu' = M^-1 f: gf = M^-1 g (symmetric), and M_jj's share -gf_j nu'_j
   const float gnu[6] = {gd.v[0], gd.v[1], gd.v[2], gd.w[0], gd.w[1], gd.w[2]};
   float gf[6], gt[6];
-  if constexpr (GEN) minv_apply(P, gnu, gf);
-  else
-    for (int j = 0; j < 6; ++j) gf[j] = P.mi[j] * gnu[j];
+  minv_apply(P, gnu, gf);
   for (int j = 0; j < 6; ++j) {
     G.mv[j] = fmaf(-gf[j], nud[j], G.mv[j]);
     gt[j] = P.kT * gf[j];
@@ -213,22 +197,20 @@ __device__ void rhs_vjp(const St<MT> &s, const float (&cs)[MT], const AdjEnv<GEN
   float gh[3] = {0.f, 0.f, 0.f}, gk[3] = {0.f, 0.f, 0.f}, gqm[3] = {0.f, 0.f, 0.f};
   float gcb[3] = {0.f, 0.f, 0.f}, ge[3] = {0.f, 0.f, 0.f}, gc[3] = {0.f, 0.f, 0.f};
   float gam[3] = {0.f, 0.f, 0.f}, gnur[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-  if constexpr (GEN) {
-    // off-diagonal current term and linear damping
+  // off-diagonal current term and linear damping
 #pragma unroll
-    for (int i = 0; i < 6; ++i)
+  for (int i = 0; i < 6; ++i)
 #pragma unroll
-      for (int j = 0; j < 6; ++j) {
-        if (j < 3 && j != i) gc[j] = fmaf(-xa(xh, i, j), gf[i], gc[j]);
-        if (j != i) gnur[j] = fmaf(-xd(xh, i, j), gf[i], gnur[j]);
-      }
-  }
+    for (int j = 0; j < 6; ++j) {
+      if (j < 3 && j != i) gc[j] = fmaf(-xa(xh, i, j), gf[i], gc[j]);
+      if (j != i) gnur[j] = fmaf(-xd(xh, i, j), gf[i], gnur[j]);
+    }
   // rotational force
   const float gfr[3] = {gf[3], gf[4], gf[5]};
   const float ngfr[3] = {-gf[3], -gf[4], -gf[5]};
   cross_vjp(r, qm, ngfr, gr, gqm);   // - r x Q1
   cross_vjp(w, k, ngfr, gw, gk);     // - w x k
-  if constexpr (GEN) cross_vjp(v, am, ngfr, gv, gam);  // - v x (w x m r_g)
+  cross_vjp(v, am, ngfr, gv, gam);  // - v x (w x m r_g)
   for (int j = 0; j < 3; ++j) {
     const float aw = fabsf(w[j]);
     gw[j] = fmaf(-fmaf(2.f * P.dq[3 + j], aw, P.dl[3 + j]), gfr[j], gw[j]);
@@ -257,26 +239,24 @@ __device__ void rhs_vjp(const St<MT> &s, const float (&cs)[MT], const AdjEnv<GEN
     }
     cross_vjp(w, cb, gc, gw, gcb);   // c = w x v_c^b
   }
-  if constexpr (GEN) {
-    // k += off-diagonal I_o w + m r_g x v;  h += w x m r_g
-    gw[0] = fmaf(P.Ixy, gk[1], fmaf(P.Ixz, gk[2], gw[0]));
-    gw[1] = fmaf(P.Ixy, gk[0], fmaf(P.Iyz, gk[2], gw[1]));
-    gw[2] = fmaf(P.Ixz, gk[0], fmaf(P.Iyz, gk[1], gw[2]));
-    gv[0] = fmaf(gk[1], mrg[2], fmaf(-gk[2], mrg[1], gv[0]));
-    gv[1] = fmaf(gk[2], mrg[0], fmaf(-gk[0], mrg[2], gv[1]));
-    gv[2] = fmaf(gk[0], mrg[1], fmaf(-gk[1], mrg[0], gv[2]));
-    for (int j = 0; j < 3; ++j) gam[j] += gh[j];
-    float gmrg[3] = {0.f, 0.f, 0.f};
-    cross_vjp(w, mrg, gam, gw, gmrg);
-    // off-diagonal added mass in the momenta (Q1 enters through h and through r x Q1)
+  // k += off-diagonal I_o w + m r_g x v;  h += w x m r_g
+  gw[0] = fmaf(P.Ixy, gk[1], fmaf(P.Ixz, gk[2], gw[0]));
+  gw[1] = fmaf(P.Ixy, gk[0], fmaf(P.Iyz, gk[2], gw[1]));
+  gw[2] = fmaf(P.Ixz, gk[0], fmaf(P.Iyz, gk[1], gw[2]));
+  gv[0] = fmaf(gk[1], mrg[2], fmaf(-gk[2], mrg[1], gv[0]));
+  gv[1] = fmaf(gk[2], mrg[0], fmaf(-gk[0], mrg[2], gv[1]));
+  gv[2] = fmaf(gk[0], mrg[1], fmaf(-gk[1], mrg[0], gv[2]));
+  for (int j = 0; j < 3; ++j) gam[j] += gh[j];
+  float gmrg[3] = {0.f, 0.f, 0.f};
+  cross_vjp(w, mrg, gam, gw, gmrg);
+  // off-diagonal added mass in the momenta (Q1 enters through h and through r x Q1)
 #pragma unroll
-    for (int i = 0; i < 3; ++i)
+  for (int i = 0; i < 3; ++i)
 #pragma unroll
-      for (int j = 0; j < 6; ++j) {
-        if (j != i) gnur[j] = fmaf(xa(xh, i, j), gqm[i] + gh[i], gnur[j]);
-        if (j != 3 + i) gnur[j] = fmaf(xa(xh, 3 + i, j), gk[i], gnur[j]);
-      }
-  }
+    for (int j = 0; j < 6; ++j) {
+      if (j != i) gnur[j] = fmaf(xa(xh, i, j), gqm[i] + gh[i], gnur[j]);
+      if (j != 3 + i) gnur[j] = fmaf(xa(xh, 3 + i, j), gk[i], gnur[j]);
+    }
   // k = J w, h = m v + Q1, Q1 = M_A r, r = v - v_c^b
   for (int j = 0; j < 3; ++j) {
     gw[j] = fmaf(J[j], gk[j], gw[j]);
@@ -326,161 +306,291 @@ __device__ void rhs_vjp(const St<MT> &s, const float (&cs)[MT], const AdjEnv<GEN
   // thrust: t = sum_i n_i|n_i| b_i
 #pragma unroll
   for (int i = 0; i < MT; ++i) {
+    en[i] = 0.f;
     if (i >= nt) continue;
     const float4 dd = gdir[i], aa = garm[i];
     const float gfi = fmaf(dd.x, gt[0], fmaf(dd.y, gt[1], fmaf(dd.z, gt[2],
                       fmaf(aa.x, gt[3], fmaf(aa.y, gt[4], aa.z * gt[5])))));
-    gs.n[i] = fmaf(2.f * fabsf(s.n[i]), gfi, gs.n[i]);
+    en[i] = 2.f * fabsf(s.n[i]) * gfi;
   }
-  for (int i = 0; i < 4; ++i) gs.q[i] += gq[i];
+  for (int i = 0; i < 4; ++i) gs.q[i] = gq[i];
   for (int i = 0; i < 3; ++i) {
-    gs.v[i] += gv[i];
-    gs.w[i] += gw[i];
+    gs.v[i] = gv[i];
+    gs.w[i] = gw[i];
   }
 }
 
-// y = x + a W k with W the rk4 weighting (the quaternion takes half of each weight because
-// rhs() stores its rate doubled):  out = a W x  or  out += a W x.
-template <int MT>
-__device__ __forceinline__ void wscale(St<MT> &out, const St<MT> &x, float a, bool add) {
-  const float aq = 0.5f * a;
-  for (int i = 0; i < 3; ++i) out.p[i] = add ? fmaf(a, x.p[i], out.p[i]) : a * x.p[i];
-  for (int i = 0; i < 4; ++i) out.q[i] = add ? fmaf(aq, x.q[i], out.q[i]) : aq * x.q[i];
-  for (int i = 0; i < 3; ++i) out.v[i] = add ? fmaf(a, x.v[i], out.v[i]) : a * x.v[i];
-  for (int i = 0; i < 3; ++i) out.w[i] = add ? fmaf(a, x.w[i], out.w[i]) : a * x.w[i];
-  for (int i = 0; i < MT; ++i) out.n[i] = add ? fmaf(a, x.n[i], out.n[i]) : a * x.n[i];
+// The transpose of the diagonal-mass right-hand side (rhs with StepDiag or StepMirrored): gs = (d
+// rhs / d s)^T gd for the pose and velocity, en[i] the adjoint of the stage throttle n_i through
+// the thrust, the sums of GradDiag accumulated.  With u_i = v_i1 + bp_i r_i1, x_i = v_i2 + bm_i r_i2
+// the rows are v'_i = ... + w_i2 u_i - w_i1 x_i - (dlt_i + dqt_i |r_i|) r_i and w'_i = ... + B_i r_i1
+// r_i2 + C_i w_i1 w_i2 - (dlr_i + dqr_i |w_i|) w_i.  About 290 operations a stage where the general
+// path's form of the same transpose (which this path used before) takes some 700: the consumer
+// warp of the two-warp kernel, a chain of these, is what bounds a small fleet's backward pass: 4,096
+// envs x 200 sub-steps 918 -> 330 us together with the re-run's single evaluation of each sub-step
+// and the 16-byte records (ncu: 2,390 instead of 4,580 instructions a sub-step in the two warps).
+template <int MT, int PATH>
+__device__ __forceinline__ void rhs_vjp_diag(const St<MT> &s, const float (&nud)[6],
+                                             const AdjEnv<PATH> &A, const float4 *gdir,
+                                             const float4 *garm, int nt, const Body &gd, Body &gs,
+                                             GradDiag &G, float (&en)[MT]) {
+  const auto &P = A.F;
+  const float qw = s.q[0], qx = s.q[1], qy = s.q[2], qz = s.q[3];
+  float R[3][3];
+  {
+    const float tx = qx + qx, ty = qy + qy, tz = qz + qz;
+    const float zd = fmaf(-qz, tz, 1.f), xy = qx * ty, xz = qx * tz, yz = qy * tz;
+    R[0][0] = fmaf(-qy, ty, zd);
+    R[1][1] = fmaf(-qx, tx, zd);
+    R[2][2] = fmaf(-qx, tx, fmaf(-qy, ty, 1.f));
+    R[0][1] = fmaf(-qw, tz, xy);
+    R[1][0] = fmaf(qw, tz, xy);
+    R[0][2] = fmaf(qw, ty, xz);
+    R[2][0] = fmaf(-qw, ty, xz);
+    R[1][2] = fmaf(-qw, tx, yz);
+    R[2][1] = fmaf(qw, tx, yz);
+  }
+  const float v[3] = {s.v[0], s.v[1], s.v[2]}, w[3] = {s.w[0], s.w[1], s.w[2]};
+  const float vc[3] = {P.vc0, P.vc1, P.vc2};
+  const float gv[3] = {gd.v[0], gd.v[1], gd.v[2]}, gw[3] = {gd.w[0], gd.w[1], gd.w[2]};
+  float cb[3], r[3], gr[3], ov[3], ow[3] = {0.f, 0.f, 0.f};  // ov, ow: adjoints of v, w
+#pragma unroll
+  for (int j = 0; j < 3; ++j) {
+    cb[j] = fmaf(R[2][j], vc[2], fmaf(R[1][j], vc[1], R[0][j] * vc[0]));
+    r[j] = v[j] - cb[j];
+  }
+  // damping
+#pragma unroll
+  for (int j = 0; j < 3; ++j) {
+    const float ar = fabsf(r[j]), aw = fabsf(w[j]);
+    const float hr = gv[j] * r[j], hw = gw[j] * w[j];
+    G.dl[j] += hr;
+    G.dl[3 + j] += hw;
+    G.dq[j] = fmaf(ar, hr, G.dq[j]);
+    G.dq[3 + j] = fmaf(aw, hw, G.dq[3 + j]);
+    gr[j] = -fmaf(P.dqt[j], ar + ar, P.dlt[j]) * gv[j];
+    ow[j] = -fmaf(P.dqr[j], aw + aw, P.dlr[j]) * gw[j];
+    G.mv[j] = fmaf(gv[j], nud[j], G.mv[j]);
+    G.mv[3 + j] = fmaf(gw[j], nud[3 + j], G.mv[3 + j]);
+    ov[j] = 0.f;
+  }
+  // translational Coriolis terms, Munk and gyroscopic products
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    const int i1 = (i + 1) % 3, i2 = (i + 2) % 3;
+    const float u = fmaf(P.bp[i], r[i1], v[i1]), x = fmaf(P.bm[i], r[i2], v[i2]);
+    const float gu = gv[i] * w[i2], gx = gv[i] * w[i1];  // adjoints of u_i and -x_i
+    ow[i2] = fmaf(gv[i], u, ow[i2]);
+    ow[i1] = fmaf(-gv[i], x, ow[i1]);
+    ov[i1] += gu;
+    ov[i2] -= gx;
+    gr[i1] = fmaf(P.bp[i], gu, gr[i1]);
+    gr[i2] = fmaf(-P.bm[i], gx, gr[i2]);
+    G.up[i] = fmaf(gu, r[i1], G.up[i]);
+    G.dn[i] = fmaf(gx, r[i2], G.dn[i]);
+    G.own[i] = fmaf(gu, cb[i1], fmaf(-gx, cb[i2], G.own[i]));
+    const float gm = gw[i] * r[i1], gg = gw[i] * w[i1];
+    G.munk[i] = fmaf(gm, r[i2], G.munk[i]);
+    G.gyro[i] = fmaf(gg, w[i2], G.gyro[i]);
+    gr[i2] = fmaf(P.B[i], gm, gr[i2]);
+    gr[i1] = fmaf(P.B[i] * gw[i], r[i2], gr[i1]);
+    ow[i2] = fmaf(P.C[i], gg, ow[i2]);
+    ow[i1] = fmaf(P.C[i] * gw[i], w[i2], ow[i1]);
+  }
+  // R: p' = R v, r = v - R^T v_c, (W - B) k_e and G x k_e with k_e the third row
+  float gR[3][3];
+#pragma unroll
+  for (int i = 0; i < 3; ++i)
+#pragma unroll
+    for (int j = 0; j < 3; ++j) gR[i][j] = fmaf(-vc[i], gr[j], gd.p[i] * v[j]);
+#pragma unroll
+  for (int j = 0; j < 3; ++j) {
+    gR[2][j] = fmaf(P.Wt[j], gv[j], gR[2][j]);
+    ov[j] += gr[j];
+    gs.v[j] = fmaf(R[0][j], gd.p[0], fmaf(R[1][j], gd.p[1], fmaf(R[2][j], gd.p[2], ov[j])));
+  }
+  if constexpr (PATH == ADJ_MIRRORED) {
+    gR[2][1] = fmaf(-P.Gr, gw[0], gR[2][1]);
+    gR[2][0] = fmaf(P.Gp, gw[1], gR[2][0]);
+  } else {
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      const int i1 = (i + 1) % 3, i2 = (i + 2) % 3;
+      gR[2][i2] = fmaf(P.Gp[i], gw[i], gR[2][i2]);
+      gR[2][i1] = fmaf(-P.Gm[i], gw[i], gR[2][i1]);
+    }
+  }
+  // d.q = q (x) (0, w)
+  const float g0 = gd.q[0], g1 = gd.q[1], g2 = gd.q[2], g3 = gd.q[3];
+  gs.w[0] = fmaf(-qx, g0, fmaf(qw, g1, fmaf(qz, g2, fmaf(-qy, g3, ow[0]))));
+  gs.w[1] = fmaf(-qy, g0, fmaf(-qz, g1, fmaf(qw, g2, fmaf(qx, g3, ow[1]))));
+  gs.w[2] = fmaf(-qz, g0, fmaf(qy, g1, fmaf(-qx, g2, fmaf(qw, g3, ow[2]))));
+  // R(q) -> q: the antisymmetric and symmetric parts of gR
+  {
+    const float a0 = gR[2][1] - gR[1][2], a1 = gR[0][2] - gR[2][0], a2 = gR[1][0] - gR[0][1];
+    const float b0 = gR[2][1] + gR[1][2], b1 = gR[0][2] + gR[2][0], b2 = gR[1][0] + gR[0][1];
+    const float d0 = gR[1][1] + gR[2][2], d1 = gR[0][0] + gR[2][2], d2 = gR[0][0] + gR[1][1];
+    const float m0 = -2.f * d0, m1 = -2.f * d1, m2 = -2.f * d2;
+    const float s0 = fmaf(qx, a0, fmaf(qy, a1, qz * a2));
+    const float s1 = fmaf(qw, a0, fmaf(qy, b2, fmaf(qz, b1, qx * m0)));
+    const float s2 = fmaf(qw, a1, fmaf(qx, b2, fmaf(qz, b0, qy * m1)));
+    const float s3 = fmaf(qw, a2, fmaf(qx, b1, fmaf(qy, b0, qz * m2)));
+    gs.q[0] = fmaf(2.f, s0, fmaf(w[0], g1, fmaf(w[1], g2, w[2] * g3)));
+    gs.q[1] = fmaf(2.f, s1, fmaf(-w[0], g0, fmaf(-w[2], g2, w[1] * g3)));
+    gs.q[2] = fmaf(2.f, s2, fmaf(-w[1], g0, fmaf(w[2], g1, -w[0] * g3)));
+    gs.q[3] = fmaf(2.f, s3, fmaf(-w[2], g0, fmaf(-w[1], g1, w[0] * g2)));
+  }
+  // thrust: n|n| of each thruster into the rows
+  float gf[MT];
+  if constexpr (PATH == ADJ_MIRRORED) {
+    const float gX = fmaf(P.At[0], gv[0], P.Mh * gw[1]), gY = fmaf(P.At[1], gv[1], P.Kh * gw[0]);
+    const float gN = P.Nh * gw[2], gZ = P.At[2] * gv[2], gK = P.Kv * gw[0];
+    const float sm = gX + gY, df = gX - gY;
+    gf[0] = sm + gN;
+    gf[1] = df - gN;
+    gf[2] = -df - gN;
+    gf[3] = gN - sm;
+    gf[4] = gZ - gK;
+    gf[5] = gZ + gK;
+    if constexpr (MT > 6) {
+      const float gM = P.Mv * gw[1];
+      gf[6] = gf[4] + gM;
+      gf[7] = gf[5] + gM;
+      gf[4] -= gM;
+      gf[5] -= gM;
+    }
+  } else {
+    float gt[6];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      gt[i] = P.At[i] * gv[i];
+      gt[3 + i] = P.Ar[i] * gw[i];
+    }
+#pragma unroll
+    for (int i = 0; i < MT; ++i) {
+      const float4 dd = gdir[i], aa = garm[i];
+      gf[i] = fmaf(dd.x, gt[0], fmaf(dd.y, gt[1], fmaf(dd.z, gt[2],
+              fmaf(aa.x, gt[3], fmaf(aa.y, gt[4], aa.z * gt[5])))));
+    }
+  }
+  (void)nt;
+#pragma unroll
+  for (int i = 0; i < MT; ++i) en[i] = 2.f * fabsf(s.n[i]) * gf[i];
 }
 
-template <int MT>
-__device__ __forceinline__ void st_zero(St<MT> &x) {
-  for (int i = 0; i < 3; ++i) x.p[i] = x.v[i] = x.w[i] = 0.f;
-  for (int i = 0; i < 4; ++i) x.q[i] = 0.f;
-  for (int i = 0; i < MT; ++i) x.n[i] = 0.f;
+// The stage states of one sub-step and the step itself: stage(i, y, nu') is called with stage i's
+// state (the same four states rk4_step evaluates, the throttles in closed form) and its nu'; zq
+// receives the quaternion before renormalisation and S the next start state.  The operations are
+// rk4_step's.
+template <int MT, int PATH, typename Stage>
+__device__ __forceinline__ void stage_step(St<MT> &S, const float (&c)[MT], const AdjEnv<PATH> &A,
+                                           const float4 *gdir, const float4 *garm, int nt, bool ca,
+                                           const RkStep &rk, float (&zq)[4], Stage stage) {
+  constexpr bool DIAG = PATH != ADJ_GEN;
+  constexpr int NH = adj_layout(PATH);
+  St<MT> k, y = S, acc;
+  float d[MT];
+#pragma unroll
+  for (int i = 0; i < MT; ++i) d[i] = S.n[i] - c[i];
+#pragma unroll
+  for (int g = 0; g < 4; ++g) {
+    rhs<MT, DIAG, true, NH, PATH == ADJ_GEN>(y, A.F, gdir, garm, nt, ca, k, A.xh);
+    const float nud[6] = {k.v[0], k.v[1], k.v[2], k.w[0], k.w[1], k.w[2]};
+    stage(g, y, nud);
+    if (g == 0) axpy<MT, false>(acc, S, rk.h6, rk.q12, k);
+    else if (g < 3) axpy<MT, false>(acc, acc, rk.h3, rk.h6, k);
+    else axpy<MT, false>(S, acc, rk.h6, rk.q12, k);
+    if (g < 2) axpy<MT, false>(y, S, rk.hh, rk.qh, k);
+    else if (g == 2) axpy<MT, false>(y, S, rk.h, rk.hh, k);
+    const float f = g == 0 ? A.L.f2 : g == 1 ? A.L.f3 : g == 2 ? A.L.f4 : A.L.P;
+#pragma unroll
+    for (int i = 0; i < MT; ++i) (g < 3 ? y.n[i] : S.n[i]) = fmaf(f, d[i], c[i]);
+  }
+#pragma unroll
+  for (int i = 0; i < 4; ++i) zq[i] = S.q[i];
+  const float inv = rsqrtf(fmaf(zq[0], zq[0], fmaf(zq[1], zq[1],
+                                fmaf(zq[2], zq[2], zq[3] * zq[3]))));
+#pragma unroll
+  for (int i = 0; i < 4; ++i) S.q[i] *= inv;
 }
 
-// The forward's right-hand side and closed-form-lag sub-step for this env (the step kernels'
-// own code: the diagonal-mass coefficients, or the general path with the staged off-diagonal
-// coefficients).
-template <int MT, bool GEN>
-__device__ __forceinline__ void fwd_rhs(const St<MT> &y, const float (&cs)[MT],
-                                        const AdjEnv<GEN> &A, const float4 *gdir,
-                                        const float4 *garm, int nt, bool ca, St<MT> &k) {
-  rhs<MT, !GEN, true, 0, GEN>(y, cs, A.F, gdir, garm, nt, ca, k, A.xh);
-}
-
-template <int MT, bool GEN>
-__device__ __forceinline__ void fwd_step(St<MT> &S, const float (&c)[MT], const LagEnv &L,
-                                         const AdjEnv<GEN> &A, const float4 *gdir,
-                                         const float4 *garm, int nt, bool ca, const RkStep &rk) {
-  rk4_step<MT, !GEN, true, 0, GEN>(S, c, L, A.F, gdir, garm, nt, ca, rk, A.xh);
-}
-
-// The RK4 stage states of one sub-step from its start state s (y1 = s):
-//   y2 = s + h/2 W k1,  y3 = s + h/2 W k2,  y4 = s + h W k3,  k_i = rhs(y_i),
-//   z  = s + h/6 W k1 + h/3 W k2 + h/3 W k3 + h/6 W k4  (before renormalisation).
-template <int MT, bool GEN>
-__device__ __forceinline__ void stage_states(const St<MT> &s, const float (&cs)[MT],
-                                             const AdjEnv<GEN> &A, const float4 *gdir,
-                                             const float4 *garm, int nt, bool current_accel,
-                                             float h, St<MT> &y2, St<MT> &y3, St<MT> &y4,
-                                             St<MT> &z) {
-  const float hh = 0.5f * h, h3 = h * (1.0f / 3.0f), h6 = h * (1.0f / 6.0f);
-  St<MT> k;
-  fwd_rhs<MT, GEN>(s, cs, A, gdir, garm, nt, current_accel, k);
-  axpy(z, s, h6, 0.5f * h6, k);
-  axpy(y2, s, hh, 0.5f * hh, k);
-  fwd_rhs<MT, GEN>(y2, cs, A, gdir, garm, nt, current_accel, k);
-  axpy(z, z, h3, 0.5f * h3, k);
-  axpy(y3, s, hh, 0.5f * hh, k);
-  fwd_rhs<MT, GEN>(y3, cs, A, gdir, garm, nt, current_accel, k);
-  axpy(z, z, h3, 0.5f * h3, k);
-  axpy(y4, s, h, hh, k);
-  fwd_rhs<MT, GEN>(y4, cs, A, gdir, garm, nt, current_accel, k);
-  axpy(z, z, h6, 0.5f * h6, k);
-}
-
-template <int MT>
-__device__ __forceinline__ void st_add(St<MT> &y, const St<MT> &x) {
-  for (int i = 0; i < 3; ++i) y.p[i] += x.p[i];
-  for (int i = 0; i < 4; ++i) y.q[i] += x.q[i];
-  for (int i = 0; i < 3; ++i) y.v[i] += x.v[i];
-  for (int i = 0; i < 3; ++i) y.w[i] += x.w[i];
-  for (int i = 0; i < MT; ++i) y.n[i] += x.n[i];
-}
-
-// lam: in, the adjoint of the sub-step's output s+; out, the adjoint of its input s.
-// stage(i, y) gives stage i's state (0: s, 1: y2, 2: y3, 3: y4; stage_states) and zq is the
-// quaternion before renormalisation.
+// lam (pose, velocity) and lamn (throttles): in, the adjoint of the sub-step's output s+; out, the
+// adjoint of its input s; gc receives the command's.  stage(i, y, nu') gives stage i's record.
 //   s+ = N(z)
 // reverse:  lk4 = h/6 W lz,            ly4 = J(y4)^T lk4
 //           lk3 = h/3 W lz + h W ly4,   ly3 = J(y3)^T lk3
 //           lk2 = h/3 W lz + h/2 W ly3, ly2 = J(y2)^T lk2
 //           lk1 = h/6 W lz + h/2 W ly2, ly1 = J(s)^T lk1
 //           ls  = lz + ly4 + ly3 + ly2 + ly1
-// The four stages share one loop body, kept a loop (UNROLL false) with a single copy of rhs_vjp:
-// a quarter of the code, which the instruction cache holds (unrolled, both backward kernels
-// stalled mostly on instruction fetch: 1.41 / 1.29 ms against 1.11 / 1.04 ms rolled at 4,096
-// envs).  The stage states are then selected or read by a runtime index.  Same operations
-// either way.
-template <int MT, bool GEN, bool UNROLL, typename Stage>
-__device__ __forceinline__ void step_vjp_stages(Stage stage, const float (&zq)[4],
-                                                const float (&cs)[MT], const AdjEnv<GEN> &A,
-                                                const float4 *gdir, const float4 *garm, int nt,
-                                                bool current_accel, float h, St<MT> &lam,
-                                                Grad &G, float (&gcs)[MT]) {
-  const float hh = 0.5f * h, h3 = h * (1.0f / 3.0f), h6 = h * (1.0f / 6.0f);
+// (W: the quaternion takes half of each weight, because rhs() stores its rate doubled; p does not
+// enter the right-hand side, so its adjoint passes through).  The four stages share one rolled
+// loop body: a quarter of the code, which the instruction cache holds.
+template <int MT, int PATH, typename Stage>
+__device__ __forceinline__ void step_vjp(Stage stage, const float (&zq)[4], const AdjEnv<PATH> &A,
+                                         const float4 *gdir, const float4 *garm, int nt, bool ca,
+                                         const RkStep &rk, Body &lam, float (&lamn)[MT],
+                                         Grad<PATH> &G, float (&gc)[MT]) {
   // renormalisation q+ = z_q / |z_q|:  lz_q = (lam_q - q+ (q+ . lam_q)) / |z_q|
-  const float nq = sqrtf(fmaf(zq[0], zq[0], fmaf(zq[1], zq[1], fmaf(zq[2], zq[2], zq[3] * zq[3]))));
+  const float inv = rsqrtf(fmaf(zq[0], zq[0], fmaf(zq[1], zq[1],
+                                fmaf(zq[2], zq[2], zq[3] * zq[3]))));
   float qn[4], dot = 0.f;
+#pragma unroll
   for (int i = 0; i < 4; ++i) {
-    qn[i] = zq[i] / nq;
+    qn[i] = zq[i] * inv;
     dot = fmaf(qn[i], lam.q[i], dot);
   }
-  St<MT> lz = lam;
-  for (int i = 0; i < 4; ++i) lz.q[i] = fmaf(-qn[i], dot, lam.q[i]) / nq;
-
-  St<MT> lk, ly;
-  St<MT> &ls = lam;
-  ls = lz;
-  st_zero(ly);
-  auto body = [&](int i) {
-    wscale(lk, lz, (i == 3 || i == 0) ? h6 : h3, false);
-    if (i < 3) wscale(lk, ly, (i == 2) ? h : hh, true);
-    St<MT> y;
-    stage(i, y);
-    st_zero(ly);
-    rhs_vjp<MT, GEN>(y, cs, A, gdir, garm, nt, current_accel, lk, ly, G, gcs);
-    st_add(ls, ly);
-  };
-  if constexpr (UNROLL) {
 #pragma unroll
-    for (int i = 3; i >= 0; --i) body(i);
-  } else {
-#pragma unroll 1
-    for (int i = 3; i >= 0; --i) body(i);
+  for (int i = 0; i < 4; ++i) lam.q[i] = fmaf(-qn[i], dot, lam.q[i]) * inv;
+  const Body lz = lam;
+  Body ly{};
+#pragma unroll
+  for (int i = 0; i < MT; ++i) {
+    gc[i] = fmaf(-A.L.P, lamn[i], lamn[i]);
+    lamn[i] *= A.L.P;
   }
-}
-
-// The whole sub-step: stage states recomputed, then their transposes.
-template <int MT, bool GEN>
-__device__ void step_vjp(const St<MT> &s, const float (&cs)[MT], const AdjEnv<GEN> &A,
-                         const float4 *gdir, const float4 *garm, int nt, bool current_accel,
-                         float h, St<MT> &lam, Grad &G, float (&gcs)[MT]) {
-  St<MT> y2, y3, y4, z;
-  stage_states<MT, GEN>(s, cs, A, gdir, garm, nt, current_accel, h, y2, y3, y4, z);
-  const float zq[4] = {z.q[0], z.q[1], z.q[2], z.q[3]};
-  auto stage = [&](int i, St<MT> &y) { y = i == 0 ? s : i == 1 ? y2 : i == 2 ? y3 : y4; };
-  step_vjp_stages<MT, GEN, false>(stage, zq, cs, A, gdir, garm, nt, current_accel, h, lam, G,
-                                  gcs);
+#pragma unroll 1
+  for (int i = 3; i >= 0; --i) {
+    const bool outer = i == 3 || i == 0;
+    const float a = outer ? rk.h6 : rk.h3, aq = outer ? rk.q12 : rk.h6;
+    const float b = i == 3 ? 0.f : i == 2 ? rk.h : rk.hh, bq = 0.5f * b;
+    const float fi = i == 3 ? A.L.f4 : i == 2 ? A.L.f3 : i == 1 ? A.L.f2 : 1.f;
+    Body lk;
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+      lk.p[j] = a * lz.p[j];
+      lk.v[j] = fmaf(b, ly.v[j], a * lz.v[j]);
+      lk.w[j] = fmaf(b, ly.w[j], a * lz.w[j]);
+    }
+#pragma unroll
+    for (int j = 0; j < 4; ++j) lk.q[j] = fmaf(bq, ly.q[j], aq * lz.q[j]);
+    St<MT> y;
+    float nud[6], en[MT];
+    stage(i, y, nud);
+    if constexpr (PATH == ADJ_GEN)
+      rhs_vjp_gen<MT>(y, nud, A, gdir, garm, nt, ca, lk, ly, G, en);
+    else
+      rhs_vjp_diag<MT, PATH>(y, nud, A, gdir, garm, nt, lk, ly, G, en);
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+      lam.v[j] += ly.v[j];
+      lam.w[j] += ly.w[j];
+    }
+#pragma unroll
+    for (int j = 0; j < 4; ++j) lam.q[j] += ly.q[j];
+#pragma unroll
+    for (int j = 0; j < MT; ++j) {
+      lamn[j] = fmaf(fi, en[j], lamn[j]);
+      gc[j] = fmaf(-fi, en[j], gc[j] + en[j]);
+    }
+  }
 }
 
 constexpr int kMaxSeg = 32;  // largest checkpoint interval
 
-// The buffered command of sub-step j (cursor position) times scale: 1 for the forward's step, 1 /
-// tau_m for the right-hand side.
+// The buffered command of sub-step j (cursor position).
 template <int MT>
 __device__ __forceinline__ void commands_at(const FleetView &fv, int64_t e, int64_t j, int nt,
-                                            float scale, float (&c)[MT]) {
+                                            float (&c)[MT]) {
   int64_t seg = j / fv.hold;
   if (seg > fv.n_seg - 1) seg = fv.n_seg - 1;
   for (int i = 0; i < MT; ++i) c[i] = 0.f;
@@ -488,17 +598,8 @@ __device__ __forceinline__ void commands_at(const FleetView &fv, int64_t e, int6
     const float *a = fv.act + (seg * fv.n + e) * fv.act_w;
     #pragma unroll
     for (int i = 0; i < MT; ++i)
-      if (i < nt) c[i] = a[i] * scale;
+      if (i < nt) c[i] = a[i];
   }
-}
-
-__global__ void k_checkpoint(const StatePlanes st, int64_t n, float *__restrict__ ck) {
-  const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= n) return;
-  const float4 a = st.s0[e], b = st.s1[e], c = st.s2[e], d = st.s3[e], f = st.s4[e];
-  const float r[MG_NSTATE] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w, c.x, c.y, c.z,
-                              c.w, d.x, d.y, d.z, d.w, f.x, f.y, f.z, f.w, st.s5[e]};
-  for (int j = 0; j < MG_NSTATE; ++j) ck[(int64_t)j * n + e] = r[j];
 }
 
 template <int MT>
@@ -513,37 +614,50 @@ __device__ __forceinline__ void load_checkpoint(const float *__restrict__ ckpt, 
 }
 
 // lam += the loss adjoint of the state after sub-step t.
-template <int MT>
-__device__ __forceinline__ void add_traj_adjoint(const float *__restrict__ dtraj, int64_t t,
-                                                 int64_t n, int64_t e, St<MT> &lam) {
-  const float *g = dtraj + t * MG_NTRAJ * n + e;
-  for (int i = 0; i < 3; ++i) lam.p[i] += g[(int64_t)i * n];
-  for (int i = 0; i < 4; ++i) lam.q[i] += g[(int64_t)(3 + i) * n];
-  for (int i = 0; i < 3; ++i) lam.v[i] += g[(int64_t)(7 + i) * n];
-  for (int i = 0; i < 3; ++i) lam.w[i] += g[(int64_t)(10 + i) * n];
+__device__ __forceinline__ void add_traj_adjoint(const float *__restrict__ g, int64_t stride,
+                                                 Body &lam) {
+  for (int i = 0; i < 3; ++i) lam.p[i] += g[i * stride];
+  for (int i = 0; i < 4; ++i) lam.q[i] += g[(3 + i) * stride];
+  for (int i = 0; i < 3; ++i) lam.v[i] += g[(7 + i) * stride];
+  for (int i = 0; i < 3; ++i) lam.w[i] += g[(10 + i) * stride];
 }
 
-// Command adjoint of sub-step t into its action segment.
+// Command adjoints of the sub-steps that share an action segment, summed in registers and added
+// to the caller's buffer when the walk leaves the segment.
 template <int MT>
-__device__ __forceinline__ void add_action_adjoint(const FleetView &fv, int64_t t, int64_t e,
-                                                   int nt, float itau, const float (&gcs)[MT],
-                                                   float *__restrict__ dact) {
-  if (!dact || fv.n_seg <= 0) return;
-  int64_t seg = t / fv.hold;
-  if (seg > fv.n_seg - 1) seg = fv.n_seg - 1;
-  float *da = dact + (seg * fv.n + e) * fv.act_w;
-  #pragma unroll
-  for (int i = 0; i < MT; ++i)
-    if (i < nt) da[i] = fmaf(itau, gcs[i], da[i]);
-}
+struct ActionAdjoint {
+  int64_t seg = -1;
+  float g[MT];
 
-// Coefficients: M_A,jj enters the momenta (Q1 for j < 3, J = diag(I_o) + M_A,rot for j >= 3),
-// the current term and M (G.mv); D_l and D_q their damping terms.
-template <int MT>
-__device__ __forceinline__ void write_gradients(const Grad &G, const St<MT> &lam, int64_t e,
-                                                float *__restrict__ dcoef,
-                                                float *__restrict__ dstate0) {
-  float *dc = dcoef + e * 18;
+  __device__ __forceinline__ void flush(const FleetView &fv, int64_t e, int nt, float *dact) {
+    if (seg < 0) return;
+    float *da = dact + (seg * fv.n + e) * fv.act_w;
+#pragma unroll
+    for (int i = 0; i < MT; ++i)
+      if (i < nt) da[i] += g[i];
+  }
+  // sub-step t (cursor position), walked backwards
+  __device__ __forceinline__ void add(const FleetView &fv, int64_t t, int64_t e, int nt,
+                                      const float (&gc)[MT], float *dact) {
+    if (!dact || fv.n_seg <= 0) return;
+    int64_t sg = t / fv.hold;
+    if (sg > fv.n_seg - 1) sg = fv.n_seg - 1;
+    if (sg != seg) {
+      flush(fv, e, nt, dact);
+      seg = sg;
+#pragma unroll
+      for (int i = 0; i < MT; ++i) g[i] = 0.f;
+    }
+#pragma unroll
+    for (int i = 0; i < MT; ++i) g[i] += gc[i];
+  }
+};
+
+// Coefficient gradients from their sums, in the order M_A, D_l, D_q.  M_A,jj enters the momenta (Q1
+// for j < 3, J = diag(I_o) + M_A,rot for j >= 3), the current term and M (mv); D_l and D_q their
+// damping terms.
+__device__ __forceinline__ void coefficient_gradients(const GradGen &G, const ParamPlanes &,
+                                                      int64_t, float *dc) {
   for (int j = 0; j < 3; ++j) {
     dc[j] = G.ma[j] + G.mv[j];
     dc[3 + j] = G.J[j] + G.mv[3 + j];
@@ -552,19 +666,45 @@ __device__ __forceinline__ void write_gradients(const Grad &G, const St<MT> &lam
     dc[6 + j] = G.dl[j];
     dc[12 + j] = G.dq[j];
   }
+}
+// Row k's terms in M_A,i are mi_k times: own_i (k = i), up_k - dn_k' (the neighbours' Coriolis
+// terms), the Munk products and, rotational, the gyroscopic products; M's share is -mi sum g nu'.
+__device__ __forceinline__ void coefficient_gradients(const GradDiag &G, const ParamPlanes &pa,
+                                                      int64_t e, float *dc) {
+  const float4 m = ldg4(pa.d7, e);
+  const float2 n = __ldg(pa.d8 + e);
+  const float mi[6] = {m.x, m.y, m.z, m.w, n.x, n.y};
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    const int b = (i + 2) % 3, f = (i + 1) % 3;  // rows in which i is i1, and i2
+    float a = mi[i] * (G.own[i] - G.mv[i]);
+    a = fmaf(mi[b], G.up[b], a);
+    a = fmaf(-mi[f], G.dn[f], a);
+    a = fmaf(mi[3 + b], G.munk[b], fmaf(-mi[3 + f], G.munk[f], a));
+    dc[i] = a;
+    dc[3 + i] = fmaf(mi[3 + b], G.gyro[b], fmaf(-mi[3 + f], G.gyro[f], -mi[3 + i] * G.mv[3 + i]));
+  }
+#pragma unroll
+  for (int j = 0; j < 6; ++j) {
+    dc[6 + j] = -mi[j] * G.dl[j];
+    dc[12 + j] = -mi[j] * G.dq[j];
+  }
+}
+
+template <int MT, typename G>
+__device__ __forceinline__ void write_gradients(const G &grad, const ParamPlanes &pa,
+                                                const Body &lam, const float (&lamn)[MT],
+                                                int64_t e, float *__restrict__ dcoef,
+                                                float *__restrict__ dstate0) {
+  coefficient_gradients(grad, pa, e, dcoef + e * 18);
   if (dstate0) {
     float *o = dstate0 + e * MG_NSTATE;
     for (int i = 0; i < 3; ++i) o[i] = lam.p[i];
     for (int i = 0; i < 4; ++i) o[3 + i] = lam.q[i];
     for (int i = 0; i < 3; ++i) o[7 + i] = lam.v[i];
     for (int i = 0; i < 3; ++i) o[10 + i] = lam.w[i];
-    for (int i = 0; i < MG_MAX_THR; ++i) o[13 + i] = i < MT ? lam.n[i] : 0.f;
+    for (int i = 0; i < MG_MAX_THR; ++i) o[13 + i] = i < MT ? lamn[i] : 0.f;
   }
-}
-
-__device__ __forceinline__ void zero_grad(Grad &G) {
-  for (int i = 0; i < 3; ++i) G.ma[i] = G.J[i] = 0.f;
-  for (int i = 0; i < 6; ++i) G.mv[i] = G.dl[i] = G.dq[i] = 0.f;
 }
 
 __device__ __forceinline__ void stage_geometry(const FleetView &fv,
@@ -586,19 +726,58 @@ __device__ __forceinline__ void stage_xh_or_zero(const FleetView &fv, int64_t en
   }
 }
 
-template <bool GEN>
-__device__ __forceinline__ void load_env(const FleetView &fv, int64_t e, bool ca,
-                                         const float *sxh_row, AdjEnv<GEN> &A) {
-  load_par<!GEN>(fv.pa, e, A.P);
-  A.F = make_coef<!GEN>(A.P, nullptr, nullptr);
-  A.xh = GEN ? sxh_row : nullptr;
+template <int PATH>
+__device__ __forceinline__ void load_env(const FleetView &fv, int64_t e, const float *sxh_row,
+                                         const float4 *gdir, const float4 *garm, AdjEnv<PATH> &A) {
+  Par<PATH != ADJ_GEN> P;
+  load_par<PATH != ADJ_GEN>(fv.pa, e, P);
+  A.F = make_coef<PATH != ADJ_GEN, adj_layout(PATH)>(P, gdir, garm);
+  A.L = lag_env(P.itau, fv.dt);
+  A.xh = PATH == ADJ_GEN ? sxh_row : nullptr;
+}
+
+// A stage record: what the transposes read of one stage, in float4 words (q, nu, nu', n), so that a
+// lane moves it in 16-byte pieces: word w of an env's record is a plane over the envs.
+template <int MT>
+__host__ __device__ constexpr int stage_words() { return (16 + MT + 3) / 4; }
+// A sub-step's: four stages and the quaternion before renormalisation.
+template <int MT>
+__host__ __device__ constexpr int rec_words() { return 4 * stage_words<MT>() + 1; }
+
+template <int MT>
+__device__ __forceinline__ void put_stage(float4 *__restrict__ r, int64_t stride, const St<MT> &y,
+                                          const float (&nud)[6]) {
+  r[0] = make_float4(y.q[0], y.q[1], y.q[2], y.q[3]);
+  r[stride] = make_float4(y.v[0], y.v[1], y.v[2], y.w[0]);
+  r[2 * stride] = make_float4(y.w[1], y.w[2], nud[0], nud[1]);
+  r[3 * stride] = make_float4(nud[2], nud[3], nud[4], nud[5]);
+  r[4 * stride] = make_float4(y.n[0], y.n[1], y.n[2], y.n[3]);
+  if constexpr (MT > 6) r[5 * stride] = make_float4(y.n[4], y.n[5], y.n[6], y.n[7]);
+  else r[5 * stride] = make_float4(y.n[4], y.n[5], 0.f, 0.f);
+}
+template <int MT>
+__device__ __forceinline__ void get_stage(const float4 *r, int64_t stride, St<MT> &y,
+                                          float (&nud)[6]) {
+  const float4 a = r[0], b = r[stride], c = r[2 * stride], d = r[3 * stride], f = r[4 * stride];
+  const float4 g = r[5 * stride];
+  y.q[0] = a.x; y.q[1] = a.y; y.q[2] = a.z; y.q[3] = a.w;
+  y.v[0] = b.x; y.v[1] = b.y; y.v[2] = b.z;
+  y.w[0] = b.w; y.w[1] = c.x; y.w[2] = c.y;
+  nud[0] = c.z; nud[1] = c.w; nud[2] = d.x; nud[3] = d.y; nud[4] = d.z; nud[5] = d.w;
+  y.n[0] = f.x; y.n[1] = f.y; y.n[2] = f.z; y.n[3] = f.w; y.n[4] = g.x; y.n[5] = g.y;
+  if constexpr (MT > 6) {
+    y.n[6] = g.z;
+    y.n[7] = g.w;
+  }
 }
 
 // One thread per env.  ckpt [n_ck][MG_NSTATE][n] (state at sub-steps 0, C, 2C, ...),
 // dtraj [T][MG_NTRAJ][n] (loss adjoint of the state after each sub-step).  Outputs: dcoef
 // [n][18] (M_A, Dl, Dq diagonals), dact [n_seg][n][w] accumulated, dstate0 [n][21] or null.
-// GEN: dynamic shared memory [blockDim.x][MG_NXPARAM] for the block's off-diagonal coefficients.
-template <int MT, bool GEN>
+// The segment's step-start states are kept in local memory, each sub-step's stages recomputed.
+// General path: dynamic shared memory [blockDim.x][MG_NXPARAM] for the block's off-diagonal
+// coefficients.
+template <int MT, int PATH>
 __global__ void __launch_bounds__(kAdjThreads)
     k_adjoint(const FleetView fv, const int32_t *__restrict__ types, const float *__restrict__ ckpt,
               const float *__restrict__ dtraj, int32_t T, int32_t C, int64_t step0,
@@ -607,7 +786,7 @@ __global__ void __launch_bounds__(kAdjThreads)
   extern __shared__ float sxh[];
   stage_geometry(fv, sgeo);
   const int64_t env0 = (int64_t)blockIdx.x * blockDim.x;
-  if constexpr (GEN)
+  if constexpr (PATH == ADJ_GEN)
     stage_xh_or_zero(fv, env0, (int)min((int64_t)blockDim.x, fv.n - env0), sxh);
   __syncthreads();
   const int64_t e = env0 + threadIdx.x;
@@ -616,18 +795,20 @@ __global__ void __launch_bounds__(kAdjThreads)
   const float4 *gdir = sgeo[type], *garm = sgeo[type] + MG_MAX_THR;
   const int nt = fv.geo[type].n_thr;
   const bool ca = !(fv.model_flags & MG_MODEL_NO_CURRENT_ACCEL);
-  const float h = fv.dt;
   const int64_t n = fv.n;
-  AdjEnv<GEN> A;
-  load_env<GEN>(fv, e, ca, sxh + threadIdx.x * MG_NXPARAM, A);
-  const LagEnv L = lag_env(A.P.itau, h);  // the forward's throttle-lag update (replay)
+  AdjEnv<PATH> A;
+  load_env<PATH>(fv, e, sxh + threadIdx.x * MG_NXPARAM, gdir, garm, A);
 
-  Grad G;
+  Grad<PATH> G;
   zero_grad(G);
-  St<MT> lam;
-  st_zero(lam);
+  Body lam{};
+  float lamn[MT];
+#pragma unroll
+  for (int i = 0; i < MT; ++i) lamn[i] = 0.f;
   St<MT> S[kMaxSeg];
-  float c[MT], gcs[MT];
+  float4 rec[4 * stage_words<MT>()];
+  float c[MT], gc[MT], zq[4];
+  ActionAdjoint<MT> act;
 
   const int32_t n_ck = (T + C - 1) / C;
   for (int32_t sg = n_ck - 1; sg >= 0; --sg) {
@@ -635,83 +816,76 @@ __global__ void __launch_bounds__(kAdjThreads)
     // re-run the segment from its checkpoint
     load_checkpoint<MT>(ckpt, sg, n, e, S[0]);
     for (int32_t j = 1; j < len; ++j) {
-      S[j] = S[j - 1];
-      commands_at<MT>(fv, e, step0 + t0 + j - 1, nt, 1.f, c);
-      fwd_step<MT, GEN>(S[j], c, L, A, gdir, garm, nt, ca, fv.rk);
+      St<MT> x = S[j - 1];
+      commands_at<MT>(fv, e, step0 + t0 + j - 1, nt, c);
+      rk4_step<MT, PATH != ADJ_GEN, true, adj_layout(PATH), PATH == ADJ_GEN>(
+          x, c, A.L, A.F, gdir, garm, nt, ca, fv.rk, A.xh);
+      S[j] = x;
     }
     // walk it backwards
     for (int32_t j = len - 1; j >= 0; --j) {
       const int64_t t = t0 + j;
-      add_traj_adjoint<MT>(dtraj, t, n, e, lam);
-      commands_at<MT>(fv, e, step0 + t, nt, A.P.itau, c);
-      for (int i = 0; i < MT; ++i) gcs[i] = 0.f;
-      step_vjp<MT, GEN>(S[j], c, A, gdir, garm, nt, ca, h, lam, G, gcs);
-      add_action_adjoint<MT>(fv, step0 + t, e, nt, A.P.itau, gcs, dact);
+      add_traj_adjoint(dtraj + t * MG_NTRAJ * n + e, n, lam);
+      commands_at<MT>(fv, e, step0 + t, nt, c);
+      St<MT> x = S[j];
+      stage_step<MT, PATH>(x, c, A, gdir, garm, nt, ca, fv.rk, zq,
+                           [&](int g, const St<MT> &y, const float (&nud)[6]) {
+                             put_stage<MT>(rec + g * stage_words<MT>(), 1, y, nud);
+                           });
+      auto stage = [&](int i, St<MT> &y, float (&nud)[6]) {
+        get_stage<MT>(rec + i * stage_words<MT>(), 1, y, nud);
+      };
+      step_vjp<MT, PATH>(stage, zq, A, gdir, garm, nt, ca, fv.rk, lam, lamn, G, gc);
+      act.add(fv, step0 + t, e, nt, gc, dact);
     }
   }
-  write_gradients<MT>(G, lam, e, dcoef, dstate0);
+  act.flush(fv, e, nt, dact);
+  write_gradients<MT>(G, fv.pa, lam, lamn, e, dcoef, dstate0);
 }
 
 // ---------------------------------------------------------------- two-warp form
 // For fleets with fewer 32-env warps than the GPU has schedulers, where the one-warp kernel
 // above leaves most of them idle and runs on instruction latency: blocks of two warps over the
-// same 32 envs.  Warp 0 re-runs each checkpoint segment and writes, for every sub-step, the
-// stage states the transposes need (q, nu and n of y1..y4, and the quaternion before
-// renormalisation) to a workspace; warp 1 applies step_vjp_stages from those records, one
-// segment behind.  The workspace holds two segments, used alternately; a block barrier at each
-// segment boundary hands one over.  The per-env arithmetic is k_adjoint's: stage_states and
-// step_vjp_stages are the two halves of step_vjp.
+// same 32 envs.  Warp 0 re-runs each checkpoint segment, one evaluation of the step per sub-step,
+// and writes the stage records the transposes need to a workspace; warp 1 applies step_vjp from
+// those records, one segment behind.  The workspace holds two segments, used alternately; a block
+// barrier at each segment boundary hands one over.  The per-env arithmetic is k_adjoint's.
 constexpr int kWsThreads = 64;
 
-template <int MT>
-__host__ __device__ constexpr int rec_words() { return 4 * (10 + MT) + 4; }
-
-template <int MT>
-__device__ __forceinline__ void put_stage(float *__restrict__ r, int64_t n, int f,
-                                          const St<MT> &y) {
-  for (int i = 0; i < 4; ++i) r[(int64_t)(f + i) * n] = y.q[i];
-  for (int i = 0; i < 3; ++i) r[(int64_t)(f + 4 + i) * n] = y.v[i];
-  for (int i = 0; i < 3; ++i) r[(int64_t)(f + 7 + i) * n] = y.w[i];
-  for (int i = 0; i < MT; ++i) r[(int64_t)(f + 10 + i) * n] = y.n[i];
-}
-
 // Warp 0: segment sg re-run from its checkpoint; record j of `rec` gets sub-step t0 + j.
-template <int MT, bool GEN>
+template <int MT, int PATH>
 __device__ __forceinline__ void produce_segment(const FleetView &fv, int64_t e,
-                                                const AdjEnv<GEN> &A, const LagEnv &L,
-                                                const float4 *gdir, const float4 *garm, int nt,
-                                                bool ca, float h, const float *__restrict__ ckpt,
-                                                int32_t sg, int32_t C, int32_t T, int64_t step0,
-                                                float *__restrict__ rec) {
-  constexpr int W = rec_words<MT>(), Y = 10 + MT;
+                                                const AdjEnv<PATH> &A, const float4 *gdir,
+                                                const float4 *garm, int nt, bool ca,
+                                                const float *__restrict__ ckpt, int32_t sg,
+                                                int32_t C, int32_t T, int64_t step0,
+                                                float4 *__restrict__ rec) {
+  constexpr int W = rec_words<MT>();
   const int64_t n = fv.n;
   const int32_t t0 = sg * C, len = min(C, T - t0);
   St<MT> S;
   load_checkpoint<MT>(ckpt, sg, n, e, S);
-  float c[MT];
+  float c[MT], zq[4];
   for (int32_t j = 0; j < len; ++j) {
-    commands_at<MT>(fv, e, step0 + t0 + j, nt, 1.f, c);
-    float cs[MT];
-    for (int i = 0; i < MT; ++i) cs[i] = c[i] * A.P.itau;
-    St<MT> y2, y3, y4, z;
-    stage_states<MT, GEN>(S, cs, A, gdir, garm, nt, ca, h, y2, y3, y4, z);
-    float *r = rec + (int64_t)j * W * n;
-    put_stage<MT>(r, n, 0, S);
-    put_stage<MT>(r, n, Y, y2);
-    put_stage<MT>(r, n, 2 * Y, y3);
-    put_stage<MT>(r, n, 3 * Y, y4);
-    for (int i = 0; i < 4; ++i) r[(int64_t)(4 * Y + i) * n] = z.q[i];
-    if (j + 1 < len) {  // the next start state, as the forward computed it
-      fwd_step<MT, GEN>(S, c, L, A, gdir, garm, nt, ca, fv.rk);
-    }
+    commands_at<MT>(fv, e, step0 + t0 + j, nt, c);
+    float4 *r = rec + (int64_t)j * W * n;
+    stage_step<MT, PATH>(S, c, A, gdir, garm, nt, ca, fv.rk, zq,
+                         [&](int g, const St<MT> &y, const float (&nud)[6]) {
+                           put_stage<MT>(r + (int64_t)g * stage_words<MT>() * n, n, y, nud);
+                         });
+    r[(int64_t)(W - 1) * n] = make_float4(zq[0], zq[1], zq[2], zq[3]);
   }
 }
 
-// Per-lane asynchronous 4-byte copies global -> shared (sm_80+ cp.async), so that the consumer
-// warp's next record is in flight while it works on the current one.
+// Per-lane asynchronous copies global -> shared (sm_80+ cp.async), so that the consumer warp's next
+// record is in flight while it works on the current one.
 __device__ __forceinline__ void cp_async4(float *smem, const float *gmem) {
   const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
   asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(sa), "l"(gmem) : "memory");
+}
+__device__ __forceinline__ void cp_async16(float4 *smem, const float4 *gmem) {
+  const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(sa), "l"(gmem) : "memory");
 }
 __device__ __forceinline__ void cp_async_commit() {
   asm volatile("cp.async.commit_group;\n" ::: "memory");
@@ -720,93 +894,80 @@ __device__ __forceinline__ void cp_async_wait_all_but_one() {
   asm volatile("cp.async.wait_group 1;\n" ::: "memory");
 }
 
-// What the consumer reads per sub-step: the stage record, the loss adjoint of the sub-step's
-// output and the sub-step's buffered command.
+// What the consumer reads per sub-step, double-buffered in shared memory: the stage records [W][32]
+// float4 and the loss adjoint of the sub-step's output [MG_NTRAJ][32].
 template <int MT>
-__host__ __device__ constexpr int fetch_words() { return rec_words<MT>() + MG_NTRAJ + MT; }
+struct Fetch {
+  float4 rec[2][rec_words<MT>()][32];
+  float adj[2][MG_NTRAJ][32];
+};
 
-// Queue the copies of sub-step t0 + j's inputs into buf [fetch_words][32] (this lane's column).
+// Queue the copies of sub-step t0 + j's inputs into slot j & 1 (this lane's column).
 template <int MT>
-__device__ __forceinline__ void fetch_substep(const FleetView &fv, int64_t e,
-                                              const float *__restrict__ rec,
+__device__ __forceinline__ void fetch_substep(const FleetView &fv, int64_t e, int lane,
+                                              const float4 *__restrict__ rec,
                                               const float *__restrict__ dtraj, int64_t t0,
-                                              int32_t j, int64_t step0, float *buf) {
+                                              int32_t j, Fetch<MT> &buf) {
   constexpr int W = rec_words<MT>();
   const int64_t n = fv.n;
-  const float *r = rec + (int64_t)j * W * n;
-  for (int f = 0; f < W; ++f) cp_async4(buf + f * 32, r + (int64_t)f * n);
+  const float4 *r = rec + (int64_t)j * W * n;
+#pragma unroll
+  for (int f = 0; f < W; ++f) cp_async16(&buf.rec[j & 1][f][lane], r + (int64_t)f * n);
   const float *g = dtraj + (t0 + j) * MG_NTRAJ * n + e;
-  for (int f = 0; f < MG_NTRAJ; ++f) cp_async4(buf + (W + f) * 32, g + (int64_t)f * n);
-  if (fv.n_seg > 0) {
-    int64_t seg = (step0 + t0 + j) / fv.hold;
-    if (seg > fv.n_seg - 1) seg = fv.n_seg - 1;
-    const float *a = fv.act + (seg * n + e) * fv.act_w;
-    for (int i = 0; i < MT; ++i) cp_async4(buf + (W + MG_NTRAJ + i) * 32, a + i);
-  }
+#pragma unroll
+  for (int f = 0; f < MG_NTRAJ; ++f) cp_async4(&buf.adj[j & 1][f][lane], g + (int64_t)f * n);
   cp_async_commit();
 }
 
-template <int MT>
-__device__ __forceinline__ void read_stage(const float *buf, int f, St<MT> &y) {
-  for (int i = 0; i < 3; ++i) y.p[i] = 0.f;  // p does not enter the right-hand side
-  for (int i = 0; i < 4; ++i) y.q[i] = buf[(f + i) * 32];
-  for (int i = 0; i < 3; ++i) y.v[i] = buf[(f + 4 + i) * 32];
-  for (int i = 0; i < 3; ++i) y.w[i] = buf[(f + 7 + i) * 32];
-  for (int i = 0; i < MT; ++i) y.n[i] = buf[(f + 10 + i) * 32];
-}
-
 // Warp 1: segment sg walked backwards from its records, each sub-step's inputs copied into
-// shared memory (double buffer sbuf [2][fetch_words][32]) while the previous one is processed.
-template <int MT, bool GEN>
+// shared memory while the previous one is processed.
+template <int MT, int PATH>
 __device__ __forceinline__ void consume_segment(const FleetView &fv, int64_t e, int lane,
-                                                const AdjEnv<GEN> &A, const float4 *gdir,
-                                                const float4 *garm, int nt, bool ca, float h,
+                                                const AdjEnv<PATH> &A, const float4 *gdir,
+                                                const float4 *garm, int nt, bool ca,
                                                 const float *__restrict__ dtraj, int32_t sg,
                                                 int32_t C, int32_t T, int64_t step0,
-                                                const float *__restrict__ rec, float *sbuf,
-                                                float *__restrict__ dact, St<MT> &lam, Grad &G) {
-  constexpr int W = rec_words<MT>(), Y = 10 + MT, F = fetch_words<MT>();
+                                                const float4 *__restrict__ rec, Fetch<MT> &buf,
+                                                float *__restrict__ dact, ActionAdjoint<MT> &act,
+                                                Body &lam, float (&lamn)[MT], Grad<PATH> &G) {
+  constexpr int W = rec_words<MT>();
   const int32_t t0 = sg * C, len = min(C, T - t0);
-  float c[MT], gcs[MT];
-  fetch_substep<MT>(fv, e, rec, dtraj, t0, len - 1, step0, sbuf + ((len - 1) & 1) * F * 32 + lane);
+  float gc[MT];
+  fetch_substep<MT>(fv, e, lane, rec, dtraj, t0, len - 1, buf);
   for (int32_t j = len - 1; j >= 0; --j) {
     if (j > 0)
-      fetch_substep<MT>(fv, e, rec, dtraj, t0, j - 1, step0, sbuf + ((j - 1) & 1) * F * 32 + lane);
+      fetch_substep<MT>(fv, e, lane, rec, dtraj, t0, j - 1, buf);
     else
       cp_async_commit();  // an empty group keeps "all but the newest" meaning sub-step j
     cp_async_wait_all_but_one();
-    const float *b = sbuf + (j & 1) * F * 32 + lane;
-    const int64_t t = t0 + j;
-    for (int i = 0; i < 3; ++i) lam.p[i] += b[(W + i) * 32];
-    for (int i = 0; i < 4; ++i) lam.q[i] += b[(W + 3 + i) * 32];
-    for (int i = 0; i < 3; ++i) lam.v[i] += b[(W + 7 + i) * 32];
-    for (int i = 0; i < 3; ++i) lam.w[i] += b[(W + 10 + i) * 32];
-    for (int i = 0; i < MT; ++i)
-      c[i] = (fv.n_seg > 0 && i < nt) ? b[(W + MG_NTRAJ + i) * 32] * A.P.itau : 0.f;
-    for (int i = 0; i < MT; ++i) gcs[i] = 0.f;
-    float zq[4];
-    for (int i = 0; i < 4; ++i) zq[i] = b[(4 * Y + i) * 32];
-    auto stage = [&](int i, St<MT> &y) { read_stage<MT>(b, i * Y, y); };
-    step_vjp_stages<MT, GEN, false>(stage, zq, c, A, gdir, garm, nt, ca, h, lam, G, gcs);
-    add_action_adjoint<MT>(fv, step0 + t, e, nt, A.P.itau, gcs, dact);
+    const float4 *b = &buf.rec[j & 1][0][lane];
+    add_traj_adjoint(&buf.adj[j & 1][0][lane], 32, lam);
+    const float4 z = b[(W - 1) * 32];
+    const float zq[4] = {z.x, z.y, z.z, z.w};
+    auto stage = [&](int i, St<MT> &y, float (&nud)[6]) {
+      get_stage<MT>(b + i * stage_words<MT>() * 32, 32, y, nud);
+    };
+    step_vjp<MT, PATH>(stage, zq, A, gdir, garm, nt, ca, fv.rk, lam, lamn, G, gc);
+    act.add(fv, step0 + t0 + j, e, nt, gc, dact);
   }
 }
 
-// ws: [2][C][rec_words<MT>()][n] floats.  Grid: one block per 32 envs.  GEN: dynamic shared
-// memory [32][MG_NXPARAM] for the block's off-diagonal coefficients (both warps read a lane's
-// row).
-template <int MT, bool GEN>
+// ws: [2][C][rec_words<MT>()][n] float4.  Grid: one block per 32 envs.  General path: dynamic
+// shared memory [32][MG_NXPARAM] for the block's off-diagonal coefficients (both warps read a
+// lane's row).
+template <int MT, int PATH>
 __global__ void __launch_bounds__(kWsThreads)
     k_adjoint_ws(const FleetView fv, const int32_t *__restrict__ types,
                  const float *__restrict__ ckpt, const float *__restrict__ dtraj, int32_t T,
                  int32_t C, int64_t step0, float *__restrict__ dcoef, float *__restrict__ dact,
-                 float *__restrict__ dstate0, float *__restrict__ ws) {
+                 float *__restrict__ dstate0, float4 *__restrict__ ws) {
   __shared__ float4 sgeo[MG_MAX_TYPES][2 * MG_MAX_THR];
-  __shared__ float sbuf[2 * fetch_words<MT>() * 32];
+  __shared__ Fetch<MT> sbuf;
   extern __shared__ float sxh[];
   stage_geometry(fv, sgeo);
   const int64_t env0 = (int64_t)blockIdx.x * 32;
-  if constexpr (GEN) stage_xh_or_zero(fv, env0, (int)min((int64_t)32, fv.n - env0), sxh);
+  if constexpr (PATH == ADJ_GEN)
+    stage_xh_or_zero(fv, env0, (int)min((int64_t)32, fv.n - env0), sxh);
   __syncthreads();
   const int warp = (int)(threadIdx.x >> 5), lane = (int)(threadIdx.x & 31);
   const int64_t e = env0 + lane;
@@ -816,44 +977,49 @@ __global__ void __launch_bounds__(kWsThreads)
   const float4 *gdir = sgeo[type], *garm = sgeo[type] + MG_MAX_THR;
   const int nt = fv.geo[type].n_thr;
   const bool ca = !(fv.model_flags & MG_MODEL_NO_CURRENT_ACCEL);
-  const float h = fv.dt;
-  AdjEnv<GEN> A;
-  load_env<GEN>(fv, el, ca, sxh + lane * MG_NXPARAM, A);
+  AdjEnv<PATH> A;
+  load_env<PATH>(fv, el, sxh + lane * MG_NXPARAM, gdir, garm, A);
   const int64_t slot = (int64_t)C * rec_words<MT>() * fv.n;
 
   const int32_t n_ck = (T + C - 1) / C;
   if (warp == 0 && live)
-    produce_segment<MT, GEN>(fv, e, A, lag_env(A.P.itau, h), gdir, garm, nt, ca, h, ckpt,
-                             n_ck - 1, C, T, step0, ws + ((n_ck - 1) & 1) * slot + e);
+    produce_segment<MT, PATH>(fv, e, A, gdir, garm, nt, ca, ckpt, n_ck - 1, C, T, step0,
+                              ws + ((n_ck - 1) & 1) * slot + e);
   __syncthreads();
-  Grad G;
+  Grad<PATH> G;
   zero_grad(G);
-  St<MT> lam;
-  st_zero(lam);
+  Body lam{};
+  float lamn[MT];
+#pragma unroll
+  for (int i = 0; i < MT; ++i) lamn[i] = 0.f;
+  ActionAdjoint<MT> act;
   for (int32_t sg = n_ck - 1; sg >= 0; --sg) {
     if (warp == 0) {
       if (live && sg > 0)
-        produce_segment<MT, GEN>(fv, e, A, lag_env(A.P.itau, h), gdir, garm, nt, ca, h, ckpt,
-                                 sg - 1, C, T, step0, ws + ((sg - 1) & 1) * slot + e);
+        produce_segment<MT, PATH>(fv, e, A, gdir, garm, nt, ca, ckpt, sg - 1, C, T, step0,
+                                  ws + ((sg - 1) & 1) * slot + e);
     } else if (live) {
-      consume_segment<MT, GEN>(fv, e, lane, A, gdir, garm, nt, ca, h, dtraj, sg, C, T, step0,
-                               ws + (sg & 1) * slot + e, sbuf, dact, lam, G);
+      consume_segment<MT, PATH>(fv, e, lane, A, gdir, garm, nt, ca, dtraj, sg, C, T, step0,
+                                ws + (sg & 1) * slot + e, sbuf, dact, act, lam, lamn, G);
     }
     __syncthreads();
   }
-  if (warp == 1 && live) write_gradients<MT>(G, lam, e, dcoef, dstate0);
+  if (warp == 1 && live) {
+    act.flush(fv, e, nt, dact);
+    write_gradients<MT>(G, fv.pa, lam, lamn, e, dcoef, dstate0);
+  }
 }
 
-template <int MT, bool GEN>
+template <int MT, int PATH>
 cudaError_t launch_adjoint_t(const FleetView &fv, const int32_t *types, const float *ckpt,
                              const float *dtraj, int32_t T, int32_t C, int64_t step0,
-                             float *dcoef, float *dact, float *dstate0, bool split, float *ws,
+                             float *dcoef, float *dact, float *dstate0, bool split, void *ws,
                              int n_sm, cudaStream_t stream) {
   if (split) {
     const int grid = (int)((fv.n + 31) / 32);
-    const size_t smem = GEN ? sizeof(float) * 32 * MG_NXPARAM : 0;
-    k_adjoint_ws<MT, GEN><<<grid, kWsThreads, smem, stream>>>(fv, types, ckpt, dtraj, T, C,
-                                                               step0, dcoef, dact, dstate0, ws);
+    const size_t smem = PATH == ADJ_GEN ? sizeof(float) * 32 * MG_NXPARAM : 0;
+    k_adjoint_ws<MT, PATH><<<grid, kWsThreads, smem, stream>>>(
+        fv, types, ckpt, dtraj, T, C, step0, dcoef, dact, dstate0, static_cast<float4 *>(ws));
     return cudaGetLastError();
   }
   // One warp per block while the fleet has fewer warps than the GPU has SMs x 4 (the backward
@@ -862,9 +1028,9 @@ cudaError_t launch_adjoint_t(const FleetView &fv, const int32_t *types, const fl
   const int64_t warps = (fv.n + 31) / 32;
   const int threads = warps <= 4 * (int64_t)n_sm ? 32 : kAdjThreads;
   const int grid = (int)((fv.n + threads - 1) / threads);
-  const size_t smem = GEN ? sizeof(float) * threads * MG_NXPARAM : 0;
-  k_adjoint<MT, GEN><<<grid, threads, smem, stream>>>(fv, types, ckpt, dtraj, T, C, step0, dcoef,
-                                                      dact, dstate0);
+  const size_t smem = PATH == ADJ_GEN ? sizeof(float) * threads * MG_NXPARAM : 0;
+  k_adjoint<MT, PATH><<<grid, threads, smem, stream>>>(fv, types, ckpt, dtraj, T, C, step0, dcoef,
+                                                       dact, dstate0);
   return cudaGetLastError();
 }
 
@@ -976,11 +1142,6 @@ cudaError_t rollout_fwd_d(const FleetView &fv, const BlockDesc *blocks, int n_bl
 
 }  // namespace
 
-cudaError_t launch_checkpoint(const StatePlanes &st, int64_t n, float *ck, cudaStream_t stream) {
-  k_checkpoint<<<(int)((n + 255) / 256), 256, 0, stream>>>(st, n, ck);
-  return cudaGetLastError();
-}
-
 cudaError_t launch_rollout_forward(const FleetView &fv, const BlockDesc *blocks, int n_blocks,
                                    int threads, NtVariant ntv, bool diag, int layout,
                                    int32_t T, int32_t C, float *traj, float *ckpt,
@@ -1012,41 +1173,47 @@ cudaError_t sm_count(int *n_sm) {
 
 }  // namespace
 
-cudaError_t adjoint_split(int64_t n, int mode, bool *split) {
+cudaError_t adjoint_split(int64_t n, bool general, int mode, bool *split) {
   if (mode == 1 || mode == 2) {
     *split = mode == 2;
     return cudaSuccess;
   }
-  // by fleet size: the two-warp form while its 2 x ceil(n / 32) warps fit one per scheduler
+  // By fleet size: the two-warp form while all its blocks are resident at once (four per SM), and
+  // twice that on the general path.  200 sub-steps, checkpoints every 20, one-warp / two-warp,
+  // us: diagonal mass 4,096 envs 544 / 335, 16,384 696 / 552, 32,768 1,004 / 1,082; general 4,096
+  // 1,283 / 736, 16,384 1,458 / 1,052, 32,768 2,425 / 2,062.
   int n_sm = 0;
   cudaError_t e = sm_count(&n_sm);
   if (e != cudaSuccess) return e;
-  *split = (n + 31) / 32 <= 2 * (int64_t)n_sm;
+  *split = (n + 31) / 32 <= (general ? 8 : 4) * (int64_t)n_sm;
   return cudaSuccess;
 }
 
 size_t adjoint_workspace_bytes(bool eight, int64_t n, int32_t C) {
   return 2 * (size_t)C * (size_t)(eight ? rec_words<8>() : rec_words<6>()) * (size_t)n *
-         sizeof(float);
+         sizeof(float4);
 }
 
 cudaError_t launch_adjoint(const FleetView &fv, const int32_t *types, bool eight, bool general,
-                           const float *ckpt, const float *dtraj, int32_t T, int32_t C,
+                           int layout, const float *ckpt, const float *dtraj, int32_t T, int32_t C,
                            int64_t step0, float *dcoef, float *dact, float *dstate0, bool split,
-                           float *ws, cudaStream_t stream) {
+                           void *ws, cudaStream_t stream) {
   if (C < 1 || C > kMaxSeg || T < 1 || (split && !ws)) return cudaErrorInvalidValue;
   int n_sm = 0;
   cudaError_t e = sm_count(&n_sm);
   if (e != cudaSuccess) return e;
+  auto run = [&](auto launch) {
+    return launch(fv, types, ckpt, dtraj, T, C, step0, dcoef, dact, dstate0, split, ws, n_sm,
+                  stream);
+  };
+  const int path = general ? ADJ_GEN : layout == MG_LAYOUT_MIRRORED ? ADJ_MIRRORED : ADJ_DENSE;
   if (eight)
-    return general ? launch_adjoint_t<8, true>(fv, types, ckpt, dtraj, T, C, step0, dcoef, dact,
-                                               dstate0, split, ws, n_sm, stream)
-                   : launch_adjoint_t<8, false>(fv, types, ckpt, dtraj, T, C, step0, dcoef,
-                                                dact, dstate0, split, ws, n_sm, stream);
-  return general ? launch_adjoint_t<6, true>(fv, types, ckpt, dtraj, T, C, step0, dcoef, dact,
-                                             dstate0, split, ws, n_sm, stream)
-                 : launch_adjoint_t<6, false>(fv, types, ckpt, dtraj, T, C, step0, dcoef, dact,
-                                              dstate0, split, ws, n_sm, stream);
+    return path == ADJ_GEN     ? run(launch_adjoint_t<8, ADJ_GEN>)
+           : path == ADJ_DENSE ? run(launch_adjoint_t<8, ADJ_DENSE>)
+                               : run(launch_adjoint_t<8, ADJ_MIRRORED>);
+  return path == ADJ_GEN     ? run(launch_adjoint_t<6, ADJ_GEN>)
+         : path == ADJ_DENSE ? run(launch_adjoint_t<6, ADJ_DENSE>)
+                             : run(launch_adjoint_t<6, ADJ_MIRRORED>);
 }
 
 int adjoint_max_interval() { return kMaxSeg; }

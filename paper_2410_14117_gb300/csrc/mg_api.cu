@@ -1236,7 +1236,8 @@ mg_status mg_rollout_backward(mg_sim *s, int32_t T, int32_t C, const float *ckpt
     return fail(MG_EINVAL, "adjoint buffers must be device memory");
   const bool eight = s->ntv != NT_6;
   bool split = false;
-  MG_CK(adjoint_split(s->n, s->adj_mode, &split));
+  const bool general = !s->diag || s->has_xh;
+  MG_CK(adjoint_split(s->n, general, s->adj_mode, &split));
   if (split) {
     const size_t bytes = adjoint_workspace_bytes(eight, s->n, C);
     if (s->adj_ws_cap < bytes) {
@@ -1247,13 +1248,15 @@ mg_status mg_rollout_backward(mg_sim *s, int32_t T, int32_t C, const float *ckpt
       if (cudaMalloc(&s->adj_ws, bytes) != cudaSuccess) {
         cudaGetLastError();
         s->adj_ws = nullptr;
-        return fail(MG_ENOMEM, "cudaMalloc(adjoint workspace)");
+        if (s->adj_mode == 2) return fail(MG_ENOMEM, "cudaMalloc(adjoint workspace)");
+        split = false;  // the one-warp form needs no workspace and gives the same results
+      } else {
+        s->adj_ws_cap = bytes;
       }
-      s->adj_ws_cap = bytes;
     }
   }
-  MG_CK(launch_adjoint(s->view(), s->types_d, eight, !s->diag || s->has_xh, ckpt, dtraj, T, C,
-                       step0, dcoef, dact, dstate0, split, s->adj_ws, s->stream));
+  MG_CK(launch_adjoint(s->view(), s->types_d, eight, general, s->layout, ckpt, dtraj,
+                       T, C, step0, dcoef, dact, dstate0, split, s->adj_ws, s->stream));
   return MG_OK;
 }
 

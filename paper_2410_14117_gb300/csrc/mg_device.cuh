@@ -326,10 +326,9 @@ __device__ __forceinline__ void store_state(const StatePlanes &sp, int64_t e, co
 }
 
 // ---------------------------------------------------------------- right-hand side of Eq. 1
-// d = f(s; c) with two storage conventions that save multiplies in the hot loop:
-//   - cs[i] = c_i / tau_m (the command divided by the lag constant by the caller), so
-//     n_i' = cs_i - n_i / tau_m is a single FMA (LAGD only);
-//   - d.q holds 2 q' (the 1/2 of q' = 1/2 q (x) (0, w) is folded into the RK4 weights).
+// d = f(s) for the pose and velocity (d.n is left unset: the linear throttle lag is integrated in
+// closed form, LagEnv).  d.q holds 2 q' (the 1/2 of q' = 1/2 q (x) (0, w) is folded into the RK4
+// weights).
 // Every sum is written as a chain of FMAs (same terms as Eq. 1; only the rounding order differs
 // from a term-by-term evaluation).  The diagonal-mass path reads the StepDiag coefficients (each
 // row's chain ends in nu'_i, no separate M^-1 multiply); the general path reads ParGen and
@@ -348,15 +347,14 @@ __device__ __forceinline__ void store_state(const StatePlanes &sp, int64_t e, co
 // XH (general path only): the env's off-diagonal hydrodynamic coefficients xh[MG_NXPARAM]
 // (M_A above its diagonal, then D_l's off-diagonal entries, both row-major; mg.h) enter the
 // added-mass momenta Q = M_A nu_r, the current term M_A [w x v_c^b; 0] and the damping D_l nu_r.
-// LAGD = false leaves d.n unset (the caller integrates the linear throttle lag in closed form).
 // The diagonal-mass path always includes the current-acceleration term (current_accel unused).
-template <int MT, bool DIAG, bool MIXED, int NH = 0, bool XH = false, bool LAGD = true>
-__device__ __forceinline__ void rhs(const St<MT> &s, const float (&cs)[MT], const Coef<DIAG, NH> &P,
+template <int MT, bool DIAG, bool MIXED, int NH = 0, bool XH = false>
+__device__ __forceinline__ void rhs(const St<MT> &s, const Coef<DIAG, NH> &P,
                                     const float4 *gdir, const float4 *garm, int nt,
                                     bool current_accel, St<MT> &d,
                                     const float *__restrict__ xh = nullptr) {
   static_assert(!(XH && DIAG), "the off-diagonal hydrodynamics use the general path");
-  // Thrusters (Eq. 3 actions): F_i = kT n_i|n_i| along d_i at r_i; n_i' = (c_i - n_i) / tau_m.
+  // Thrusters (Eq. 3 actions): F_i = kT n_i|n_i| along d_i at r_i.
   constexpr bool MIRRORED = DIAG && NH == MG_LAYOUT_MIRRORED;
   float t0 = 0.f, t1 = 0.f, t2 = 0.f, t3 = 0.f, t4 = 0.f, t5 = 0.f;
   if constexpr (MIRRORED) {
@@ -375,10 +373,6 @@ __device__ __forceinline__ void rhs(const St<MT> &s, const float (&cs)[MT], cons
       t2 += s67;
       t3 += add(7, -f6);
     }
-    if constexpr (LAGD) {
-#pragma unroll
-      for (int i = 0; i < MT; ++i) d.n[i] = fmaf(-s.n[i], P.itau, cs[i]);
-    }
   } else
 #pragma unroll
   for (int i = 0; i < MT; ++i) {
@@ -394,7 +388,6 @@ __device__ __forceinline__ void rhs(const St<MT> &s, const float (&cs)[MT], cons
       } else {
         t2 = fmaf(f, dd.z, t2); t3 = fmaf(f, aa.x, t3); t4 = fmaf(f, aa.y, t4);
       }
-      if constexpr (LAGD) d.n[i] = fmaf(-s.n[i], P.itau, cs[i]);
     }
   }
   (void)nt;
@@ -623,22 +616,22 @@ __device__ __forceinline__ void rk4_step(St<MT> &s, const float (&c)[MT], const 
   float d[MT];
 #pragma unroll
   for (int i = 0; i < MT; ++i) d[i] = s.n[i] - c[i];
-  rhs<MT, DIAG, MIXED, NH, XH, false>(s, c, P, gdir, garm, nt, current_accel, k, xh);
+  rhs<MT, DIAG, MIXED, NH, XH>(s, P, gdir, garm, nt, current_accel, k, xh);
   axpy<MT, false>(acc, s, rk.h6, rk.q12, k);
   axpy<MT, false>(y, s, rk.hh, rk.qh, k);
 #pragma unroll
   for (int i = 0; i < MT; ++i) y.n[i] = fmaf(L.f2, d[i], c[i]);
-  rhs<MT, DIAG, MIXED, NH, XH, false>(y, c, P, gdir, garm, nt, current_accel, k, xh);
+  rhs<MT, DIAG, MIXED, NH, XH>(y, P, gdir, garm, nt, current_accel, k, xh);
   axpy<MT, false>(acc, acc, rk.h3, rk.h6, k);
   axpy<MT, false>(y, s, rk.hh, rk.qh, k);
 #pragma unroll
   for (int i = 0; i < MT; ++i) y.n[i] = fmaf(L.f3, d[i], c[i]);
-  rhs<MT, DIAG, MIXED, NH, XH, false>(y, c, P, gdir, garm, nt, current_accel, k, xh);
+  rhs<MT, DIAG, MIXED, NH, XH>(y, P, gdir, garm, nt, current_accel, k, xh);
   axpy<MT, false>(acc, acc, rk.h3, rk.h6, k);
   axpy<MT, false>(y, s, rk.h, rk.hh, k);
 #pragma unroll
   for (int i = 0; i < MT; ++i) y.n[i] = fmaf(L.f4, d[i], c[i]);
-  rhs<MT, DIAG, MIXED, NH, XH, false>(y, c, P, gdir, garm, nt, current_accel, k, xh);
+  rhs<MT, DIAG, MIXED, NH, XH>(y, P, gdir, garm, nt, current_accel, k, xh);
   axpy<MT, false>(s, acc, rk.h6, rk.q12, k);
 #pragma unroll
   for (int i = 0; i < MT; ++i) s.n[i] = fmaf(L.P, d[i], c[i]);

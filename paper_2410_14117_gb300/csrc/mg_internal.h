@@ -208,7 +208,6 @@ cudaStream_t pool_stream(const mg_pool *p);
 int64_t pool_capacity(const mg_pool *p);
 
 // ---------------------------------------------------------------- launchers (mg_adjoint.cu)
-cudaError_t launch_checkpoint(const StatePlanes &st, int64_t n, float *ck, cudaStream_t stream);
 // The rollout's forward in one launch on the static grid (mg_adjoint.cu): T sub-steps, ckpt
 // [ceil(T / C)][MG_NSTATE][n] before sub-steps 0, C, ..., traj [T][MG_NTRAJ][n] after each.
 cudaError_t launch_rollout_forward(const FleetView &fv, const BlockDesc *blocks, int n_blocks,
@@ -216,14 +215,15 @@ cudaError_t launch_rollout_forward(const FleetView &fv, const BlockDesc *blocks,
                                    int32_t T, int32_t C, float *traj, float *ckpt,
                                    cudaStream_t stream);
 // Backward kernel: mode 1 one warp per 32 envs, 2 the two-warp form (producer and consumer warps
-// per 32 envs, through a workspace of adjoint_workspace_bytes), 0 chosen by fleet size.
-cudaError_t adjoint_split(int64_t n, int mode, bool *split);
+// per 32 envs, through a workspace of adjoint_workspace_bytes), 0 chosen by fleet size and path.
+cudaError_t adjoint_split(int64_t n, bool general, int mode, bool *split);
 size_t adjoint_workspace_bytes(bool eight, int64_t n, int32_t C);
 // general: the general-path kernels (off-centre gravity, off-diagonal extension, full M^-1).
+// layout: as launch_fleet (the forward's).
 cudaError_t launch_adjoint(const FleetView &fv, const int32_t *types, bool eight, bool general,
-                           const float *ckpt, const float *dtraj, int32_t T, int32_t C,
+                           int layout, const float *ckpt, const float *dtraj, int32_t T, int32_t C,
                            int64_t step0, float *dcoef, float *dact, float *dstate0, bool split,
-                           float *ws, cudaStream_t stream);
+                           void *ws, cudaStream_t stream);
 int adjoint_max_interval();
 
 // ---------------------------------------------------------------- launchers (mg_task.cu)

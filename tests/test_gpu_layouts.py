@@ -10,6 +10,7 @@ import torch
 from _helpers import TOL_ROLLOUT, TOL_STEP, oracle_nominal, rel_err, vehicles
 from oracle import oracle as O
 from paper_2410_14117_gb300 import inputs as I
+from paper_2410_14117_gb300.adjoint import rollout
 from test_gpu_parity import H, gpu_state, make_sim, oracle_types_geo
 
 pytestmark = pytest.mark.gpu
@@ -99,3 +100,38 @@ def test_recorded_and_rolled_out_states_equal_the_step():
         got.append(gpu_state(sim))
         sim.close()
     np.testing.assert_array_equal(got[0], got[1])
+
+
+@pytest.mark.parametrize("mode", [1, 2])
+@pytest.mark.parametrize("which", [0, 1])
+def test_adjoint_of_renumbered_thrusters(which, mode):
+    """The same vehicles with thrusters 0 and 1 numbered the other way round: not a mirrored frame,
+    so the dense transposes, whose gradients are the mirrored ones' with the actions permuted.
+    Both sides sum the same terms in FP32 over 60 sub-steps: 1e-4 of each env's vector norm."""
+    n, T, C = 97, 60, 16
+    v = [ROV, HEAVY][which]
+    perm = np.array([1, 0, 2, 3, 4, 5, 6, 7])
+    types = np.zeros(n, np.int32)
+    params = I.perturbed_params(5, oracle_nominal([v])[types], n)
+    states = I.random_states(6, n, np.full(n, v.n_thr))
+    cmds = I.commands(7, 6, n, v.n_thr)
+    g = torch.randn((T, n, 13), generator=torch.Generator().manual_seed(3)).cuda()
+    got = []
+    for veh, p in ((v, np.arange(8)), (_swapped(v, 0, 1), perm)):
+        sim = make_sim(types, [veh], queue=False)
+        sim.set_adjoint_mode(mode)
+        sim.set_params(torch.tensor(params, dtype=torch.float32, device="cuda"))
+        coef = torch.tensor(params[:, 4:22], dtype=torch.float32, device="cuda", requires_grad=True)
+        s = states.copy()
+        s[:, 13:] = s[:, 13 + p]
+        s = torch.tensor(s, dtype=torch.float32, device="cuda", requires_grad=True)
+        a = torch.tensor(np.ascontiguousarray(cmds[:, :, p]), device="cuda", requires_grad=True)
+        traj = rollout(sim, coef, a, s, 10, T, C)
+        dc, da, ds = torch.autograd.grad(traj, (coef, a, s), g)
+        ds = torch.cat([ds[:, :13], ds[:, 13 + p]], dim=1)
+        got.append([x.double().cpu().numpy() for x in (dc, da[:, :, p].permute(1, 0, 2), ds)])
+        sim.close()
+    for x, y in zip(*got):
+        x, y = x.reshape(n, -1), y.reshape(n, -1)
+        err = np.linalg.norm(x - y, axis=1) / np.linalg.norm(y, axis=1)
+        assert err.max() <= 1e-4
