@@ -427,8 +427,8 @@ mg_status mg_task_step(mg_sim *sim, int32_t k, float *obs, float *err, uint8_t *
  * one-segment schedule, held over all k >= 1 sub-steps, and the task step of mg_task_step
  * follows, writing reward = -(Eq. 4 position error) instead of err.  The schedule replaces the
  * sim's actions on the first call (and after any other action call) and is rewritten in place
- * by the later ones, so a policy loop pays one small copy kernel per step.  actions may be
- * reused once the stream has passed the call.  obs, reward, done, episode_err: device, as
+ * by the later ones: by the step's one launch for k <= steps_per_launch, by a small copy kernel
+ * ahead of the launches for larger k.  actions may be reused once the stream has passed the call.  obs, reward, done, episode_err: device, as
  * mg_task_step.  Asynchronous.  Errors: MG_ESTATE (no task), MG_EINVAL (k < 1, NULL, host
  * memory), MG_ENOMEM (the schedule's first allocation). */
 mg_status mg_env_step(mg_sim *sim, int32_t k, const float *actions, float *obs, float *reward,

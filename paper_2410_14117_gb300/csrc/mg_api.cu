@@ -1299,9 +1299,10 @@ mg_status mg_task_obs_dim(mg_sim *s, int32_t *obs_dim) {
 
 namespace {
 
-// A task step (mg_task_step) with its outputs; err and reward may each be null.
+// A task step (mg_task_step) with its outputs; err and reward may each be null.  actions: the
+// throttles of an environment step (mg_env_step), to be clamped into the schedule env_act.
 mg_status task_step_outputs(mg_sim *s, int32_t k, float *obs, float *err, float *reward,
-                            uint8_t *done, float *episode_err) {
+                            uint8_t *done, float *episode_err, const float *actions = nullptr) {
   if (!s->has_task) return fail(MG_ESTATE, "no task set");
   if (k < 0) return fail(MG_EINVAL, "k must be >= 0");
   // a policy loop passes the same output buffers every call: check them once (a pointer query
@@ -1321,13 +1322,16 @@ mg_status task_step_outputs(mg_sim *s, int32_t k, float *obs, float *err, float 
   // Leading sub-steps as mg_step; the last static chunk carries the fused task epilogue.
   const int32_t k_last = (k - 1) % s->spl + 1;
   if (k > k_last) {
+    if (actions)
+      MG_CK(launch_clamp_actions(actions, s->env_act, s->n * (int64_t)s->act_w, s->stream));
+    actions = nullptr;  // the schedule holds them from here on
     mg_status st = mg_step(s, k - k_last);
     if (st != MG_OK) return st;
   }
   int32_t obs_dim = 0;
   mg_task_obs_dim(s, &obs_dim);
   TaskOut to{obs, err, done, episode_err, obs_dim, 0, s->reset_seed, s->nu0_sigma, s->episode,
-             reward};
+             reward, actions, actions ? s->env_act : nullptr};
   FleetView v = s->view();
   v.cursor_adv = k_last;
   MG_CK(launch_fleet_task(v, s->blocks_d, s->n_blocks, s->threads, s->ntv, s->diag,
@@ -1389,8 +1393,7 @@ mg_status mg_env_step(mg_sim *s, int32_t k, const float *actions, float *obs, fl
     s->hold = 1 << 30;
     if ((st = rewind_cursor(s)) != MG_OK) return st;
   }
-  MG_CK(launch_clamp_actions(actions, s->env_act, (int64_t)floats, s->stream));
-  return task_step_outputs(s, k, obs, nullptr, reward, done, episode_err);
+  return task_step_outputs(s, k, obs, nullptr, reward, done, episode_err, actions);
 }
 
 mg_status mg_get_state(mg_sim *s, float *out) {

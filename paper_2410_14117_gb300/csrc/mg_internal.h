@@ -255,6 +255,10 @@ struct TaskOut {
   double sigma;
   uint32_t *episode;
   float *reward;     // [n] or null: the negative error
+  // Environment step: the policy's throttles [n][fv.act_w], clamped by this launch into the
+  // schedule act_out of the same shape and held over it; null: the sim's own action schedule.
+  const float *act_in;
+  float *act_out;
 };
 
 // Final launch of a task step: k_launch sub-steps (static grid), then the task epilogue for a

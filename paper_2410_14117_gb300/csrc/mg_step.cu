@@ -69,10 +69,14 @@ __global__ void __maxnreg__(XH ? kRegsXH : !DIAG ? kRegsGeneral : WIDE ? kRegsWi
   if ((int)threadIdx.x >= bd.count) return;
   const int64_t e = (int64_t)bd.env0 + threadIdx.x;
   St<MT> st;
-  advance_env<MT, DIAG, MIXED, REC, false, NH, XH>(fv, e, MIXED ? bd.n_thr : MT, sdir, sarm,
-                                                   s_cursor + fv.cursor_off, k, traj, st,
-                                                   XH ? sxh + threadIdx.x * MG_NXPARAM
-                                                      : nullptr);
+  const int nt = MIXED ? bd.n_thr : MT;
+  const int64_t step0 = s_cursor + fv.cursor_off;
+  advance_env<MT, DIAG, MIXED, REC, false, NH, XH>(
+      fv, e, nt, sdir, sarm,
+      [&](float (&c)[MT], int64_t &seg, int32_t &left) {
+        scheduled_start<MT>(fv, e, nt, step0, c, seg, left);
+      },
+      k, traj, st, XH ? sxh + threadIdx.x * MG_NXPARAM : nullptr);
   store_and_flag<MT, false>(fv, e, st);
   if (fv.cursor_adv) finish_envs(fv, &s_done, bd.count, fv.cursor_adv);
 }
@@ -130,10 +134,13 @@ __global__ void __maxnreg__(XH ? kRegsXH : !DIAG ? kRegsGeneral : WIDE ? kRegsWi
       if constexpr (XH)
         for (int j = 0; j < MG_NXPARAM; ++j) row[j] = __ldg(fv.xh + (int64_t)j * fv.n + e);
       St<MT> st;
-      advance_env<MT, DIAG, MIXED, false, true, NH, XH>(fv, e, MIXED ? bd.n_thr : MT, gdir, garm,
-                                                        step0 + (int64_t)c * chunk,
-                                                        min(chunk, k_total - c * chunk),
-                                                        nullptr, st, XH ? row : nullptr);
+      const int nt = MIXED ? bd.n_thr : MT;
+      advance_env<MT, DIAG, MIXED, false, true, NH, XH>(
+          fv, e, nt, gdir, garm,
+          [&](float (&cmd)[MT], int64_t &seg, int32_t &left) {
+            scheduled_start<MT>(fv, e, nt, step0 + (int64_t)c * chunk, cmd, seg, left);
+          },
+          min(chunk, k_total - c * chunk), nullptr, st, XH ? row : nullptr);
       store_and_flag<MT, true>(fv, e, st);
     }
     __syncwarp();

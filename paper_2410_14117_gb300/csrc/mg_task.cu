@@ -242,6 +242,34 @@ __device__ __forceinline__ void copy_rows(const float *src, float *dst, int n_ro
   for (int i = i0 + lane; i < total; i += n_act) dst[i] = src[i];
 }
 
+// Throttles clamped to [-1, 1] (NaN kept).
+__device__ __forceinline__ float clamp_throttle(float x) {
+  return x < -1.f ? -1.f : (x > 1.f ? 1.f : x);
+}
+
+// The env's throttles of an environment step: clamped into the schedule's row, and into c (entries
+// past the vehicle's thruster count zero).  The policy's buffer may have any 4-byte alignment; the
+// schedule's rows start 8-byte (w = 6) or 16-byte (w = 8) aligned.
+template <int MT>
+__device__ __forceinline__ void env_commands(const FleetView &fv, const TaskOut &to, int64_t e,
+                                             int nt, float (&c)[MT]) {
+  const int w = MT == 6 && fv.act_w == 6 ? 6 : MG_MAX_THR;
+  const float *in = to.act_in + e * w;
+  float x[MG_MAX_THR];
+#pragma unroll
+  for (int i = 0; i < MG_MAX_THR; ++i) x[i] = i < 6 || w > 6 ? clamp_throttle(in[i]) : 0.f;
+  float2 *out = reinterpret_cast<float2 *>(to.act_out + e * w);
+#pragma unroll
+  for (int i = 0; i < 3; ++i) out[i] = make_float2(x[2 * i], x[2 * i + 1]);
+  if (w > 6) out[3] = make_float2(x[6], x[7]);
+#pragma unroll
+  for (int i = 0; i < MT; ++i) c[i] = i < nt ? x[i] : 0.f;
+}
+
+__device__ __forceinline__ void prefetch_l1(const void *p) {
+  asm volatile("prefetch.global.L1 [%0];" ::"l"(p));
+}
+
 // The last launch of a task step: the env's final sub-steps as in k_fleet, then the task
 // epilogue from the state still in registers, so the state is stored once and never re-read.
 // Each warp stages its 32 rows of the observation in shared memory (when they fit) and writes
@@ -267,21 +295,38 @@ __global__ void __maxnreg__(XH ? kRegsXH : DIAG ? kRegsDiag : kRegsGeneral)
     sarm[threadIdx.x] = fv.geo[bd.type].arm[threadIdx.x];
   }
   // Programmatic dependent launch: the block descriptors and the geometry above are written
-  // before any step; everything below waits for the previous kernel in the stream (the action
-  // copy of mg_env_step, or the task step's leading launches) to complete.
+  // before any step; everything below waits for the previous kernel in the stream to complete,
+  // and the next step's launch may run up to its own wait beside this one.
+  cudaTriggerProgrammaticLaunchCompletion();
   cudaGridDependencySynchronize();
   if (threadIdx.x == 0) {
     s_done = 0u;
-    s_cursor = launch_cursor(fv);
+    if (!to.act_in) s_cursor = launch_cursor(fv);
   }
   if constexpr (XH) stage_xh(fv.xh, fv.n, bd.env0, bd.count, sxh);
   __syncthreads();
   if ((int)threadIdx.x >= bd.count) return;
   const int64_t e = (int64_t)bd.env0 + threadIdx.x;
+  const int nt = MIXED ? bd.n_thr : MT;
+  // what the epilogue reads, on its way while the sub-steps run
+  prefetch_l1(tv.centre + e);
+  prefetch_l1(tv.clock + e);
+  prefetch_l1(tv.err_sum + e);
+  prefetch_l1(fv.flags + e);
+  prefetch_l1(to.episode + e);
   St<MT> s;
   advance_env<MT, DIAG, MIXED, false, false, NH, XH>(
-      fv, e, MIXED ? bd.n_thr : MT, sdir, sarm, s_cursor + fv.cursor_off, k_launch, nullptr, s,
-      XH ? sxh + threadIdx.x * MG_NXPARAM : nullptr);
+      fv, e, nt, sdir, sarm,
+      [&](float (&c)[MT], int64_t &seg, int32_t &left) {
+        if (to.act_in) {  // one command for the whole launch, no cursor
+          seg = 0;
+          left = k_launch;
+          env_commands<MT>(fv, to, e, nt, c);
+        } else {
+          scheduled_start<MT>(fv, e, nt, s_cursor + fv.cursor_off, c, seg, left);
+        }
+      },
+      k_launch, nullptr, s, XH ? sxh + threadIdx.x * MG_NXPARAM : nullptr);
 
   const int obs_dim = to.obs_dim;
   task_epilogue<MT>(fv, tv, to, k_task, e, task_in(fv, tv, to, e), s,
@@ -346,8 +391,7 @@ __global__ void k_clamp_actions(const float *__restrict__ in, float *__restrict_
   cudaTriggerProgrammaticLaunchCompletion();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= count) return;
-  const float x = in[i];
-  out[i] = x < -1.f ? -1.f : (x > 1.f ? 1.f : x);
+  out[i] = clamp_throttle(in[i]);
 }
 
 }  // namespace
