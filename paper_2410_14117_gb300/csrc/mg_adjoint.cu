@@ -587,20 +587,26 @@ __device__ __forceinline__ void step_vjp(Stage stage, const float (&zq)[4], cons
 
 constexpr int kMaxSeg = 32;  // largest checkpoint interval
 
-// The buffered command of sub-step j (cursor position).
+// The held command along a forward walk over sub-steps (the forward's own schedule).
 template <int MT>
-__device__ __forceinline__ void commands_at(const FleetView &fv, int64_t e, int64_t j, int nt,
-                                            float (&c)[MT]) {
-  int64_t seg = j / fv.hold;
-  if (seg > fv.n_seg - 1) seg = fv.n_seg - 1;
-  for (int i = 0; i < MT; ++i) c[i] = 0.f;
-  if (fv.n_seg > 0) {
-    const float *a = fv.act + (seg * fv.n + e) * fv.act_w;
-    #pragma unroll
-    for (int i = 0; i < MT; ++i)
-      if (i < nt) c[i] = a[i];
+struct CommandWalk {
+  int64_t seg;
+  int32_t left;
+  float c[MT];
+
+  __device__ __forceinline__ CommandWalk(const FleetView &fv, int64_t e, int nt, int64_t step0) {
+    scheduled_start<MT>(fv, e, nt, step0, c, seg, left);
+    prefetch_commands(fv, e, seg);
   }
-}
+  __device__ __forceinline__ void next(const FleetView &fv, int64_t e, int nt) {
+    if (--left == 0) {
+      ++seg;
+      left = fv.hold;
+      load_commands<MT>(fv, e, seg, nt, c);
+      prefetch_commands(fv, e, seg);
+    }
+  }
+};
 
 template <int MT>
 __device__ __forceinline__ void load_checkpoint(const float *__restrict__ ckpt, int32_t sg,
@@ -623,33 +629,40 @@ __device__ __forceinline__ void add_traj_adjoint(const float *__restrict__ g, in
 }
 
 // Command adjoints of the sub-steps that share an action segment, summed in registers and added
-// to the caller's buffer when the walk leaves the segment.
+// to the caller's buffer when the backward walk leaves the segment.
 template <int MT>
 struct ActionAdjoint {
-  int64_t seg = -1;
+  int64_t seg;   // the segment being summed
+  int64_t left;  // its sub-steps still ahead of the walk
   float g[MT];
 
+  // The walk starts at cursor position t.
+  __device__ __forceinline__ ActionAdjoint(const FleetView &fv, int64_t t) {
+    seg = t / fv.hold;
+    if (seg > fv.n_seg - 1) seg = fv.n_seg - 1;  // the last segment holds for good
+    left = t - seg * fv.hold + 1;
+#pragma unroll
+    for (int i = 0; i < MT; ++i) g[i] = 0.f;
+  }
   __device__ __forceinline__ void flush(const FleetView &fv, int64_t e, int nt, float *dact) {
-    if (seg < 0) return;
+    if (!dact || seg < 0) return;
     float *da = dact + (seg * fv.n + e) * fv.act_w;
 #pragma unroll
-    for (int i = 0; i < MT; ++i)
+    for (int i = 0; i < MT; ++i) {
       if (i < nt) da[i] += g[i];
-  }
-  // sub-step t (cursor position), walked backwards
-  __device__ __forceinline__ void add(const FleetView &fv, int64_t t, int64_t e, int nt,
-                                      const float (&gc)[MT], float *dact) {
-    if (!dact || fv.n_seg <= 0) return;
-    int64_t sg = t / fv.hold;
-    if (sg > fv.n_seg - 1) sg = fv.n_seg - 1;
-    if (sg != seg) {
-      flush(fv, e, nt, dact);
-      seg = sg;
-#pragma unroll
-      for (int i = 0; i < MT; ++i) g[i] = 0.f;
+      g[i] = 0.f;
     }
+  }
+  // One sub-step's command adjoint.
+  __device__ __forceinline__ void add(const FleetView &fv, int64_t e, int nt,
+                                      const float (&gc)[MT], float *dact) {
 #pragma unroll
     for (int i = 0; i < MT; ++i) g[i] += gc[i];
+    if (--left == 0) {
+      flush(fv, e, nt, dact);
+      --seg;
+      left = fv.hold;
+    }
   }
 };
 
@@ -807,26 +820,32 @@ __global__ void __launch_bounds__(kAdjThreads)
   for (int i = 0; i < MT; ++i) lamn[i] = 0.f;
   St<MT> S[kMaxSeg];
   float4 rec[4 * stage_words<MT>()];
-  float c[MT], gc[MT], zq[4];
-  ActionAdjoint<MT> act;
+  float gc[MT], zq[4];
+  ActionAdjoint<MT> act(fv, step0 + T - 1);
 
   const int32_t n_ck = (T + C - 1) / C;
   for (int32_t sg = n_ck - 1; sg >= 0; --sg) {
     const int32_t t0 = sg * C, len = min(C, T - t0);
     // re-run the segment from its checkpoint
     load_checkpoint<MT>(ckpt, sg, n, e, S[0]);
-    for (int32_t j = 1; j < len; ++j) {
-      St<MT> x = S[j - 1];
-      commands_at<MT>(fv, e, step0 + t0 + j - 1, nt, c);
-      rk4_step<MT, PATH != ADJ_GEN, true, adj_layout(PATH), PATH == ADJ_GEN>(
-          x, c, A.L, A.F, gdir, garm, nt, ca, fv.rk, A.xh);
-      S[j] = x;
+    {
+      CommandWalk<MT> cmd(fv, e, nt, step0 + t0);
+      St<MT> x = S[0];
+      for (int32_t j = 1; j < len; ++j) {
+        rk4_step<MT, PATH != ADJ_GEN, true, adj_layout(PATH), PATH == ADJ_GEN>(
+            x, cmd.c, A.L, A.F, gdir, garm, nt, ca, fv.rk, A.xh);
+        S[j] = x;
+        cmd.next(fv, e, nt);
+      }
     }
     // walk it backwards
     for (int32_t j = len - 1; j >= 0; --j) {
       const int64_t t = t0 + j;
       add_traj_adjoint(dtraj + t * MG_NTRAJ * n + e, n, lam);
-      commands_at<MT>(fv, e, step0 + t, nt, c);
+      int64_t cs;
+      int32_t cl;
+      float c[MT];
+      scheduled_start<MT>(fv, e, nt, step0 + t, c, cs, cl);
       St<MT> x = S[j];
       stage_step<MT, PATH>(x, c, A, gdir, garm, nt, ca, fv.rk, zq,
                            [&](int g, const St<MT> &y, const float (&nud)[6]) {
@@ -836,7 +855,7 @@ __global__ void __launch_bounds__(kAdjThreads)
         get_stage<MT>(rec + i * stage_words<MT>(), 1, y, nud);
       };
       step_vjp<MT, PATH>(stage, zq, A, gdir, garm, nt, ca, fv.rk, lam, lamn, G, gc);
-      act.add(fv, step0 + t, e, nt, gc, dact);
+      act.add(fv, e, nt, gc, dact);
     }
   }
   act.flush(fv, e, nt, dact);
@@ -865,15 +884,16 @@ __device__ __forceinline__ void produce_segment(const FleetView &fv, int64_t e,
   const int32_t t0 = sg * C, len = min(C, T - t0);
   St<MT> S;
   load_checkpoint<MT>(ckpt, sg, n, e, S);
-  float c[MT], zq[4];
+  float zq[4];
+  CommandWalk<MT> cmd(fv, e, nt, step0 + t0);
   for (int32_t j = 0; j < len; ++j) {
-    commands_at<MT>(fv, e, step0 + t0 + j, nt, c);
     float4 *r = rec + (int64_t)j * W * n;
-    stage_step<MT, PATH>(S, c, A, gdir, garm, nt, ca, fv.rk, zq,
+    stage_step<MT, PATH>(S, cmd.c, A, gdir, garm, nt, ca, fv.rk, zq,
                          [&](int g, const St<MT> &y, const float (&nud)[6]) {
                            put_stage<MT>(r + (int64_t)g * stage_words<MT>() * n, n, y, nud);
                          });
     r[(int64_t)(W - 1) * n] = make_float4(zq[0], zq[1], zq[2], zq[3]);
+    cmd.next(fv, e, nt);
   }
 }
 
@@ -926,7 +946,7 @@ __device__ __forceinline__ void consume_segment(const FleetView &fv, int64_t e, 
                                                 const AdjEnv<PATH> &A, const float4 *gdir,
                                                 const float4 *garm, int nt, bool ca,
                                                 const float *__restrict__ dtraj, int32_t sg,
-                                                int32_t C, int32_t T, int64_t step0,
+                                                int32_t C, int32_t T,
                                                 const float4 *__restrict__ rec, Fetch<MT> &buf,
                                                 float *__restrict__ dact, ActionAdjoint<MT> &act,
                                                 Body &lam, float (&lamn)[MT], Grad<PATH> &G) {
@@ -948,7 +968,7 @@ __device__ __forceinline__ void consume_segment(const FleetView &fv, int64_t e, 
       get_stage<MT>(b + i * stage_words<MT>() * 32, 32, y, nud);
     };
     step_vjp<MT, PATH>(stage, zq, A, gdir, garm, nt, ca, fv.rk, lam, lamn, G, gc);
-    act.add(fv, step0 + t0 + j, e, nt, gc, dact);
+    act.add(fv, e, nt, gc, dact);
   }
 }
 
@@ -992,14 +1012,14 @@ __global__ void __launch_bounds__(kWsThreads)
   float lamn[MT];
 #pragma unroll
   for (int i = 0; i < MT; ++i) lamn[i] = 0.f;
-  ActionAdjoint<MT> act;
+  ActionAdjoint<MT> act(fv, step0 + T - 1);
   for (int32_t sg = n_ck - 1; sg >= 0; --sg) {
     if (warp == 0) {
       if (live && sg > 0)
         produce_segment<MT, PATH>(fv, e, A, gdir, garm, nt, ca, ckpt, sg - 1, C, T, step0,
                                   ws + ((sg - 1) & 1) * slot + e);
     } else if (live) {
-      consume_segment<MT, PATH>(fv, e, lane, A, gdir, garm, nt, ca, dtraj, sg, C, T, step0,
+      consume_segment<MT, PATH>(fv, e, lane, A, gdir, garm, nt, ca, dtraj, sg, C, T,
                                 ws + (sg & 1) * slot + e, sbuf, dact, act, lam, lamn, G);
     }
     __syncthreads();
@@ -1095,12 +1115,14 @@ __global__ void __maxnreg__(XH ? kRegsXH : DIAG ? kRegsWide : kRegsGeneral)
   const LagEnv L = lag_env(P.itau, fv.dt);
   float c[MT];
   load_commands<MT>(fv, e, seg, nt, c);
+  if (left < T) prefetch_commands(fv, e, seg);
   for (int32_t it = 0; it < T; ++it) {
     if (it % C == 0) write_checkpoint<MT>(ckpt + (int64_t)(it / C) * MG_NSTATE * n, n, e, s);
     if (left == 0) {
       ++seg;
       left = fv.hold;
       load_commands<MT>(fv, e, seg, nt, c);
+      if (left < T - it) prefetch_commands(fv, e, seg);
     }
     rk4_step<MT, DIAG, MIXED, NH, XH>(s, c, L, P, sdir, sarm, nt, current_accel, fv.rk, xh);
     --left;

@@ -266,10 +266,6 @@ __device__ __forceinline__ void env_commands(const FleetView &fv, const TaskOut 
   for (int i = 0; i < MT; ++i) c[i] = i < nt ? x[i] : 0.f;
 }
 
-__device__ __forceinline__ void prefetch_l1(const void *p) {
-  asm volatile("prefetch.global.L1 [%0];" ::"l"(p));
-}
-
 // The last launch of a task step: the env's final sub-steps as in k_fleet, then the task
 // epilogue from the state still in registers, so the state is stored once and never re-read.
 // Each warp stages its 32 rows of the observation in shared memory (when they fit) and writes
