@@ -139,11 +139,14 @@ SIGNATURES = {
 
 _lock = threading.Lock()
 _lib = None
+_functions = {}  # entry points with their signatures declared, by name
 
 
 def load() -> ctypes.CDLL:
     """Build (if needed) and load libmg.so, declaring every entry point's signature."""
     global _lib
+    if _lib is not None:
+        return _lib
     with _lock:
         if _lib is None:
             path = _build.build()
@@ -152,6 +155,7 @@ def load() -> ctypes.CDLL:
                 fn = getattr(L, name)
                 fn.argtypes = args
                 fn.restype = ctypes.c_int
+                _functions[name] = fn
             L.mg_last_error.argtypes = []
             L.mg_last_error.restype = ctypes.c_char_p
             _lib = L
@@ -160,8 +164,9 @@ def load() -> ctypes.CDLL:
 
 def call(name: str, *args, ok=(0,)) -> int:
     """Call an entry point; raise MGError unless its status is in ``ok``."""
-    L = load()
-    st = getattr(L, name)(*args)
+    if _lib is None:
+        load()
+    st = _functions[name](*args)
     if st not in ok:
-        raise MGError(st, name, L.mg_last_error().decode(errors="replace"))
+        raise MGError(st, name, _lib.mg_last_error().decode(errors="replace"))
     return st

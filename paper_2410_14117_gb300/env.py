@@ -114,6 +114,8 @@ class MarineEnv:
         self._done = torch.zeros(self.n, dtype=torch.uint8, device=dev)
         self._ep = torch.zeros(self.n, dtype=torch.float32, device=dev)
         self._lib = _lib.load()
+        self._done_flags = self._done.view(torch.bool)
+        self._shape = (self.n, self.n_thr)
         p = lambda t: ctypes.c_void_p(t.data_ptr())  # noqa: E731
         self._step_outs = (p(self._obs), p(self._rew), p(self._done), p(self._ep))
         self._obs_outs = (p(self._obs), p(self._err), p(self._done), p(self._ep))
@@ -136,11 +138,12 @@ class MarineEnv:
         if not (isinstance(a, torch.Tensor) and a.is_cuda and a.dtype == torch.float32
                 and a.is_contiguous()):
             a = torch.as_tensor(a, dtype=torch.float32).to(self._obs.device).contiguous()
-        if tuple(a.shape) != (self.n, self.n_thr):
+        if a.shape != self._shape:
             raise ValueError(f"actions must be [{self.n}, {self.n_thr}]")
-        self._check(self._lib.mg_env_step(self.sim._h, self.k, ctypes.c_void_p(a.data_ptr()),
-                                          *self._step_outs), "mg_env_step")
-        return self._obs, self._rew, self._done.view(torch.bool), self._info
+        st = self._lib.mg_env_step(self.sim._h, self.k, a.data_ptr(), *self._step_outs)
+        if st != 0:
+            self._check(st, "mg_env_step")
+        return self._obs, self._rew, self._done_flags, self._info
 
     def close(self):
         if self.sim is not None:
