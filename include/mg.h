@@ -148,7 +148,8 @@ mg_status mg_set_timestep(mg_sim *sim, float dt);
 
 /* Launch shape: envs_per_block in [32, 256] (one thread per env), steps_per_launch >= 1 (RK4
  * steps a kernel keeps state in registers for; 1 gives the plain per-step form), use_graph
- * != 0 to replay mg_step's launch sequence from a cached CUDA graph.  Defaults 128, 50, 1. */
+ * != 0 to replay mg_step's launch sequence from a cached CUDA graph (a call that is a single
+ * static-grid launch is launched as it is).  Defaults 128, 50, 1. */
 mg_status mg_set_launch(mg_sim *sim, int32_t envs_per_block, int32_t steps_per_launch,
                         int32_t use_graph);
 

@@ -44,6 +44,13 @@ __device__ __forceinline__ void finish_launch(const FleetView &fv, int32_t k) {
   }
 }
 
+// The cursor a static-grid step launch starts at: 0 when the launch carries a rewind that the device
+// has not seen (rewinding is then true), else the device's word.
+__device__ __forceinline__ int64_t start_cursor(const FleetView &fv, bool &rewinding) {
+  rewinding = fv.rewind && __ldcg(fv.rewind_gen) != fv.rewind;
+  return rewinding ? 0 : launch_cursor(fv);
+}
+
 // Static-grid form of finish_launch, for kernels whose idle threads have already returned (no
 // block barrier possible): each warp adds its live lanes to the block's shared counter s_done
 // (zeroed before the block's first barrier); the warp that completes the block's count of live
@@ -51,14 +58,20 @@ __device__ __forceinline__ void finish_launch(const FleetView &fv, int32_t k) {
 // advances the cursor by k and re-arms the counter.  Every thread read the cursor before its
 // warp counted itself, so every block saw the launch's starting value.
 __device__ __forceinline__ void finish_envs(const FleetView &fv, unsigned *s_done, int count,
-                                            int32_t k) {
+                                            int32_t k, bool rewinding = false) {
   const unsigned mask = __activemask();
   __syncwarp(mask);
   if ((threadIdx.x & 31) == (unsigned)(__ffs(mask) - 1)) {
     const unsigned add = __popc(mask);
     if (atomicAdd(s_done, add) + add == (unsigned)count &&
         atomicAdd(fv.done_blocks, 1u) == gridDim.x - 1) {
-      atomicAdd(reinterpret_cast<unsigned long long *>(fv.cursor), (unsigned long long)k);
+      unsigned long long *cursor = reinterpret_cast<unsigned long long *>(fv.cursor);
+      if (rewinding) {
+        atomicExch(cursor, (unsigned long long)k);
+        atomicExch(fv.rewind_gen, fv.rewind);
+      } else {
+        atomicAdd(cursor, (unsigned long long)k);
+      }
       atomicExch(fv.done_blocks, 0u);
     }
   }

@@ -149,7 +149,8 @@ struct mg_sim {
   uint32_t *episode = nullptr;
   unsigned long long *counters = nullptr;  // [0] non-finite envs, [1] non-SPD envs,
                                            // [2] work-queue wait time-outs, [3] action
-                                           // cursor, [4] finished-block count
+                                           // cursor, [4] finished-block count, [5] last
+                                           // rewind carried by a launch
   unsigned int *offdiag = nullptr;
   // off-diagonal hydrodynamics, [MG_NXPARAM][n] planes (mg_set_hydro_offdiag), and whether set
   float *xh = nullptr;
@@ -196,6 +197,14 @@ struct mg_sim {
   int32_t proc = 0;
   uint64_t cmd_seed = 0;
   int64_t cursor = 0;  // host copy of the device cursor (counters[3])
+  // A rewind not yet in device memory (rewind_cursor): number rewind_gen, carried by the next direct
+  // step launch, or settled before any other use of the cursor; whichever runs first on the device
+  // applies it.  captured: the sim's stream has been captured into a user's graph, whose replays
+  // read the cursor at times the host does not see, so rewinds go to device memory at once from
+  // then on; a rewind pending when a capture starts stays pending beside the captured launch.
+  bool rewind_pending = false;
+  uint32_t rewind_gen = 0;
+  bool captured = false;
 
   // knobs
   int32_t epb = 128, spl = 50;
@@ -277,6 +286,7 @@ struct mg_sim {
     v.spin_limit = wait_limit;
     v.cursor = reinterpret_cast<int64_t *>(counters + 3);
     v.done_blocks = reinterpret_cast<unsigned int *>(counters + 4);
+    v.rewind_gen = reinterpret_cast<uint32_t *>(counters + 5);
     return v;
   }
 
@@ -473,10 +483,48 @@ mg_status finish_params(mg_sim *s) {
   return MG_OK;
 }
 
-// Rewind the action cursor (host copy and the device word the step kernels read).
+// Whether the sim's stream is being captured into a user's graph; remembered (mg_sim::captured).
+bool capturing(mg_sim *s) {
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s->stream, &st) != cudaSuccess) cudaGetLastError();
+  if (st != cudaStreamCaptureStatusNone) s->captured = true;
+  return st != cudaStreamCaptureStatusNone;
+}
+
+cudaError_t apply_rewind(mg_sim *s, bool always) {
+  return launch_rewind(s->counters + 3, reinterpret_cast<uint32_t *>(s->counters + 5),
+                       s->rewind_gen, always, s->stream);
+}
+
+// Before any use of the device's cursor other than a direct step launch: apply a pending rewind
+// (and notice a capture).
+mg_status settle_cursor(mg_sim *s) {
+  const bool cap = capturing(s);
+  if (!s->rewind_pending) return MG_OK;
+  if (s->captured)
+    MG_CK(apply_rewind(s, false));
+  else
+    MG_CK(cudaMemsetAsync(s->counters + 3, 0, sizeof(unsigned long long), s->stream));
+  if (!cap) s->rewind_pending = false;
+  return MG_OK;
+}
+
+// Rewind the action cursor: the host copy now, the device word with the next step launch (a
+// control loop that sets its throttles every sub-step would otherwise pay a memset, and its place
+// in the stream, per sub-step).
 mg_status rewind_cursor(mg_sim *s) {
   s->cursor = 0;
-  MG_CK(cudaMemsetAsync(s->counters + 3, 0, sizeof(unsigned long long), s->stream));
+  if (capturing(s)) {  // every replay rewinds
+    MG_CK(apply_rewind(s, true));
+    return MG_OK;
+  }
+  if (s->captured) {
+    MG_CK(apply_rewind(s, true));
+    s->rewind_pending = false;
+    return MG_OK;
+  }
+  s->rewind_pending = true;
+  if (++s->rewind_gen == 0) s->rewind_gen = 1;
   return MG_OK;
 }
 
@@ -542,6 +590,7 @@ mg_status mg_step_noalloc(mg_sim *s, int32_t k) {
   uint32_t *sched = nullptr;
   mg_status st = noalloc_scratch(s->dev, &sched);
   if (st != MG_OK) return st;
+  if ((st = settle_cursor(s)) != MG_OK) return st;
   FleetView v = s->view();
   v.cursor_adv = k;
   MG_CK(launch_fleet_queue(v, s->slices_d, s->n_slices, s->ntv, s->diag, s->layout,
@@ -613,7 +662,7 @@ mg_status mg_create(int64_t n_envs, const int32_t *vehicle_types,
   s->n_slices = (int)slices.size();
   const size_t o_slices = take(sizeof(BlockDesc) * slices.size());
   const size_t o_sched = take(queue_sched_bytes(s->n_slices));
-  const size_t o_cnt = take(5 * sizeof(unsigned long long));
+  const size_t o_cnt = take(6 * sizeof(unsigned long long));
   const size_t o_off = take(sizeof(unsigned int));
   cudaError_t e = cudaMalloc(&s->arena, off);
   if (e != cudaSuccess) {
@@ -704,7 +753,7 @@ mg_status mg_create(int64_t n_envs, const int32_t *vehicle_types,
   MG_CKB(cudaMemcpy(s->types_d, s->types_h.data(), 4 * n, cudaMemcpyHostToDevice));
   MG_CKB(cudaMemset(s->flags, 0, 4 * n));
   MG_CKB(cudaMemset(s->episode, 0, 4 * n));
-  MG_CKB(cudaMemset(s->counters, 0, 5 * sizeof(unsigned long long)));
+  MG_CKB(cudaMemset(s->counters, 0, 6 * sizeof(unsigned long long)));
   MG_CKB(cudaMemcpy(s->slices_d, slices.data(), sizeof(BlockDesc) * slices.size(),
                     cudaMemcpyHostToDevice));
   MG_CKB(cudaMemset(s->offdiag, 0, sizeof(unsigned int)));
@@ -1123,8 +1172,25 @@ mg_status mg_step(mg_sim *s, int32_t k) {
   MG_NONNULL(s);
   NvtxRange nvtx("mg_step");
   if (k < 1) return fail(MG_EINVAL, "k must be >= 1");
+  mg_status st;
+  const bool single = !s->queue && k <= s->spl;
+  if (single) {
+    // One static-grid launch: as it is, carrying a pending rewind.  A graph of this one kernel is no
+    // cheaper for the host and takes twice as long on the device (256 envs, back to back: 6.2 us a
+    // step against 3.1, the launches overlapping).
+    const bool cap = capturing(s);
+    FleetView v = s->view();
+    v.cursor_adv = k;
+    v.rewind = s->rewind_pending ? s->rewind_gen : 0;
+    MG_CK(launch_fleet(v, s->blocks_d, s->n_blocks, s->threads, s->ntv, s->diag, s->layout, s->wide,
+                       k, nullptr, s->stream));
+    if (!cap) s->rewind_pending = false;
+    s->cursor += k;
+    return MG_OK;
+  }
+  if ((st = settle_cursor(s)) != MG_OK) return st;
   if (!s->use_graph) {
-    mg_status st = launch_chunks(s, k, nullptr, s->stream);
+    st = launch_chunks(s, k, nullptr, s->stream);
     if (st != MG_OK) return st;
     s->cursor += k;
     return MG_OK;
@@ -1147,7 +1213,7 @@ mg_status mg_step(mg_sim *s, int32_t k) {
     }
     cudaGraph_t graph = nullptr;
     MG_CK(cudaStreamBeginCapture(s->cap_stream, cudaStreamCaptureModeThreadLocal));
-    mg_status st = launch_chunks(s, k, nullptr, s->cap_stream);
+    st = launch_chunks(s, k, nullptr, s->cap_stream);
     cudaError_t ce = cudaStreamEndCapture(s->cap_stream, &graph);
     if (st != MG_OK) {
       if (graph) cudaGraphDestroy(graph);
@@ -1173,6 +1239,8 @@ mg_status mg_step_split(mg_sim *s, int32_t k, float *accel) {
   MG_NONNULL(accel);
   if (k < 1) return fail(MG_EINVAL, "k must be >= 1");
   if (!is_device_ptr(accel)) return fail(MG_EINVAL, "accel must be device memory");
+  mg_status st = settle_cursor(s);
+  if (st != MG_OK) return st;
   FleetView v = s->view();
   for (int32_t done = 0; done < k;) {
     const int32_t kk = std::min(s->spl, k - done);
@@ -1192,7 +1260,8 @@ mg_status mg_step_record(mg_sim *s, int32_t k, float *traj) {
   MG_NONNULL(traj);
   if (k < 1) return fail(MG_EINVAL, "k must be >= 1");
   if (!is_device_ptr(traj)) return fail(MG_EINVAL, "traj must be device memory");
-  mg_status st = launch_chunks(s, k, traj, s->stream);
+  mg_status st = settle_cursor(s);
+  if (st == MG_OK) st = launch_chunks(s, k, traj, s->stream);
   if (st != MG_OK) return st;
   s->cursor += k;
   return MG_OK;
@@ -1208,6 +1277,8 @@ mg_status mg_rollout_forward(mg_sim *s, int32_t T, int32_t C, float *traj, float
     return fail(MG_EINVAL, "need T >= 1 and 1 <= C <= 32");
   if (!is_device_ptr(traj) || !is_device_ptr(ckpt))
     return fail(MG_EINVAL, "traj and ckpt must be device memory");
+  mg_status st = settle_cursor(s);
+  if (st != MG_OK) return st;
   FleetView v = s->view();
   const int64_t step0 = s->cursor;
   v.cursor_off = 0;
@@ -1319,6 +1390,8 @@ mg_status task_step_outputs(mg_sim *s, int32_t k, float *obs, float *err, float 
                       s->counters, s->stream));
     return MG_OK;
   }
+  mg_status cs = settle_cursor(s);
+  if (cs != MG_OK) return cs;
   // Leading sub-steps as mg_step; the last static chunk carries the fused task epilogue.
   const int32_t k_last = (k - 1) % s->spl + 1;
   if (k > k_last) {

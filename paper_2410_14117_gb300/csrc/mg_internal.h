@@ -117,6 +117,12 @@ struct FleetView {
   // cursor_adv once all its blocks are done.  Only that launch pays for the completion count.
   int32_t cursor_off;
   int32_t cursor_adv;
+  // Pending rewind of the cursor (static-grid step kernel only): nonzero, and different from the
+  // device's word *rewind_gen, the launch starts at cursor 0 instead of *cursor and its last block
+  // stores both words.  A replay of the same launch in a user's graph then finds the word equal and
+  // goes on from *cursor.
+  uint32_t rewind;
+  uint32_t *rewind_gen;
   // Work-queue schedule: polls of ~128 ns a unit's wait for its slice's previous chunk may take
   // before it gives up (counted in counters[2] and reported by mg_sync as MG_ETIMEOUT).
   uint32_t spin_limit;
@@ -193,6 +199,10 @@ cudaError_t launch_export_params(const SetupView &v, float *out /*dev [n][35]*/,
 cudaError_t launch_reset(const StatePlanes &st, int64_t n, int64_t gid0, const uint8_t *mask,
                          uint64_t seed, double nu0_sigma, uint32_t *episode, uint32_t *flags,
                          unsigned long long *nonfinite_count, cudaStream_t stream);
+// *cursor = 0 and *gen_word = gen, always or only where *gen_word differs (the rewind that a step
+// launch carries, FleetView::rewind).
+cudaError_t launch_rewind(unsigned long long *cursor, uint32_t *gen_word, uint32_t gen, bool always,
+                          cudaStream_t stream);
 cudaError_t launch_export_state(const StatePlanes &st, int64_t n, float *out,
                                 cudaStream_t stream);
 cudaError_t launch_import_state(const StatePlanes &st, int64_t n, const float *in,

@@ -374,6 +374,10 @@ __global__ void __launch_bounds__(kRowThreads)
   const int64_t e0 = (int64_t)blockIdx.x * kRowThreads;
   const int t = (int)threadIdx.x;
   const int64_t e = e0 + t;
+  // Programmatic dependent launch, both ways: this kernel's launch overlaps the step that writes the
+  // state, and the next step's launch overlaps this kernel (each waits here for the one before it).
+  cudaTriggerProgrammaticLaunchCompletion();
+  cudaGridDependencySynchronize();
   if (e < n) {
     const float4 a = st.s0[e], b = st.s1[e], c = st.s2[e], d = st.s3[e], f = st.s4[e];
     const float r[MG_NSTATE] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w, c.x, c.y, c.z,
@@ -419,6 +423,13 @@ __global__ void __launch_bounds__(kRowThreads)
   st.s3[e] = make_float4(r[12], r[13], r[14], r[15]);
   st.s4[e] = make_float4(r[16], r[17], r[18], r[19]);
   st.s5[e] = r[20];
+}
+
+__global__ void k_rewind(unsigned long long *cursor, uint32_t *gen_word, uint32_t gen, bool always) {
+  if (always || *gen_word != gen) {
+    *cursor = 0;
+    *gen_word = gen;
+  }
 }
 
 __global__ void k_flags_to_bytes(const uint32_t *__restrict__ flags, int64_t n,
@@ -495,11 +506,24 @@ cudaError_t launch_reset(const StatePlanes &st, int64_t n, int64_t gid0, const u
   return cudaGetLastError();
 }
 
+cudaError_t launch_rewind(unsigned long long *cursor, uint32_t *gen_word, uint32_t gen, bool always,
+                          cudaStream_t stream) {
+  k_rewind<<<1, 1, 0, stream>>>(cursor, gen_word, gen, always);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_export_state(const StatePlanes &st, int64_t n, float *out,
                                 cudaStream_t stream) {
-  k_export_state<<<(int)((n + kRowThreads - 1) / kRowThreads), kRowThreads, 0, stream>>>(st, n,
-                                                                                      out);
-  return cudaGetLastError();
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)((n + kRowThreads - 1) / kRowThreads));
+  cfg.blockDim = dim3(kRowThreads);
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, k_export_state, st, n, out);
 }
 
 cudaError_t launch_import_state(const StatePlanes &st, int64_t n, const float *in,

@@ -48,6 +48,7 @@ __global__ void __maxnreg__(XH ? kRegsXH : !DIAG ? kRegsGeneral : WIDE ? kRegsWi
   __shared__ float4 sdir[MG_MAX_THR], sarm[MG_MAX_THR];
   __shared__ unsigned s_done;
   __shared__ int64_t s_cursor;
+  __shared__ bool s_rewinding;
   extern __shared__ float sxh[];
 
   const BlockDesc bd = blocks[blockIdx.x];
@@ -62,7 +63,9 @@ __global__ void __maxnreg__(XH ? kRegsXH : !DIAG ? kRegsGeneral : WIDE ? kRegsWi
   cudaGridDependencySynchronize();
   if (threadIdx.x == 0) {
     s_done = 0u;
-    s_cursor = launch_cursor(fv);
+    bool rewinding;
+    s_cursor = start_cursor(fv, rewinding);
+    s_rewinding = rewinding;
   }
   if constexpr (XH) stage_xh(fv.xh, fv.n, bd.env0, bd.count, sxh);
   __syncthreads();
@@ -78,7 +81,7 @@ __global__ void __maxnreg__(XH ? kRegsXH : !DIAG ? kRegsGeneral : WIDE ? kRegsWi
       },
       k, traj, st, XH ? sxh + threadIdx.x * MG_NXPARAM : nullptr);
   store_and_flag<MT, false>(fv, e, st);
-  if (fv.cursor_adv) finish_envs(fv, &s_done, bd.count, fv.cursor_adv);
+  if (fv.cursor_adv) finish_envs(fv, &s_done, bd.count, fv.cursor_adv, s_rewinding);
 }
 
 // XH (general path): each warp stages the off-diagonal hydrodynamic coefficients of the slice it
