@@ -171,13 +171,17 @@ __device__ __forceinline__ void scheduled_start(const FleetView &fv, int64_t e, 
 // XH: xh is the env's row of staged off-diagonal hydrodynamic coefficients.
 // start(c, seg, left) sets the first sub-step's command c, its segment and the sub-steps left in it
 // (scheduled_start, or a fused kernel's own source).
-template <int MT, bool DIAG, bool MIXED, bool REC, bool L2, int NH, bool XH, typename Start>
+// loaded: the parameters, where the caller has loaded them and the state s already (the task kernel,
+// before its block barrier; the step kernels' loops come out 2 % slower that way).
+template <int MT, bool DIAG, bool MIXED, bool REC, bool L2, int NH, bool XH, bool LOADED = false,
+          typename Start = void>
 __device__ __forceinline__ void advance_env(const FleetView &fv, int64_t e, int nt,
                                             const float4 *gdir, const float4 *garm, Start start,
-                                            int32_t k, float *traj, St<MT> &s, const float *xh) {
+                                            int32_t k, float *traj, St<MT> &s, const float *xh,
+                                            const Par<DIAG> *loaded = nullptr) {
   const bool current_accel = !(fv.model_flags & MG_MODEL_NO_CURRENT_ACCEL);
 
-  load_state<MT, L2>(fv.st, e, s);
+  if constexpr (!LOADED) load_state<MT, L2>(fv.st, e, s);
   float c[MT];
   int64_t seg;
   int32_t left;
@@ -190,7 +194,8 @@ __device__ __forceinline__ void advance_env(const FleetView &fv, int64_t e, int 
   Coef<DIAG, NH> P;
   {
     Par<DIAG> raw;
-    load_par<DIAG>(fv.pa, e, raw);
+    if constexpr (LOADED) raw = *loaded;
+    else load_par<DIAG>(fv.pa, e, raw);
     P = make_coef<DIAG, NH>(raw, gdir, garm);
   }
   const LagEnv L = lag_env(P.itau, fv.dt);

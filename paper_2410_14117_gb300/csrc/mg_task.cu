@@ -300,18 +300,25 @@ __global__ void __maxnreg__(XH ? kRegsXH : DIAG ? kRegsDiag : kRegsGeneral)
     if (!to.act_in) s_cursor = launch_cursor(fv);
   }
   if constexpr (XH) stage_xh(fv.xh, fv.n, bd.env0, bd.count, sxh);
-  __syncthreads();
-  if ((int)threadIdx.x >= bd.count) return;
+  // the env's loads are on their way while the block waits for the cursor
   const int64_t e = (int64_t)bd.env0 + threadIdx.x;
-  const int nt = MIXED ? bd.n_thr : MT;
-  // what the epilogue reads, on its way while the sub-steps run
-  prefetch_l1(tv.centre + e);
-  prefetch_l1(tv.clock + e);
-  prefetch_l1(tv.err_sum + e);
-  prefetch_l1(fv.flags + e);
-  prefetch_l1(to.episode + e);
+  const bool live = (int)threadIdx.x < bd.count;
   St<MT> s;
-  advance_env<MT, DIAG, MIXED, false, false, NH, XH>(
+  Par<DIAG> raw;
+  if (live) {
+    load_state<MT>(fv.st, e, s);
+    load_par<DIAG>(fv.pa, e, raw);
+    // what the epilogue reads, moved while the sub-steps run
+    prefetch_l1(tv.centre + e);
+    prefetch_l1(tv.clock + e);
+    prefetch_l1(tv.err_sum + e);
+    prefetch_l1(fv.flags + e);
+    prefetch_l1(to.episode + e);
+  }
+  __syncthreads();
+  if (!live) return;
+  const int nt = MIXED ? bd.n_thr : MT;
+  advance_env<MT, DIAG, MIXED, false, false, NH, XH, true>(
       fv, e, nt, sdir, sarm,
       [&](float (&c)[MT], int64_t &seg, int32_t &left) {
         if (to.act_in) {  // one command for the whole launch, no cursor
@@ -322,7 +329,7 @@ __global__ void __maxnreg__(XH ? kRegsXH : DIAG ? kRegsDiag : kRegsGeneral)
           scheduled_start<MT>(fv, e, nt, s_cursor + fv.cursor_off, c, seg, left);
         }
       },
-      k_launch, nullptr, s, XH ? sxh + threadIdx.x * MG_NXPARAM : nullptr);
+      k_launch, nullptr, s, XH ? sxh + threadIdx.x * MG_NXPARAM : nullptr, &raw);
 
   const int obs_dim = to.obs_dim;
   task_epilogue<MT>(fv, tv, to, k_task, e, task_in(fv, tv, to, e), s,
