@@ -39,8 +39,9 @@ constexpr int kAdjThreads = 128;
 // Which transpose a kernel is compiled for.
 enum AdjPath { ADJ_GEN = 0, ADJ_DENSE = 1, ADJ_MIRRORED = 2 };
 
-// The thruster allocation of the re-run: the forward's (the vectored one only skips exact zeros of
-// the dense one, so the states are the forward's bit for bit either way).
+// The thruster allocation of the re-run.  Diagonal mass: the forward's (the vectored one only skips
+// exact zeros of the dense one, so the states are the forward's bit for bit).  General path: the
+// dense one, the forward's within the rounding of the thrust sums where that was mirrored.
 __host__ __device__ constexpr int adj_layout(int path) {
   return path == ADJ_MIRRORED ? MG_LAYOUT_MIRRORED : MG_LAYOUT_DENSE;
 }
@@ -1146,9 +1147,12 @@ template <int NTV>
 cudaError_t rollout_fwd_d(const FleetView &fv, const BlockDesc *blocks, int n_blocks,
                           int threads, bool diag, int layout, int32_t T, int32_t C,
                           float *traj, float *ckpt, cudaStream_t stream) {
+  constexpr int M = MG_LAYOUT_MIRRORED;
   if (fv.xh)
-    return rollout_fwd_t<NTV, false, 0, true>(fv, blocks, n_blocks, threads, T, C, traj, ckpt,
-                                              stream);
+    return layout == M ? rollout_fwd_t<NTV, false, M, true>(fv, blocks, n_blocks, threads, T, C,
+                                                            traj, ckpt, stream)
+                       : rollout_fwd_t<NTV, false, 0, true>(fv, blocks, n_blocks, threads, T, C,
+                                                            traj, ckpt, stream);
   if (diag && layout == MG_LAYOUT_MIRRORED)
     return rollout_fwd_t<NTV, true, MG_LAYOUT_MIRRORED, false>(fv, blocks, n_blocks, threads, T, C,
                                                                traj, ckpt, stream);
@@ -1158,8 +1162,10 @@ cudaError_t rollout_fwd_d(const FleetView &fv, const BlockDesc *blocks, int n_bl
   if (diag)
     return rollout_fwd_t<NTV, true, 0, false>(fv, blocks, n_blocks, threads, T, C, traj, ckpt,
                                               stream);
-  return rollout_fwd_t<NTV, false, 0, false>(fv, blocks, n_blocks, threads, T, C, traj, ckpt,
-                                             stream);
+  return layout == M ? rollout_fwd_t<NTV, false, M, false>(fv, blocks, n_blocks, threads, T, C, traj,
+                                                           ckpt, stream)
+                     : rollout_fwd_t<NTV, false, 0, false>(fv, blocks, n_blocks, threads, T, C, traj,
+                                                           ckpt, stream);
 }
 
 }  // namespace

@@ -38,11 +38,7 @@ bool mg::vectored_layout(const Geo &g) {
   return true;
 }
 
-namespace {
-
-// Mirror images (MG_LAYOUT_MIRRORED): six or eight thrusters whose rows repeat one magnitude each
-// with the signs given there.
-bool mirrored_layout(const Geo &g) {
+bool mg::mirrored_layout(const Geo &g) {
   if ((g.n_thr != 6 && g.n_thr != 8) || !vectored_layout(g)) return false;
   const float4 *d = g.dir, *a = g.arm;
   auto rows = [](float x0, float x1, float x2, float x3, int s1, int s2, int s3) {
@@ -60,8 +56,6 @@ bool mirrored_layout(const Geo &g) {
          rows(a[4].x, a[5].x, a[6].x, a[7].x, -1, 1, -1) &&
          rows(a[4].y, a[5].y, a[6].y, a[7].y, 1, -1, -1);
 }
-
-}  // namespace
 
 int mg::thruster_layout(const Geo &g, const mg_vehicle_params &v) {
   if (mirrored_layout(g) && v.rb[0] == 0.f && v.rb[1] == 0.f) return MG_LAYOUT_MIRRORED;
@@ -126,9 +120,11 @@ struct mg_sim {
   // current-acceleration term, so a sim that switches that term off takes the general path.
   bool mass_diag = true;
   bool diag = true;
-  // Thruster allocation of the diagonal-mass step (MG_LAYOUT_*): by the geometry and nominal r_b of
-  // the types present, and the one in use, which is the vectored one at most while some env's r_b is
-  // off the z axis (mg_set_params).
+  // Thruster allocation (MG_LAYOUT_*): the diagonal-mass step's by the geometry and nominal r_b of
+  // the types present (mirrored: by the geometry alone, the general path's), and the one in use,
+  // which for a diagonal mass is the vectored one at most while some env's r_b is off the z axis
+  // (mg_set_params).
+  bool mirrored = true;
   int type_layout = MG_LAYOUT_DENSE;
   int layout = MG_LAYOUT_DENSE;
   bool on_axis = true;          // every env's r_b lies on the body's z axis
@@ -459,8 +455,9 @@ void set_mass_diag(mg_sim *s, bool mass_diag, bool on_axis) {
   s->mass_diag = mass_diag;
   s->on_axis = on_axis;
   const bool diag = mass_diag && !(s->model_flags & MG_MODEL_NO_CURRENT_ACCEL);
-  const int layout =
-      on_axis ? s->type_layout : std::min<int>(s->type_layout, MG_LAYOUT_VECTORED);
+  const int layout = !diag     ? (s->mirrored ? MG_LAYOUT_MIRRORED : MG_LAYOUT_DENSE)
+                     : on_axis ? s->type_layout
+                               : std::min<int>(s->type_layout, MG_LAYOUT_VECTORED);
   if (diag != s->diag || layout != s->layout) s->drop_graphs();
   s->diag = diag;
   s->layout = layout;
@@ -715,7 +712,10 @@ mg_status mg_create(int64_t n_envs, const int32_t *vehicle_types,
       g.arm[i] = make_float4(r[1] * d[2] - r[2] * d[1], r[2] * d[0] - r[0] * d[2],
                              r[0] * d[1] - r[1] * d[0], 0.f);
     }
-    if (seen[t]) s->type_layout = std::min(s->type_layout, thruster_layout(g, v));
+    if (seen[t]) {
+      s->type_layout = std::min(s->type_layout, thruster_layout(g, v));
+      s->mirrored = s->mirrored && mirrored_layout(g);
+    }
     if (seen[t] && (v.rb[0] != 0.f || v.rb[1] != 0.f)) s->nominal_on_axis = false;
     if (v.rg[0] != 0.f || v.rg[1] != 0.f || v.rg[2] != 0.f) s->nominal_diag = false;
     float *p = &nom[(size_t)t * MG_NPARAM];

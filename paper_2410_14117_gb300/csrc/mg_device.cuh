@@ -204,11 +204,13 @@ struct StepMirrored {
   float vc0, vc1, vc2, itau;
 };
 
-// Thruster allocations of the diagonal-mass step (the NH parameter of the kernels).
+// Thruster allocations (the NH parameter of the kernels; the general path has the dense and the
+// mirrored one).
 //   MG_LAYOUT_DENSE     any geometry: all six rows of every thruster.
 //   MG_LAYOUT_VECTORED  thrusters [0, 4) horizontal (d_z = 0), the rest vertical (d_x = d_y = 0).
 //   MG_LAYOUT_MIRRORED  vectored with 6 or 8 thrusters placed by mirror images (see
-//                       mirrored_layout), and r_b on the body's z axis in every env: the
+//                       mirrored_layout), and, for a diagonal mass matrix, r_b on the body's z
+//                       axis in every env: the
 //                       horizontals' force and moment rows are d_x (+ + - -), d_y (+ - + -),
 //                       arm_x (+ - + -), arm_y (+ + - -), arm_z (+ - - +) times one magnitude each,
 //                       the verticals' d_z (+ +), arm_x (- + [- +]), arm_y (- - [+ +]; zero with
@@ -250,18 +252,41 @@ __device__ __forceinline__ StepMirrored step_mirrored(const ParDiag &P, const fl
   return C;
 }
 
+// The general path with a mirrored frame: kT times the type's directions and moment arms, which
+// weight the same thrust sums (its G stays general, so r_b may be anywhere).  19 operations and no
+// geometry reads for the dense allocation's 48.
+struct ParGenMirrored : ParGen {
+  float tx, ty, tz, Kh, Kv, Mh, Mv, Nh;
+};
+
+__device__ __forceinline__ ParGenMirrored gen_mirrored(const ParGen &P, const float4 *gdir,
+                                                       const float4 *garm) {
+  ParGenMirrored C;
+  static_cast<ParGen &>(C) = P;
+  C.tx = P.kT * gdir[0].x;
+  C.ty = P.kT * gdir[0].y;
+  C.tz = P.kT * gdir[4].z;
+  C.Kh = P.kT * garm[0].x;
+  C.Kv = P.kT * garm[5].x;
+  C.Mh = P.kT * garm[0].y;
+  C.Mv = -(P.kT * garm[4].y);
+  C.Nh = P.kT * garm[0].z;
+  return C;
+}
+
 // What the step's right-hand side reads: the diagonal-mass coefficients above, or the general
-// parameters as loaded.
+// parameters as loaded (with the mirrored frame's weights).
 template <bool DIAG, int NH = MG_LAYOUT_DENSE>
 using Coef = typename std::conditional<
     DIAG, typename std::conditional<NH == MG_LAYOUT_MIRRORED, StepMirrored, StepDiag>::type,
-    ParGen>::type;
+    typename std::conditional<NH == MG_LAYOUT_MIRRORED, ParGenMirrored, ParGen>::type>::type;
 
 template <bool DIAG, int NH = MG_LAYOUT_DENSE>
 __device__ __forceinline__ Coef<DIAG, NH> make_coef(const Par<DIAG> &P, const float4 *gdir,
                                                     const float4 *garm) {
   if constexpr (DIAG && NH == MG_LAYOUT_MIRRORED) return step_mirrored(P, gdir, garm);
   else if constexpr (DIAG) return step_diag(P);
+  else if constexpr (NH == MG_LAYOUT_MIRRORED) return gen_mirrored(P, gdir, garm);
   else return P;
 }
 
@@ -355,7 +380,7 @@ __device__ __forceinline__ void rhs(const St<MT> &s, const Coef<DIAG, NH> &P,
                                     const float *__restrict__ xh = nullptr) {
   static_assert(!(XH && DIAG), "the off-diagonal hydrodynamics use the general path");
   // Thrusters (Eq. 3 actions): F_i = kT n_i|n_i| along d_i at r_i.
-  constexpr bool MIRRORED = DIAG && NH == MG_LAYOUT_MIRRORED;
+  constexpr bool MIRRORED = NH == MG_LAYOUT_MIRRORED;
   float t0 = 0.f, t1 = 0.f, t2 = 0.f, t3 = 0.f, t4 = 0.f, t5 = 0.f;
   if constexpr (MIRRORED) {
     auto f = [&](int i) { return s.n[i] * fabsf(s.n[i]); };
@@ -482,9 +507,23 @@ __device__ __forceinline__ void rhs(const St<MT> &s, const Coef<DIAG, NH> &P,
     // Translational generalised force:
     //   kT t + (W - B) k_e - w x h - (Dl + Dq |v_r|) v_r [- M_A,lin (w x v_c^b)],
     // with k_e = R^T e3 = (R20, R21, R22) the restoring direction.
-    float f0 = fmaf(P.wb, R20, P.kT * t0);
-    float f1 = fmaf(P.wb, R21, P.kT * t1);
-    float f2 = fmaf(P.wb, R22, P.kT * t2);
+    float f0, f1, f2, f3, f4, f5;
+    if constexpr (MIRRORED) {
+      f0 = fmaf(P.wb, R20, P.tx * t0);
+      f1 = fmaf(P.wb, R21, P.ty * t1);
+      f2 = fmaf(P.wb, R22, P.tz * t2);
+      f3 = fmaf(P.Kv, t3, P.Kh * t1);
+      f4 = P.Mh * t0;
+      if constexpr (MT > 6) f4 = fmaf(P.Mv, t4, f4);
+      f5 = P.Nh * t5;
+    } else {
+      f0 = fmaf(P.wb, R20, P.kT * t0);
+      f1 = fmaf(P.wb, R21, P.kT * t1);
+      f2 = fmaf(P.wb, R22, P.kT * t2);
+      f3 = P.kT * t3;
+      f4 = P.kT * t4;
+      f5 = P.kT * t5;
+    }
     f0 = fmaf(w2, h1, fmaf(-w1, h2, f0));
     f1 = fmaf(w0, h2, fmaf(-w2, h0, f1));
     f2 = fmaf(w1, h0, fmaf(-w0, h1, f2));
@@ -514,9 +553,9 @@ __device__ __forceinline__ void rhs(const St<MT> &s, const Coef<DIAG, NH> &P,
                fmaf(-Dl[14], w2, f2)))));
     }
     // Rotational: kT t' - v_r x Q1 - w x k - v x (w x m r_g) - (Dl + Dq|w|) w + G x k_e.
-    float f3 = fmaf(r2, q1, fmaf(-r1, q2, P.kT * t3));
-    float f4 = fmaf(r0, q2, fmaf(-r2, q0, P.kT * t4));
-    float f5 = fmaf(r1, q0, fmaf(-r0, q1, P.kT * t5));
+    f3 = fmaf(r2, q1, fmaf(-r1, q2, f3));
+    f4 = fmaf(r0, q2, fmaf(-r2, q0, f4));
+    f5 = fmaf(r1, q0, fmaf(-r0, q1, f5));
     f3 = fmaf(w2, k1, fmaf(-w1, k2, f3));
     f4 = fmaf(w0, k2, fmaf(-w2, k0, f4));
     f5 = fmaf(w1, k0, fmaf(-w0, k1, f5));

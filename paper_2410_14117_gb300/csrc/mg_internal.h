@@ -137,8 +137,8 @@ enum NtVariant { NT_6 = 0, NT_8 = 1, NT_MIXED = 2 };
 
 // ---------------------------------------------------------------- launchers (mg_step.cu)
 // Static schedule: one block per BlockDesc, k sub-steps per launch.
-// layout: MG_LAYOUT_* (mg_device.cuh), the thruster allocation of the diagonal-mass step: the
-// fastest one that every vehicle type present has.
+// layout: MG_LAYOUT_* (mg_device.cuh), the thruster allocation: the fastest one of the path that
+// every vehicle type present has.
 // wide: the diagonal-mass kernel without recording gets 200 registers instead of 128.
 cudaError_t launch_fleet(const FleetView &fv, const BlockDesc *blocks, int n_blocks, int threads,
                          NtVariant ntv, bool diag, int layout, bool wide, int32_t k,
@@ -164,7 +164,10 @@ cudaError_t queue_kernel_attributes(NtVariant ntv, bool diag, bool wide, int lay
 
 // True when thrusters [0, 4) of the geometry have d_z = 0 and the rest d_x = d_y = 0.
 bool vectored_layout(const Geo &g);
-// The fastest MG_LAYOUT_* that vehicle type v with geometry g has (mirrored asks for r_b on the
+// True for mirror images (MG_LAYOUT_MIRRORED in mg_device.cuh): six or eight thrusters whose rows
+// repeat one magnitude each with the signs given there.
+bool mirrored_layout(const Geo &g);
+// The fastest MG_LAYOUT_* of the diagonal-mass step that vehicle type v with geometry g has (mirrored asks for r_b on the
 // z axis too).
 int thruster_layout(const Geo &g, const mg_vehicle_params &v);
 

@@ -198,6 +198,7 @@ struct mg_pool {
   std::vector<mg_vehicle_params> vp;
   bool diag = true;
   int layout = MG_LAYOUT_MIRRORED;  // the fastest one that every vehicle type has
+  bool mirrored = true;             // every type's geometry is (the general path's condition)
   cudaStream_t stream = nullptr;
   void *arena = nullptr;
   StatePlanes st{};
@@ -369,6 +370,7 @@ mg_status mg_pool_create(int64_t capacity_envs, const mg_vehicle_params *params,
                              r[0] * d[1] - r[1] * d[0], 0.f);
     }
     p->layout = std::min(p->layout, thruster_layout(g, v));
+    p->mirrored = p->mirrored && mirrored_layout(g);
     float *q = &nom[(size_t)t * MG_NPARAM];
     q[MG_P_M] = v.m;
     q[MG_P_IG] = v.Ixx;
@@ -612,13 +614,19 @@ mg_status mg_pool_tick(mg_pool *p, int32_t k, int32_t *n_running) {
     ;
   else if (p->diag)
     launch_serve_diag(p->layout, wide, g, v, jt, bl, p->stream);
+  else if (p->mirrored)
+    k_serve<false, MG_LAYOUT_MIRRORED><<<g, kServeThreads, 0, p->stream>>>(v, jt, bl);
   else
     k_serve<false, 0><<<g, kServeThreads, 0, p->stream>>>(v, jt, bl);
   PK(cudaGetLastError());
   if (nx > 0) {
     constexpr size_t kXhBytes = sizeof(float) * kServeThreads * MG_NXPARAM;  // 23,040 B
-    k_serve<false, 0, false, true>
-        <<<(int)nx, kServeThreads, kXhBytes, p->stream>>>(v, jt, bl + nb);
+    if (p->mirrored)
+      k_serve<false, MG_LAYOUT_MIRRORED, false, true>
+          <<<(int)nx, kServeThreads, kXhBytes, p->stream>>>(v, jt, bl + nb);
+    else
+      k_serve<false, 0, false, true>
+          <<<(int)nx, kServeThreads, kXhBytes, p->stream>>>(v, jt, bl + nb);
     PK(cudaGetLastError());
   }
   return MG_OK;

@@ -173,19 +173,25 @@ cudaError_t launch_pdl(Kernel kernel, int n_blocks, int threads, size_t smem, cu
   return cudaLaunchKernelEx(&cfg, kernel, fv, blocks, k, traj);
 }
 
-// The vectored and mirrored allocations are only instantiated for the diagonal-mass step, the
-// off-diagonal hydrodynamics (XH) only for the general one, the wide register budget only for
-// the diagonal-mass step without recording.
+// The vectored allocation is only instantiated for the diagonal-mass step, the off-diagonal
+// hydrodynamics (XH) only for the general one, the wide register budget only for the diagonal-mass
+// step without recording.
 template <int NTV, bool DIAG, bool REC, bool WIDE>
 cudaError_t launch_t(const FleetView &fv, const BlockDesc *blocks, int n_blocks, int threads,
                      int layout, int32_t k, float *traj, cudaStream_t stream) {
-  if constexpr (!DIAG) if (fv.xh)
-    return launch_pdl(k_fleet<NTV, false, REC, 0, true>, n_blocks, threads,
-                      sizeof(float) * MG_NXPARAM * threads, stream, fv, blocks, k, traj);
+  if constexpr (!DIAG)
+    if (fv.xh) {
+      const size_t smem = sizeof(float) * MG_NXPARAM * threads;
+      if (layout == MG_LAYOUT_MIRRORED)
+        return launch_pdl(k_fleet<NTV, false, REC, MG_LAYOUT_MIRRORED, true>, n_blocks, threads, smem,
+                          stream, fv, blocks, k, traj);
+      return launch_pdl(k_fleet<NTV, false, REC, 0, true>, n_blocks, threads, smem, stream, fv,
+                        blocks, k, traj);
+    }
+  if (layout == MG_LAYOUT_MIRRORED)
+    return launch_pdl(k_fleet<NTV, DIAG, REC, MG_LAYOUT_MIRRORED, false, WIDE>, n_blocks, threads, 0,
+                      stream, fv, blocks, k, traj);
   if constexpr (DIAG) {
-    if (layout == MG_LAYOUT_MIRRORED)
-      return launch_pdl(k_fleet<NTV, true, REC, MG_LAYOUT_MIRRORED, false, WIDE>, n_blocks, threads,
-                        0, stream, fv, blocks, k, traj);
     if (layout == MG_LAYOUT_VECTORED)
       return launch_pdl(k_fleet<NTV, true, REC, MG_LAYOUT_VECTORED, false, WIDE>, n_blocks, threads,
                         0, stream, fv, blocks, k, traj);
@@ -220,10 +226,10 @@ cudaError_t launch_d(const FleetView &fv, const BlockDesc *blocks, int n_blocks,
 
 template <int NTV, bool DIAG, bool REC, bool WIDE = false>
 const void *kernel_ptr(int layout) {
+  if (layout == MG_LAYOUT_MIRRORED)
+    return reinterpret_cast<const void *>(
+        &k_fleet<NTV, DIAG, REC, MG_LAYOUT_MIRRORED, false, WIDE>);
   if constexpr (DIAG) {
-    if (layout == MG_LAYOUT_MIRRORED)
-      return reinterpret_cast<const void *>(
-          &k_fleet<NTV, true, REC, MG_LAYOUT_MIRRORED, false, WIDE>);
     if (layout == MG_LAYOUT_VECTORED)
       return reinterpret_cast<const void *>(
           &k_fleet<NTV, true, REC, MG_LAYOUT_VECTORED, false, WIDE>);
@@ -234,13 +240,16 @@ const void *kernel_ptr(int layout) {
 template <int NTV, bool DIAG>
 const void *queue_ptr(bool wide, int layout, bool xh) {
   constexpr int S = DIAG ? 4 : 0;
+  constexpr int M = MG_LAYOUT_MIRRORED, V = MG_LAYOUT_VECTORED;
   if constexpr (!DIAG)
-    if (xh) return reinterpret_cast<const void *>(&k_fleet_queue<NTV, false, false, 0, true>);
+    if (xh)
+      return layout == M
+                 ? reinterpret_cast<const void *>(&k_fleet_queue<NTV, false, false, M, true>)
+                 : reinterpret_cast<const void *>(&k_fleet_queue<NTV, false, false, 0, true>);
+  if (layout == M)
+    return wide ? reinterpret_cast<const void *>(&k_fleet_queue<NTV, DIAG, true, M>)
+                : reinterpret_cast<const void *>(&k_fleet_queue<NTV, DIAG, false, M>);
   if constexpr (DIAG) {
-    constexpr int M = MG_LAYOUT_MIRRORED, V = MG_LAYOUT_VECTORED;
-    if (layout == M)
-      return wide ? reinterpret_cast<const void *>(&k_fleet_queue<NTV, true, true, M>)
-                  : reinterpret_cast<const void *>(&k_fleet_queue<NTV, true, false, M>);
     if (layout == V)
       return wide ? reinterpret_cast<const void *>(&k_fleet_queue<NTV, true, true, V>)
                   : reinterpret_cast<const void *>(&k_fleet_queue<NTV, true, false, V>);
@@ -253,13 +262,13 @@ const void *queue_kernel(NtVariant ntv, bool diag, bool wide, int layout, bool x
   switch (ntv) {
     case NT_6:
       return diag ? queue_ptr<NT_6, true>(wide, layout, false)
-                  : queue_ptr<NT_6, false>(wide, MG_LAYOUT_DENSE, xh);
+                  : queue_ptr<NT_6, false>(wide, layout, xh);
     case NT_8:
       return diag ? queue_ptr<NT_8, true>(wide, layout, false)
-                  : queue_ptr<NT_8, false>(wide, MG_LAYOUT_DENSE, xh);
+                  : queue_ptr<NT_8, false>(wide, layout, xh);
     default:
       return diag ? queue_ptr<NT_MIXED, true>(wide, layout, false)
-                  : queue_ptr<NT_MIXED, false>(wide, MG_LAYOUT_DENSE, xh);
+                  : queue_ptr<NT_MIXED, false>(wide, layout, xh);
   }
 }
 
@@ -272,7 +281,7 @@ void queue_launch_w(bool wide, int grid, size_t smem, const FleetView &fv, const
                     cudaStream_t stream) {
   if constexpr (!DIAG)
     if (fv.xh) {
-      k_fleet_queue<NTV, false, false, 0, true><<<grid, kQueueWarps * 32, smem, stream>>>(
+      k_fleet_queue<NTV, false, false, NH, true><<<grid, kQueueWarps * 32, smem, stream>>>(
           fv, slices, n_slices, k, chunk, sched);
       return;
     }
@@ -327,6 +336,9 @@ void queue_launch(bool diag, bool wide, int layout, int grid, size_t smem, const
   else if (diag)
     queue_launch_w<NTV, true, MG_LAYOUT_DENSE>(wide, grid, smem, fv, slices, n_slices, k, chunk, sched,
                                                stream);
+  else if (layout == MG_LAYOUT_MIRRORED)
+    queue_launch_w<NTV, false, MG_LAYOUT_MIRRORED>(wide, grid, smem, fv, slices, n_slices, k, chunk,
+                                                   sched, stream);
   else
     queue_launch_w<NTV, false, 0>(wide, grid, smem, fv, slices, n_slices, k, chunk, sched,
                                                stream);
@@ -360,7 +372,7 @@ cudaError_t fleet_kernel_attributes(NtVariant ntv, bool diag, int layout, bool r
   f = diag ? (rec ? kernel_ptr<N, true, true>(layout)                               \
                   : wide ? kernel_ptr<N, true, false, true>(layout)                 \
                          : kernel_ptr<N, true, false>(layout))                      \
-           : (rec ? kernel_ptr<N, false, true>(0) : kernel_ptr<N, false, false>(0));
+           : (rec ? kernel_ptr<N, false, true>(layout) : kernel_ptr<N, false, false>(layout));
   switch (ntv) {
     case NT_6: MG_PICK(NT_6) break;
     case NT_8: MG_PICK(NT_8) break;

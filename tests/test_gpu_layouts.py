@@ -56,8 +56,9 @@ FLEETS = {
 }
 
 
+@pytest.mark.parametrize("general", [False, True])  # True: off-centre gravity, full mass matrices
 @pytest.mark.parametrize("name", FLEETS)
-def test_allocation_matches_oracle_on_every_kernel(name):
+def test_allocation_matches_oracle_on_every_kernel(name, general):
     vs, only = FLEETS[name]
     n = 700
     types = np.full(n, 0, np.int32) if only == 0 else I.mixed_fleet(4, n, max_group=90)
@@ -65,6 +66,9 @@ def test_allocation_matches_oracle_on_every_kernel(name):
     params = I.perturbed_params(5, oracle_nominal(vs)[types], n)
     if name == "record off axis":
         params[n // 2, I.P_RB + 1] = 0.0078125
+    if general:
+        params[:, I.P_RG:I.P_RG + 3] = I.round_f32(
+            np.random.default_rng(2).uniform(-0.02, 0.02, (n, 3)))
     states = I.random_states(6, n, nt)
     cmds = I.commands(7, 4, n, nt).astype(np.float64)
     t, geo = oracle_types_geo(types, vs)
