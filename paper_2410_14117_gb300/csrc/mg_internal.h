@@ -191,6 +191,11 @@ struct SetupView {
 cudaError_t launch_randomize(const SetupView &v, const float *nominal /*dev [n_types][35]*/,
                              uint64_t seed, double lo, double hi, double current_sigma,
                              double rg_halfwidth, cudaStream_t stream, int background_blocks = 0);
+// Admission of a serving job's envs (v and st at the job's first env): types, a draw with the job's
+// seeds and ranges, and the start state of its first episode, in one launch.
+cudaError_t launch_admit(const SetupView &v, const float *nominal, const mg_job_spec &job,
+                         int32_t *types, const StatePlanes &st, uint32_t *episode, uint32_t *flags,
+                         unsigned long long *nonfinite_count, cudaStream_t stream);
 cudaError_t launch_import_params(const SetupView &v, const float *in /*dev [n][35]*/,
                                  cudaStream_t stream);
 // [n][MG_NXPARAM] records <-> [MG_NXPARAM][stride] planes (to_planes: records -> planes); the

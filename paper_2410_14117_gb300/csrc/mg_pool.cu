@@ -42,14 +42,15 @@ struct ServeBlock {
 
 namespace {
 
-constexpr int kServeThreads = 128;
-// Register cap of the tick kernel for ticks of many blocks: the diagonal-mass step coefficients
-// do not fit 128 registers beside the trajectory record without spilling; 144 (three blocks per
-// SM) served the 200 req/s job mix at p99 2.0 ms against 2.25 ms at 128, and the 10x stream at
-// 6.7 against 8.4 ms.
+// Two warps per block: a tick's blocks come in any number, and the last ones leave SMs idle by whole
+// blocks (6 jobs of up to 4,000 envs served in 274-280 us with 64 threads, 289 with 128, 281 with
+// 32; 12 jobs of up to 32,768 in 909, 909, 897).
+constexpr int kServeThreads = 64;
+// Register cap of the tick kernel for ticks of many blocks: 144 (seven blocks per SM) served those
+// 12 jobs in 909 us against 960 at 128, where the vectored and dense allocations also spill.
 constexpr int kRegsServe = 144;
 
-// WIDE (diagonal mass): 200 registers, for ticks whose blocks all fit at two per SM.  Few envs
+// WIDE (diagonal mass): 200 registers, for ticks of at most 256 envs per SM.  Few envs
 // (a warp per scheduler or fewer) run latency-bound and gain from the extra registers; a tick of
 // more blocks keeps more per SM resident with kRegsServe.  Measured on the 200 req/s job mix: p50
 // 0.60 -> 0.56 ms with this choice per tick; the wide kernel for every tick gave the same p50 but
@@ -134,11 +135,6 @@ void launch_serve_diag(int layout, bool wide, int grid, const FleetView &v, cons
     launch_serve<MG_LAYOUT_VECTORED>(wide, grid, v, jobs, blocks, stream);
   else
     launch_serve<MG_LAYOUT_DENSE>(wide, grid, v, jobs, blocks, stream);
-}
-
-__global__ void k_fill_i32(int32_t *p, int64_t n, int32_t v) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) p[i] = v;
 }
 
 }  // namespace
@@ -441,12 +437,8 @@ namespace {
 // [n_envs][MG_NXPARAM], or null) into its columns of the pool's planes, randomised parameters
 // and derived planes, episode counters and start states.
 cudaError_t init_job(mg_pool *p, const mg_job_spec &s, int64_t env0, const float *xh) {
-  const mg_ranges &r = s.ranges;
   const int64_t n = s.n_envs;
-  const int grid = (int)((n + 255) / 256);
-  k_fill_i32<<<grid, 256, 0, p->stream>>>(p->types + env0, n, s.vehicle_type);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
+  cudaError_t e = cudaSuccess;
   SetupView v{};
   v.n = n;
   v.gid0 = 0;
@@ -473,13 +465,8 @@ cudaError_t init_job(mg_pool *p, const mg_job_spec &s, int64_t env0, const float
     v.xh = p->xh + env0;
     v.xh_stride = p->cap;
   }
-  e = launch_randomize(v, p->nominal, s.param_seed, (double)r.lo, (double)r.hi,
-                       (double)r.current_sigma, (double)r.rg_halfwidth, p->stream);
-  if (e == cudaSuccess) e = cudaMemsetAsync(p->episode + env0, 0, 4 * n, p->stream);
-  if (e == cudaSuccess)
-    e = launch_reset(sub_state(p->st, env0), n, 0, nullptr, s.param_seed, (double)r.nu0_sigma,
-                     p->episode + env0, p->flags + env0, p->counters, p->stream);
-  return e;
+  return launch_admit(v, p->nominal, s, p->types + env0, sub_state(p->st, env0),
+                      p->episode + env0, p->flags + env0, p->counters, p->stream);
 }
 
 mg_status admit_job(mg_pool *p, const mg_job_spec *spec, float *traj, const float *xh,
@@ -609,7 +596,7 @@ mg_status mg_pool_tick(mg_pool *p, int32_t k, int32_t *n_running) {
       reinterpret_cast<const ServeBlock *>(static_cast<char *>(p->dev_table) + tb);
   const FleetView v = pool_view(p);
   const int g = (int)nb;
-  const bool wide = g <= 2 * p->n_sm;
+  const bool wide = (int64_t)g * kServeThreads <= 256 * (int64_t)p->n_sm;
   if (g == 0)
     ;
   else if (p->diag)
@@ -620,7 +607,7 @@ mg_status mg_pool_tick(mg_pool *p, int32_t k, int32_t *n_running) {
     k_serve<false, 0><<<g, kServeThreads, 0, p->stream>>>(v, jt, bl);
   PK(cudaGetLastError());
   if (nx > 0) {
-    constexpr size_t kXhBytes = sizeof(float) * kServeThreads * MG_NXPARAM;  // 23,040 B
+    constexpr size_t kXhBytes = sizeof(float) * kServeThreads * MG_NXPARAM;  // 11,520 B
     if (p->mirrored)
       k_serve<false, MG_LAYOUT_MIRRORED, false, true>
           <<<(int)nx, kServeThreads, kXhBytes, p->stream>>>(v, jt, bl + nb);
