@@ -548,6 +548,15 @@ mg_status mg_server_submit(mg_server *srv, const mg_job_spec *spec, int64_t *tic
 mg_status mg_server_submit_offdiag(mg_server *srv, const mg_job_spec *spec, const float *xh,
                                    int64_t *ticket);
 
+/* mg_server_submit (xh NULL) or mg_server_submit_offdiag for a server that records, with the job's
+ * trajectory record kept in the caller's buffer traj, device [horizon][MG_NTRAJ][n_envs], instead
+ * of one of the server's: the ticks write it in place, so collecting it costs no copy.  Its bytes
+ * count against the budget all the same.  The caller keeps traj alive until the job has been
+ * handed back and released, or the server is destroyed.  Errors as those calls, and MG_EINVAL
+ * (traj NULL or host memory, a server with record = 0). */
+mg_status mg_server_submit_record(mg_server *srv, const mg_job_spec *spec, const float *xh,
+                                  float *traj, int64_t *ticket);
+
 /* One round of the loop (above); the counts (any may be NULL) are those after it: jobs queued,
  * admitted and not yet handed back, ticks in flight.  Errors: MG_ETIMEOUT, MG_ECUDA, and those of
  * the pool calls. */

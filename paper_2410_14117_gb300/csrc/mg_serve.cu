@@ -33,6 +33,7 @@ struct ServeJob {
   double submit_s = 0.0, admit_s = -1.0, done_s = -1.0;
   int32_t job_id = -1;       // pool handle while admitted
   float *traj = nullptr;     // trajectory record (stream-ordered allocation) or null
+  float *caller_traj = nullptr;  // the caller's buffer to record into instead, or null
   double traj_bytes = 0.0;
   bool last_tick_issued = false;
   JobState state = QUEUED;
@@ -97,7 +98,7 @@ mg_status finish_front(mg_server *s) {
     if (!s->cfg.keep_done) {
       mg_status st = mg_pool_release(s->pool, j.job_id);
       if (st != MG_OK) return st;
-      if (j.traj) SK(cudaFreeAsync(j.traj, s->stream));
+      if (j.traj && !j.caller_traj) SK(cudaFreeAsync(j.traj, s->stream));
       j.traj = nullptr;
       s->used -= j.traj_bytes;
       j.state = RELEASED;
@@ -129,7 +130,9 @@ mg_status admit_queued(mg_server *s) {
     const double need = s->cfg.record ? traj_bytes_of(j.spec) : 0.0;
     if (s->used + need > s->cfg.budget_bytes) break;
     float *traj = nullptr;
-    if (s->cfg.record) {
+    if (j.caller_traj) {
+      traj = j.caller_traj;
+    } else if (s->cfg.record) {
       const cudaError_t e = cudaMallocFromPoolAsync(reinterpret_cast<void **>(&traj),
                                                     (size_t)need, s->mempool, s->stream);
       if (e == cudaErrorMemoryAllocation) {
@@ -143,11 +146,11 @@ mg_status admit_queued(mg_server *s) {
         j.xh.empty() ? mg_pool_admit(s->pool, &j.spec, traj, &jid)
                      : mg_pool_admit_offdiag(s->pool, &j.spec, traj, j.xh.data(), &jid);
     if (st == MG_ENOMEM) {  // no free arena range large enough yet
-      if (traj) SK(cudaFreeAsync(traj, s->stream));
+      if (traj && !j.caller_traj) SK(cudaFreeAsync(traj, s->stream));
       break;
     }
     if (st != MG_OK) {
-      if (traj) cudaFreeAsync(traj, s->stream);
+      if (traj && !j.caller_traj) cudaFreeAsync(traj, s->stream);
       return st;
     }
     j.job_id = jid;
@@ -205,7 +208,7 @@ mg_status mg_server_destroy(mg_server *s) {
   cudaStreamSynchronize(s->stream);
   for (ServeJob &j : s->jobs) {
     if (j.state == RUNNING || j.state == DONE) mg_pool_release(s->pool, j.job_id);
-    if (j.traj) cudaFreeAsync(j.traj, s->stream);
+    if (j.traj && !j.caller_traj) cudaFreeAsync(j.traj, s->stream);
   }
   cudaStreamSynchronize(s->stream);
   for (Inflight &f : s->inflight) cudaEventDestroy(f.ev);
@@ -219,15 +222,27 @@ mg_status mg_server_destroy(mg_server *s) {
 
 namespace {
 
-mg_status submit_job(mg_server *s, const mg_job_spec *spec, const float *xh, int64_t *ticket) {
+mg_status submit_job(mg_server *s, const mg_job_spec *spec, const float *xh, float *traj,
+                     int64_t *ticket) {
   if (!s || !spec || !ticket) return sfail(MG_EINVAL, "NULL argument");
   if (spec->n_envs < 1 || spec->n_envs > s->capacity || spec->horizon < 1 ||
       spec->hold_steps < 1)
     return sfail(MG_EINVAL, "bad job spec (n_envs outside [1, pool capacity], horizon or hold < 1)");
   if (s->cfg.record && traj_bytes_of(*spec) > s->cfg.budget_bytes)
     return sfail(MG_EINVAL, "the job's trajectory record alone exceeds the budget");
+  if (traj) {
+    if (!s->cfg.record) return sfail(MG_EINVAL, "the server does not record trajectories");
+    cudaPointerAttributes a;
+    if (cudaPointerGetAttributes(&a, traj) != cudaSuccess) {
+      cudaGetLastError();
+      a.type = cudaMemoryTypeUnregistered;
+    }
+    if (a.type != cudaMemoryTypeDevice && a.type != cudaMemoryTypeManaged)
+      return sfail(MG_EINVAL, "traj must be device memory");
+  }
   ServeJob j;
   j.spec = *spec;
+  j.caller_traj = traj;
   if (xh) {  // a copy of the records, kept until the job is admitted
     j.xh.resize((size_t)spec->n_envs * MG_NXPARAM);
     SK(cudaMemcpy(j.xh.data(), xh, j.xh.size() * sizeof(float), cudaMemcpyDefault));
@@ -244,12 +259,18 @@ mg_status submit_job(mg_server *s, const mg_job_spec *spec, const float *xh, int
 extern "C" {
 
 mg_status mg_server_submit(mg_server *s, const mg_job_spec *spec, int64_t *ticket) {
-  return submit_job(s, spec, nullptr, ticket);
+  return submit_job(s, spec, nullptr, nullptr, ticket);
 }
 
 mg_status mg_server_submit_offdiag(mg_server *s, const mg_job_spec *spec, const float *xh,
                                    int64_t *ticket) {
-  return submit_job(s, spec, xh, ticket);
+  return submit_job(s, spec, xh, nullptr, ticket);
+}
+
+mg_status mg_server_submit_record(mg_server *s, const mg_job_spec *spec, const float *xh,
+                                  float *traj, int64_t *ticket) {
+  if (!traj) return sfail(MG_EINVAL, "traj is NULL");
+  return submit_job(s, spec, xh, traj, ticket);
 }
 
 mg_status mg_server_poll(mg_server *s, int32_t *n_queued, int32_t *n_running,
@@ -342,7 +363,7 @@ mg_status mg_server_release(mg_server *s, int64_t ticket) {
   if (j.state != DONE) return sfail(MG_ESTATE, "the job is not finished and kept");
   mg_status st = mg_pool_release(s->pool, j.job_id);
   if (st != MG_OK) return st;
-  if (j.traj) SK(cudaFreeAsync(j.traj, s->stream));
+  if (j.traj && !j.caller_traj) SK(cudaFreeAsync(j.traj, s->stream));
   j.traj = nullptr;
   s->used -= j.traj_bytes;
   j.state = RELEASED;

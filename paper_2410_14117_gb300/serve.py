@@ -283,6 +283,7 @@ class NativeServer:
             raise ValueError("the arena alone exceeds the budget")
         self.peak_used = self.arena_bytes
         self._servers = {}  # mode -> native server, kept so its record memory pool stays warm
+        self._records = {}  # (mode, ticket) -> tensor an unreleased job records into
 
     def _server(self, mode):
         if mode not in self._servers:
@@ -294,10 +295,21 @@ class NativeServer:
             self._servers[mode] = h
         return self._servers[mode]
 
+    def _record_buffer(self, r):
+        """Tensor for a job's trajectory, written on the pool's stream."""
+        traj = torch.empty((r.horizon, MG_NTRAJ, r.n_envs), dtype=torch.float32,
+                           device=self.pool.device)
+        current = torch.cuda.current_stream(self.pool.device)
+        if current != self.pool.stream:
+            self.pool.stream.wait_stream(current)  # the block's earlier use
+            traj.record_stream(self.pool.stream)
+        return traj
+
     def close(self):
         for h in self._servers.values():
             call("mg_server_destroy", h)
         self._servers = {}
+        self._records = {}
         self.pool.close()
 
     def run(self, requests, mode: str = "batched", realtime: bool = True):
@@ -330,7 +342,14 @@ class NativeServer:
                                int(r.param_seed), int(r.cmd_seed),
                                Ranges(0.8, 1.2, 0.2, 0.3, 0))
                 tk = ctypes.c_int64()
-                if r.xh is None:
+                if self.keep_results and self.record:
+                    # the job records into the tensor its caller gets; the server keeps it alive
+                    # while ticks may write it, also past an exception here
+                    traj = self._record_buffer(r)
+                    call("mg_server_submit_record", h, ctypes.byref(spec),
+                         None if r.xh is None else _ptr(r.xh), _ptr(traj), ctypes.byref(tk))
+                    self._records[mode, tk.value] = traj
+                elif r.xh is None:
                     call("mg_server_submit", h, ctypes.byref(spec), ctypes.byref(tk))
                 else:
                     call("mg_server_submit_offdiag", h, ctypes.byref(spec), _ptr(r.xh),
@@ -355,12 +374,12 @@ class NativeServer:
             if self.keep_results:
                 r.final_state = torch.empty((r.n_envs, MG_NSTATE), dtype=torch.float32,
                                             device=self.pool.device)
-                r.traj = (torch.empty((r.horizon, MG_NTRAJ, r.n_envs), dtype=torch.float32,
-                                      device=self.pool.device) if self.record else None)
-                call("mg_server_job_result", h, tk, _ptr(r.final_state),
-                     _ptr(r.traj) if r.traj is not None else None)
+                call("mg_server_job_result", h, tk, _ptr(r.final_state), None)
                 call("mg_server_release", h, tk)
+                r.traj = self._records.pop((mode, tk), None)
             done.append(r)
+        if self.keep_results:
+            self.pool.sync()  # the state exports (the records were complete with their ticks)
         call("mg_server_info", h, None, None, ctypes.byref(d[0]))
         self.peak_used = max(self.peak_used, self.arena_bytes + d[0].value)
         makespan = max(r.done_s for r in done) - min(r.arrival_s for r in done)
