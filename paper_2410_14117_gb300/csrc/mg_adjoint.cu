@@ -498,11 +498,11 @@ __device__ __forceinline__ void stage_step(St<MT> &S, const float (&c)[MT], cons
     rhs<MT, DIAG, true, NH, PATH == ADJ_GEN>(y, A.F, gdir, garm, nt, ca, k, A.xh);
     const float nud[6] = {k.v[0], k.v[1], k.v[2], k.w[0], k.w[1], k.w[2]};
     stage(g, y, nud);
-    if (g == 0) axpy<MT, false>(acc, S, rk.h6, rk.q12, k);
-    else if (g < 3) axpy<MT, false>(acc, acc, rk.h3, rk.h6, k);
-    else axpy<MT, false>(S, acc, rk.h6, rk.q12, k);
-    if (g < 2) axpy<MT, false>(y, S, rk.hh, rk.qh, k);
-    else if (g == 2) axpy<MT, false>(y, S, rk.h, rk.hh, k);
+    if (g == 0) axpy<MT>(acc, S, rk.h6, rk.q12, k);
+    else if (g < 3) axpy<MT>(acc, acc, rk.h3, rk.h6, k);
+    else axpy<MT>(S, acc, rk.h6, rk.q12, k);
+    if (g < 2) axpy<MT>(y, S, rk.hh, rk.qh, k);
+    else if (g == 2) axpy<MT>(y, S, rk.h, rk.hh, k);
     const float f = g == 0 ? A.L.f2 : g == 1 ? A.L.f3 : g == 2 ? A.L.f4 : A.L.P;
 #pragma unroll
     for (int i = 0; i < MT; ++i) (g < 3 ? y.n[i] : S.n[i]) = fmaf(f, d[i], c[i]);
@@ -1125,7 +1125,10 @@ __global__ void __maxnreg__(XH ? kRegsXH : DIAG ? kRegsWide : kRegsGeneral)
       load_commands<MT>(fv, e, seg, nt, c);
       if (left < T - it) prefetch_commands(fv, e, seg);
     }
-    rk4_step<MT, DIAG, MIXED, NH, XH>(s, c, L, P, sdir, sarm, nt, current_accel, fv.rk, xh);
+    if constexpr (XH || MT > 6)
+      rk4_step<MT, DIAG, MIXED, NH, XH>(s, c, L, P, sdir, sarm, nt, current_accel, fv.rk2, xh);
+    else
+      rk4_step<MT, DIAG, MIXED, NH, XH>(s, c, L, P, sdir, sarm, nt, current_accel, fv.rk, xh);
     --left;
     record<MT>(traj + (int64_t)it * MG_NTRAJ * n, n, e, s);
   }

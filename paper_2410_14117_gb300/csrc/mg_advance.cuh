@@ -173,8 +173,9 @@ __device__ __forceinline__ void scheduled_start(const FleetView &fv, int64_t e, 
 // (scheduled_start, or a fused kernel's own source).
 // loaded: the parameters, where the caller has loaded them and the state s already (the task kernel,
 // before its block barrier; the step kernels' loops come out 2 % slower that way).
-template <int MT, bool DIAG, bool MIXED, bool REC, bool L2, int NH, bool XH, bool LOADED = false,
-          typename Start = void>
+// PACK: packed stage updates (see axpy).
+template <int MT, bool DIAG, bool MIXED, bool REC, bool L2, int NH, bool XH, bool PACK,
+          bool LOADED = false, typename Start = void>
 __device__ __forceinline__ void advance_env(const FleetView &fv, int64_t e, int nt,
                                             const float4 *gdir, const float4 *garm, Start start,
                                             int32_t k, float *traj, St<MT> &s, const float *xh,
@@ -211,7 +212,10 @@ __device__ __forceinline__ void advance_env(const FleetView &fv, int64_t e, int 
       if constexpr (REC)
         if (left < k - it) prefetch_commands(fv, e, seg);
     }
-    rk4_step<MT, DIAG, MIXED, NH, XH>(s, c, L, P, gdir, garm, nt, current_accel, fv.rk, xh);
+    if constexpr (PACK)
+      rk4_step<MT, DIAG, MIXED, NH, XH>(s, c, L, P, gdir, garm, nt, current_accel, fv.rk2, xh);
+    else
+      rk4_step<MT, DIAG, MIXED, NH, XH>(s, c, L, P, gdir, garm, nt, current_accel, fv.rk, xh);
     --left;
     if constexpr (REC) record<MT>(traj + (int64_t)it * MG_NTRAJ * fv.n, fv.n, e, s);
   }

@@ -276,6 +276,7 @@ struct mg_sim {
     v.model_flags = model_flags;
     v.dt = dt;
     v.rk = rk_step(dt);
+    v.rk2 = rk_pairs(v.rk);
     v.flags = flags;
     v.counters = counters;
     v.xh = has_xh ? xh : nullptr;

@@ -73,19 +73,21 @@ struct BlockDesc {
 // RK4's weights for sub-step size h.  They travel with the kernel parameters so that the stage
 // updates can take them as constant-bank operands: the step's issue rate is bound by register
 // operand reads, and a multiply-add with one constant reads two registers instead of three.
+// The packed updates (axpy) read each weight twice, from RkPairs.
 struct RkStep {
   float h, hh, h3, h6;  // h, h/2, h/3, h/6
   float qh, q12;        // h/4 and h/12: the quaternion's halves of hh and h6 (its rate is doubled)
 };
+struct RkPairs {
+  float2 h, hh, h3, h6, qh, q12;
+};
 inline RkStep rk_step(float h) {
-  RkStep r;
-  r.h = h;
-  r.hh = 0.5f * h;
-  r.h3 = h * (1.0f / 3.0f);
-  r.h6 = h * (1.0f / 6.0f);
-  r.qh = 0.5f * r.hh;
-  r.q12 = 0.5f * r.h6;
-  return r;
+  const float hh = 0.5f * h, h6 = h * (1.0f / 6.0f);
+  return {h, hh, h * (1.0f / 3.0f), h6, 0.5f * hh, 0.5f * h6};
+}
+inline RkPairs rk_pairs(const RkStep &r) {
+  auto twice = [](float x) { return make_float2(x, x); };
+  return {twice(r.h), twice(r.hh), twice(r.h3), twice(r.h6), twice(r.qh), twice(r.q12)};
 }
 
 // Everything a step kernel reads besides its block list; passed by value.
@@ -130,6 +132,7 @@ struct FleetView {
   // and task kernels then run their XH variants (general path), staging each block's
   // coefficients in shared memory.
   const float *xh;
+  RkPairs rk2;               // rk_pairs(rk)
 };
 
 // Kernel variants: thruster count fixed at 6 or 8, or mixed (up to 8, read per block).

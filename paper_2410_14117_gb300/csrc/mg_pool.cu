@@ -103,7 +103,7 @@ __global__ void __maxnreg__(XH ? kRegsXH : !DIAG ? kRegsGeneral : WIDE ? kRegsWi
       left = jd.hold;
       load(seg);
     }
-    rk4_step<MT, DIAG, true, NH, XH>(s, c, L, P, sdir, sarm, nt, current_accel, fv.rk,
+    rk4_step<MT, DIAG, true, NH, XH>(s, c, L, P, sdir, sarm, nt, current_accel, fv.rk2,
                                      XH ? sxh + threadIdx.x * MG_NXPARAM : nullptr);
     --left;
     if (jd.traj) {
@@ -230,6 +230,7 @@ FleetView pool_view(const mg_pool *p) {
   v.n = p->cap;
   v.dt = p->dt;
   v.rk = rk_step(p->dt);
+  v.rk2 = rk_pairs(v.rk);
   v.flags = p->flags;
   v.counters = p->counters;
   v.hold = 1;

@@ -74,7 +74,7 @@ __global__ void __maxnreg__(XH ? kRegsXH : !DIAG ? kRegsGeneral : WIDE ? kRegsWi
   St<MT> st;
   const int nt = MIXED ? bd.n_thr : MT;
   const int64_t step0 = s_cursor + fv.cursor_off;
-  advance_env<MT, DIAG, MIXED, REC, false, NH, XH>(
+  advance_env<MT, DIAG, MIXED, REC, false, NH, XH, XH || (REC && MT > 6)>(
       fv, e, nt, sdir, sarm,
       [&](float (&c)[MT], int64_t &seg, int32_t &left) {
         scheduled_start<MT>(fv, e, nt, step0, c, seg, left);
@@ -138,7 +138,7 @@ __global__ void __maxnreg__(XH ? kRegsXH : !DIAG ? kRegsGeneral : WIDE ? kRegsWi
         for (int j = 0; j < MG_NXPARAM; ++j) row[j] = __ldg(fv.xh + (int64_t)j * fv.n + e);
       St<MT> st;
       const int nt = MIXED ? bd.n_thr : MT;
-      advance_env<MT, DIAG, MIXED, false, true, NH, XH>(
+      advance_env<MT, DIAG, MIXED, false, true, NH, XH, XH>(
           fv, e, nt, gdir, garm,
           [&](float (&cmd)[MT], int64_t &seg, int32_t &left) {
             scheduled_start<MT>(fv, e, nt, step0 + (int64_t)c * chunk, cmd, seg, left);

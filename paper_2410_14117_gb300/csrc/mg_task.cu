@@ -318,7 +318,7 @@ __global__ void __maxnreg__(XH ? kRegsXH : DIAG ? kRegsDiag : kRegsGeneral)
   __syncthreads();
   if (!live) return;
   const int nt = MIXED ? bd.n_thr : MT;
-  advance_env<MT, DIAG, MIXED, false, false, NH, XH, true>(
+  advance_env<MT, DIAG, MIXED, false, false, NH, XH, XH || (MT > 6), true>(
       fv, e, nt, sdir, sarm,
       [&](float (&c)[MT], int64_t &seg, int32_t &left) {
         if (to.act_in) {  // one command for the whole launch, no cursor
