@@ -100,6 +100,7 @@ bool is_device_ptr(const void *p) {
 struct GraphEntry {
   int32_t k;
   const float *act_src;
+  const char *par;  // the parameter range the kernels read (mg_randomize_prefetch exchanges two)
   int32_t n_seg, hold, proc;
   uint64_t cmd_seed;
   cudaGraphExec_t exec;
@@ -155,15 +156,21 @@ struct mg_sim {
   int32_t adj_mode = 0;
   float *adj_ws = nullptr;
   size_t adj_ws_cap = 0;
-  // the arena's parameter range (derived planes, then the raw records): one contiguous span
-  size_t par_off = 0, par_bytes = 0;
+  // the parameter range in use (derived planes, then the raw records): one contiguous span, the
+  // arena's until an install exchanges it
+  char *par = nullptr;
+  size_t par_bytes = 0;
 
   // background randomisation (mg_randomize_prefetch): a second parameter range of the same
-  // layout, followed by its own non-SPD count and off-diagonal word, drawn on the library's own
-  // stream; pf_done orders the install after the draw, pf_consumed the next draw after the
-  // install's copy.  Keyed by everything the draw depends on.  Created on first use.
+  // layout and a non-SPD count and off-diagonal word of its own, drawn on the library's own
+  // stream.  An install exchanges the two ranges (1,048,576 envs: a copy of the 360 bytes per env
+  // would take 110 us, more than drawing them does), or copies once a user's graph has captured
+  // the range in use.  pf_done orders the install after the draw, pf_consumed the next draw after
+  // the last work that reads the range it writes.  Keyed by everything the draw depends on.
+  // Created on first use.
   cudaStream_t pf_stream = nullptr;
-  char *pf_buf = nullptr;
+  char *pf_alloc = nullptr;  // [par_bytes] range, then the two check words
+  char *pf_buf = nullptr;    // the range not in use
   cudaEvent_t pf_done = nullptr, pf_consumed = nullptr;
   bool pf_valid = false;
   uint64_t pf_seed = 0;
@@ -301,21 +308,24 @@ struct mg_sim {
     return v;
   }
 
-  // setup_view() with every parameter pointer moved into the background range
+  // Move v's parameter pointers from range `from` to range `to`.
+  static void rebase(ParamPlanes &pa, float *&raw, const char *from, char *to) {
+    auto move = [&](auto *&ptr) {
+      using P = std::remove_reference_t<decltype(ptr)>;
+      ptr = reinterpret_cast<P>(to + (reinterpret_cast<const char *>(ptr) - from));
+    };
+    move(raw);
+    move(pa.d0); move(pa.d1); move(pa.d2); move(pa.d3); move(pa.d4); move(pa.d5); move(pa.d6);
+    move(pa.d7); move(pa.d8);
+    move(pa.g0); move(pa.g1); move(pa.g2); move(pa.g3); move(pa.g4); move(pa.g5);
+  }
+
+  // setup_view() on the range not in use, with its own check words
   SetupView staged_setup_view() const {
     SetupView v = setup_view();
-    const char *base = static_cast<const char *>(arena) + par_off;
-    auto move = [&](auto *ptr) {
-      return reinterpret_cast<decltype(ptr)>(pf_buf + (reinterpret_cast<const char *>(ptr) - base));
-    };
-    v.raw = move(v.raw);
-    v.pa.d0 = move(v.pa.d0); v.pa.d1 = move(v.pa.d1); v.pa.d2 = move(v.pa.d2);
-    v.pa.d3 = move(v.pa.d3); v.pa.d4 = move(v.pa.d4); v.pa.d5 = move(v.pa.d5);
-    v.pa.d6 = move(v.pa.d6); v.pa.d7 = move(v.pa.d7); v.pa.d8 = move(v.pa.d8);
-    v.pa.g0 = move(v.pa.g0); v.pa.g1 = move(v.pa.g1); v.pa.g2 = move(v.pa.g2);
-    v.pa.g3 = move(v.pa.g3); v.pa.g4 = move(v.pa.g4); v.pa.g5 = move(v.pa.g5);
-    v.n_not_spd = reinterpret_cast<unsigned long long *>(pf_buf + par_bytes);
-    v.any_offdiag = reinterpret_cast<unsigned int *>(pf_buf + par_bytes + 8);
+    rebase(v.pa, v.raw, par, pf_buf);
+    v.n_not_spd = reinterpret_cast<unsigned long long *>(pf_alloc + par_bytes);
+    v.any_offdiag = reinterpret_cast<unsigned int *>(pf_alloc + par_bytes + 8);
     return v;
   }
 
@@ -682,7 +692,7 @@ mg_status mg_create(int64_t n_envs, const int32_t *vehicle_types,
   for (int i = 0; i < 5; ++i) *gp[i] = (float4 *)(a + o_g[i]);
   s->pa.g5 = (float *)(a + o_g5);
   s->raw = (float *)(a + o_raw);
-  s->par_off = o_d[0];
+  s->par = a + o_d[0];
   s->par_bytes = o_types - o_d[0];
   s->types_d = (int32_t *)(a + o_types);
   s->geo_d = (Geo *)(a + o_geo);
@@ -784,7 +794,7 @@ mg_status mg_destroy(mg_sim *s) {
     cudaStreamDestroy(s->pf_stream);
     cudaEventDestroy(s->pf_done);
     cudaEventDestroy(s->pf_consumed);
-    cudaFree(s->pf_buf);
+    cudaFree(s->pf_alloc);
   }
   if (s->h2d_stream) {
     cudaStreamSynchronize(s->h2d_stream);
@@ -917,23 +927,25 @@ mg_status mg_randomize_prefetch(mg_sim *s, uint64_t seed, const mg_ranges *r) {
     MG_CK(cudaStreamCreateWithFlags(&s->pf_stream, cudaStreamNonBlocking));
     MG_CK(cudaEventCreateWithFlags(&s->pf_done, cudaEventDisableTiming));
     MG_CK(cudaEventCreateWithFlags(&s->pf_consumed, cudaEventDisableTiming));
-    if (cudaMalloc(&s->pf_buf, s->par_bytes + 16) != cudaSuccess) {
+    if (cudaMalloc(&s->pf_alloc, s->par_bytes + 16) != cudaSuccess) {
       cudaGetLastError();
-      s->pf_buf = nullptr;
+      s->pf_alloc = nullptr;
       cudaEventDestroy(s->pf_done);
       cudaEventDestroy(s->pf_consumed);
       cudaStreamDestroy(s->pf_stream);
       s->pf_stream = nullptr;
       return fail(MG_ENOMEM, "cudaMalloc(background parameter range)");
     }
+    s->pf_buf = s->pf_alloc;
   }
   s->pf_valid = false;
-  // the last install's copy must have read the range (a never-recorded event is no wait)
+  // everything that reads this range was queued before the last install (a never-recorded event is
+  // no wait)
   MG_CK(cudaStreamWaitEvent(s->pf_stream, s->pf_consumed, 0));
   const SetupView v = s->staged_setup_view();
   MG_CK(cudaMemsetAsync(v.n_not_spd, 0, 16, s->pf_stream));
   MG_CK(launch_randomize(v, s->nominal_d, seed, (double)r->lo, (double)r->hi,
-                         (double)r->current_sigma, 0.0, s->pf_stream, s->n_sm));
+                         (double)r->current_sigma, 0.0, s->pf_stream, 16 * s->n_sm));
   MG_CK(cudaEventRecord(s->pf_done, s->pf_stream));
   s->pf_valid = true;
   s->pf_seed = seed;
@@ -955,13 +967,18 @@ mg_status mg_randomize(mg_sim *s, uint64_t seed, const mg_ranges *r) {
     return fail(MG_EINVAL, "MG_RANDOMIZE_ASYNC needs mass matrices known to be diagonal "
                            "(r_g = 0 for every type, rg_halfwidth = 0, no extension)");
   if (staged_matches(s, seed, r)) {
-    // install the background draw: one copy of the parameter range and its two check words
-    char *live = static_cast<char *>(s->arena) + s->par_off;
+    // install the background draw and its two check words
     MG_CK(cudaStreamWaitEvent(s->stream, s->pf_done, 0));
-    MG_CK(cudaMemcpyAsync(live, s->pf_buf, s->par_bytes, cudaMemcpyDeviceToDevice, s->stream));
-    MG_CK(cudaMemcpyAsync(s->counters + 1, s->pf_buf + s->par_bytes, 8,
+    if (capturing(s) || s->captured) {
+      MG_CK(cudaMemcpyAsync(s->par, s->pf_buf, s->par_bytes, cudaMemcpyDeviceToDevice, s->stream));
+    } else {
+      mg_sim::rebase(s->pa, s->raw, s->par, s->pf_buf);
+      std::swap(s->par, s->pf_buf);
+      s->pf_valid = false;  // the range not in use holds the previous parameters now
+    }
+    MG_CK(cudaMemcpyAsync(s->counters + 1, s->pf_alloc + s->par_bytes, 8,
                           cudaMemcpyDeviceToDevice, s->stream));
-    MG_CK(cudaMemcpyAsync(s->offdiag, s->pf_buf + s->par_bytes + 8, 4,
+    MG_CK(cudaMemcpyAsync(s->offdiag, s->pf_alloc + s->par_bytes + 8, 4,
                           cudaMemcpyDeviceToDevice, s->stream));
     MG_CK(cudaEventRecord(s->pf_consumed, s->stream));
   } else {
@@ -996,6 +1013,7 @@ mg_status mg_get_params(mg_sim *s, float *out) {
   MG_NONNULL(out);
   const size_t bytes = (size_t)s->n * MG_NPARAM * 4;
   if (is_device_ptr(out)) {
+    capturing(s);  // a user's graph then reads this parameter range
     MG_CK(launch_export_params(s->setup_view(), out, s->stream));
     return MG_OK;
   }
@@ -1200,7 +1218,7 @@ mg_status mg_step(mg_sim *s, int32_t k) {
   const float *src = s->proc ? nullptr : s->act_src;
   const uint64_t seed = s->proc ? s->cmd_seed : 0;
   for (auto &g : s->graphs)
-    if (g.k == k && g.act_src == src && g.n_seg == s->n_seg && g.hold == s->hold &&
+    if (g.k == k && g.act_src == src && g.par == s->par && g.n_seg == s->n_seg && g.hold == s->hold &&
         g.proc == s->proc && g.cmd_seed == seed)
       hit = &g;
   if (!hit) {
@@ -1221,7 +1239,7 @@ mg_status mg_step(mg_sim *s, int32_t k) {
       return st;
     }
     MG_CK(ce);
-    GraphEntry g{k, src, s->n_seg, s->hold, s->proc, seed, nullptr, 0};
+    GraphEntry g{k, src, s->par, s->n_seg, s->hold, s->proc, seed, nullptr, 0};
     ce = cudaGraphInstantiate(&g.exec, graph, 0);
     cudaGraphDestroy(graph);
     MG_CK(ce);
@@ -1307,6 +1325,7 @@ mg_status mg_rollout_backward(mg_sim *s, int32_t T, int32_t C, const float *ckpt
   if ((dact && !is_device_ptr(dact)) || (dstate0 && !is_device_ptr(dstate0)))
     return fail(MG_EINVAL, "adjoint buffers must be device memory");
   const bool eight = s->ntv != NT_6;
+  capturing(s);  // a user's graph then reads this parameter range
   bool split = false;
   const bool general = !s->diag || s->has_xh;
   MG_CK(adjoint_split(s->n, general, s->adj_mode, &split));

@@ -108,3 +108,39 @@ def test_captured_steps_replay_around_rewinds(k, schedule_inside, step_before_re
         assert torch.equal(a.get_state(), b.get_state())
         a.close()
         b.close()
+
+
+def test_exchanged_parameters_around_a_captured_step():
+    """Prefetched draws installed before and after step(5) is captured into a user's graph, whose
+    replays must see each installed draw; an unmatched draw in between; graph-cached long steps."""
+    s = torch.cuda.Stream()
+    with torch.cuda.stream(s):
+        a, b = _sim(s), _sim(s)
+        for sim in (a, b):
+            sim.set_launch(64, 20, True)  # step(45) replays a cached graph
+            sim.set_procedural_actions(7, 5)
+        g = None
+        for ep in range(6):
+            for sim in (a, b):
+                if ep != 3:
+                    if sim is a:
+                        sim.randomize_prefetch(50 + ep)
+                    sim.randomize(50 + ep, nu0_sigma=0.3, wait=False)
+                else:  # a draw for another seed stays in the buffer
+                    if sim is a:
+                        sim.randomize_prefetch(99)
+                    sim.randomize(7, nu0_sigma=0.3)
+                sim.reset()
+                sim.step(45)
+            if ep == 2:
+                torch.cuda.synchronize()
+                g = torch.cuda.CUDAGraph()
+                with torch.cuda.graph(g, stream=s, capture_error_mode="thread_local"):
+                    a.step(5)
+            if g is not None:
+                g.replay()
+                b.step(5)
+            assert torch.equal(a.get_params(), b.get_params())
+            assert torch.equal(a.get_state(), b.get_state()), ep
+        a.close()
+        b.close()
