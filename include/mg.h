@@ -189,18 +189,18 @@ mg_status mg_randomize(mg_sim *sim, uint64_t seed, const mg_ranges *ranges);
 /* Background randomisation (§METHOD's per-episode domain randomisation, drawn ahead): draws the
  * parameters mg_randomize(sim, seed, ranges) would draw into a second parameter buffer of the
  * sim, on the library's own stream, so that the draw runs while the sim's stream is still
- * stepping the current episode (small blocks striding over the fleet).  The draw waits only for the work queued before the previous
- * install, which reads the buffer it writes.  A later mg_randomize with the same seed, lo, hi and current_sigma, the same
- * env-id offset and rg_halfwidth 0 installs the buffer (ordered after the draw) instead of
- * drawing, by exchanging it with the one in use, or, once the sim's stream has been captured into
- * a user's CUDA graph, with one device-to-device copy: the parameters are bit-identical to
- * a direct draw, and the rest of mg_randomize (nu0_sigma and the seed recorded for mg_reset,
- * episode counters zeroed, MG_RANDOMIZE_ASYNC) applies as usual.  Any other mg_randomize draws
- * directly and leaves a buffer not yet installed in place; a new prefetch replaces it.  ranges->nu0_sigma and
- * ranges->flags are not used here.  The buffer (the sim's parameter planes and records, 360 B
- * per env) is allocated on first use.  Errors: MG_EINVAL (ranges as mg_randomize, or mass matrices
- * that may be full: some type with r_g != 0, rg_halfwidth != 0, or the off-diagonal extension
- * set), MG_ENOMEM, MG_ECUDA. */
+ * stepping the current episode (small blocks striding over the fleet).  The draw waits only for
+ * the work queued before the previous install, which reads the buffer it writes.  A later
+ * mg_randomize with the same seed, lo, hi and current_sigma, the same env-id offset and
+ * rg_halfwidth 0 installs the buffer (ordered after the draw) instead of drawing, by exchanging it
+ * with the one in use, or, once the sim's stream has been captured into a user's CUDA graph, with
+ * one device-to-device copy: the parameters are bit-identical to a direct draw, and the rest of
+ * mg_randomize (nu0_sigma and the seed recorded for mg_reset, episode counters zeroed,
+ * MG_RANDOMIZE_ASYNC) applies as usual.  Any other mg_randomize draws directly and leaves a buffer
+ * not yet installed in place; a new prefetch replaces it.  ranges->nu0_sigma and ranges->flags are
+ * not used here.  The buffer (the sim's parameter planes and records, 360 B per env) is allocated
+ * on first use.  Errors: MG_EINVAL (ranges as mg_randomize, or mass matrices that may be full: some
+ * type with r_g != 0, rg_halfwidth != 0, or the off-diagonal extension set), MG_ENOMEM, MG_ECUDA. */
 mg_status mg_randomize_prefetch(mg_sim *sim, uint64_t seed, const mg_ranges *ranges);
 
 /* Set every env's parameters from a [n][MG_NPARAM] record (host or device); inverts the mass
