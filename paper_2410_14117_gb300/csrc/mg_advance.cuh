@@ -77,6 +77,28 @@ __device__ __forceinline__ void finish_envs(const FleetView &fv, unsigned *s_don
   }
 }
 
+// The task kernel's form, called by one thread of every block after its dependency wait: the cursor
+// the launch starts at, which that thread alone reads for its block.  The block is counted at once,
+// by an increment that depends on the value read, so the last block to begin knows that all have
+// read the cursor and advances it (the next launch looks after this one's end).  In a kernel of a
+// few sub-steps the count's round trip at the end stands between the last sub-step and the next
+// launch: 1,000-env environment steps 5.60 us with it there, 5.39 here, 65,536-env mixed ones 22.2
+// and 21.9.  The step kernels keep theirs at the end: their loops come out slower with this one
+// (1,048,576 envs x 50 on the static grid 937 against 957 us).
+// use_cursor = false: the launch only counts (it has its own command).
+__device__ __forceinline__ int64_t begin_launch(const FleetView &fv, bool use_cursor) {
+  const int64_t at = use_cursor ? launch_cursor(fv) : 0;
+  if (fv.cursor_adv) {
+    const unsigned one = at < 0 ? 2u : 1u;  // 1: the cursor is never negative
+    if (atomicAdd(fv.done_blocks, one) == gridDim.x - 1) {
+      atomicAdd(reinterpret_cast<unsigned long long *>(fv.cursor),
+                (unsigned long long)fv.cursor_adv);
+      atomicExch(fv.done_blocks, 0u);
+    }
+  }
+  return at;
+}
+
 // Stage a block's off-diagonal hydrodynamic coefficients in shared memory: row t of sx (stride
 // MG_NXPARAM, coprime with the 32 banks) receives env env0 + t's coefficients from the
 // component-major planes xh [MG_NXPARAM][n] (each component read coalesced).

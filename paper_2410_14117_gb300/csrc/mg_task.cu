@@ -277,7 +277,6 @@ __global__ void __maxnreg__(XH ? kRegsXH : DIAG ? kRegsDiag : kRegsGeneral)
   constexpr int MT = (NTV == NT_6) ? 6 : 8;
   constexpr bool MIXED = (NTV == NT_MIXED);
   __shared__ float4 sdir[MG_MAX_THR], sarm[MG_MAX_THR];
-  __shared__ unsigned s_done;
   __shared__ int64_t s_cursor;
   // dynamic: [blockDim.x][MG_NXPARAM] off-diagonal hydrodynamics (XH), then
   // [blockDim.x][obs_dim] observation rows (to.stage)
@@ -295,10 +294,7 @@ __global__ void __maxnreg__(XH ? kRegsXH : DIAG ? kRegsDiag : kRegsGeneral)
   // and the next step's launch may run up to its own wait beside this one.
   cudaTriggerProgrammaticLaunchCompletion();
   cudaGridDependencySynchronize();
-  if (threadIdx.x == 0) {
-    s_done = 0u;
-    if (!to.act_in) s_cursor = launch_cursor(fv);
-  }
+  if (threadIdx.x == 0) s_cursor = begin_launch(fv, !to.act_in);
   if constexpr (XH) stage_xh(fv.xh, fv.n, bd.env0, bd.count, sxh);
   // the env's loads are on their way while the block waits for the cursor
   const int64_t e = (int64_t)bd.env0 + threadIdx.x;
@@ -334,7 +330,6 @@ __global__ void __maxnreg__(XH ? kRegsXH : DIAG ? kRegsDiag : kRegsGeneral)
   const int obs_dim = to.obs_dim;
   task_epilogue<MT>(fv, tv, to, k_task, e, task_in(fv, tv, to, e), s,
                     to.stage ? sobs + threadIdx.x * obs_dim : to.obs + e * obs_dim);
-  if (fv.cursor_adv) finish_envs(fv, &s_done, bd.count, fv.cursor_adv);
   if (!to.stage) return;
   // Warp copy-out: the warp's live lanes are its low lanes (threads below bd.count).
   const int lane = threadIdx.x & 31;
