@@ -1629,7 +1629,8 @@ mg_status mg_kernel_info(mg_sim *s, int32_t *regs, int32_t *max_threads, int32_t
     MG_CK(queue_kernel_attributes(s->ntv, s->diag, s->wide, s->layout, s->has_xh, &a,
                                   &per_sm));
   else
-    MG_CK(fleet_kernel_attributes(s->ntv, s->diag, s->layout, false, s->wide, &a));
+    MG_CK(fleet_kernel_attributes(s->ntv, s->diag, s->layout, false, s->wide, s->n_blocks,
+                                  s->threads, &a));
   if (regs) *regs = a.numRegs;
   if (max_threads) *max_threads = a.maxThreadsPerBlock;
   if (local_bytes) *local_bytes = (int32_t)a.localSizeBytes;

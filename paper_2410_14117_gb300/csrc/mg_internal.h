@@ -36,7 +36,7 @@ struct StatePlanes {
 };
 
 // ---------------------------------------------------------------- derived parameter planes
-// What the step needs, derived once per parameter change (FP64 on the device, stored FP32).
+// What the step needs, derived once per parameter change (to FP64's rounding, stored FP32).
 // Diagonal-mass fleets (r_g = 0 everywhere, so M = M_RB + M_A is diagonal) read D0..D8 only:
 //   D0 (m, Ma_u, Ma_v, Ma_w)       D1 (Jx, Jy, Jz, W - B)   J = diag(I_o) + Ma_rot
 //   D2 (Dl_u, Dl_v, Dl_w, Dl_p)    D3 (Dl_q, Dl_r, Dq_u, Dq_v)   D4 (Dq_w, Dq_p, Dq_q, Dq_r)
@@ -142,12 +142,13 @@ enum NtVariant { NT_6 = 0, NT_8 = 1, NT_MIXED = 2 };
 // Static schedule: one block per BlockDesc, k sub-steps per launch.
 // layout: MG_LAYOUT_* (mg_device.cuh), the thruster allocation: the fastest one of the path that
 // every vehicle type present has.
-// wide: the diagonal-mass kernel without recording gets 200 registers instead of 128.
+// wide: the diagonal-mass kernel without recording gets 200 registers instead of 128 (the mirrored
+// allocation only where that pays).
 cudaError_t launch_fleet(const FleetView &fv, const BlockDesc *blocks, int n_blocks, int threads,
                          NtVariant ntv, bool diag, int layout, bool wide, int32_t k,
                          float *traj, cudaStream_t stream);
-cudaError_t fleet_kernel_attributes(NtVariant ntv, bool diag, int layout, bool record,
-                                    bool wide, cudaFuncAttributes *attr);
+cudaError_t fleet_kernel_attributes(NtVariant ntv, bool diag, int layout, bool record, bool wide,
+                                    int n_blocks, int threads, cudaFuncAttributes *attr);
 
 // Work-queue schedule: warps claim (32-env slice, chunk of sub-steps) units in chunk-major
 // order.  sched: device words, zeroed by the launcher: [0] next unit, [1..3] unused,

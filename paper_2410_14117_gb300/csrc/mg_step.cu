@@ -56,10 +56,8 @@ __global__ void __maxnreg__(XH ? kRegsXH : !DIAG ? kRegsGeneral : WIDE ? kRegsWi
     sdir[threadIdx.x] = fv.geo[bd.type].dir[threadIdx.x];
     sarm[threadIdx.x] = fv.geo[bd.type].arm[threadIdx.x];
   }
-  // Programmatic dependent launch: the next launch in the stream may start (and run up to its
-  // own wait) now; everything above reads only buffers written before any step launch, and
-  // everything below waits for the previous launch in the stream to complete.
-  cudaTriggerProgrammaticLaunchCompletion();
+  // Programmatic dependent launch: everything above reads only buffers written before any step
+  // launch, and everything below waits for the previous launch in the stream to complete.
   cudaGridDependencySynchronize();
   if (threadIdx.x == 0) {
     s_done = 0u;
@@ -80,6 +78,13 @@ __global__ void __maxnreg__(XH ? kRegsXH : !DIAG ? kRegsGeneral : WIDE ? kRegsWi
         scheduled_start<MT>(fv, e, nt, step0, c, seg, left);
       },
       k, traj, st, XH ? sxh + threadIdx.x * MG_NXPARAM : nullptr);
+  // The next launch's blocks may be placed once every block of this one has come here (k = 1) or
+  // ended.  Placed earlier they take the slots that happen to be free, two on one SM and none on
+  // another, and the launch runs as long as its fullest SM: with the trigger before the sub-steps,
+  // launches of 10 took 16.2 us for 30,000 envs instead of 10.6, and 9.5 instead of 7.4 for 15,000.
+  // After them it is still too early where the last blocks run on (19,456 envs x 10: 9.8 instead
+  // of 7.5), and only pays for one sub-step (65,536 envs in a graph: 3.8 us, without it 4.0).
+  if (k == 1) cudaTriggerProgrammaticLaunchCompletion();
   store_and_flag<MT, false>(fv, e, st);
   if (fv.cursor_adv) finish_envs(fv, &s_done, bd.count, fv.cursor_adv, s_rewinding);
 }
@@ -188,9 +193,10 @@ cudaError_t launch_t(const FleetView &fv, const BlockDesc *blocks, int n_blocks,
       return launch_pdl(k_fleet<NTV, false, REC, 0, true>, n_blocks, threads, smem, stream, fv,
                         blocks, k, traj);
     }
+  constexpr bool MWIDE = WIDE && NTV != NT_6;  // wide_kernel
   if (layout == MG_LAYOUT_MIRRORED)
-    return launch_pdl(k_fleet<NTV, DIAG, REC, MG_LAYOUT_MIRRORED, false, WIDE>, n_blocks, threads, 0,
-                      stream, fv, blocks, k, traj);
+    return launch_pdl(k_fleet<NTV, DIAG, REC, MG_LAYOUT_MIRRORED, false, MWIDE>, n_blocks, threads,
+                      0, stream, fv, blocks, k, traj);
   if constexpr (DIAG) {
     if (layout == MG_LAYOUT_VECTORED)
       return launch_pdl(k_fleet<NTV, true, REC, MG_LAYOUT_VECTORED, false, WIDE>, n_blocks, threads,
@@ -200,6 +206,21 @@ cudaError_t launch_t(const FleetView &fv, const BlockDesc *blocks, int n_blocks,
                     blocks, k, traj);
 }
 
+// Whether the static grid takes the 200-register kernel.  The mirrored allocation fits 128 registers
+// without spilling, which puts four 128-thread blocks on an SM against three: 65,536 envs x 200 in
+// 288 us against 373, 1,048,576 x 50 in 937 against 966; six thrusters gain nothing by more
+// registers at any size (1,000 envs x 200: 90 us both, 50,000: 223 against 233).  Eight, and mixed
+// fleets, do while all blocks are resident at once (1,000 envs: 95 against 102 us; 50,000: 241
+// against 246).  The other allocations spill at 128.
+template <int NTV>
+bool wide_kernel(bool wide, int layout, int n_blocks, int threads) {
+  if (!wide || layout != MG_LAYOUT_MIRRORED) return wide;
+  int dev = 0, n_sm = 0;
+  return NTV != NT_6 && cudaGetDevice(&dev) == cudaSuccess &&
+         cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess &&
+         n_blocks <= n_sm * (12 / (threads / 32));
+}
+
 template <int NTV, bool DIAG>
 cudaError_t launch_r(const FleetView &fv, const BlockDesc *blocks, int n_blocks, int threads,
                      int layout, bool wide, int32_t k, float *traj, cudaStream_t stream) {
@@ -207,7 +228,7 @@ cudaError_t launch_r(const FleetView &fv, const BlockDesc *blocks, int n_blocks,
     return launch_t<NTV, DIAG, true, false>(fv, blocks, n_blocks, threads, layout, k, traj,
                                             stream);
   if constexpr (DIAG)
-    if (wide)
+    if (wide_kernel<NTV>(wide, layout, n_blocks, threads))
       return launch_t<NTV, true, false, true>(fv, blocks, n_blocks, threads, layout, k,
                                               traj, stream);
   return launch_t<NTV, DIAG, false, false>(fv, blocks, n_blocks, threads, layout, k, traj,
@@ -228,7 +249,7 @@ template <int NTV, bool DIAG, bool REC, bool WIDE = false>
 const void *kernel_ptr(int layout) {
   if (layout == MG_LAYOUT_MIRRORED)
     return reinterpret_cast<const void *>(
-        &k_fleet<NTV, DIAG, REC, MG_LAYOUT_MIRRORED, false, WIDE>);
+        &k_fleet<NTV, DIAG, REC, MG_LAYOUT_MIRRORED, false, WIDE && NTV != NT_6>);
   if constexpr (DIAG) {
     if (layout == MG_LAYOUT_VECTORED)
       return reinterpret_cast<const void *>(
@@ -365,13 +386,14 @@ cudaError_t launch_fleet(const FleetView &fv, const BlockDesc *blocks, int n_blo
   }
 }
 
-cudaError_t fleet_kernel_attributes(NtVariant ntv, bool diag, int layout, bool rec,
-                                    bool wide, cudaFuncAttributes *attr) {
+cudaError_t fleet_kernel_attributes(NtVariant ntv, bool diag, int layout, bool rec, bool wide,
+                                    int n_blocks, int threads, cudaFuncAttributes *attr) {
   const void *f = nullptr;
 #define MG_PICK(N)                                                                      \
   f = diag ? (rec ? kernel_ptr<N, true, true>(layout)                               \
-                  : wide ? kernel_ptr<N, true, false, true>(layout)                 \
-                         : kernel_ptr<N, true, false>(layout))                      \
+                  : wide_kernel<N>(wide, layout, n_blocks, threads)                     \
+                      ? kernel_ptr<N, true, false, true>(layout)                        \
+                      : kernel_ptr<N, true, false>(layout))                             \
            : (rec ? kernel_ptr<N, false, true>(layout) : kernel_ptr<N, false, false>(layout));
   switch (ntv) {
     case NT_6: MG_PICK(NT_6) break;

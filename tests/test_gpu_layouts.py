@@ -139,3 +139,24 @@ def test_adjoint_of_renumbered_thrusters(which, mode):
         x, y = x.reshape(n, -1), y.reshape(n, -1)
         err = np.linalg.norm(x - y, axis=1) / np.linalg.norm(y, axis=1)
         assert err.max() <= 1e-4
+
+
+@pytest.mark.parametrize("kind", [0, 1, "mixed"])
+@pytest.mark.parametrize("over", [0, 1])  # blocks past the static grid's register-budget line
+def test_static_grid_register_budgets_give_the_same_bits(kind, over):
+    n_sm = torch.cuda.get_device_properties(0).multi_processor_count
+    n = 32 * 12 * n_sm + over
+    types = np.arange(n, dtype=np.int32) * 2 // n if kind == "mixed" else np.full(n, kind, np.int32)
+    states = []
+    for wide in (True, False):
+        sim = make_sim(types, [ROV, HEAVY])
+        sim.set_launch(32, 3, False)
+        sim.set_schedule(False, wide)
+        sim.randomize(7, 0.8, 1.2, 0.2, 0.3)
+        sim.reset()
+        sim.set_procedural_actions(11, 2)
+        for k in (1, 5):
+            sim.step(k)
+        states.append(sim.get_state())
+        sim.close()
+    assert torch.equal(*states)
