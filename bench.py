@@ -1,7 +1,7 @@
 #!/usr/bin/env python
 """Benchmark: env-steps/s of the fused persistent Fossen step on domain-randomised fleets.
 
-One benchmark step is one episode over the whole hot path: domain randomisation with the FP64
+One benchmark step is one episode over the whole hot path: domain randomisation with the
 mass-matrix inverse, reset, loading the episode's throttle schedule, 1,000 RK4 sub-steps
 (persistent kernel, 50 sub-steps per launch, replayed from one CUDA graph) and the state
 read-back.  Prints one JSON line.
@@ -31,13 +31,14 @@ METRIC = "env-steps/s at 64K envs (fused vs per-step, same GPU); p50/p99 serve l
 
 # Algorithmic FP32 work per env and sub-step of the diagonal-mass step (FMA = 2 flops, a product
 # into a zero accumulator 1), counted from the arithmetic of Eq. 1 + RK4 as the kernel performs
-# it for the vectored thruster layout (the allocation's known zeros are not multiplied): 4
-# right-hand sides without the lag derivative (6 thrusters: 223 flops each = thrust 52, R(q) 28,
-# relative velocity 18, translational rows 45, rotational rows 45, kinematics 35; 8 thrusters:
-# 237) + RK4 stage updates and combination of p, q, nu (164; the unused stage values of p are
-# not formed) + the throttle lag in its closed form (12 per thruster) + quaternion
-# renormalisation (15).
-FLOPS_PER_ENV_STEP = {6: 4 * 223 + 164 + 6 * 12 + 15, 8: 4 * 237 + 164 + 8 * 12 + 15}
+# it for a layout mirrored fore-aft and port-starboard (both vehicles': one multiplier per force
+# or moment component over sums and differences of n|n|): 4 right-hand sides without the lag
+# derivative (6 thrusters: 183 flops each = thrust sums 18, R(q) 28, relative velocity 18,
+# translational rows 45, rotational rows 39, kinematics 35; 8 thrusters: 193, of which thrust
+# sums 26 and rotational rows 41) + RK4 stage updates and combination of p, q, nu (164; the
+# unused stage values of p are not formed) + the throttle lag as a deviation from the command
+# (9 per thruster) + quaternion renormalisation (15).
+FLOPS_PER_ENV_STEP = {6: 4 * 183 + 164 + 6 * 9 + 15, 8: 4 * 193 + 164 + 8 * 9 + 15}
 # Algorithmic HBM bytes per env of one launch: state read + written ((13 + n_thr) floats each),
 # the 34 parameter floats of the diagonal-mass step, and one command row (unpadded for a fleet of
 # 6-thruster vehicles: mg_set_action_width 6).
@@ -378,7 +379,7 @@ def run_ours(args):
 
     # Each episode's parameters are drawn while the previous episode steps
     # (mg_randomize_prefetch on the library's own stream); the episode's mg_randomize installs
-    # them with one device copy.
+    # them by exchanging the two parameter buffers.
     def episode(seed, a, out):
         sim.randomize(seed, 0.8, 1.2, 0.2, 0.3, wait=False)
         sim.reset()

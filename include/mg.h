@@ -24,7 +24,8 @@
  *     mg_last_error() gives a thread-local message.  Argument errors are found on the host and
  *     change nothing.
  *   - All floating-point state and parameters are FP32 on the device.  The 6x6 mass matrix is
- *     inverted in FP64 when parameters change (mg_randomize, mg_set_params).
+ *     inverted when parameters change (mg_randomize, mg_set_params): in FP64 where it is full,
+ *     and where it is diagonal by reciprocals that round as FP64's do.
  */
 #ifndef MG_H
 #define MG_H
@@ -159,9 +160,10 @@ mg_status mg_set_launch(mg_sim *sim, int32_t envs_per_block, int32_t steps_per_l
  * warps take more units, which balances the SMs when the fleet has more 32-env slices than
  * resident warps.  wide != 0 (default) gives that kernel, and the static grid's kernel
  * outside mg_step_record, up to 200 registers per thread instead of 128 (diagonal-mass fleets;
- * the general kernels always have 168): the queue at 8 warps/SM runs best with it, and a static
- * grid of few envs (a warp per scheduler or fewer) gains 6-7 %, while a large static grid
- * keeps more warps resident at 128; warps_per_sm > 0 caps the queue kernel's resident warps
+ * the general kernels always have 168): the queue at 8 warps/SM runs best with it; a static grid
+ * of vehicles whose thrusters mirror each other fore-aft and port-starboard needs no more than 128
+ * and takes the larger budget only where it is faster (fleets with 8-thruster vehicles, while
+ * every block is resident); warps_per_sm > 0 caps the queue kernel's resident warps
  * per SM (0 = as many as fit).  work_queue = 0 (default) launches a static grid of
  * envs_per_block-env blocks per steps_per_launch sub-steps (steps_per_launch = 1: the plain
  * per-step form).  All choices give bit-identical results.  mg_step_record always uses the
@@ -178,9 +180,9 @@ mg_status mg_set_schedule(mg_sim *sim, int32_t work_queue, int32_t wide, int32_t
 mg_status mg_set_wait_limit(mg_sim *sim, uint32_t polls);
 
 /* Domain randomisation (§METHOD; §EXPERIMENTS "supports domain randomization"): per env, draws
- * from Philox4x32-10 keyed by (seed, env id + offset), then builds M = M_RB + M_A in FP64 and
- * inverts it by Cholesky.  Also records (seed, nu0_sigma) for mg_reset and zeroes every env's
- * episode counter.  Synchronous unless ranges->flags has MG_RANDOMIZE_ASYNC.  Errors: MG_EINVAL
+ * from Philox4x32-10 keyed by (seed, env id + offset), then builds M = M_RB + M_A and inverts it
+ * (FP64 Cholesky, or reciprocals where it is diagonal).  Also records (seed, nu0_sigma) for
+ * mg_reset and zeroes every env's episode counter.  Synchronous unless ranges->flags has MG_RANDOMIZE_ASYNC.  Errors: MG_EINVAL
  * (ranges NULL, lo > hi, lo <= 0, negative sigma or half-width, unknown flags, MG_RANDOMIZE_ASYNC
  * for a fleet whose mass matrices may be full), MG_ENOTSPD (parameters are stored but some mass
  * matrix has a pivot <= 0), MG_ECUDA. */
@@ -429,9 +431,9 @@ mg_status mg_task_step(mg_sim *sim, int32_t k, float *obs, float *err, uint8_t *
  * follows, writing reward = -(Eq. 4 position error) instead of err.  The schedule replaces the
  * sim's actions on the first call (and after any other action call) and is rewritten in place
  * by the later ones: by the step's one launch for k <= steps_per_launch, by a small copy kernel
- * ahead of the launches for larger k.  actions may be reused once the stream has passed the call.  obs, reward, done, episode_err: device, as
- * mg_task_step.  Asynchronous.  Errors: MG_ESTATE (no task), MG_EINVAL (k < 1, NULL, host
- * memory), MG_ENOMEM (the schedule's first allocation). */
+ * ahead of the launches for larger k.  actions may be reused once the stream has passed the call.
+ * obs, reward, done, episode_err: device, as mg_task_step.  Asynchronous.  Errors: MG_ESTATE (no
+ * task), MG_EINVAL (k < 1, NULL, host memory), MG_ENOMEM (the schedule's first allocation). */
 mg_status mg_env_step(mg_sim *sim, int32_t k, const float *actions, float *obs, float *reward,
                       uint8_t *done, float *episode_err);
 

@@ -7,16 +7,15 @@
 
 namespace mg {
 
-// Register caps: the narrow diagonal-mass step keeps 128 registers (16 resident warps per SM,
-// for the per-step form and large per-step grids; about 100 bytes of the step coefficients
-// spill to L1 at this cap); the general step keeps 168.
+// Register caps: the narrow diagonal-mass step keeps 128 registers (16 resident warps per SM, for
+// the per-step form and large per-step grids; no spills with the mirrored allocation, 40-280 bytes
+// with the others); the general step keeps 168.
 constexpr int kRegsDiag = 128;
 constexpr int kRegsGeneral = 168;
 // The wide diagonal-mass variants (mg_set_schedule's wide): the work-queue kernel runs at 8
-// warps/SM, where 256 registers per thread would fit; a 200 cap measured best (ptxas uses 181;
-// +1.7 % over 168, none at 255).  The static-grid kernel with the same cap runs small fleets
-// (one warp per scheduler or fewer, latency-bound) 6-7 % faster than at 128: the extra
-// registers let the compiler interleave more independent work.
+// warps/SM, where 256 registers per thread would fit; with the mirrored allocation ptxas uses
+// 164-178 (65,536 envs x 1,000 sub-steps: 1.29 ms; the static grid at 128 registers 1.38 ms).  The
+// static grid takes it where that pays (wide_kernel in mg_step.cu).
 constexpr int kRegsWide = 200;
 // With the off-diagonal hydrodynamics the 45 extra coefficients stay in registers too (no
 // spills up to 255; 8 resident warps per SM).

@@ -9,8 +9,8 @@
 //     the cross products.
 //   - Restoring vector from the third row of R(q): k = R^T e3, g = -[(W - B) k ; G x k],
 //     G = W r_g - B r_b.
-//   - The mass matrix M = M_RB + M_A is inverted once per parameter change (FP64 Cholesky, see
-//     mg_setup.cu); the step multiplies by the stored FP32 inverse.
+//   - The mass matrix M = M_RB + M_A is inverted once per parameter change (mg_setup.cu); the step
+//     multiplies by the stored FP32 inverse.
 #pragma once
 
 #include <type_traits>

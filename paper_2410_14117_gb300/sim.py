@@ -142,7 +142,7 @@ class Sim:
                            current_sigma: float = 0.2):
         """Draw randomize(seed, lo, hi, current_sigma) ahead, on the library's own stream, into a
         second parameter buffer (mg_randomize_prefetch); the matching randomize() call installs
-        it with one device copy.  Diagonal-mass fleets."""
+        it by exchanging it with the one in use.  Diagonal-mass fleets."""
         r = Ranges(lo, hi, current_sigma, 0.0, 0, 0.0)
         call("mg_randomize_prefetch", self._h, ctypes.c_uint64(seed), ctypes.byref(r))
 
