@@ -337,7 +337,7 @@ mg_status mg_rollout_backward(mg_sim *sim, int32_t T, int32_t C, const float *ck
 mg_status mg_set_adjoint_mode(mg_sim *sim, int32_t mode);
 
 /* State in the record layout [n][MG_NSTATE] = p(3) q(4: w,x,y,z) nu(6) n(8, zero past n_thr);
- * host or device. */
+ * host or device.  Whatever mg_set_state is given past n_thr drives nothing. */
 mg_status mg_get_state(mg_sim *sim, float *out);
 mg_status mg_set_state(mg_sim *sim, const float *in);
 

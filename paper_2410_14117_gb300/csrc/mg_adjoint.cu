@@ -617,15 +617,16 @@ struct CommandWalk {
   }
 };
 
-template <int MT>
+template <int MT, int PATH>
 __device__ __forceinline__ void load_checkpoint(const float *__restrict__ ckpt, int32_t sg,
-                                                int64_t n, int64_t e, St<MT> &S) {
+                                                int64_t n, int64_t e, int nt, St<MT> &S) {
   const float *ck = ckpt + (int64_t)sg * MG_NSTATE * n + e;
   for (int i = 0; i < 3; ++i) S.p[i] = ck[(int64_t)(i)*n];
   for (int i = 0; i < 4; ++i) S.q[i] = ck[(int64_t)(3 + i) * n];
   for (int i = 0; i < 3; ++i) S.v[i] = ck[(int64_t)(7 + i) * n];
   for (int i = 0; i < 3; ++i) S.w[i] = ck[(int64_t)(10 + i) * n];
   for (int i = 0; i < MT; ++i) S.n[i] = ck[(int64_t)(13 + i) * n];
+  drop_unused_lag<MT, true, adj_layout(PATH)>(S, nt);
 }
 
 // lam += the loss adjoint of the state after sub-step t.
@@ -836,7 +837,7 @@ __global__ void __launch_bounds__(kAdjThreads)
   for (int32_t sg = n_ck - 1; sg >= 0; --sg) {
     const int32_t t0 = sg * C, len = min(C, T - t0);
     // re-run the segment from its checkpoint
-    load_checkpoint<MT>(ckpt, sg, n, e, S[0]);
+    load_checkpoint<MT, PATH>(ckpt, sg, n, e, nt, S[0]);
     {
       CommandWalk<MT> cmd(fv, e, nt, step0 + t0);
       St<MT> x = S[0];
@@ -892,7 +893,7 @@ __device__ __forceinline__ void produce_segment(const FleetView &fv, int64_t e,
   const int64_t n = fv.n;
   const int32_t t0 = sg * C, len = min(C, T - t0);
   St<MT> S;
-  load_checkpoint<MT>(ckpt, sg, n, e, S);
+  load_checkpoint<MT, PATH>(ckpt, sg, n, e, nt, S);
   float zq[4];
   CommandWalk<MT> cmd(fv, e, nt, step0 + t0);
   for (int32_t j = 0; j < len; ++j) {
@@ -1112,6 +1113,7 @@ __global__ void __maxnreg__(XH ? kRegsXH : DIAG ? kRegsWide : kRegsGeneral)
 
   St<MT> s;
   load_state<MT>(fv.st, e, s);
+  drop_unused_lag<MT, MIXED, NH>(s, nt);
   Coef<DIAG, NH> P;
   {
     Par<DIAG> raw;

@@ -138,6 +138,17 @@ __device__ __forceinline__ void load_commands(const FleetView &fv, int64_t e, in
   for (int i = 0; i < MT; ++i) c[i] = (i < nt) ? c[i] : 0.f;
 }
 
+// Lag entries past a six-thruster vehicle's thrusters in a mixed fleet's eight-entry loop, as zero:
+// the mirrored sums add the forces of all eight (the other allocations multiply each by its own
+// direction, which is zero there), and a caller's state may hold anything in them.
+template <int MT, bool MIXED, int NH>
+__device__ __forceinline__ void drop_unused_lag(St<MT> &s, int nt) {
+  if constexpr (MIXED && MT > 6 && NH == MG_LAYOUT_MIRRORED) {
+#pragma unroll
+    for (int i = 6; i < MT; ++i) s.n[i] = i < nt ? s.n[i] : 0.f;
+  }
+}
+
 __device__ __forceinline__ void prefetch_l1(const void *p) {
   asm volatile("prefetch.global.L1 [%0];" ::"l"(p));
 }
@@ -204,6 +215,7 @@ __device__ __forceinline__ void advance_env(const FleetView &fv, int64_t e, int 
   const bool current_accel = !(fv.model_flags & MG_MODEL_NO_CURRENT_ACCEL);
 
   if constexpr (!LOADED) load_state<MT, L2>(fv.st, e, s);
+  drop_unused_lag<MT, MIXED, NH>(s, nt);
   float c[MT];
   int64_t seg;
   int32_t left;

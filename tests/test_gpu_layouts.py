@@ -160,3 +160,41 @@ def test_static_grid_register_budgets_give_the_same_bits(kind, over):
         states.append(sim.get_state())
         sim.close()
     assert torch.equal(*states)
+
+
+@pytest.mark.parametrize("general", [False, True])
+@pytest.mark.parametrize("how", ["static", "queue", "record", "task", "rollout"])
+def test_lag_entries_past_the_thrusters_push_nothing(how, general):
+    """A state whose throttle entries past a vehicle's thruster count are not zero moves as the same
+    state with zeros there: those entries belong to no thruster."""
+    n, k = 300, 12
+    types = I.mixed_fleet(4, n, max_group=60)
+    nt = np.array([(ROV, HEAVY)[t].n_thr for t in types])
+    clean = torch.tensor(I.random_states(6, n, nt), dtype=torch.float32, device="cuda")
+    dirty = clean.clone()
+    dirty[torch.tensor(nt == 6, device="cuda"), 19:] = torch.tensor([0.75, -0.5], device="cuda")
+    acts = torch.tensor(I.commands(7, 2, n, nt), device="cuda")
+    got = []
+    for start in (clean, dirty):
+        sim = make_sim(types, [ROV, HEAVY], queue=how == "queue")
+        sim.randomize(3, 0.8, 1.2, 0.2, 0.3, rg_halfwidth=0.02 if general else 0.0)
+        sim.set_state(start)
+        sim.set_actions(acts, 10)
+        if how == "record":
+            got.append([sim.step_record(k)])
+        elif how == "task":
+            sim.set_task(0, torch.zeros((n, 4), device="cuda"))
+            got.append([sim.task_step(k)[0].clone()])
+        elif how == "rollout":
+            coef = sim.get_params()[:, 4:22].clone().requires_grad_(True)
+            s = start.clone().requires_grad_(True)
+            traj = rollout(sim, coef, acts, s, 10, k, 5)
+            dc, ds = torch.autograd.grad(traj, (coef, s), torch.ones_like(traj))
+            got.append([traj.detach(), dc, ds])
+        else:
+            sim.step(k)
+            got.append([])
+        got[-1].append(sim.get_state()[:, :19])
+        sim.close()
+    for x, y in zip(*got):
+        assert torch.equal(x, y)
