@@ -256,7 +256,9 @@ mg_status mg_set_procedural_actions(mg_sim *sim, uint64_t cmd_seed, int32_t hold
  * stream; non-finite states are reported by mg_sync.  The action cursor is a word in the sim's
  * device memory: each step launch reads it when it starts and its last block advances it, so the
  * CUDA graph cached for a given k replays correctly at any cursor (one graph per distinct k, at
- * most 16 kept).  Steps of one sim must therefore stay ordered on its stream. */
+ * most 16 kept).  Steps of one sim must therefore stay ordered on its stream.  A step captured
+ * into a user's own graph keeps the path of its capture: its replays follow later parameters as
+ * long as the mass matrices stay diagonal (or full) as they were then, r_b anywhere. */
 mg_status mg_step(mg_sim *sim, int32_t k);
 
 /* Split-integration comparison step (§METHOD: the physics engine integrates the rigid-body term

@@ -37,13 +37,15 @@ namespace {
 constexpr int kAdjThreads = 128;
 
 // Which transpose a kernel is compiled for.
-enum AdjPath { ADJ_GEN = 0, ADJ_DENSE = 1, ADJ_MIRRORED = 2 };
+enum AdjPath { ADJ_GEN = 0, ADJ_DENSE = 1, ADJ_MIRRORED = 2, ADJ_MIRRORED_G = 3 };
 
 // The thruster allocation of the re-run.  Diagonal mass: the forward's (the vectored one only skips
 // exact zeros of the dense one, so the states are the forward's bit for bit).  General path: the
 // dense one, the forward's within the rounding of the thrust sums where that was mirrored.
 __host__ __device__ constexpr int adj_layout(int path) {
-  return path == ADJ_MIRRORED ? MG_LAYOUT_MIRRORED : MG_LAYOUT_DENSE;
+  return path == ADJ_MIRRORED     ? MG_LAYOUT_MIRRORED
+         : path == ADJ_MIRRORED_G ? MG_LAYOUT_MIRRORED_G
+                                  : MG_LAYOUT_DENSE;
 }
 
 // Sums over stages and sub-steps that the coefficient gradients are formed from at the end.
@@ -410,9 +412,14 @@ __device__ __forceinline__ void rhs_vjp_diag(const St<MT> &s, const float (&nud)
     ov[j] += gr[j];
     gs.v[j] = fmaf(R[0][j], gd.p[0], fmaf(R[1][j], gd.p[1], fmaf(R[2][j], gd.p[2], ov[j])));
   }
-  if constexpr (PATH == ADJ_MIRRORED) {
+  if constexpr (mirrored_sums(adj_layout(PATH))) {
     gR[2][1] = fmaf(-P.Gr, gw[0], gR[2][1]);
     gR[2][0] = fmaf(P.Gp, gw[1], gR[2][0]);
+    if constexpr (PATH == ADJ_MIRRORED_G) {
+      gR[2][0] = fmaf(-P.Gyy, gw[2], gR[2][0]);
+      gR[2][1] = fmaf(P.Gyx, gw[2], gR[2][1]);
+      gR[2][2] = fmaf(P.Gry, gw[0], fmaf(-P.Gpx, gw[1], gR[2][2]));
+    }
   } else {
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
@@ -443,7 +450,7 @@ __device__ __forceinline__ void rhs_vjp_diag(const St<MT> &s, const float (&nud)
   }
   // thrust: n|n| of each thruster into the rows
   float gf[MT];
-  if constexpr (PATH == ADJ_MIRRORED) {
+  if constexpr (mirrored_sums(adj_layout(PATH))) {
     const float gX = fmaf(P.At[0], gv[0], P.Mh * gw[1]), gY = fmaf(P.At[1], gv[1], P.Kh * gw[0]);
     const float gN = P.Nh * gw[2], gZ = P.At[2] * gv[2], gK = P.Kv * gw[0];
     const float sm = gX + gY, df = gX - gY;
@@ -1160,25 +1167,18 @@ template <int NTV>
 cudaError_t rollout_fwd_d(const FleetView &fv, const BlockDesc *blocks, int n_blocks,
                           int threads, bool diag, int layout, int32_t T, int32_t C,
                           float *traj, float *ckpt, cudaStream_t stream) {
-  constexpr int M = MG_LAYOUT_MIRRORED;
-  if (fv.xh)
-    return layout == M ? rollout_fwd_t<NTV, false, M, true>(fv, blocks, n_blocks, threads, T, C,
-                                                            traj, ckpt, stream)
-                       : rollout_fwd_t<NTV, false, 0, true>(fv, blocks, n_blocks, threads, T, C,
-                                                            traj, ckpt, stream);
-  if (diag && layout == MG_LAYOUT_MIRRORED)
-    return rollout_fwd_t<NTV, true, MG_LAYOUT_MIRRORED, false>(fv, blocks, n_blocks, threads, T, C,
-                                                               traj, ckpt, stream);
-  if (diag && layout == MG_LAYOUT_VECTORED)
-    return rollout_fwd_t<NTV, true, MG_LAYOUT_VECTORED, false>(fv, blocks, n_blocks, threads, T, C, traj, ckpt,
-                                              stream);
   if (diag)
-    return rollout_fwd_t<NTV, true, 0, false>(fv, blocks, n_blocks, threads, T, C, traj, ckpt,
-                                              stream);
-  return layout == M ? rollout_fwd_t<NTV, false, M, false>(fv, blocks, n_blocks, threads, T, C, traj,
-                                                           ckpt, stream)
-                     : rollout_fwd_t<NTV, false, 0, false>(fv, blocks, n_blocks, threads, T, C, traj,
-                                                           ckpt, stream);
+    return with_layout<true>(layout, [&](auto l) {
+      return rollout_fwd_t<NTV, true, decltype(l)::value, false>(fv, blocks, n_blocks, threads, T, C,
+                                                                 traj, ckpt, stream);
+    });
+  return with_layout<false>(layout, [&](auto l) {
+    constexpr int L = decltype(l)::value;
+    return fv.xh ? rollout_fwd_t<NTV, false, L, true>(fv, blocks, n_blocks, threads, T, C, traj, ckpt,
+                                                      stream)
+                 : rollout_fwd_t<NTV, false, L, false>(fv, blocks, n_blocks, threads, T, C, traj,
+                                                       ckpt, stream);
+  });
 }
 
 }  // namespace
@@ -1247,14 +1247,14 @@ cudaError_t launch_adjoint(const FleetView &fv, const int32_t *types, bool eight
     return launch(fv, types, ckpt, dtraj, T, C, step0, dcoef, dact, dstate0, split, ws, n_sm,
                   stream);
   };
-  const int path = general ? ADJ_GEN : layout == MG_LAYOUT_MIRRORED ? ADJ_MIRRORED : ADJ_DENSE;
-  if (eight)
-    return path == ADJ_GEN     ? run(launch_adjoint_t<8, ADJ_GEN>)
-           : path == ADJ_DENSE ? run(launch_adjoint_t<8, ADJ_DENSE>)
-                               : run(launch_adjoint_t<8, ADJ_MIRRORED>);
-  return path == ADJ_GEN     ? run(launch_adjoint_t<6, ADJ_GEN>)
-         : path == ADJ_DENSE ? run(launch_adjoint_t<6, ADJ_DENSE>)
-                             : run(launch_adjoint_t<6, ADJ_MIRRORED>);
+  auto on_path = [&](auto p) {
+    return eight ? run(launch_adjoint_t<8, decltype(p)::value>)
+                 : run(launch_adjoint_t<6, decltype(p)::value>);
+  };
+  if (general) return on_path(std::integral_constant<int, ADJ_GEN>());
+  if (layout == MG_LAYOUT_MIRRORED) return on_path(std::integral_constant<int, ADJ_MIRRORED>());
+  if (layout == MG_LAYOUT_MIRRORED_G) return on_path(std::integral_constant<int, ADJ_MIRRORED_G>());
+  return on_path(std::integral_constant<int, ADJ_DENSE>());
 }
 
 int adjoint_max_interval() { return kMaxSeg; }

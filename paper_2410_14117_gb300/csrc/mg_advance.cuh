@@ -43,6 +43,19 @@ __device__ __forceinline__ void finish_launch(const FleetView &fv, int32_t k) {
   }
 }
 
+// f(std::integral_constant<int, L>()) for the allocation `layout`: those the diagonal-mass kernels
+// are compiled for, or the general ones (dense, mirrored).
+template <bool DIAG, typename F>
+auto with_layout(int layout, F f) {
+  if (layout == MG_LAYOUT_MIRRORED) return f(std::integral_constant<int, MG_LAYOUT_MIRRORED>());
+  if constexpr (DIAG) {
+    if (layout == MG_LAYOUT_MIRRORED_G)
+      return f(std::integral_constant<int, MG_LAYOUT_MIRRORED_G>());
+    if (layout == MG_LAYOUT_VECTORED) return f(std::integral_constant<int, MG_LAYOUT_VECTORED>());
+  }
+  return f(std::integral_constant<int, MG_LAYOUT_DENSE>());
+}
+
 // The cursor a static-grid step launch starts at: 0 when the launch carries a rewind that the device
 // has not seen (rewinding is then true), else the device's word.
 __device__ __forceinline__ int64_t start_cursor(const FleetView &fv, bool &rewinding) {
@@ -143,7 +156,7 @@ __device__ __forceinline__ void load_commands(const FleetView &fv, int64_t e, in
 // direction, which is zero there), and a caller's state may hold anything in them.
 template <int MT, bool MIXED, int NH>
 __device__ __forceinline__ void drop_unused_lag(St<MT> &s, int nt) {
-  if constexpr (MIXED && MT > 6 && NH == MG_LAYOUT_MIRRORED) {
+  if constexpr (MIXED && MT > 6 && mirrored_sums(NH)) {
 #pragma unroll
     for (int i = 6; i < MT; ++i) s.n[i] = i < nt ? s.n[i] : 0.f;
   }

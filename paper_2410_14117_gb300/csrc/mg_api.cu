@@ -58,7 +58,8 @@ bool mg::mirrored_layout(const Geo &g) {
 }
 
 int mg::thruster_layout(const Geo &g, const mg_vehicle_params &v) {
-  if (mirrored_layout(g) && v.rb[0] == 0.f && v.rb[1] == 0.f) return MG_LAYOUT_MIRRORED;
+  if (mirrored_layout(g))
+    return v.rb[0] == 0.f && v.rb[1] == 0.f ? MG_LAYOUT_MIRRORED : MG_LAYOUT_MIRRORED_G;
   return vectored_layout(g) ? MG_LAYOUT_VECTORED : MG_LAYOUT_DENSE;
 }
 
@@ -101,6 +102,7 @@ struct GraphEntry {
   int32_t k;
   const float *act_src;
   const char *par;  // the parameter range the kernels read (mg_randomize_prefetch exchanges two)
+  int layout;       // launch_layout()
   int32_t n_seg, hold, proc;
   uint64_t cmd_seed;
   cudaGraphExec_t exec;
@@ -123,8 +125,8 @@ struct mg_sim {
   bool diag = true;
   // Thruster allocation (MG_LAYOUT_*): the diagonal-mass step's by the geometry and nominal r_b of
   // the types present (mirrored: by the geometry alone, the general path's), and the one in use,
-  // which for a diagonal mass is the vectored one at most while some env's r_b is off the z axis
-  // (mg_set_params).
+  // which for a diagonal mass is the mirrored one of any r_b at most while some env's is off the z
+  // axis (mg_set_params).
   bool mirrored = true;
   int type_layout = MG_LAYOUT_DENSE;
   int layout = MG_LAYOUT_DENSE;
@@ -208,6 +210,7 @@ struct mg_sim {
   bool rewind_pending = false;
   uint32_t rewind_gen = 0;
   bool captured = false;
+  bool in_capture = false;  // being captured, as of the last capturing()
 
   // knobs
   int32_t epb = 128, spl = 50;
@@ -320,6 +323,13 @@ struct mg_sim {
     move(pa.g0); move(pa.g1); move(pa.g2); move(pa.g3); move(pa.g4); move(pa.g5);
   }
 
+  // The allocation of a launch: while the stream is captured into a user's graph, one that stays
+  // right when mg_set_params later moves r_b off the z axis (the library's own graphs are dropped
+  // then, the user's are not).  Same bits as `layout` while r_b is on it.
+  int launch_layout() const {
+    return in_capture && diag ? std::min<int>(layout, MG_LAYOUT_MIRRORED_G) : layout;
+  }
+
   // setup_view() on the range not in use, with its own check words
   SetupView staged_setup_view() const {
     SetupView v = setup_view();
@@ -405,7 +415,7 @@ mg_status launch_chunks(mg_sim *s, int32_t k, float *traj, cudaStream_t stream) 
   FleetView v = s->view();
   if (s->queue && !traj) {
     v.cursor_adv = k;
-    MG_CK(launch_fleet_queue(v, s->slices_d, s->n_slices, s->ntv, s->diag, s->layout,
+    MG_CK(launch_fleet_queue(v, s->slices_d, s->n_slices, s->ntv, s->diag, s->launch_layout(),
                              s->wide, s->queue_warps_per_sm, k, s->spl, s->sched, s->n_sm,
                              stream));
     return MG_OK;
@@ -415,7 +425,7 @@ mg_status launch_chunks(mg_sim *s, int32_t k, float *traj, cudaStream_t stream) 
     float *t = traj ? traj + (int64_t)done * MG_NTRAJ * s->n : nullptr;
     v.cursor_off = done;
     v.cursor_adv = (done + kk == k) ? k : 0;
-    MG_CK(launch_fleet(v, s->blocks_d, s->n_blocks, s->threads, s->ntv, s->diag, s->layout,
+    MG_CK(launch_fleet(v, s->blocks_d, s->n_blocks, s->threads, s->ntv, s->diag, s->launch_layout(),
                        s->wide, kk, t, stream));
     done += kk;
   }
@@ -468,7 +478,7 @@ void set_mass_diag(mg_sim *s, bool mass_diag, bool on_axis) {
   const bool diag = mass_diag && !(s->model_flags & MG_MODEL_NO_CURRENT_ACCEL);
   const int layout = !diag     ? (s->mirrored ? MG_LAYOUT_MIRRORED : MG_LAYOUT_DENSE)
                      : on_axis ? s->type_layout
-                               : std::min<int>(s->type_layout, MG_LAYOUT_VECTORED);
+                               : std::min<int>(s->type_layout, MG_LAYOUT_MIRRORED_G);
   if (diag != s->diag || layout != s->layout) s->drop_graphs();
   s->diag = diag;
   s->layout = layout;
@@ -495,8 +505,9 @@ mg_status finish_params(mg_sim *s) {
 bool capturing(mg_sim *s) {
   cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing(s->stream, &st) != cudaSuccess) cudaGetLastError();
-  if (st != cudaStreamCaptureStatusNone) s->captured = true;
-  return st != cudaStreamCaptureStatusNone;
+  s->in_capture = st != cudaStreamCaptureStatusNone;
+  s->captured = s->captured || s->in_capture;
+  return s->in_capture;
 }
 
 cudaError_t apply_rewind(mg_sim *s, bool always) {
@@ -601,7 +612,7 @@ mg_status mg_step_noalloc(mg_sim *s, int32_t k) {
   if ((st = settle_cursor(s)) != MG_OK) return st;
   FleetView v = s->view();
   v.cursor_adv = k;
-  MG_CK(launch_fleet_queue(v, s->slices_d, s->n_slices, s->ntv, s->diag, s->layout,
+  MG_CK(launch_fleet_queue(v, s->slices_d, s->n_slices, s->ntv, s->diag, s->launch_layout(),
                            s->wide, s->queue_warps_per_sm, k, s->spl, sched, s->n_sm,
                            s->stream));
   s->cursor += k;
@@ -1201,8 +1212,8 @@ mg_status mg_step(mg_sim *s, int32_t k) {
     FleetView v = s->view();
     v.cursor_adv = k;
     v.rewind = s->rewind_pending ? s->rewind_gen : 0;
-    MG_CK(launch_fleet(v, s->blocks_d, s->n_blocks, s->threads, s->ntv, s->diag, s->layout, s->wide,
-                       k, nullptr, s->stream));
+    MG_CK(launch_fleet(v, s->blocks_d, s->n_blocks, s->threads, s->ntv, s->diag, s->launch_layout(),
+                       s->wide, k, nullptr, s->stream));
     if (!cap) s->rewind_pending = false;
     s->cursor += k;
     return MG_OK;
@@ -1218,8 +1229,8 @@ mg_status mg_step(mg_sim *s, int32_t k) {
   const float *src = s->proc ? nullptr : s->act_src;
   const uint64_t seed = s->proc ? s->cmd_seed : 0;
   for (auto &g : s->graphs)
-    if (g.k == k && g.act_src == src && g.par == s->par && g.n_seg == s->n_seg && g.hold == s->hold &&
-        g.proc == s->proc && g.cmd_seed == seed)
+    if (g.k == k && g.act_src == src && g.par == s->par && g.layout == s->launch_layout() &&
+        g.n_seg == s->n_seg && g.hold == s->hold && g.proc == s->proc && g.cmd_seed == seed)
       hit = &g;
   if (!hit) {
     if (s->graphs.size() >= 16) {
@@ -1239,7 +1250,7 @@ mg_status mg_step(mg_sim *s, int32_t k) {
       return st;
     }
     MG_CK(ce);
-    GraphEntry g{k, src, s->par, s->n_seg, s->hold, s->proc, seed, nullptr, 0};
+    GraphEntry g{k, src, s->par, s->launch_layout(), s->n_seg, s->hold, s->proc, seed, nullptr, 0};
     ce = cudaGraphInstantiate(&g.exec, graph, 0);
     cudaGraphDestroy(graph);
     MG_CK(ce);
@@ -1303,7 +1314,7 @@ mg_status mg_rollout_forward(mg_sim *s, int32_t T, int32_t C, float *traj, float
   v.cursor_off = 0;
   v.cursor_adv = T;
   MG_CK(launch_rollout_forward(v, s->blocks_d, s->n_blocks, s->threads, s->ntv, s->diag,
-                               s->layout, T, C, traj, ckpt, s->stream));
+                               s->launch_layout(), T, C, traj, ckpt, s->stream));
   s->cursor += T;
   if (step0_out) *step0_out = step0;
   return MG_OK;
@@ -1346,7 +1357,7 @@ mg_status mg_rollout_backward(mg_sim *s, int32_t T, int32_t C, const float *ckpt
       }
     }
   }
-  MG_CK(launch_adjoint(s->view(), s->types_d, eight, general, s->layout, ckpt, dtraj,
+  MG_CK(launch_adjoint(s->view(), s->types_d, eight, general, s->launch_layout(), ckpt, dtraj,
                        T, C, step0, dcoef, dact, dstate0, split, s->adj_ws, s->stream));
   return MG_OK;
 }
@@ -1428,7 +1439,7 @@ mg_status task_step_outputs(mg_sim *s, int32_t k, float *obs, float *err, float 
   FleetView v = s->view();
   v.cursor_adv = k_last;
   MG_CK(launch_fleet_task(v, s->blocks_d, s->n_blocks, s->threads, s->ntv, s->diag,
-                          s->layout, k_last, k, s->task_view(), to, s->stream));
+                          s->launch_layout(), k_last, k, s->task_view(), to, s->stream));
   s->cursor += k_last;
   return MG_OK;
 }

@@ -216,17 +216,40 @@ struct StepMirrored {
 //                       the verticals' d_z (+ +), arm_x (- + [- +]), arm_y (- - [+ +]; zero with
 //                       two verticals).  Every such frame with the centres on the z axis, which is
 //                       what the vehicles of the experiments are.
+//   MG_LAYOUT_MIRRORED_G  the same with r_b anywhere (diagonal mass only): the four products of G_x
+//                       and G_y follow in their chains, so that the results are
+//                       MG_LAYOUT_MIRRORED's bit for bit where those are zero.  Taken while some
+//                       r_b is off the axis, and by launches captured into a user's graph, whose
+//                       replays may come after such parameters were set.
 // Vectored against mirrored, CUDA events: 65,536 six-thruster envs x 1,000 sub-steps on the work
 // queue 1.69 -> 1.40 ms; 262,144 mixed envs x 500 on the static grid 3.38 -> 2.85 ms; no spills at
 // 128 registers (vectored: about 100 bytes with six thrusters, 200 with eight), so 65,536-env
 // environment steps of 10 sub-steps 40.7 -> 28.7 us and 30,000 recorded 8-thruster envs x 200
 // 413 -> 283 us.
-enum : int { MG_LAYOUT_DENSE = 0, MG_LAYOUT_VECTORED = 4, MG_LAYOUT_MIRRORED = 5 };
+enum : int {
+  MG_LAYOUT_DENSE = 0, MG_LAYOUT_VECTORED = 4, MG_LAYOUT_MIRRORED_G = 5, MG_LAYOUT_MIRRORED = 6
+};
+__host__ __device__ constexpr bool mirrored_sums(int layout) {
+  return layout >= MG_LAYOUT_MIRRORED_G;
+}
 
-__device__ __forceinline__ StepMirrored step_mirrored(const ParDiag &P, const float4 *gdir,
-                                                      const float4 *garm) {
+// MG_LAYOUT_MIRRORED_G: and mi G_y of the roll row, mi G_x of the pitch row, mi G_x and mi G_y of the
+// yaw row.
+struct StepMirroredG : StepMirrored {
+  float Gry, Gpx, Gyx, Gyy;
+};
+
+template <int NH>
+__device__ __forceinline__ auto step_mirrored(const ParDiag &P, const float4 *gdir,
+                                              const float4 *garm) {
   const StepDiag D = step_diag(P);
-  StepMirrored C;
+  typename std::conditional<NH == MG_LAYOUT_MIRRORED_G, StepMirroredG, StepMirrored>::type C;
+  if constexpr (NH == MG_LAYOUT_MIRRORED_G) {
+    C.Gry = D.Gp[0];
+    C.Gpx = D.Gm[1];
+    C.Gyx = D.Gp[2];
+    C.Gyy = D.Gm[2];
+  }
   const float d[3] = {gdir[0].x, gdir[0].y, gdir[4].z};
 #pragma unroll
   for (int i = 0; i < 3; ++i) {
@@ -278,13 +301,16 @@ __device__ __forceinline__ ParGenMirrored gen_mirrored(const ParGen &P, const fl
 // parameters as loaded (with the mirrored frame's weights).
 template <bool DIAG, int NH = MG_LAYOUT_DENSE>
 using Coef = typename std::conditional<
-    DIAG, typename std::conditional<NH == MG_LAYOUT_MIRRORED, StepMirrored, StepDiag>::type,
+    DIAG,
+    typename std::conditional<
+        NH == MG_LAYOUT_MIRRORED, StepMirrored,
+        typename std::conditional<NH == MG_LAYOUT_MIRRORED_G, StepMirroredG, StepDiag>::type>::type,
     typename std::conditional<NH == MG_LAYOUT_MIRRORED, ParGenMirrored, ParGen>::type>::type;
 
 template <bool DIAG, int NH = MG_LAYOUT_DENSE>
 __device__ __forceinline__ Coef<DIAG, NH> make_coef(const Par<DIAG> &P, const float4 *gdir,
                                                     const float4 *garm) {
-  if constexpr (DIAG && NH == MG_LAYOUT_MIRRORED) return step_mirrored(P, gdir, garm);
+  if constexpr (DIAG && mirrored_sums(NH)) return step_mirrored<NH>(P, gdir, garm);
   else if constexpr (DIAG) return step_diag(P);
   else if constexpr (NH == MG_LAYOUT_MIRRORED) return gen_mirrored(P, gdir, garm);
   else return P;
@@ -380,7 +406,7 @@ __device__ __forceinline__ void rhs(const St<MT> &s, const Coef<DIAG, NH> &P,
                                     const float *__restrict__ xh = nullptr) {
   static_assert(!(XH && DIAG), "the off-diagonal hydrodynamics use the general path");
   // Thrusters (Eq. 3 actions): F_i = kT n_i|n_i| along d_i at r_i.
-  constexpr bool MIRRORED = NH == MG_LAYOUT_MIRRORED;
+  constexpr bool MIRRORED = mirrored_sums(NH);
   float t0 = 0.f, t1 = 0.f, t2 = 0.f, t3 = 0.f, t4 = 0.f, t5 = 0.f;
   if constexpr (MIRRORED) {
     auto f = [&](int i) { return s.n[i] * fabsf(s.n[i]); };
@@ -457,11 +483,17 @@ __device__ __forceinline__ void rhs(const St<MT> &s, const Coef<DIAG, NH> &P,
     {
       float b0, b1, b2;
       if constexpr (MIRRORED) {
-        b0 = fmaf(-P.Gr, R21, fmaf(P.Kv, t3, P.Kh * t1));
+        b0 = fmaf(P.Kv, t3, P.Kh * t1);
+        if constexpr (NH == MG_LAYOUT_MIRRORED_G) b0 = fmaf(P.Gry, R22, b0);
+        b0 = fmaf(-P.Gr, R21, b0);
         b1 = P.Mh * t0;
         if constexpr (MT > 6) b1 = fmaf(P.Mv, t4, b1);
         b1 = fmaf(P.Gp, R20, b1);
         b2 = P.Nh * t5;
+        if constexpr (NH == MG_LAYOUT_MIRRORED_G) {
+          b1 = fmaf(-P.Gpx, R22, b1);
+          b2 = fmaf(-P.Gyy, R20, fmaf(P.Gyx, R21, b2));
+        }
       } else {
         b0 = fmaf(-P.Gm[0], R21, fmaf(P.Gp[0], R22, P.Ar[0] * t3));
         b1 = fmaf(-P.Gm[1], R22, fmaf(P.Gp[1], R20, P.Ar[1] * t4));

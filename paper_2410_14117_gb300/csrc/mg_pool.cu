@@ -129,12 +129,9 @@ void launch_serve(bool wide, int grid, const FleetView &v, const JobDesc *jobs,
 
 void launch_serve_diag(int layout, bool wide, int grid, const FleetView &v, const JobDesc *jobs,
                        const ServeBlock *blocks, cudaStream_t stream) {
-  if (layout == MG_LAYOUT_MIRRORED)
-    launch_serve<MG_LAYOUT_MIRRORED>(wide, grid, v, jobs, blocks, stream);
-  else if (layout == MG_LAYOUT_VECTORED)
-    launch_serve<MG_LAYOUT_VECTORED>(wide, grid, v, jobs, blocks, stream);
-  else
-    launch_serve<MG_LAYOUT_DENSE>(wide, grid, v, jobs, blocks, stream);
+  with_layout<true>(layout, [&](auto l) {
+    launch_serve<decltype(l)::value>(wide, grid, v, jobs, blocks, stream);
+  });
 }
 
 }  // namespace

@@ -184,26 +184,16 @@ cudaError_t launch_pdl(Kernel kernel, int n_blocks, int threads, size_t smem, cu
 template <int NTV, bool DIAG, bool REC, bool WIDE>
 cudaError_t launch_t(const FleetView &fv, const BlockDesc *blocks, int n_blocks, int threads,
                      int layout, int32_t k, float *traj, cudaStream_t stream) {
-  if constexpr (!DIAG)
-    if (fv.xh) {
-      const size_t smem = sizeof(float) * MG_NXPARAM * threads;
-      if (layout == MG_LAYOUT_MIRRORED)
-        return launch_pdl(k_fleet<NTV, false, REC, MG_LAYOUT_MIRRORED, true>, n_blocks, threads, smem,
-                          stream, fv, blocks, k, traj);
-      return launch_pdl(k_fleet<NTV, false, REC, 0, true>, n_blocks, threads, smem, stream, fv,
-                        blocks, k, traj);
-    }
-  constexpr bool MWIDE = WIDE && NTV != NT_6;  // wide_kernel
-  if (layout == MG_LAYOUT_MIRRORED)
-    return launch_pdl(k_fleet<NTV, DIAG, REC, MG_LAYOUT_MIRRORED, false, MWIDE>, n_blocks, threads,
-                      0, stream, fv, blocks, k, traj);
-  if constexpr (DIAG) {
-    if (layout == MG_LAYOUT_VECTORED)
-      return launch_pdl(k_fleet<NTV, true, REC, MG_LAYOUT_VECTORED, false, WIDE>, n_blocks, threads,
-                        0, stream, fv, blocks, k, traj);
-  }
-  return launch_pdl(k_fleet<NTV, DIAG, REC, 0, false, WIDE>, n_blocks, threads, 0, stream, fv,
-                    blocks, k, traj);
+  return with_layout<DIAG>(layout, [&](auto l) {
+    constexpr int L = decltype(l)::value;
+    if constexpr (!DIAG)
+      if (fv.xh)
+        return launch_pdl(k_fleet<NTV, false, REC, L, true>, n_blocks, threads,
+                          sizeof(float) * MG_NXPARAM * threads, stream, fv, blocks, k, traj);
+    constexpr bool W = WIDE && !(mirrored_sums(L) && NTV == NT_6);  // wide_kernel
+    return launch_pdl(k_fleet<NTV, DIAG, REC, L, false, W>, n_blocks, threads, 0, stream, fv,
+                      blocks, k, traj);
+  });
 }
 
 // Whether the static grid takes the 200-register kernel.  The mirrored allocation fits 128 registers
@@ -214,7 +204,7 @@ cudaError_t launch_t(const FleetView &fv, const BlockDesc *blocks, int n_blocks,
 // against 246).  The other allocations spill at 128.
 template <int NTV>
 bool wide_kernel(bool wide, int layout, int n_blocks, int threads) {
-  if (!wide || layout != MG_LAYOUT_MIRRORED) return wide;
+  if (!wide || !mirrored_sums(layout)) return wide;
   int dev = 0, n_sm = 0;
   return NTV != NT_6 && cudaGetDevice(&dev) == cudaSuccess &&
          cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess &&
@@ -247,36 +237,22 @@ cudaError_t launch_d(const FleetView &fv, const BlockDesc *blocks, int n_blocks,
 
 template <int NTV, bool DIAG, bool REC, bool WIDE = false>
 const void *kernel_ptr(int layout) {
-  if (layout == MG_LAYOUT_MIRRORED)
+  return with_layout<DIAG>(layout, [](auto l) {
+    constexpr int L = decltype(l)::value;
     return reinterpret_cast<const void *>(
-        &k_fleet<NTV, DIAG, REC, MG_LAYOUT_MIRRORED, false, WIDE && NTV != NT_6>);
-  if constexpr (DIAG) {
-    if (layout == MG_LAYOUT_VECTORED)
-      return reinterpret_cast<const void *>(
-          &k_fleet<NTV, true, REC, MG_LAYOUT_VECTORED, false, WIDE>);
-  }
-  return reinterpret_cast<const void *>(&k_fleet<NTV, DIAG, REC, 0, false, WIDE>);
+        &k_fleet<NTV, DIAG, REC, L, false, WIDE && !(mirrored_sums(L) && NTV == NT_6)>);
+  });
 }
 
 template <int NTV, bool DIAG>
 const void *queue_ptr(bool wide, int layout, bool xh) {
-  constexpr int S = DIAG ? 4 : 0;
-  constexpr int M = MG_LAYOUT_MIRRORED, V = MG_LAYOUT_VECTORED;
-  if constexpr (!DIAG)
-    if (xh)
-      return layout == M
-                 ? reinterpret_cast<const void *>(&k_fleet_queue<NTV, false, false, M, true>)
-                 : reinterpret_cast<const void *>(&k_fleet_queue<NTV, false, false, 0, true>);
-  if (layout == M)
-    return wide ? reinterpret_cast<const void *>(&k_fleet_queue<NTV, DIAG, true, M>)
-                : reinterpret_cast<const void *>(&k_fleet_queue<NTV, DIAG, false, M>);
-  if constexpr (DIAG) {
-    if (layout == V)
-      return wide ? reinterpret_cast<const void *>(&k_fleet_queue<NTV, true, true, V>)
-                  : reinterpret_cast<const void *>(&k_fleet_queue<NTV, true, false, V>);
-  }
-  return wide ? reinterpret_cast<const void *>(&k_fleet_queue<NTV, DIAG, true, 0>)
-              : reinterpret_cast<const void *>(&k_fleet_queue<NTV, DIAG, false, 0>);
+  return with_layout<DIAG>(layout, [&](auto l) {
+    constexpr int L = decltype(l)::value;
+    if constexpr (!DIAG)
+      if (xh) return reinterpret_cast<const void *>(&k_fleet_queue<NTV, false, false, L, true>);
+    return wide ? reinterpret_cast<const void *>(&k_fleet_queue<NTV, DIAG, true, L>)
+                : reinterpret_cast<const void *>(&k_fleet_queue<NTV, DIAG, false, L>);
+  });
 }
 
 const void *queue_kernel(NtVariant ntv, bool diag, bool wide, int layout, bool xh) {
@@ -348,21 +324,16 @@ template <int NTV>
 void queue_launch(bool diag, bool wide, int layout, int grid, size_t smem, const FleetView &fv,
                   const BlockDesc *slices, int32_t n_slices, int32_t k, int32_t chunk,
                   uint32_t *sched, cudaStream_t stream) {
-  if (diag && layout == MG_LAYOUT_MIRRORED)
-    queue_launch_w<NTV, true, MG_LAYOUT_MIRRORED>(wide, grid, smem, fv, slices, n_slices, k, chunk,
-                                                  sched, stream);
-  else if (diag && layout == MG_LAYOUT_VECTORED)
-    queue_launch_w<NTV, true, MG_LAYOUT_VECTORED>(wide, grid, smem, fv, slices, n_slices, k, chunk,
-                                                  sched, stream);
-  else if (diag)
-    queue_launch_w<NTV, true, MG_LAYOUT_DENSE>(wide, grid, smem, fv, slices, n_slices, k, chunk, sched,
-                                               stream);
-  else if (layout == MG_LAYOUT_MIRRORED)
-    queue_launch_w<NTV, false, MG_LAYOUT_MIRRORED>(wide, grid, smem, fv, slices, n_slices, k, chunk,
-                                                   sched, stream);
+  if (diag)
+    with_layout<true>(layout, [&](auto l) {
+      queue_launch_w<NTV, true, decltype(l)::value>(wide, grid, smem, fv, slices, n_slices, k, chunk,
+                                                    sched, stream);
+    });
   else
-    queue_launch_w<NTV, false, 0>(wide, grid, smem, fv, slices, n_slices, k, chunk, sched,
-                                               stream);
+    with_layout<false>(layout, [&](auto l) {
+      queue_launch_w<NTV, false, decltype(l)::value>(wide, grid, smem, fv, slices, n_slices, k,
+                                                     chunk, sched, stream);
+    });
 }
 
 }  // namespace

@@ -368,25 +368,18 @@ cudaError_t fleet_task_d(const FleetView &fv, const BlockDesc *blocks, int n_blo
                          bool diag, int layout, int32_t k_launch, int32_t k_task,
                          const TaskView &tv, const TaskOut &to, size_t smem,
                          cudaStream_t stream) {
-  constexpr int M = MG_LAYOUT_MIRRORED;
-  if (fv.xh)
-    return layout == M ? fleet_task_t<NTV, false, M, true>(fv, blocks, n_blocks, threads, k_launch,
-                                                           k_task, tv, to, smem, stream)
-                       : fleet_task_t<NTV, false, 0, true>(fv, blocks, n_blocks, threads, k_launch,
-                                                           k_task, tv, to, smem, stream);
-  if (diag && layout == MG_LAYOUT_MIRRORED)
-    return fleet_task_t<NTV, true, MG_LAYOUT_MIRRORED>(fv, blocks, n_blocks, threads, k_launch,
-                                                       k_task, tv, to, smem, stream);
-  if (diag && layout == MG_LAYOUT_VECTORED)
-    return fleet_task_t<NTV, true, MG_LAYOUT_VECTORED>(fv, blocks, n_blocks, threads, k_launch,
-                                                       k_task, tv, to, smem, stream);
   if (diag)
-    return fleet_task_t<NTV, true, 0>(fv, blocks, n_blocks, threads, k_launch, k_task, tv, to,
-                                      smem, stream);
-  return layout == M ? fleet_task_t<NTV, false, M>(fv, blocks, n_blocks, threads, k_launch, k_task,
-                                                   tv, to, smem, stream)
-                     : fleet_task_t<NTV, false, 0>(fv, blocks, n_blocks, threads, k_launch, k_task,
-                                                   tv, to, smem, stream);
+    return with_layout<true>(layout, [&](auto l) {
+      return fleet_task_t<NTV, true, decltype(l)::value>(fv, blocks, n_blocks, threads, k_launch,
+                                                         k_task, tv, to, smem, stream);
+    });
+  return with_layout<false>(layout, [&](auto l) {
+    constexpr int L = decltype(l)::value;
+    return fv.xh ? fleet_task_t<NTV, false, L, true>(fv, blocks, n_blocks, threads, k_launch, k_task,
+                                                     tv, to, smem, stream)
+                 : fleet_task_t<NTV, false, L>(fv, blocks, n_blocks, threads, k_launch, k_task, tv,
+                                               to, smem, stream);
+  });
 }
 
 __global__ void k_clamp_actions(const float *__restrict__ in, float *__restrict__ out,
