@@ -977,10 +977,11 @@ mg_status mg_randomize(mg_sim *s, uint64_t seed, const mg_ranges *r) {
   if (async && !diagonal_by_construction(s, r))
     return fail(MG_EINVAL, "MG_RANDOMIZE_ASYNC needs mass matrices known to be diagonal "
                            "(r_g = 0 for every type, rg_halfwidth = 0, no extension)");
+  capturing(s);  // a user's graph then draws into, or installs over, this parameter range
   if (staged_matches(s, seed, r)) {
     // install the background draw and its two check words
     MG_CK(cudaStreamWaitEvent(s->stream, s->pf_done, 0));
-    if (capturing(s) || s->captured) {
+    if (s->captured) {
       MG_CK(cudaMemcpyAsync(s->par, s->pf_buf, s->par_bytes, cudaMemcpyDeviceToDevice, s->stream));
     } else {
       mg_sim::rebase(s->pa, s->raw, s->par, s->pf_buf);
@@ -1001,7 +1002,8 @@ mg_status mg_randomize(mg_sim *s, uint64_t seed, const mg_ranges *r) {
   s->reset_seed = seed;
   s->nu0_sigma = (double)r->nu0_sigma;
   if (async) {  // diagonal by construction; a pivot <= 0 is left to mg_sync
-    set_mass_diag(s, true, s->nominal_on_axis);
+    // captured, the draw runs with a replay: an r_b off the axis is still in use until then
+    set_mass_diag(s, true, s->nominal_on_axis && (s->on_axis || !s->in_capture));
     return MG_OK;
   }
   return finish_params(s);

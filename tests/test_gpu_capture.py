@@ -125,3 +125,68 @@ def test_captured_step_follows_buoyancy_off_the_axis(how, kind):
                 assert rel_err(got, ref).max() <= TOL_STEP * T
         for sim in sims:
             sim.close()
+
+
+@pytest.mark.parametrize("also_step", [False, True])
+def test_captured_draw_writes_the_parameters_in_use(also_step):
+    """randomize(wait=False) and reset() in a user's graph; prefetched draws installed outside it
+    before and after; each replay redraws what the next step reads."""
+    vs = vehicles()
+    s = torch.cuda.Stream()
+    with torch.cuda.stream(s):
+        a, b = (Sim(N, np.zeros(N, np.int32), vs, stream=s) for _ in range(2))
+        for sim in (a, b):
+            sim.randomize(1)
+            sim.set_procedural_actions(7, HOLD)
+
+        def draw(sim):
+            sim.randomize(5, wait=False)
+            sim.reset()
+            if also_step:
+                sim.step(3)
+        g = _capture(s, lambda: draw(a))
+        for ep in range(4):
+            a.randomize_prefetch(50 + ep)
+            for sim in (a, b):
+                sim.randomize(50 + ep, wait=False)
+                sim.reset()
+                sim.step(11)
+            assert torch.equal(a.get_params(), b.get_params()), ep
+            assert torch.equal(a.get_state(), b.get_state()), ep
+            if ep % 2:
+                a.randomize_prefetch(70 + ep)  # drawn beside the replay, installed later
+            g.replay()
+            draw(b)
+            for sim in (a, b):
+                sim.step(9)
+            assert torch.equal(a.get_params(), b.get_params()), ep
+            assert torch.equal(a.get_state(), b.get_state()), ep
+            if ep % 2:
+                for sim in (a, b):
+                    sim.randomize(70 + ep, wait=False)
+                assert torch.equal(a.get_params(), b.get_params()), ep
+        a.close()
+        b.close()
+
+
+def test_parameters_off_the_axis_stay_in_use_until_a_captured_draw_is_replayed():
+    vs = vehicles()
+    off = I.perturbed_params(5, oracle_nominal(vs)[np.zeros(N, int)], N)
+    off[:, I.P_RB] = 0.015625
+    s = torch.cuda.Stream()
+    with torch.cuda.stream(s):
+        a, b = (Sim(N, np.zeros(N, np.int32), vs, stream=s) for _ in range(2))
+        for sim in (a, b):
+            sim.set_procedural_actions(7, HOLD)
+            sim.set_params(torch.tensor(off, dtype=torch.float32, device="cuda"))
+        g = _capture(s, lambda: a.randomize(5, wait=False))
+        for sim in (a, b):
+            sim.step(T)
+        assert torch.equal(a.get_state(), b.get_state())
+        g.replay()
+        b.randomize(5, wait=False)
+        for sim in (a, b):
+            sim.step(T)
+        assert torch.equal(a.get_state(), b.get_state())
+        a.close()
+        b.close()
