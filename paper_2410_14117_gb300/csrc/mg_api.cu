@@ -158,6 +158,7 @@ struct mg_sim {
   int32_t adj_mode = 0;
   float *adj_ws = nullptr;
   size_t adj_ws_cap = 0;
+  std::vector<float *> adj_ws_old;  // outgrown, but a user's graph may write them
   // the parameter range in use (derived planes, then the raw records): one contiguous span, the
   // arena's until an install exchanges it
   char *par = nullptr;
@@ -828,6 +829,7 @@ mg_status mg_destroy(mg_sim *s) {
   cudaFree(s->xh);
   cudaFree(s->env_act);
   cudaFree(s->adj_ws);
+  for (float *p : s->adj_ws_old) cudaFree(p);
   cudaFree(s->arena);
   delete s;
   return MG_OK;
@@ -1322,6 +1324,30 @@ mg_status mg_rollout_forward(mg_sim *s, int32_t T, int32_t C, float *traj, float
   return MG_OK;
 }
 
+}  // extern "C"
+
+namespace {
+
+// The backward pass's workspace is no longer wanted: give it back, or set it aside where a user's
+// graph may use it.
+cudaError_t drop_adjoint_workspace(mg_sim *s) {
+  if (!s->adj_ws) return cudaSuccess;
+  if (s->captured) {
+    s->adj_ws_old.push_back(s->adj_ws);
+  } else {
+    const cudaError_t e = cudaStreamSynchronize(s->stream);
+    if (e != cudaSuccess) return e;
+    cudaFree(s->adj_ws);
+  }
+  s->adj_ws = nullptr;
+  s->adj_ws_cap = 0;
+  return cudaSuccess;
+}
+
+}  // namespace
+
+extern "C" {
+
 mg_status mg_rollout_backward(mg_sim *s, int32_t T, int32_t C, const float *ckpt,
                               const float *dtraj, int64_t step0, float *dcoef, float *dact,
                               float *dstate0) {
@@ -1338,22 +1364,22 @@ mg_status mg_rollout_backward(mg_sim *s, int32_t T, int32_t C, const float *ckpt
   if ((dact && !is_device_ptr(dact)) || (dstate0 && !is_device_ptr(dstate0)))
     return fail(MG_EINVAL, "adjoint buffers must be device memory");
   const bool eight = s->ntv != NT_6;
-  capturing(s);  // a user's graph then reads this parameter range
+  const bool cap = capturing(s);  // a user's graph then reads this parameter range
   bool split = false;
   const bool general = !s->diag || s->has_xh;
   MG_CK(adjoint_split(s->n, general, s->adj_mode, &split));
   if (split) {
     const size_t bytes = adjoint_workspace_bytes(eight, s->n, C);
-    if (s->adj_ws_cap < bytes) {
-      MG_CK(cudaStreamSynchronize(s->stream));
-      cudaFree(s->adj_ws);
-      s->adj_ws = nullptr;
-      s->adj_ws_cap = 0;
+    if (s->adj_ws_cap < bytes && cap) {  // nothing can be allocated
+      if (s->adj_mode == 2) return fail(MG_ENOMEM, "no adjoint workspace, and a capture is on");
+      split = false;  // the one-warp form needs none and gives the same results
+    } else if (s->adj_ws_cap < bytes) {
+      MG_CK(drop_adjoint_workspace(s));
       if (cudaMalloc(&s->adj_ws, bytes) != cudaSuccess) {
         cudaGetLastError();
         s->adj_ws = nullptr;
         if (s->adj_mode == 2) return fail(MG_ENOMEM, "cudaMalloc(adjoint workspace)");
-        split = false;  // the one-warp form needs no workspace and gives the same results
+        split = false;
       } else {
         s->adj_ws_cap = bytes;
       }
