@@ -336,7 +336,9 @@ mg_status mg_rollout_backward(mg_sim *sim, int32_t T, int32_t C, const float *ck
  * schedulers busy.  mode 0 (default): mode 2 while ceil(n_envs / 32) is at most 4 times the GPU's
  * SMs (8 times on the general path) and the workspace can be had, else mode 1 (under stream
  * capture, mode 1 too while the sim holds no workspace large enough).  The per-env arithmetic is
- * the same in both.  MG_EINVAL unless 0 <= mode <= 2. */
+ * the same in both.  The sim keeps the workspace until it is destroyed or mode 1 is set, which
+ * gives it back (with a stream that was ever captured: at destruction, since a user's graph may
+ * use it).  MG_EINVAL unless 0 <= mode <= 2. */
 mg_status mg_set_adjoint_mode(mg_sim *sim, int32_t mode);
 
 /* State in the record layout [n][MG_NSTATE] = p(3) q(4: w,x,y,z) nu(6) n(8, zero past n_thr);

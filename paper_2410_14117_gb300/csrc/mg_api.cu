@@ -1394,6 +1394,7 @@ mg_status mg_set_adjoint_mode(mg_sim *s, int32_t mode) {
   MG_NONNULL(s);
   if (mode < 0 || mode > 2) return fail(MG_EINVAL, "adjoint mode must be 0, 1 or 2");
   s->adj_mode = mode;
+  if (mode == 1 && s->adj_ws && !capturing(s) && !s->captured) MG_CK(drop_adjoint_workspace(s));
   return MG_OK;
 }
 

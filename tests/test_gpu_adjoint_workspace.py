@@ -103,3 +103,19 @@ def test_graph_keeps_its_workspace_when_a_larger_one_is_allocated():
             del fill
         assert torch.cuda.mem_get_info()[0] <= free
         case.sim.close()
+
+
+def test_workspace_is_given_back():
+    case = _Case(16384, False)
+    torch.cuda.synchronize()
+    before = torch.cuda.mem_get_info()[0]
+    case.backward(12)
+    want = case.result()
+    held = before - torch.cuda.mem_get_info()[0]
+    assert held >= 2 * 12 * 100 * 4 * 16384
+    case.sim.set_adjoint_mode(1)
+    assert before - torch.cuda.mem_get_info()[0] <= held - 2 * 12 * 100 * 4 * 16384
+    case.sim.set_adjoint_mode(0)
+    case.backward(12)
+    assert all(torch.equal(x, y) for x, y in zip(want, case.result()))
+    case.sim.close()
