@@ -11,11 +11,11 @@
 // rhs(), written out below).  It is the adjoint of the discrete map the forward computes, so it
 // matches finite differences of the rollout itself, not of the continuous equations.
 //
-// The throttle lag is linear with the command held (LagEnv): the stage throttles are c + f_i d
-// with d = n - c and the step gives c + P d.  So with e_i the adjoint of stage i's throttle
-// through the thrust, the throttle's own adjoint goes lambda_n <- P lambda_n + sum f_i e_i and the
-// command's gains (1 - P) lambda_n + sum (1 - f_i) e_i (f_1 = 1); the throttles stay out of the
-// stage combinations.
+// The throttle lag is linear with the command held (LagEnv): with d = n - c the step gives n+ = n +
+// g d, and the later stages' throttles are n+ + h_i d.  So with e_i the adjoint of stage i's throttle
+// through the thrust, n+ has mu = lambda_n + e_2 + e_3 + e_4, d has delta = g mu + sum h_i e_i, the
+// throttle's own adjoint goes lambda_n <- mu + delta + e_1 and the command's gains -delta; the
+// throttles stay out of the stage combinations.
 //
 // Parameter paths, as the forward has:
 //   - diagonal mass (r_g = 0, no off-diagonal extension): rhs_vjp_diag, the transpose of the step's
@@ -499,8 +499,6 @@ __device__ __forceinline__ void stage_step(St<MT> &S, const float (&c)[MT], cons
   St<MT> k, y = S, acc;
   float d[MT];
 #pragma unroll
-  for (int i = 0; i < MT; ++i) d[i] = S.n[i] - c[i];
-#pragma unroll
   for (int g = 0; g < 4; ++g) {
     rhs<MT, DIAG, true, NH, PATH == ADJ_GEN>(y, A.F, gdir, garm, nt, ca, k, A.xh);
     const float nud[6] = {k.v[0], k.v[1], k.v[2], k.w[0], k.w[1], k.w[2]};
@@ -510,9 +508,15 @@ __device__ __forceinline__ void stage_step(St<MT> &S, const float (&c)[MT], cons
     else axpy<MT>(S, acc, rk.h6, rk.q12, k);
     if (g < 2) axpy<MT>(y, S, rk.hh, rk.qh, k);
     else if (g == 2) axpy<MT>(y, S, rk.h, rk.hh, k);
-    const float f = g == 0 ? A.L.f2 : g == 1 ? A.L.f3 : g == 2 ? A.L.f4 : A.L.P;
+    const float hi = g == 0 ? A.L.h2 : g == 1 ? A.L.h3 : A.L.h4;
 #pragma unroll
-    for (int i = 0; i < MT; ++i) (g < 3 ? y.n[i] : S.n[i]) = fmaf(f, d[i], c[i]);
+    for (int i = 0; i < MT; ++i) {
+      if (g == 0) {
+        d[i] = S.n[i] - c[i];
+        S.n[i] = fmaf(A.L.g, d[i], S.n[i]);
+      }
+      if (g < 3) y.n[i] = fmaf(hi, d[i], S.n[i]);
+    }
   }
 #pragma unroll
   for (int i = 0; i < 4; ++i) zq[i] = S.q[i];
@@ -554,15 +558,12 @@ __device__ __forceinline__ void step_vjp(Stage stage, const float (&zq)[4], cons
   const Body lz = lam;
   Body ly{};
 #pragma unroll
-  for (int i = 0; i < MT; ++i) {
-    gc[i] = fmaf(-A.L.P, lamn[i], lamn[i]);
-    lamn[i] *= A.L.P;
-  }
+  for (int i = 0; i < MT; ++i) gc[i] = 0.f;  // sum h_i e_i, until the first stage
   auto transpose = [&](int i) {
     const bool outer = i == 3 || i == 0;
     const float a = outer ? rk.h6 : rk.h3, aq = outer ? rk.q12 : rk.h6;
     const float b = i == 3 ? 0.f : i == 2 ? rk.h : rk.hh, bq = 0.5f * b;
-    const float fi = i == 3 ? A.L.f4 : i == 2 ? A.L.f3 : i == 1 ? A.L.f2 : 1.f;
+    const float hi = i == 3 ? A.L.h4 : i == 2 ? A.L.h3 : A.L.h2;
     Body lk;
 #pragma unroll
     for (int j = 0; j < 3; ++j) {
@@ -588,8 +589,14 @@ __device__ __forceinline__ void step_vjp(Stage stage, const float (&zq)[4], cons
     for (int j = 0; j < 4; ++j) lam.q[j] += ly.q[j];
 #pragma unroll
     for (int j = 0; j < MT; ++j) {
-      lamn[j] = fmaf(fi, en[j], lamn[j]);
-      gc[j] = fmaf(-fi, en[j], gc[j] + en[j]);
+      if (i > 0) {
+        lamn[j] += en[j];
+        gc[j] = fmaf(hi, en[j], gc[j]);
+      } else {
+        const float delta = fmaf(A.L.g, lamn[j], gc[j]);
+        lamn[j] = (lamn[j] + delta) + en[j];
+        gc[j] = -delta;
+      }
     }
   };
   if constexpr (PATH == ADJ_GEN) {
