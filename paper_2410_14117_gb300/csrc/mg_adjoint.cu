@@ -37,15 +37,17 @@ namespace {
 constexpr int kAdjThreads = 128;
 
 // Which transpose a kernel is compiled for.
-enum AdjPath { ADJ_GEN = 0, ADJ_DENSE = 1, ADJ_MIRRORED = 2, ADJ_MIRRORED_G = 3 };
+enum AdjPath {
+  ADJ_GEN = 0, ADJ_GEN_MIRRORED = 1, ADJ_DENSE = 2, ADJ_MIRRORED = 3, ADJ_MIRRORED_G = 4
+};
+__host__ __device__ constexpr bool adj_general(int path) { return path <= ADJ_GEN_MIRRORED; }
 
-// The thruster allocation of the re-run.  Diagonal mass: the forward's (the vectored one only skips
-// exact zeros of the dense one, so the states are the forward's bit for bit).  General path: the
-// dense one, the forward's within the rounding of the thrust sums where that was mirrored.
+// The thruster allocation of the re-run: the forward's (the vectored one only skips exact zeros of
+// the dense one), so the states are the forward's bit for bit.
 __host__ __device__ constexpr int adj_layout(int path) {
-  return path == ADJ_MIRRORED     ? MG_LAYOUT_MIRRORED
-         : path == ADJ_MIRRORED_G ? MG_LAYOUT_MIRRORED_G
-                                  : MG_LAYOUT_DENSE;
+  return path == ADJ_MIRRORED || path == ADJ_GEN_MIRRORED ? MG_LAYOUT_MIRRORED
+         : path == ADJ_MIRRORED_G                         ? MG_LAYOUT_MIRRORED_G
+                                                          : MG_LAYOUT_DENSE;
 }
 
 // Sums over stages and sub-steps that the coefficient gradients are formed from at the end.
@@ -62,7 +64,7 @@ struct GradDiag {
   float dl[6], dq[6], own[3], up[3], dn[3], munk[3], gyro[3], mv[6];
 };
 template <int PATH>
-using Grad = typename std::conditional<PATH == ADJ_GEN, GradGen, GradDiag>::type;
+using Grad = typename std::conditional<adj_general(PATH), GradGen, GradDiag>::type;
 
 template <typename G>
 __device__ __forceinline__ void zero_grad(G &g) {
@@ -76,7 +78,7 @@ __device__ __forceinline__ void zero_grad(G &g) {
 // memory).
 template <int PATH>
 struct AdjEnv {
-  Coef<PATH != ADJ_GEN, adj_layout(PATH)> F;
+  Coef<!adj_general(PATH), adj_layout(PATH)> F;
   LagEnv L;
   const float *xh;
 };
@@ -134,8 +136,8 @@ struct Body {
 // stage's recorded nu'.  The forward quantities are recomputed from Eq. 1 in the general path's
 // Kirchhoff form; gd.q is the adjoint of d.q = q (x) (0, w) (the doubled quaternion rate rhs()
 // stores).
-template <int MT>
-__device__ void rhs_vjp_gen(const St<MT> &s, const float (&nud)[6], const AdjEnv<ADJ_GEN> &A,
+template <int MT, int PATH>
+__device__ void rhs_vjp_gen(const St<MT> &s, const float (&nud)[6], const AdjEnv<PATH> &A,
                             const float4 *gdir, const float4 *garm, int nt, bool current_accel,
                             const Body &gd, Body &gs, GradGen &G, float (&en)[MT]) {
   const auto &P = A.F;
@@ -494,13 +496,13 @@ template <int MT, int PATH, typename Stage>
 __device__ __forceinline__ void stage_step(St<MT> &S, const float (&c)[MT], const AdjEnv<PATH> &A,
                                            const float4 *gdir, const float4 *garm, int nt, bool ca,
                                            const RkStep &rk, float (&zq)[4], Stage stage) {
-  constexpr bool DIAG = PATH != ADJ_GEN;
+  constexpr bool DIAG = !adj_general(PATH);
   constexpr int NH = adj_layout(PATH);
   St<MT> k, y = S, acc;
   float d[MT];
 #pragma unroll
   for (int g = 0; g < 4; ++g) {
-    rhs<MT, DIAG, true, NH, PATH == ADJ_GEN>(y, A.F, gdir, garm, nt, ca, k, A.xh);
+    rhs<MT, DIAG, true, NH, !DIAG>(y, A.F, gdir, garm, nt, ca, k, A.xh);
     const float nud[6] = {k.v[0], k.v[1], k.v[2], k.w[0], k.w[1], k.w[2]};
     stage(g, y, nud);
     if (g == 0) axpy<MT>(acc, S, rk.h6, rk.q12, k);
@@ -576,8 +578,8 @@ __device__ __forceinline__ void step_vjp(Stage stage, const float (&zq)[4], cons
     St<MT> y;
     float nud[6], en[MT];
     stage(i, y, nud);
-    if constexpr (PATH == ADJ_GEN)
-      rhs_vjp_gen<MT>(y, nud, A, gdir, garm, nt, ca, lk, ly, G, en);
+    if constexpr (adj_general(PATH))
+      rhs_vjp_gen<MT, PATH>(y, nud, A, gdir, garm, nt, ca, lk, ly, G, en);
     else
       rhs_vjp_diag<MT, PATH>(y, nud, A, gdir, garm, nt, lk, ly, G, en);
 #pragma unroll
@@ -599,7 +601,7 @@ __device__ __forceinline__ void step_vjp(Stage stage, const float (&zq)[4], cons
       }
     }
   };
-  if constexpr (PATH == ADJ_GEN) {
+  if constexpr (adj_general(PATH)) {
 #pragma unroll 1
     for (int i = 3; i >= 0; --i) transpose(i);
   } else {
@@ -766,11 +768,12 @@ __device__ __forceinline__ void stage_xh_or_zero(const FleetView &fv, int64_t en
 template <int PATH>
 __device__ __forceinline__ void load_env(const FleetView &fv, int64_t e, const float *sxh_row,
                                          const float4 *gdir, const float4 *garm, AdjEnv<PATH> &A) {
-  Par<PATH != ADJ_GEN> P;
-  load_par<PATH != ADJ_GEN>(fv.pa, e, P);
-  A.F = make_coef<PATH != ADJ_GEN, adj_layout(PATH)>(P, gdir, garm);
+  constexpr bool DIAG = !adj_general(PATH);
+  Par<DIAG> P;
+  load_par<DIAG>(fv.pa, e, P);
+  A.F = make_coef<DIAG, adj_layout(PATH)>(P, gdir, garm);
   A.L = lag_env(P.itau, fv.dt);
-  A.xh = PATH == ADJ_GEN ? sxh_row : nullptr;
+  A.xh = DIAG ? nullptr : sxh_row;
 }
 
 // A stage record: what the transposes read of one stage, in float4 words (q, nu, nu', n), so that a
@@ -823,7 +826,7 @@ __global__ void __launch_bounds__(kAdjThreads)
   extern __shared__ float sxh[];
   stage_geometry(fv, sgeo);
   const int64_t env0 = (int64_t)blockIdx.x * blockDim.x;
-  if constexpr (PATH == ADJ_GEN)
+  if constexpr (adj_general(PATH))
     stage_xh_or_zero(fv, env0, (int)min((int64_t)blockDim.x, fv.n - env0), sxh);
   __syncthreads();
   const int64_t e = env0 + threadIdx.x;
@@ -856,7 +859,7 @@ __global__ void __launch_bounds__(kAdjThreads)
       CommandWalk<MT> cmd(fv, e, nt, step0 + t0);
       St<MT> x = S[0];
       for (int32_t j = 1; j < len; ++j) {
-        rk4_step<MT, PATH != ADJ_GEN, true, adj_layout(PATH), PATH == ADJ_GEN>(
+        rk4_step<MT, !adj_general(PATH), true, adj_layout(PATH), adj_general(PATH)>(
             x, cmd.c, A.L, A.F, gdir, garm, nt, ca, fv.rk, A.xh);
         S[j] = x;
         cmd.next(fv, e, nt);
@@ -1010,7 +1013,7 @@ __global__ void __launch_bounds__(kWsThreads)
   extern __shared__ float sxh[];
   stage_geometry(fv, sgeo);
   const int64_t env0 = (int64_t)blockIdx.x * 32;
-  if constexpr (PATH == ADJ_GEN)
+  if constexpr (adj_general(PATH))
     stage_xh_or_zero(fv, env0, (int)min((int64_t)32, fv.n - env0), sxh);
   __syncthreads();
   const int warp = (int)(threadIdx.x >> 5), lane = (int)(threadIdx.x & 31);
@@ -1061,7 +1064,7 @@ cudaError_t launch_adjoint_t(const FleetView &fv, const int32_t *types, const fl
                              int n_sm, cudaStream_t stream) {
   if (split) {
     const int grid = (int)((fv.n + 31) / 32);
-    const size_t smem = PATH == ADJ_GEN ? sizeof(float) * 32 * MG_NXPARAM : 0;
+    const size_t smem = adj_general(PATH) ? sizeof(float) * 32 * MG_NXPARAM : 0;
     k_adjoint_ws<MT, PATH><<<grid, kWsThreads, smem, stream>>>(
         fv, types, ckpt, dtraj, T, C, step0, dcoef, dact, dstate0, static_cast<float4 *>(ws));
     return cudaGetLastError();
@@ -1072,7 +1075,7 @@ cudaError_t launch_adjoint_t(const FleetView &fv, const int32_t *types, const fl
   const int64_t warps = (fv.n + 31) / 32;
   const int threads = warps <= 4 * (int64_t)n_sm ? 32 : kAdjThreads;
   const int grid = (int)((fv.n + threads - 1) / threads);
-  const size_t smem = PATH == ADJ_GEN ? sizeof(float) * threads * MG_NXPARAM : 0;
+  const size_t smem = adj_general(PATH) ? sizeof(float) * threads * MG_NXPARAM : 0;
   k_adjoint<MT, PATH><<<grid, threads, smem, stream>>>(fv, types, ckpt, dtraj, T, C, step0, dcoef,
                                                        dact, dstate0);
   return cudaGetLastError();
@@ -1258,7 +1261,10 @@ cudaError_t launch_adjoint(const FleetView &fv, const int32_t *types, bool eight
     return eight ? run(launch_adjoint_t<8, decltype(p)::value>)
                  : run(launch_adjoint_t<6, decltype(p)::value>);
   };
-  if (general) return on_path(std::integral_constant<int, ADJ_GEN>());
+  if (general)
+    return layout == MG_LAYOUT_MIRRORED
+               ? on_path(std::integral_constant<int, ADJ_GEN_MIRRORED>())
+               : on_path(std::integral_constant<int, ADJ_GEN>());
   if (layout == MG_LAYOUT_MIRRORED) return on_path(std::integral_constant<int, ADJ_MIRRORED>());
   if (layout == MG_LAYOUT_MIRRORED_G) return on_path(std::integral_constant<int, ADJ_MIRRORED_G>());
   return on_path(std::integral_constant<int, ADJ_DENSE>());

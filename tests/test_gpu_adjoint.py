@@ -276,3 +276,38 @@ def test_forward_equals_recorded_steps(general):
     assert torch.equal(a.get_state(), b.get_state())
     a.close()
     b.close()
+
+
+@pytest.mark.parametrize("mode", [1, 2])
+@pytest.mark.parametrize("general", [False, "cg", "coupled"])
+@pytest.mark.parametrize("frame", ["mirrored", "renumbered"])
+def test_gradients_do_not_depend_on_the_checkpoint_interval(frame, general, mode):
+    """The re-run from a checkpoint repeats the forward's states bit for bit (every frame's thrust
+    sums, both paths), so the gradients are those with a checkpoint at every sub-step."""
+    vs = vehicles()
+    if frame == "renumbered":  # two thrusters swapped: no longer a mirrored frame
+        for v in vs:
+            v.r[[0, 1]], v.d[[0, 1]] = v.r[[1, 0]], v.d[[1, 0]]
+    n, T, hold = 200, 45, 10
+    types = I.mixed_fleet(3, n, max_group=60)
+    nt = np.array([vs[t].n_thr for t in types])
+    outs = []
+    for C in (1, 20):
+        sim = Sim(n, types, vs)
+        sim.set_adjoint_mode(mode)
+        sim.randomize(77, 0.8, 1.2, 0.2, 0.3, rg_halfwidth=0.02 if general else 0.0)
+        if general == "coupled":
+            p = sim.get_params().double().cpu().numpy()
+            sim.set_hydro_offdiag(torch.tensor(I.hydro_offdiag(8, p), dtype=torch.float32,
+                                               device="cuda"))
+        coeffs = sim.get_params()[:, COEF_SLICE].clone().requires_grad_(True)
+        acts = torch.tensor(I.commands(5, -(-T // hold), n, nt), device="cuda", requires_grad=True)
+        s0 = torch.tensor(I.initial_states(21, n), dtype=torch.float32, device="cuda",
+                          requires_grad=True)
+        traj = rollout(sim, coeffs, acts, s0, hold, T, C)
+        g = torch.randn(traj.shape, generator=torch.Generator(device="cuda").manual_seed(3),
+                        device="cuda")
+        outs.append(torch.autograd.grad(traj, (coeffs, acts, s0), g))
+        sim.close()
+    for name, a, b in zip(("coefficients", "actions", "initial state"), *outs):
+        torch.testing.assert_close(b, a, rtol=0, atol=0, msg=name)
