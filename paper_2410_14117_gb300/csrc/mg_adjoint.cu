@@ -94,9 +94,11 @@ __device__ __forceinline__ float xd(const float *xh, int i, int j) {
   return xh[15 + 5 * i + (j < i ? j : j - 1)];
 }
 
-// Every multiply-add of the adjoint code below is written as an explicit fmaf, so the compiler
+// Every multiply-add of the adjoint code below, and of the right-hand side it re-runs, is written as
+// an explicit fmaf, and a product that only a plain addition follows as __fmul_rn, so the compiler
 // forms no fused operation of its own: the results do not depend on the surrounding code the
-// functions are inlined into (the one-warp and two-warp backward kernels agree bit for bit).
+// functions are inlined into (the one-warp and two-warp backward kernels agree bit for bit; so does
+// this file compiled without contraction).
 
 __device__ __forceinline__ void cross_vjp(const float a[3], const float b[3], const float gc[3],
                                           float ga[3], float gb[3]) {
@@ -316,7 +318,7 @@ __device__ void rhs_vjp_gen(const St<MT> &s, const float (&nud)[6], const AdjEnv
     const float4 dd = gdir[i], aa = garm[i];
     const float gfi = fmaf(dd.x, gt[0], fmaf(dd.y, gt[1], fmaf(dd.z, gt[2],
                       fmaf(aa.x, gt[3], fmaf(aa.y, gt[4], aa.z * gt[5])))));
-    en[i] = 2.f * fabsf(s.n[i]) * gfi;
+    en[i] = __fmul_rn(2.f * fabsf(s.n[i]), gfi);
   }
   for (int i = 0; i < 4; ++i) gs.q[i] = gq[i];
   for (int i = 0; i < 3; ++i) {
@@ -369,8 +371,8 @@ __device__ __forceinline__ void rhs_vjp_diag(const St<MT> &s, const float (&nud)
   for (int j = 0; j < 3; ++j) {
     const float ar = fabsf(r[j]), aw = fabsf(w[j]);
     const float hr = gv[j] * r[j], hw = gw[j] * w[j];
-    G.dl[j] += hr;
-    G.dl[3 + j] += hw;
+    G.dl[j] = fmaf(gv[j], r[j], G.dl[j]);
+    G.dl[3 + j] = fmaf(gw[j], w[j], G.dl[3 + j]);
     G.dq[j] = fmaf(ar, hr, G.dq[j]);
     G.dq[3 + j] = fmaf(aw, hw, G.dq[3 + j]);
     gr[j] = -fmaf(P.dqt[j], ar + ar, P.dlt[j]) * gv[j];
@@ -387,8 +389,8 @@ __device__ __forceinline__ void rhs_vjp_diag(const St<MT> &s, const float (&nud)
     const float gu = gv[i] * w[i2], gx = gv[i] * w[i1];  // adjoints of u_i and -x_i
     ow[i2] = fmaf(gv[i], u, ow[i2]);
     ow[i1] = fmaf(-gv[i], x, ow[i1]);
-    ov[i1] += gu;
-    ov[i2] -= gx;
+    ov[i1] = fmaf(gv[i], w[i2], ov[i1]);
+    ov[i2] = fmaf(-gv[i], w[i1], ov[i2]);
     gr[i1] = fmaf(P.bp[i], gu, gr[i1]);
     gr[i2] = fmaf(-P.bm[i], gx, gr[i2]);
     G.up[i] = fmaf(gu, r[i1], G.up[i]);
@@ -454,20 +456,19 @@ __device__ __forceinline__ void rhs_vjp_diag(const St<MT> &s, const float (&nud)
   float gf[MT];
   if constexpr (mirrored_sums(adj_layout(PATH))) {
     const float gX = fmaf(P.At[0], gv[0], P.Mh * gw[1]), gY = fmaf(P.At[1], gv[1], P.Kh * gw[0]);
-    const float gN = P.Nh * gw[2], gZ = P.At[2] * gv[2], gK = P.Kv * gw[0];
+    const float gZ = P.At[2] * gv[2];
     const float sm = gX + gY, df = gX - gY;
-    gf[0] = sm + gN;
-    gf[1] = df - gN;
-    gf[2] = -df - gN;
-    gf[3] = gN - sm;
-    gf[4] = gZ - gK;
-    gf[5] = gZ + gK;
+    gf[0] = fmaf(P.Nh, gw[2], sm);
+    gf[1] = fmaf(-P.Nh, gw[2], df);
+    gf[2] = fmaf(-P.Nh, gw[2], -df);
+    gf[3] = fmaf(P.Nh, gw[2], -sm);
+    gf[4] = fmaf(-P.Kv, gw[0], gZ);
+    gf[5] = fmaf(P.Kv, gw[0], gZ);
     if constexpr (MT > 6) {
-      const float gM = P.Mv * gw[1];
-      gf[6] = gf[4] + gM;
-      gf[7] = gf[5] + gM;
-      gf[4] -= gM;
-      gf[5] -= gM;
+      gf[6] = fmaf(P.Mv, gw[1], gf[4]);
+      gf[7] = fmaf(P.Mv, gw[1], gf[5]);
+      gf[4] = fmaf(-P.Mv, gw[1], gf[4]);
+      gf[5] = fmaf(-P.Mv, gw[1], gf[5]);
     }
   } else {
     float gt[6];
@@ -485,7 +486,7 @@ __device__ __forceinline__ void rhs_vjp_diag(const St<MT> &s, const float (&nud)
   }
   (void)nt;
 #pragma unroll
-  for (int i = 0; i < MT; ++i) en[i] = 2.f * fabsf(s.n[i]) * gf[i];
+  for (int i = 0; i < MT; ++i) en[i] = __fmul_rn(2.f * fabsf(s.n[i]), gf[i]);
 }
 
 // The stage states of one sub-step and the step itself: stage(i, y, nu') is called with stage i's

@@ -616,12 +616,15 @@ __device__ __forceinline__ void rhs(const St<MT> &s, const Coef<DIAG, NH> &P,
 
     // nu' = M^-1 f.
     const float *o = P.mo;
-    d.v[0] = P.mi[0] * f0 + o[0] * f1 + o[1] * f2 + o[2] * f3 + o[3] * f4 + o[4] * f5;
-    d.v[1] = o[0] * f0 + P.mi[1] * f1 + o[5] * f2 + o[6] * f3 + o[7] * f4 + o[8] * f5;
-    d.v[2] = o[1] * f0 + o[5] * f1 + P.mi[2] * f2 + o[9] * f3 + o[10] * f4 + o[11] * f5;
-    d.w[0] = o[2] * f0 + o[6] * f1 + o[9] * f2 + P.mi[3] * f3 + o[12] * f4 + o[13] * f5;
-    d.w[1] = o[3] * f0 + o[7] * f1 + o[10] * f2 + o[12] * f3 + P.mi[4] * f4 + o[14] * f5;
-    d.w[2] = o[4] * f0 + o[8] * f1 + o[11] * f2 + o[13] * f3 + o[14] * f4 + P.mi[5] * f5;
+    auto row = [&](float m0, float m1, float m2, float m3, float m4, float m5) {
+      return fmaf(m5, f5, fmaf(m4, f4, fmaf(m3, f3, fmaf(m2, f2, fmaf(m1, f1, m0 * f0)))));
+    };
+    d.v[0] = row(P.mi[0], o[0], o[1], o[2], o[3], o[4]);
+    d.v[1] = row(o[0], P.mi[1], o[5], o[6], o[7], o[8]);
+    d.v[2] = row(o[1], o[5], P.mi[2], o[9], o[10], o[11]);
+    d.w[0] = row(o[2], o[6], o[9], P.mi[3], o[12], o[13]);
+    d.w[1] = row(o[3], o[7], o[10], o[12], P.mi[4], o[14]);
+    d.w[2] = row(o[4], o[8], o[11], o[13], o[14], P.mi[5]);
   }
 
   // Kinematics: p' = R v; 2 q' = q (x) (0, w).

@@ -311,3 +311,37 @@ def test_gradients_do_not_depend_on_the_checkpoint_interval(frame, general, mode
         sim.close()
     for name, a, b in zip(("coefficients", "actions", "initial state"), *outs):
         torch.testing.assert_close(b, a, rtol=0, atol=0, msg=name)
+
+
+@pytest.mark.parametrize("frame", ["renumbered", "buoyancy off the axis"])
+@pytest.mark.parametrize("mixed", [False, True])
+def test_backward_kernels_agree_for_other_frames(mixed, frame):
+    """As test_backward_kernels_agree, for the diagonal-mass transposes of a frame that is no longer
+    mirrored, and of a mirrored one with r_b off the z axis."""
+    vs = vehicles()
+    if frame == "renumbered":
+        for v in vs:
+            v.r[[0, 1]], v.d[[0, 1]] = v.r[[1, 0]], v.d[[1, 0]]
+    n, T, C, hold = 300, 93, 7, 10
+    types = I.mixed_fleet(3, n, max_group=60) if mixed else np.zeros(n, dtype=np.int32)
+    nt = np.array([vs[t].n_thr for t in types])
+    outs = []
+    for mode in (1, 2):
+        sim = Sim(n, types, vs)
+        sim.set_adjoint_mode(mode)
+        sim.randomize(77, 0.8, 1.2, 0.2, 0.3)
+        if frame != "renumbered":
+            p = sim.get_params()
+            p[:, I.P_RB] = 0.01
+            sim.set_params(p)
+        coeffs = sim.get_params()[:, COEF_SLICE].clone().requires_grad_(True)
+        acts = torch.tensor(I.commands(5, -(-T // hold), n, nt), device="cuda", requires_grad=True)
+        s0 = torch.tensor(I.initial_states(21, n), dtype=torch.float32, device="cuda",
+                          requires_grad=True)
+        traj = rollout(sim, coeffs, acts, s0, hold, T, C)
+        g = torch.randn(traj.shape, generator=torch.Generator(device="cuda").manual_seed(3),
+                        device="cuda")
+        outs.append(torch.autograd.grad(traj, (coeffs, acts, s0), g))
+        sim.close()
+    for name, a, b in zip(("coefficients", "actions", "initial state"), *outs):
+        torch.testing.assert_close(b, a, rtol=0, atol=0, msg=name)
