@@ -132,6 +132,7 @@ struct mg_sim {
   int layout = MG_LAYOUT_DENSE;
   bool on_axis = true;          // every env's r_b lies on the body's z axis
   bool nominal_on_axis = true;  // so do the types' present (randomised r_b stays there)
+  bool nominal_plain = true;  // plain_record() for every type's
   bool nominal_diag = true;  // every type has r_g = 0 (randomised M_RB + M_A stays diagonal)
   cudaStream_t stream = nullptr;
   cudaStream_t cap_stream = nullptr;
@@ -308,6 +309,7 @@ struct mg_sim {
     v.n_not_spd = counters + 1;
     v.any_offdiag = offdiag;
     v.xh = has_xh ? xh : nullptr;
+    v.plain = nominal_plain;
     v.diag_only = nominal_diag && !has_xh;
     return v;
   }
@@ -759,6 +761,7 @@ mg_status mg_create(int64_t n_envs, const int32_t *vehicle_types,
     }
     p[MG_P_KT] = v.kT;
     p[MG_P_TAU] = v.tau_m;
+    s->nominal_plain = s->nominal_plain && plain_record(p);
   }
   auto bail = [&](mg_status st) {
     mg_destroy(s);

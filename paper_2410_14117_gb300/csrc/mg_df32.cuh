@@ -1,10 +1,11 @@
 // Two-float arithmetic for the set-up kernels: a value is the unevaluated sum h + l of two FP32
 // numbers, |l| <= ulp(h) / 2.  GB300 executes FP64 at a 64th of the FP32 rate, which made the domain
 // randomisation (some 380 FP64 warp instructions per 32 envs) a quarter of a 100-sub-step episode
-// of a 1,048,576-env fleet.  The sums and products below are exact or good to about 2^-45, the
-// elementary functions to 2^-35 or better, so that a result rounded once to FP32 at the end is
-// what FP64 arithmetic rounds to but for ties within 2^-35 (the error bound stays 0.5 FP32 ulp to
-// three digits).
+// of a 1,048,576-env fleet.  The sums and products below are exact or good to 2^-45, the elementary
+// functions to 2^-41 (every uniform draw checked against 64-bit mantissas: radius 2^-41.4, sine and
+// cosine 2^-41.8).  A result is rounded to FP32 from here only where both ends of its error bound
+// round alike (round_df); the few others are left to FP64, so what is stored is what FP64
+// arithmetic stores, bit for bit.
 //
 // Published methods: Knuth's two-sum, Dekker's fast two-sum and the FMA two-product; the series of
 // atanh, sin and cos.  Every operation is an explicit round-to-nearest intrinsic, so the compiler
@@ -43,16 +44,32 @@ __device__ __forceinline__ df32 df_add_small(df32 c, df32 p) {
   return fast_two_sum(s.h, __fadd_rn(s.l, __fadd_rn(c.l, p.l)));
 }
 
-// 1 / (a.h + a.l) rounded to FP32 (0, infinities and NaN as FP32's reciprocal gives them).
-__device__ __forceinline__ float df_rcp(df32 a) {
+// A double constant in two floats.
+__device__ __forceinline__ constexpr df32 df_const(double c) {
+  return {(float)c, (float)(c - (double)(float)c)};
+}
+
+// q + r, |r| << |q|, rounded to FP32.  open: some number within w rel of it rounds otherwise (or it is
+// not finite).
+__device__ __forceinline__ float round_df(float q, float r, float w, float rel, bool &open) {
+  const float f = __fadd_rn(q, __fmaf_rn(w, rel, r));
+  open = !(f == __fadd_rn(q, __fmaf_rn(-w, rel, r)));
+  return f;
+}
+
+// 1 / (a.h + a.l) rounded to FP32; open as in round_df.  The residual is exact but for its last
+// rounding (2^-47 of the result), the neglected square of it 2^-47.
+__device__ __forceinline__ float df_rcp(df32 a, bool &open) {
   const float r = __frcp_rn(a.h);
   const float e = __fmaf_rn(-a.l, r, __fmaf_rn(-a.h, r, 1.f));
-  return isfinite(e) ? __fmaf_rn(r, e, r) : r;
+  const float f = round_df(r, __fmul_rn(r, e), r, 0x1p-43f, open);
+  open = open || !(a.h > 1e-20f && a.h < 1e20f);
+  return f;
 }
 
 // sqrt(-2 ln u) for u in (0, 1).  u = 2^e m with m in [sqrt(1/2), sqrt(2)); with s = (m - 1) /
-// (m + 1), ln m = 2 atanh s = 2 s (1 + z/3 + z^2/5 + ...), z = s^2 <= 0.0295; the terms past z/3
-// are summed in FP32 (they are below 2^-10 of the total).
+// (m + 1), ln m = 2 atanh s = 2 s (1 + z/3 + z^2/5 + ...), z = s^2 <= 0.0295; the terms past z^2/5
+// are summed in FP32 (they are below 2^-17 of the total).
 __device__ __forceinline__ df32 df_normal_radius(float u) {
   const int bits = __float_as_int(u);
   const int e = (bits - __float_as_int(0.70710677f)) >> 23;
@@ -64,14 +81,16 @@ __device__ __forceinline__ df32 df_normal_radius(float u) {
   s.h = __fmul_rn(f, r);
   s.l = __fmul_rn(__fmaf_rn(-s.h, g.l, __fmaf_rn(-s.h, g.h, f)), r);
   const df32 z = df_mul(s, s);
-  float q = 1.f / 15.f;
+  float q = 1.f / 17.f;
+  q = __fmaf_rn(q, z.h, 1.f / 15.f);
   q = __fmaf_rn(q, z.h, 1.f / 13.f);
   q = __fmaf_rn(q, z.h, 1.f / 11.f);
   q = __fmaf_rn(q, z.h, 1.f / 9.f);
   q = __fmaf_rn(q, z.h, 1.f / 7.f);
-  q = __fmaf_rn(q, z.h, 1.f / 5.f);
-  constexpr float third = 1.f / 3.f, third_l = (float)(1.0 / 3.0 - (double)third);
-  const df32 p = df_add_small({third, third_l}, two_prod(z.h, q));
+  df32 p = two_prod(z.h, q);
+  p.l = __fmaf_rn(z.l, q, p.l);
+  p = df_add_small(df_const(1.0 / 5.0), p);
+  p = df_add_small(df_const(1.0 / 3.0), df_mul(z, p));
   const df32 t = df_mul(z, p);
   const df32 lm = df_add_small(s, df_mul(s, t));  // atanh s
   // e ln 2 with the leading part of ln 2 in 15 bits, so that its product with e is exact
@@ -86,7 +105,7 @@ __device__ __forceinline__ df32 df_normal_radius(float u) {
 }
 
 // cos(2 pi u) and sin(2 pi u) for a u in (0, 1) with 24 bits.  The argument is reduced exactly to
-// t in [-1/4, 1/4] half turns; x = pi t, y = x^2 <= 0.617, and the first three coefficients of each
+// t in [-1/4, 1/4] half turns; x = pi t, y = x^2 <= 0.617, and the first four coefficients of each
 // series are applied in two floats, the rest in FP32.
 __device__ __forceinline__ void df_cos_sin_turn(float u, df32 &c, df32 &s) {
   const float v = __fadd_rn(u, u);
@@ -98,24 +117,23 @@ __device__ __forceinline__ void df_cos_sin_turn(float u, df32 &c, df32 &s) {
   df32 x = two_prod(t, pi_h);
   x.l = __fmaf_rn(t, pi_l, x.l);
   const df32 y = df_mul(x, x);
-  auto horner = [&](float tail, double c2, double c1) {  // y (c1 + y (c2 + y tail))
-    const float c2h = (float)c2, c1h = (float)c1;
-    df32 p = two_prod(y.h, tail);
-    p.l = __fmaf_rn(y.l, tail, p.l);
-    p = df_add_small({c2h, (float)(c2 - (double)c2h)}, p);
-    p = df_add_small({c1h, (float)(c1 - (double)c1h)}, df_mul(y, p));
-    return df_mul(y, p);
+  auto tail = [&](double c, float t) {  // c + y t
+    df32 p = two_prod(y.h, t);
+    p.l = __fmaf_rn(y.l, t, p.l);
+    return df_add_small(df_const(c), p);
   };
+  auto term = [&](double c, df32 p) { return df_add_small(df_const(c), df_mul(y, p)); };
   float ts = 1.f / 6227020800.f;
   ts = __fmaf_rn(ts, y.h, -1.f / 39916800.f);
   ts = __fmaf_rn(ts, y.h, 1.f / 362880.f);
-  ts = __fmaf_rn(ts, y.h, -1.f / 5040.f);
-  float tc = 1.f / 479001600.f;
+  float tc = -1.f / 87178291200.f;
+  tc = __fmaf_rn(tc, y.h, 1.f / 479001600.f);
   tc = __fmaf_rn(tc, y.h, -1.f / 3628800.f);
   tc = __fmaf_rn(tc, y.h, 1.f / 40320.f);
-  tc = __fmaf_rn(tc, y.h, -1.f / 720.f);
-  const df32 sn = df_add_small(x, df_mul(x, horner(ts, 1.0 / 120.0, -1.0 / 6.0)));
-  const df32 cs = df_add_small({1.f, 0.f}, horner(tc, 1.0 / 24.0, -0.5));
+  const df32 ps = term(-1.0 / 6.0, term(1.0 / 120.0, tail(-1.0 / 5040.0, ts)));
+  const df32 pc = term(-0.5, term(1.0 / 24.0, tail(-1.0 / 720.0, tc)));
+  const df32 sn = df_add_small(x, df_mul(x, df_mul(y, ps)));
+  const df32 cs = df_add_small({1.f, 0.f}, df_mul(y, pc));
   // rotate by j quarter turns
   const bool odd = j & 1, neg_c = (j + 1) & 2, neg_s = j & 2;
   c = odd ? sn : cs;

@@ -186,9 +186,19 @@ struct SetupView {
   unsigned int *any_offdiag;  // bit 0: some mass matrix is full; bit 1: some r_b is off the z axis
   const float *xh;           // device [MG_NXPARAM][xh_stride] off-diagonal hydrodynamics, or null
   int64_t xh_stride;         // floats between xh's component planes (0: n)
+  bool plain;                // plain_record() for every type's nominal record
   bool diag_only;            // nominal mass matrices are diagonal and xh is null: a draw without r_g
                              // keeps them so
 };
+
+// Whether a nominal record's magnitudes are ordinary (zero, or within [1e-25, 1e25]).
+inline bool plain_record(const float *p) {
+  for (int j = 0; j < MG_NPARAM; ++j) {
+    const float a = p[j] < 0.f ? -p[j] : p[j];
+    if (a != 0.f && !(a >= 1e-25f && a <= 1e25f)) return false;
+  }
+  return true;
+}
 
 // background_blocks > 0: at most that many 64-thread blocks striding over the fleet (leaves room
 // for a step kernel running concurrently on another stream); 0: one env per thread.

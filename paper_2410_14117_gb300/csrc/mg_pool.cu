@@ -191,6 +191,7 @@ struct mg_pool {
   std::vector<mg_vehicle_params> vp;
   bool diag = true;
   int layout = MG_LAYOUT_MIRRORED;  // the fastest one that every vehicle type has
+  bool plain = true;                // plain_record() for every type's
   bool mirrored = true;             // every type's geometry is (the general path's condition)
   cudaStream_t stream = nullptr;
   void *arena = nullptr;
@@ -383,6 +384,7 @@ mg_status mg_pool_create(int64_t capacity_envs, const mg_vehicle_params *params,
     }
     q[MG_P_KT] = v.kT;
     q[MG_P_TAU] = v.tau_m;
+    p->plain = p->plain && plain_record(q);
   }
   e = cudaMemset(p->arena, 0, off);
   if (e == cudaSuccess)
@@ -445,6 +447,7 @@ cudaError_t init_job(mg_pool *p, const mg_job_spec &s, int64_t env0, const float
   v.pa = sub_params(p->pa, env0);
   v.n_not_spd = p->counters + 1;
   v.any_offdiag = p->offdiag;
+  v.plain = p->plain;
   v.diag_only = p->diag && !xh;
   if (xh) {
     // stride of the planes: the capacity

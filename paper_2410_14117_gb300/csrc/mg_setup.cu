@@ -1,6 +1,6 @@
 // Set-up kernels, run when parameters or episodes change (not per sub-step):
-//   - domain randomisation (§METHOD) from Philox4x32-10 draws, each value rounded once to FP32
-//     from two-float arithmetic (mg_df32.cuh);
+//   - domain randomisation (§METHOD) from Philox4x32-10 draws, the values FP64 arithmetic stores,
+//     formed in two-float arithmetic (mg_df32.cuh) where that decides their rounding to FP32;
 //   - derivation of what the step reads, including M^-1 of the 6x6 mass matrix M_RB + M_A of
 //     Eq. 1: its reciprocals where it is diagonal, else by an FP64 Cholesky factorisation (M is
 //     symmetric positive definite for any physical vehicle; a non-positive pivot is counted and
@@ -33,7 +33,7 @@ __host__ __device__ constexpr int rand_idx(int j) {
 }
 // Block size of the randomisation kernel and of the record copies.
 constexpr int kRandThreads = 128;
-// Background form: 64-thread blocks (two warps, 4 K registers) striding over the fleet, which fit
+// Background form: 64-thread blocks (two warps, 4.6 K registers) striding over the fleet, which fit
 // beside the work queue's resident blocks on every SM.
 constexpr int kRandBgThreads = 64;
 
@@ -57,22 +57,38 @@ __device__ __forceinline__ void note_off_axis(const SetupView &v, const float *p
   if (p[MG_P_RB] != 0.f || p[MG_P_RB + 1] != 0.f) atomicOr(v.any_offdiag, 2u);
 }
 
+// M^-1 of a diagonal mass matrix in FP64, for the few envs with a reciprocal whose rounding df_rcp
+// leaves open.
+__device__ __noinline__ void invert_diag_fp64(const ParamPlanes &pa, int64_t e, float m, float Ix,
+                                              float Iy, float Iz, float a0, float a1, float a2,
+                                              float a3, float a4, float a5) {
+  auto inv = [](float a, float b) {
+    const double M = (double)a + (double)b;
+    return M > 0.0 ? (float)(1.0 / M) : 0.f;
+  };
+  pa.d7[e] = make_float4(inv(m, a0), inv(m, a1), inv(m, a2), inv(Ix, a3));
+  pa.d8[e] = make_float2(inv(Iy, a4), inv(Iz, a5));
+}
+
 // The step's parameter planes of an env whose mass matrix is diagonal (r_g = 0, no off-diagonal
 // added mass) from its record p[MG_NPARAM]: I_o = I_g exactly, M^-1 = diag(1 / M_jj) and every
 // off-diagonal entry is +0.  Each stored value is the FP64 expression's, rounded once: a sum,
-// difference or product of two FP32 numbers is one FP32 operation, and 1 / (a + b) takes the sum
-// in two floats.
+// difference or product of two FP32 numbers is one FP32 operation, and 1 / (a + b) is formed in two
+// floats, or in FP64 where those leave its rounding open.
 __device__ __forceinline__ void derive_diag(const SetupView &v, int64_t e, const float *p) {
   const float m = p[MG_P_M];
   const float *ma = p + MG_P_MA, *rg = p + MG_P_RG, *rb = p + MG_P_RB;
   float J[3], mi[6];
-  bool spd = true;
+  bool spd = true, open = false;
 #pragma unroll
   for (int j = 0; j < 6; ++j) {
     const df32 M = two_sum(j < 3 ? m : p[MG_P_IG + j - 3], ma[j]);
     if (j >= 3) J[j - 3] = M.h;
     if (!(M.h > 0.f)) spd = false;
-    mi[j] = M.h > 0.f ? df_rcp(M) : 0.f;
+    bool o;
+    const float r = df_rcp(M, o);
+    mi[j] = M.h > 0.f ? r : 0.f;
+    open = open || o;
   }
   if (!spd) atomicAdd(v.n_not_spd, 1ull);
   note_off_axis(v, p);
@@ -90,6 +106,9 @@ __device__ __forceinline__ void derive_diag(const SetupView &v, int64_t e, const
   pa.d6[e] = make_float4(p[MG_P_VC], p[MG_P_VC + 1], p[MG_P_VC + 2], __frcp_rn(p[MG_P_TAU]));
   pa.d7[e] = make_float4(mi[0], mi[1], mi[2], mi[3]);
   pa.d8[e] = make_float2(mi[4], mi[5]);
+  if (open)
+    invert_diag_fp64(pa, e, m, p[MG_P_IG], p[MG_P_IG + 1], p[MG_P_IG + 2], ma[0], ma[1], ma[2], ma[3],
+                     ma[4], ma[5]);
   const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
   pa.g0[e] = make_float4(__fmul_rn(m, rg[0]), __fmul_rn(m, rg[1]), __fmul_rn(m, rg[2]), 0.f);
   pa.g1[e] = z;
@@ -211,37 +230,66 @@ __device__ void derive(const SetupView &v, int64_t e, const float *f32) {
 // floats, the current's sigma and the half-width of r_g.
 struct Draw {
   uint64_t seed;
-  float lo;
+  float lo, hi;
   df32 width;
   float sigma;
+  uint32_t open;  // draws that FP64 alone does: none, or all where magnitudes are extreme
   double rg_halfwidth;
 };
+constexpr int kDraws = 30;  // 27 scalars, three of the current
 
-// nominal x (lo + (hi - lo) u), rounded once.
-__device__ __forceinline__ float scaled(const Draw &d, float nominal, float u) {
+// nominal x (lo + (hi - lo) u), rounded once; open: two floats (error 2^-45) leave the rounding
+// undecided.
+__device__ __forceinline__ float scaled(const Draw &d, float nominal, float u, bool &open) {
   df32 p = two_prod(d.width.h, u);
   p.l = __fmaf_rn(d.width.l, u, p.l);
-  df32 s = two_sum(d.lo, p.h);
+  df32 s = fast_two_sum(fmaxf(d.lo, p.h), fminf(d.lo, p.h));
   s.l = __fadd_rn(s.l, p.l);
   const float q = __fmul_rn(s.h, nominal);
   const float r = __fmaf_rn(s.l, nominal, __fmaf_rn(s.h, nominal, -q));
-  return isfinite(q) ? __fadd_rn(q, r) : q;
+  return round_df(q, r, q, 0x1p-43f, open);
 }
 
-// c + sigma r x, rounded once.
-__device__ __forceinline__ float current(const Draw &d, float c, df32 r, df32 x) {
+// c + sigma r x, rounded once; open as above (error of the normal 2^-40.6).
+__device__ __forceinline__ float current(const Draw &d, float c, df32 r, df32 x, bool &open) {
   const df32 z = df_mul(r, x);
   df32 p = two_prod(d.sigma, z.h);
   p.l = __fmaf_rn(d.sigma, z.l, p.l);
   const df32 s = two_sum(c, p.h);
-  return __fadd_rn(s.h, __fadd_rn(s.l, p.l));
+  return round_df(s.h, __fadd_rn(s.l, p.l), __fadd_rn(fabsf(c), fabsf(p.h)), 0x1p-39f, open);
 }
 
-// Draw one tile of blockDim.x envs from e0 on (of the given vehicle type, or of v.types): each thread draws and derives its env, the records
-// are staged in rows [blockDim.x][MG_NPARAM] and leave as one contiguous run (a thread's own row is
-// 140 bytes, so direct stores would touch 32 sectors each).  Everything is FP32 pairs: the FP64
-// form of the same draws took 840 us for 1,048,576 envs, FP64-pipe bound, against 55 us for the
-// 360 bytes per env it stores; this takes 63 us.
+// Word j of an env's parameter draws from its block x of four.
+__device__ __forceinline__ uint32_t draw_word(const uint4 &x, int j) {
+  return (j % 4 == 0) ? x.x : (j % 4 == 1) ? x.y : (j % 4 == 2) ? x.z : x.w;
+}
+
+// The draws whose bits are set in `open` again, in FP64, into the record `row`: the 27 scalars, then
+// the current.  One env in 3,000 comes here, mostly for one value.
+__device__ __noinline__ void redraw_fp64(uint32_t open, const float *__restrict__ nom, const Draw &d,
+                                         uint64_t gid, float *row) {
+  for (; open; open &= open - 1u) {
+    const int j = __ffs(open) - 1;
+    if (j < 27) {
+      const uint4 x = draw4(d.seed, gid, STREAM_PARAMS, (uint32_t)(j / 4));
+      const double lo = (double)d.lo, u = u01d(draw_word(x, j));
+      row[rand_idx(j)] = (float)((double)nom[rand_idx(j)] * (lo + ((double)d.hi - lo) * u));
+    } else {
+      const uint4 x = draw4(d.seed, gid, STREAM_CURRENT, 0u);
+      const double r = sqrt(-2.0 * log(u01d(j < 29 ? x.x : x.z)));
+      const double a = 2.0 * u01d(j < 29 ? x.y : x.w);
+      const int i = MG_P_VC + j - 27;
+      row[i] = (float)((double)nom[i] + (double)d.sigma * (r * (j == 28 ? sinpi(a) : cospi(a))));
+    }
+  }
+}
+
+// Draw one tile of blockDim.x envs from e0 on (of the given vehicle type, or of v.types): each thread
+// draws and derives its env, the records are staged in rows [blockDim.x][MG_NPARAM] and leave as one
+// contiguous run (a thread's own row is 140 bytes, so direct stores would touch 32 sectors each).
+// FP32 pairs but where they leave a rounding open: the FP64 form of the same draws took 840 us for
+// 1,048,576 envs, FP64-pipe bound, against 55 us for the 360 bytes per env it stores; this takes
+// 71 us (63 without the test of each rounding, which left 7 of 3.5 million values off by an ulp).
 // DIAG: every mass matrix is diagonal (no r_g, no extension), so the FP64 Cholesky is not compiled
 // in (it doubles the registers).
 template <bool DIAG>
@@ -253,25 +301,30 @@ __device__ __forceinline__ void randomize_tile(const SetupView &v,
     const uint64_t gid = (uint64_t)(v.gid0 + e);
     const float *nom = nominal + (int64_t)(type < 0 ? v.types[e] : type) * MG_NPARAM;
     float p[MG_NPARAM];
+    uint32_t open = d.open;  // draws left to FP64
+    bool o;
 #pragma unroll
     for (int j = 0; j < MG_NPARAM; ++j) p[j] = nom[j];
     uint4 x = make_uint4(0, 0, 0, 0);
 #pragma unroll
     for (int j = 0; j < 27; ++j) {
       if (j % 4 == 0) x = draw4(d.seed, gid, STREAM_PARAMS, (uint32_t)(j / 4));
-      const uint32_t w = (j % 4 == 0) ? x.x : (j % 4 == 1) ? x.y : (j % 4 == 2) ? x.z : x.w;
-      p[rand_idx(j)] = scaled(d, p[rand_idx(j)], u01f(w));
+      p[rand_idx(j)] = scaled(d, p[rand_idx(j)], u01f(draw_word(x, j)), o);
+      if (o) open |= 1u << j;
     }
     // Box-Muller normals of the current: two of the first pair, the cosine of the second
     const uint4 c = draw4(d.seed, gid, STREAM_CURRENT, 0u);
     df32 cs, sn;
     df32 r = df_normal_radius(u01f(c.x));
     df_cos_sin_turn(u01f(c.y), cs, sn);
-    p[MG_P_VC] = current(d, p[MG_P_VC], r, cs);
-    p[MG_P_VC + 1] = current(d, p[MG_P_VC + 1], r, sn);
+    p[MG_P_VC] = current(d, p[MG_P_VC], r, cs, o);
+    if (o) open |= 1u << 27;
+    p[MG_P_VC + 1] = current(d, p[MG_P_VC + 1], r, sn, o);
+    if (o) open |= 1u << 28;
     r = df_normal_radius(u01f(c.z));
     df_cos_sin_turn(u01f(c.w), cs, sn);
-    p[MG_P_VC + 2] = current(d, p[MG_P_VC + 2], r, cs);
+    p[MG_P_VC + 2] = current(d, p[MG_P_VC + 2], r, cs, o);
+    if (o) open |= 1u << 29;
     if constexpr (!DIAG) {
       if (d.rg_halfwidth > 0.0) {  // off-centre gravity: nominal + U[-w, w] per axis
         const uint4 g = draw4(d.seed, gid, STREAM_PARAMS, 7u);
@@ -284,8 +337,14 @@ __device__ __forceinline__ void randomize_tile(const SetupView &v,
     }
     // Everything the step reads is derived from the stored FP32 values, so that it is consistent
     // with what mg_get_params reports.
+    float *row = rows + threadIdx.x * MG_NPARAM;
 #pragma unroll
-    for (int j = 0; j < MG_NPARAM; ++j) rows[threadIdx.x * MG_NPARAM + j] = p[j];
+    for (int j = 0; j < MG_NPARAM; ++j) row[j] = p[j];
+    if (open) {
+      redraw_fp64(open, nom, d, gid, row);
+#pragma unroll
+      for (int j = 0; j < MG_NPARAM; ++j) p[j] = row[j];
+    }
     if constexpr (DIAG) derive_diag(v, e, p);
     else derive(v, e, p);
   }
@@ -304,7 +363,7 @@ __global__ void __launch_bounds__(kRandThreads)
 }
 
 // Background form: up to 16 small blocks per SM stride over the fleet beside a step kernel on another
-// stream.  Beside the work queue five of them fit an SM at a time; a static grid lets them in at
+// stream.  Beside the work queue four of them fit an SM at a time; a static grid lets them in at
 // its tail, which they then fill (one block per SM ran on alone after it: whole episodes of
 // 1,048,576 envs x 50 sub-steps 1,225 us against 1,054, of 65,536 x 10 55.6 against 42.7).  Same
 // per-env arithmetic.
@@ -476,14 +535,19 @@ __global__ void k_philox(const uint32_t *__restrict__ ctr, const uint32_t *__res
 
 namespace {
 
-Draw make_draw(uint64_t seed, double lo, double hi, double current_sigma, double rg_halfwidth) {
+Draw make_draw(const SetupView &v, uint64_t seed, double lo, double hi, double current_sigma, double rg_halfwidth) {
   Draw d{};
   d.seed = seed;
   d.lo = (float)lo;  // the bounds are FP32 numbers
+  d.hi = (float)hi;
   const double width = hi - lo;
   d.width.h = (float)width;
   d.width.l = (float)(width - (double)d.width.h);
   d.sigma = (float)current_sigma;
+  // Two floats hold 48 bits only while the lower one is a normal number.
+  const bool plain = v.plain && lo >= 1e-6 && hi <= 1e6 &&
+                     (current_sigma == 0.0 || (current_sigma >= 1e-25 && current_sigma <= 1e25));
+  d.open = plain ? 0u : (1u << kDraws) - 1u;
   d.rg_halfwidth = rg_halfwidth;
   return d;
 }
@@ -494,7 +558,7 @@ cudaError_t launch_admit(const SetupView &v, const float *nominal, const mg_job_
                          int32_t *types, const StatePlanes &st, uint32_t *episode, uint32_t *flags,
                          unsigned long long *nonfinite_count, cudaStream_t stream) {
   const mg_ranges &r = job.ranges;
-  const Draw d = make_draw(job.param_seed, (double)r.lo, (double)r.hi, (double)r.current_sigma,
+  const Draw d = make_draw(v, job.param_seed, (double)r.lo, (double)r.hi, (double)r.current_sigma,
                            (double)r.rg_halfwidth);
   const int blocks = (int)((v.n + kRandThreads - 1) / kRandThreads);
   const auto kernel = v.diag_only && r.rg_halfwidth == 0.f ? k_admit<true> : k_admit<false>;
@@ -507,7 +571,7 @@ cudaError_t launch_admit(const SetupView &v, const float *nominal, const mg_job_
 cudaError_t launch_randomize(const SetupView &v, const float *nominal, uint64_t seed, double lo,
                              double hi, double current_sigma, double rg_halfwidth,
                              cudaStream_t stream, int background_blocks) {
-  const Draw d = make_draw(seed, lo, hi, current_sigma, rg_halfwidth);
+  const Draw d = make_draw(v, seed, lo, hi, current_sigma, rg_halfwidth);
   if (background_blocks > 0) {
     if (!v.diag_only || rg_halfwidth != 0.0) return cudaErrorInvalidValue;
     const int64_t full = (v.n + kRandBgThreads - 1) / kRandBgThreads;

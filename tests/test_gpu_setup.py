@@ -31,6 +31,29 @@ def test_draws_are_the_fp64_values_rounded_once(n, lo, hi, sigma, background):
     np.testing.assert_allclose(got, ref, rtol=2.0 ** -24 + 2.0 ** -34, atol=1e-30)
 
 
+@pytest.mark.parametrize("lo,hi,sigma", [(0.8, 1.2, 0.2), (0.003, 7.5, 5.0), (1e-3, 1e3, 1e-4),
+                                         (1.0, 1.0, 0.0)])
+@pytest.mark.parametrize("background", [False, True])
+@pytest.mark.parametrize("extreme", [False, True])
+def test_draws_round_as_fp64_does(lo, hi, sigma, background, extreme):
+    """Every stored value is the one FP64 arithmetic stores: a two-float value whose rounding its
+    error leaves open is drawn again in FP64, and so is every value where a vehicle's are too small
+    for two floats to hold."""
+    vs = vehicles()
+    n = 5003 if extreme else 100003
+    if extreme:
+        vs[0].params[I.P_DL:I.P_DL + 2] = 1e-33, 0.0
+    types = I.mixed_fleet(3, n, max_group=9000)
+    sim = Sim(n, types, vs)
+    if background:
+        sim.randomize_prefetch(78, lo, hi, sigma)
+    sim.randomize(78, lo, hi, sigma, 0.3)
+    got = sim.get_params().cpu().numpy()
+    sim.close()
+    ref = O.randomize(78, oracle_nominal(vs), types, f32(lo), f32(hi), f32(sigma))
+    np.testing.assert_array_equal(got, ref.astype(np.float32))
+
+
 @pytest.mark.parametrize("n", [1, 33, 128, 257, 1000])
 @pytest.mark.parametrize("off", [0, 1, 2])
 def test_records_round_trip_any_alignment(n, off):
