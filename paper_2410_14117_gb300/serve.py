@@ -295,15 +295,14 @@ class NativeServer:
             self._servers[mode] = h
         return self._servers[mode]
 
-    def _record_buffer(self, r):
-        """Tensor for a job's trajectory, written on the pool's stream."""
-        traj = torch.empty((r.horizon, MG_NTRAJ, r.n_envs), dtype=torch.float32,
-                           device=self.pool.device)
+    def _buffer(self, *shape):
+        """Tensor of the caller's stream that the pool's stream writes."""
+        t = torch.empty(shape, dtype=torch.float32, device=self.pool.device)
         current = torch.cuda.current_stream(self.pool.device)
         if current != self.pool.stream:
             self.pool.stream.wait_stream(current)  # the block's earlier use
-            traj.record_stream(self.pool.stream)
-        return traj
+            t.record_stream(self.pool.stream)
+        return t
 
     def close(self):
         for h in self._servers.values():
@@ -345,7 +344,7 @@ class NativeServer:
                 if self.keep_results and self.record:
                     # the job records into the tensor its caller gets; the server keeps it alive
                     # while ticks may write it, also past an exception here
-                    traj = self._record_buffer(r)
+                    traj = self._buffer(r.horizon, MG_NTRAJ, r.n_envs)
                     call("mg_server_submit_record", h, ctypes.byref(spec),
                          None if r.xh is None else _ptr(r.xh), _ptr(traj), ctypes.byref(tk))
                     self._records[mode, tk.value] = traj
@@ -372,8 +371,7 @@ class NativeServer:
             r.job_id = tk
             r.admitted_s, r.done_s = d[1].value - t_start, d[2].value - t_start
             if self.keep_results:
-                r.final_state = torch.empty((r.n_envs, MG_NSTATE), dtype=torch.float32,
-                                            device=self.pool.device)
+                r.final_state = self._buffer(r.n_envs, MG_NSTATE)
                 call("mg_server_job_result", h, tk, _ptr(r.final_state), None)
                 call("mg_server_release", h, tk)
                 r.traj = self._records.pop((mode, tk), None)

@@ -85,3 +85,25 @@ def test_results_on_another_stream():
     for x, y in zip(*out):
         assert torch.equal(x[0], y[0]) and torch.equal(x[1], y[1])
     srv.close()
+
+
+def test_final_states_wait_for_the_memorys_earlier_use():
+    """run() under a stream with work still queued: the final states come in memory that this work
+    may yet write, and are written on the pool's stream after it."""
+    n = 4001
+    srv = NativeServer(I.fleet_vehicles(), budget_bytes=1e9, capacity_envs=1 << 14, k=20,
+                       record=False, keep_results=True)
+    req = lambda: [Request(0.0, n, 40, 0, 3, 9)]  # noqa: E731
+    want = srv.run(req(), realtime=False)[0][0].final_state.cpu()
+    s = torch.cuda.Stream()
+    with torch.cuda.stream(s):
+        x = torch.empty((n, 21), device="cuda")
+        torch.cuda._sleep(400_000_000)  # 0.2 s, longer than the job takes
+        x.fill_(7.0)
+        at = x.data_ptr()
+        del x
+        got = srv.run(req(), realtime=False)[0][0].final_state
+        assert got.data_ptr() == at
+        s.synchronize()
+        assert torch.equal(got.cpu(), want)
+    srv.close()
