@@ -4,10 +4,10 @@ import numpy as np
 import pytest
 import torch
 
-from _helpers import f32, oracle_nominal, vehicles
+from _helpers import TOL_STEP, f32, oracle_geo, oracle_nominal, rel_err, vehicles
 from oracle import oracle as O
 from paper_2410_14117_gb300 import inputs as I
-from paper_2410_14117_gb300.sim import Sim
+from paper_2410_14117_gb300.sim import MGError, Sim
 
 pytestmark = pytest.mark.gpu
 
@@ -71,14 +71,55 @@ def test_records_round_trip_any_alignment(n, off):
     sim.close()
 
 
-def test_not_spd_and_off_axis_records_are_seen():
+def test_not_spd_records_are_seen():
     vs = vehicles()
     n = 300
     p = np.ascontiguousarray(I.perturbed_params(5, oracle_nominal(vs)[np.zeros(n, int)], n))
     p[17, I.P_MA + 2] = -p[17, I.P_M]  # M_33 = 0
     sim = Sim(n, np.zeros(n, np.int32), vs)
-    from paper_2410_14117_gb300.sim import MGError
-    with pytest.raises(MGError):
+    with pytest.raises(MGError) as e:
         sim.set_params(torch.tensor(p, dtype=torch.float32, device="cuda"))
+    assert e.value.code == "MG_ENOTSPD"
     assert np.array_equal(sim.get_params().double().cpu().numpy(), p)
     sim.close()
+
+
+@pytest.mark.parametrize("back", ["set_params", "randomize", "randomize async", "prefetch"])
+@pytest.mark.parametrize("axis", [0, 1])
+def test_off_axis_records_are_seen_and_forgotten(axis, back):
+    """One env's r_b off the z axis: the step keeps its moments (the oracle's step); with r_b back on
+    the axis, by every way there, the steps are those of a sim that never left it."""
+    vs = vehicles()
+    n = 300
+    types = I.mixed_fleet(4, n, max_group=60)
+    nt = np.array([vs[t].n_thr for t in types])
+    on = I.perturbed_params(5, oracle_nominal(vs)[types], n)
+    off = on.copy()
+    off[n - 1, I.P_RB + axis] = 0.03125
+    states, cmds = I.random_states(6, n, nt), I.commands(7, 1, n, nt)
+    dev = lambda x: torch.tensor(x, dtype=torch.float32, device="cuda")  # noqa: E731
+
+    def step(sim):
+        sim.set_state(dev(states))
+        sim.set_actions(dev(cmds), 10)
+        sim.step(5)
+        return sim.get_state()
+
+    def on_axis(sim):
+        if back == "set_params":
+            sim.set_params(dev(on))
+        else:
+            if back == "prefetch":
+                sim.randomize_prefetch(9)
+            sim.randomize(9, wait=back != "randomize async")
+    sim, fresh = Sim(n, types, vs), Sim(n, types, vs)
+    for params in (off, off):
+        sim.set_params(dev(params))
+        ref = O.rollout(params, oracle_geo(vs), types, states, cmds.astype(np.float64), 10, 5, h=0.01)
+        assert rel_err(step(sim).double().cpu().numpy(), ref).max() <= 5 * TOL_STEP
+        on_axis(sim)
+        on_axis(fresh)
+        assert torch.equal(step(sim), step(fresh))
+        assert sim.kernel_info() == fresh.kernel_info()
+    sim.close()
+    fresh.close()
