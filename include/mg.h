@@ -334,8 +334,8 @@ mg_status mg_rollout_backward(mg_sim *sim, int32_t T, int32_t C, const float *ck
  * x 100 floats per env, allocated by mg_rollout_backward on first use), the other applying the
  * transposes from those records one segment behind, so that a small fleet keeps twice as many
  * schedulers busy.  mode 0 (default): mode 2 while ceil(n_envs / 32) is at most 4 times the GPU's
- * SMs (8 times on the general path) and the workspace can be had, else mode 1 (under stream
- * capture, mode 1 too while the sim holds no workspace large enough).  The per-env arithmetic is
+ * SMs and the workspace can be had, else mode 1 (under stream capture, mode 1 too while the sim
+ * holds no workspace large enough).  The per-env arithmetic is
  * the same in both.  The sim keeps the workspace until it is destroyed or mode 1 is set, which
  * gives it back (with a stream that was ever captured: at destruction, since a user's graph may
  * use it).  MG_EINVAL unless 0 <= mode <= 2. */

@@ -1225,19 +1225,19 @@ cudaError_t sm_count(int *n_sm) {
 
 }  // namespace
 
-cudaError_t adjoint_split(int64_t n, bool general, int mode, bool *split) {
+cudaError_t adjoint_split(int64_t n, int mode, bool *split) {
   if (mode == 1 || mode == 2) {
     *split = mode == 2;
     return cudaSuccess;
   }
-  // By fleet size: the two-warp form while all its blocks are resident at once (four per SM), and
-  // twice that on the general path.  200 sub-steps, checkpoints every 20, one-warp / two-warp,
-  // us: diagonal mass 4,096 envs 544 / 335, 16,384 696 / 552, 32,768 1,004 / 1,082; general 4,096
-  // 1,283 / 736, 16,384 1,458 / 1,052, 32,768 2,425 / 2,062.
+  // By fleet size: the two-warp form while all its blocks are resident at once (four per SM, 19,456
+  // envs).  200 sub-steps, checkpoints every 20, one-warp / two-warp, us: diagonal mass 4,096 envs
+  // 453 / 303, 18,000 568 / 516, 20,480 787 / 935, 32,768 837 / 987; general 4,096 1,148 / 695,
+  // 18,000 1,349 / 1,005, 20,480 1,794 / 1,935, 32,768 1,968 / 1,973.
   int n_sm = 0;
   cudaError_t e = sm_count(&n_sm);
   if (e != cudaSuccess) return e;
-  *split = (n + 31) / 32 <= (general ? 8 : 4) * (int64_t)n_sm;
+  *split = (n + 31) / 32 <= 4 * (int64_t)n_sm;
   return cudaSuccess;
 }
 

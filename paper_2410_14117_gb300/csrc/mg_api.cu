@@ -1370,7 +1370,7 @@ mg_status mg_rollout_backward(mg_sim *s, int32_t T, int32_t C, const float *ckpt
   const bool cap = capturing(s);  // a user's graph then reads this parameter range
   bool split = false;
   const bool general = !s->diag || s->has_xh;
-  MG_CK(adjoint_split(s->n, general, s->adj_mode, &split));
+  MG_CK(adjoint_split(s->n, s->adj_mode, &split));
   if (split) {
     const size_t bytes = adjoint_workspace_bytes(eight, s->n, C);
     if (s->adj_ws_cap < bytes && cap) {  // nothing can be allocated

@@ -247,8 +247,8 @@ cudaError_t launch_rollout_forward(const FleetView &fv, const BlockDesc *blocks,
                                    int32_t T, int32_t C, float *traj, float *ckpt,
                                    cudaStream_t stream);
 // Backward kernel: mode 1 one warp per 32 envs, 2 the two-warp form (producer and consumer warps
-// per 32 envs, through a workspace of adjoint_workspace_bytes), 0 chosen by fleet size and path.
-cudaError_t adjoint_split(int64_t n, bool general, int mode, bool *split);
+// per 32 envs, through a workspace of adjoint_workspace_bytes), 0 chosen by fleet size.
+cudaError_t adjoint_split(int64_t n, int mode, bool *split);
 size_t adjoint_workspace_bytes(bool eight, int64_t n, int32_t C);
 // general: the general-path kernels (off-centre gravity, off-diagonal extension, full M^-1).
 // layout: as launch_fleet (the forward's).

@@ -49,7 +49,7 @@ class _Case:
         return [x.clone() for x in self.out]
 
 
-# fleets that the default runs with one thread per env, and with two warps per 32 envs
+# fleets that the default runs with two warps per 32 envs, and with one thread per env
 @pytest.mark.parametrize("n,general", [(97, False), (12000, False), (12000, True), (30000, True),
                                        (30000, False)])
 def test_first_backward_can_be_captured(n, general):
@@ -119,3 +119,16 @@ def test_workspace_is_given_back():
     case.backward(12)
     assert all(torch.equal(x, y) for x, y in zip(want, case.result()))
     case.sim.close()
+
+
+@pytest.mark.parametrize("general", [False, True])
+def test_default_holds_a_workspace_only_while_every_block_is_resident(general):
+    line = 32 * 4 * torch.cuda.get_device_properties(0).multi_processor_count
+    for n, held in ((line, True), (line + 1, False)):
+        case = _Case(n, general)
+        torch.cuda.synchronize()
+        before = torch.cuda.mem_get_info()[0]
+        case.backward(12)
+        torch.cuda.synchronize()
+        assert (before - torch.cuda.mem_get_info()[0] >= 2 * 12 * 100 * 4 * n) == held
+        case.sim.close()
