@@ -181,11 +181,12 @@ mg_status mg_set_wait_limit(mg_sim *sim, uint32_t polls);
 
 /* Domain randomisation (§METHOD; §EXPERIMENTS "supports domain randomization"): per env, draws
  * from Philox4x32-10 keyed by (seed, env id + offset), then builds M = M_RB + M_A and inverts it
- * (FP64 Cholesky, or reciprocals where it is diagonal).  Also records (seed, nu0_sigma) for
- * mg_reset and zeroes every env's episode counter.  Synchronous unless ranges->flags has MG_RANDOMIZE_ASYNC.  Errors: MG_EINVAL
- * (ranges NULL, lo > hi, lo <= 0, negative sigma or half-width, unknown flags, MG_RANDOMIZE_ASYNC
- * for a fleet whose mass matrices may be full), MG_ENOTSPD (parameters are stored but some mass
- * matrix has a pivot <= 0), MG_ECUDA. */
+ * (FP64 Cholesky, or reciprocals where it is diagonal).  The stored FP32 values are those of FP64
+ * arithmetic.  Also records (seed, nu0_sigma) for mg_reset and zeroes every env's episode counter.
+ * Synchronous unless ranges->flags has MG_RANDOMIZE_ASYNC.  Errors: MG_EINVAL (ranges NULL, lo >
+ * hi, lo <= 0, negative sigma or half-width, unknown flags, MG_RANDOMIZE_ASYNC for a fleet whose
+ * mass matrices may be full), MG_ENOTSPD (parameters are stored but some mass matrix has a pivot
+ * <= 0), MG_ECUDA. */
 mg_status mg_randomize(mg_sim *sim, uint64_t seed, const mg_ranges *ranges);
 
 /* Background randomisation (§METHOD's per-episode domain randomisation, drawn ahead): draws the
@@ -202,7 +203,8 @@ mg_status mg_randomize(mg_sim *sim, uint64_t seed, const mg_ranges *ranges);
  * not yet installed in place; a new prefetch replaces it.  ranges->nu0_sigma and ranges->flags are
  * not used here.  The buffer (the sim's parameter planes and records, 360 B per env) is allocated
  * on first use.  Errors: MG_EINVAL (ranges as mg_randomize, or mass matrices that may be full: some
- * type with r_g != 0, rg_halfwidth != 0, or the off-diagonal extension set), MG_ENOMEM, MG_ECUDA. */
+ * type with r_g != 0, rg_halfwidth != 0, or the off-diagonal extension set), MG_ENOMEM,
+ * MG_ECUDA. */
 mg_status mg_randomize_prefetch(mg_sim *sim, uint64_t seed, const mg_ranges *ranges);
 
 /* Set every env's parameters from a [n][MG_NPARAM] record (host or device); inverts the mass
@@ -217,8 +219,8 @@ mg_status mg_get_params(mg_sim *sim, float *out);
  * The mass matrices are re-inverted in FP64 with the off-diagonal added mass; a fleet with a
  * non-zero extension steps on the general path (static grid or work queue, each block or warp
  * staging its envs' coefficients in shared memory; mg_step_split runs its general form).
- * mg_randomize and mg_set_params keep the extension.  Synchronous.  Errors: MG_EINVAL, MG_ENOMEM, MG_ENOTSPD
- * (stored, but some M_RB + M_A is not positive definite), MG_ECUDA. */
+ * mg_randomize and mg_set_params keep the extension.  Synchronous.  Errors: MG_EINVAL, MG_ENOMEM,
+ * MG_ENOTSPD (stored, but some M_RB + M_A is not positive definite), MG_ECUDA. */
 mg_status mg_set_hydro_offdiag(mg_sim *sim, const float *x);
 
 /* Copy every env's off-diagonal extension into out [n][MG_NXPARAM] (host or device; zeros when

@@ -12,10 +12,10 @@
 // matches finite differences of the rollout itself, not of the continuous equations.
 //
 // The throttle lag is linear with the command held (LagEnv): with d = n - c the step gives n+ = n +
-// g d, and the later stages' throttles are n+ + h_i d.  So with e_i the adjoint of stage i's throttle
-// through the thrust, n+ has mu = lambda_n + e_2 + e_3 + e_4, d has delta = g mu + sum h_i e_i, the
-// throttle's own adjoint goes lambda_n <- mu + delta + e_1 and the command's gains -delta; the
-// throttles stay out of the stage combinations.
+// g d, and the later stages' throttles are n+ + h_i d.  So with e_i the adjoint of stage i's
+// throttle through the thrust, n+ has mu = lambda_n + e_2 + e_3 + e_4, d has delta = g mu + sum h_i
+// e_i, the throttle's own adjoint goes lambda_n <- mu + delta + e_1 and the command's gains -delta;
+// the throttles stay out of the stage combinations.
 //
 // Parameter paths, as the forward has:
 //   - diagonal mass (r_g = 0, no off-diagonal extension): rhs_vjp_diag, the transpose of the step's
@@ -24,8 +24,8 @@
 //     off-diagonal I_o) and the off-diagonal added mass and linear damping of the extension record
 //     (zeros when the fleet has none), with the full M^-1.
 // A diagonal coefficient theta = M_A,jj enters M = M_RB + M_A, so nu' = M^-1 f gets d nu'/d theta =
-// -M^-1 e_j nu'_j, whose contribution to the gradient is -(M^-1 g)_j nu'_j for the loss adjoint g of
-// nu' (M^-1 is symmetric).  nu' itself comes recorded with the stage states.
+// -M^-1 e_j nu'_j, whose contribution to the gradient is -(M^-1 g)_j nu'_j for the loss adjoint g
+// of nu' (M^-1 is symmetric).  nu' itself comes recorded with the stage states.
 #include <type_traits>
 
 #include "mg_advance.cuh"
@@ -55,7 +55,8 @@ __host__ __device__ constexpr int adj_layout(int path) {
 struct GradGen {
   float ma[3], J[3], mv[6], dl[6], dq[6];
 };
-// Diagonal mass, with g the loss adjoint of nu' (trans/rotational rows i, i1 = i+1, i2 = i+2 mod 3):
+// Diagonal mass, with g the loss adjoint of nu' (trans/rotational rows i, i1 = i+1, i2 = i+2 mod
+// 3):
 //   dl, dq   sum g_j x_j, sum g_j |x_j| x_j         (x = r, w)
 //   own      sum g_i (w_i2 c_i1 - w_i1 c_i2), c = v - r the current seen from the body
 //   up, dn   sum g_i w_i2 r_i1, sum g_i w_i1 r_i2
@@ -94,11 +95,11 @@ __device__ __forceinline__ float xd(const float *xh, int i, int j) {
   return xh[15 + 5 * i + (j < i ? j : j - 1)];
 }
 
-// Every multiply-add of the adjoint code below, and of the right-hand side it re-runs, is written as
-// an explicit fmaf, and a product that only a plain addition follows as __fmul_rn, so the compiler
-// forms no fused operation of its own: the results do not depend on the surrounding code the
-// functions are inlined into (the one-warp and two-warp backward kernels agree bit for bit; so does
-// this file compiled without contraction).
+// Every multiply-add of the adjoint code below, and of the right-hand side it re-runs, is written
+// as an explicit fmaf, and a product that only a plain addition follows as __fmul_rn, so the
+// compiler forms no fused operation of its own: the results do not depend on the surrounding code
+// the functions are inlined into (the one-warp and two-warp backward kernels agree bit for bit; so
+// does this file compiled without contraction).
 
 __device__ __forceinline__ void cross_vjp(const float a[3], const float b[3], const float gc[3],
                                           float ga[3], float gb[3]) {
@@ -329,13 +330,14 @@ __device__ void rhs_vjp_gen(const St<MT> &s, const float (&nud)[6], const AdjEnv
 
 // The transpose of the diagonal-mass right-hand side (rhs with StepDiag or StepMirrored): gs = (d
 // rhs / d s)^T gd for the pose and velocity, en[i] the adjoint of the stage throttle n_i through
-// the thrust, the sums of GradDiag accumulated.  With u_i = v_i1 + bp_i r_i1, x_i = v_i2 + bm_i r_i2
-// the rows are v'_i = ... + w_i2 u_i - w_i1 x_i - (dlt_i + dqt_i |r_i|) r_i and w'_i = ... + B_i r_i1
-// r_i2 + C_i w_i1 w_i2 - (dlr_i + dqr_i |w_i|) w_i.  About 290 operations a stage where the general
-// path's form of the same transpose (which this path used before) takes some 700: the consumer
-// warp of the two-warp kernel, a chain of these, is what bounds a small fleet's backward pass: 4,096
-// envs x 200 sub-steps 918 -> 330 us together with the re-run's single evaluation of each sub-step
-// and the 16-byte records (ncu: 2,390 instead of 4,580 instructions a sub-step in the two warps).
+// the thrust, the sums of GradDiag accumulated.  With u_i = v_i1 + bp_i r_i1, x_i = v_i2 + bm_i
+// r_i2 the rows are v'_i = ... + w_i2 u_i - w_i1 x_i - (dlt_i + dqt_i |r_i|) r_i and w'_i = ... +
+// B_i r_i1 r_i2 + C_i w_i1 w_i2 - (dlr_i + dqr_i |w_i|) w_i.  About 290 operations a stage where
+// the general path's form of the same transpose (which this path used before) takes some 700: the
+// consumer warp of the two-warp kernel, a chain of these, is what bounds a small fleet's backward
+// pass: 4,096 envs x 200 sub-steps 918 -> 330 us together with the re-run's single evaluation of
+// each sub-step and the 16-byte records (ncu: 2,390 instead of 4,580 instructions a sub-step in the
+// two warps).
 template <int MT, int PATH>
 __device__ __forceinline__ void rhs_vjp_diag(const St<MT> &s, const float (&nud)[6],
                                              const AdjEnv<PATH> &A, const float4 *gdir,
@@ -1153,6 +1155,8 @@ __global__ void __maxnreg__(XH ? kRegsXH : DIAG ? kRegsWide : kRegsGeneral)
       load_commands<MT>(fv, e, seg, nt, c);
       if (left < T - it) prefetch_commands(fv, e, seg);
     }
+    // packed updates (axpy), packed / not, 200 sub-steps: eight thrusters 179 / 187 us at 30,000
+    // envs, 109 / 109 at 4,096 (general path 269 / 277, 158 / 162); six 173 / 175 and 105 / 103
     if constexpr (XH || MT > 6)
       rk4_step<MT, DIAG, MIXED, NH, XH>(s, c, L, P, sdir, sarm, nt, current_accel, fv.rk2, xh);
     else
@@ -1180,13 +1184,13 @@ cudaError_t rollout_fwd_d(const FleetView &fv, const BlockDesc *blocks, int n_bl
                           float *traj, float *ckpt, cudaStream_t stream) {
   if (diag)
     return with_layout<true>(layout, [&](auto l) {
-      return rollout_fwd_t<NTV, true, decltype(l)::value, false>(fv, blocks, n_blocks, threads, T, C,
-                                                                 traj, ckpt, stream);
+      return rollout_fwd_t<NTV, true, decltype(l)::value, false>(fv, blocks, n_blocks, threads, T,
+                                                                 C, traj, ckpt, stream);
     });
   return with_layout<false>(layout, [&](auto l) {
     constexpr int L = decltype(l)::value;
-    return fv.xh ? rollout_fwd_t<NTV, false, L, true>(fv, blocks, n_blocks, threads, T, C, traj, ckpt,
-                                                      stream)
+    return fv.xh ? rollout_fwd_t<NTV, false, L, true>(fv, blocks, n_blocks, threads, T, C, traj,
+                                                      ckpt, stream)
                  : rollout_fwd_t<NTV, false, L, false>(fv, blocks, n_blocks, threads, T, C, traj,
                                                        ckpt, stream);
   });

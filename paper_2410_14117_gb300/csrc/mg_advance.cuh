@@ -56,8 +56,8 @@ auto with_layout(int layout, F f) {
   return f(std::integral_constant<int, MG_LAYOUT_DENSE>());
 }
 
-// The cursor a static-grid step launch starts at: 0 when the launch carries a rewind that the device
-// has not seen (rewinding is then true), else the device's word.
+// The cursor a static-grid step launch starts at: 0 when the launch carries a rewind that the
+// device has not seen (rewinding is then true), else the device's word.
 __device__ __forceinline__ int64_t start_cursor(const FleetView &fv, bool &rewinding) {
   rewinding = fv.rewind && __ldcg(fv.rewind_gen) != fv.rewind;
   return rewinding ? 0 : launch_cursor(fv);
@@ -216,9 +216,9 @@ __device__ __forceinline__ void scheduled_start(const FleetView &fv, int64_t e, 
 // XH: xh is the env's row of staged off-diagonal hydrodynamic coefficients.
 // start(c, seg, left) sets the first sub-step's command c, its segment and the sub-steps left in it
 // (scheduled_start, or a fused kernel's own source).
-// loaded: the parameters, where the caller has loaded them and the state s already (the task kernel,
-// before its block barrier; the step kernels' loops come out 2 % slower that way).
-// PACK: packed stage updates (see axpy).
+// loaded: the parameters, where the caller has loaded them and the state s already (the task
+// kernel, before its block barrier; the step kernels' loops come out 2 % slower that way). PACK:
+// packed stage updates (see axpy).
 template <int MT, bool DIAG, bool MIXED, bool REC, bool L2, int NH, bool XH, bool PACK,
           bool LOADED = false, typename Start = void>
 __device__ __forceinline__ void advance_env(const FleetView &fv, int64_t e, int nt,
@@ -233,10 +233,10 @@ __device__ __forceinline__ void advance_env(const FleetView &fv, int64_t e, int 
   int64_t seg;
   int32_t left;
   // The command's address depends on the action cursor and starts its load before the parameters'
-  // 34 floats arrive; the work queue, whose warps overlap one another's loads, runs faster the other
-  // way round (registers: 65,536 envs x 1,000 sub-steps 1.29 against 1.35 ms; the static grid 1.39
-  // against 1.44 ms in this order), and so do mixed fleets on the static grid (262,144 x 500 2.65
-  // against 2.67 ms).
+  // 34 floats arrive; the work queue, whose warps overlap one another's loads, runs faster the
+  // other way round (registers: 65,536 envs x 1,000 sub-steps 1.29 against 1.35 ms; the static grid
+  // 1.39 against 1.44 ms in this order), and so do mixed fleets on the static grid (262,144 x 500
+  // 2.65 against 2.67 ms).
   if constexpr (!L2 && !MIXED) start(c, seg, left);
   Coef<DIAG, NH> P;
   {

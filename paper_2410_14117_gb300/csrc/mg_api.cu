@@ -204,11 +204,11 @@ struct mg_sim {
   int32_t proc = 0;
   uint64_t cmd_seed = 0;
   int64_t cursor = 0;  // host copy of the device cursor (counters[3])
-  // A rewind not yet in device memory (rewind_cursor): number rewind_gen, carried by the next direct
-  // step launch, or settled before any other use of the cursor; whichever runs first on the device
-  // applies it.  captured: the sim's stream has been captured into a user's graph, whose replays
-  // read the cursor at times the host does not see, so rewinds go to device memory at once from
-  // then on; a rewind pending when a capture starts stays pending beside the captured launch.
+  // A rewind not yet in device memory (rewind_cursor): number rewind_gen, carried by the next
+  // direct step launch, or settled before any other use of the cursor; whichever runs first on the
+  // device applies it.  captured: the sim's stream has been captured into a user's graph, whose
+  // replays read the cursor at times the host does not see, so rewinds go to device memory at once
+  // from then on; a rewind pending when a capture starts stays pending beside the captured launch.
   bool rewind_pending = false;
   uint32_t rewind_gen = 0;
   bool captured = false;
@@ -1212,9 +1212,9 @@ mg_status mg_step(mg_sim *s, int32_t k) {
   mg_status st;
   const bool single = !s->queue && k <= s->spl;
   if (single) {
-    // One static-grid launch: as it is, carrying a pending rewind.  A graph of this one kernel is no
-    // cheaper for the host and takes twice as long on the device (256 envs, back to back: 6.2 us a
-    // step against 3.1, the launches overlapping).
+    // One static-grid launch: as it is, carrying a pending rewind.  A graph of this one kernel is
+    // no cheaper for the host and takes twice as long on the device (256 envs, back to back: 6.2 us
+    // a step against 3.1, the launches overlapping).
     const bool cap = capturing(s);
     FleetView v = s->view();
     v.cursor_adv = k;

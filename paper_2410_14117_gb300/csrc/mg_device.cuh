@@ -233,8 +233,8 @@ __host__ __device__ constexpr bool mirrored_sums(int layout) {
   return layout >= MG_LAYOUT_MIRRORED_G;
 }
 
-// MG_LAYOUT_MIRRORED_G: and mi G_y of the roll row, mi G_x of the pitch row, mi G_x and mi G_y of the
-// yaw row.
+// MG_LAYOUT_MIRRORED_G: and mi G_y of the roll row, mi G_x of the pitch row, mi G_x and mi G_y of
+// the yaw row.
 struct StepMirroredG : StepMirrored {
   float Gry, Gpx, Gyx, Gyy;
 };
@@ -648,12 +648,13 @@ __device__ __forceinline__ void fma2(float &o0, float &o1, float2 a, float k0, f
 }
 
 // y = x + a k for the pose and velocity, with the quaternion taking aq = a / 2 (its derivative is
-// stored doubled).  Packed (W = float2): velocity and attitude in five packed multiply-adds instead of ten.  The
-// same bits; a pair reads its operands without bank conflicts and takes one issue slot, but ties its
-// registers together, so it pays only in the larger loops.  200 sub-steps of 30,000 recorded
-// 8-thruster envs 241 -> 210 us, 12 served jobs 911 -> 891, 16,384 envs with the full hydrodynamics
-// 203.5 -> 199.4, 65,536 mixed environment steps 22.6 -> 22.2; but 65,536 six-thruster envs x 1,000
-// on the work queue 1,303 -> 1,440, 1,024 x 500 227.6 -> 230.2, 262,144 mixed x 100 520 -> 527.
+// stored doubled).  Packed (W = float2): velocity and attitude in five packed multiply-adds instead
+// of ten.  The same bits; a pair reads its operands without bank conflicts and takes one issue
+// slot, but ties its registers together, so it pays only in the larger loops.  200 sub-steps of
+// 30,000 recorded 8-thruster envs 180 -> 176 us, 12 served jobs 911 -> 891, 16,384 envs with the
+// full hydrodynamics 203.5 -> 199.4, 65,536 mixed environment steps 22.6 -> 22.2; but 65,536
+// six-thruster envs x 1,000 on the work queue 1,303 -> 1,440, 1,024 x 500 227.6 -> 230.2, 262,144
+// mixed x 100 520 -> 527, and 30,000 recorded six-thruster ones 170 -> 171.
 __device__ __forceinline__ float scalar(float a) { return a; }
 __device__ __forceinline__ float scalar(float2 a) { return a.x; }
 
@@ -679,8 +680,8 @@ __device__ __forceinline__ void axpy(St<MT> &y, const St<MT> &x, W a, W aq, cons
 }
 
 // The throttle lag n' = (c - n) / tau_m is linear with the command held, so RK4 applied to it has
-// closed forms in the deviation d = n - c: with z = -h / tau_m the step gives n + g d, 1 + g = 1 + z
-// + z^2/2 + z^3/6 + z^4/24 (RK4's stability polynomial), and the stage values differ from that by
+// closed forms in the deviation d = n - c: with z = -h / tau_m the step gives n + g d, 1 + g = 1 +
+// z + z^2/2 + z^3/6 + z^4/24 (RK4's stability polynomial), and the stage values differ from that by
 // h2 d, h3 d and h4 d (1 + g + h2 = 1 + z/2, 1 + g + h3 = 1 + z/2 + z^2/4, 1 + g + h4 = 1 + z +
 // z^2/2 + z^3/4) — the same numbers as RK4's stage updates and weighted sum, in 5 operations per
 // thruster instead of 11 (a form in n and h c / tau_m takes 7).  With the RK4 weights as kernel

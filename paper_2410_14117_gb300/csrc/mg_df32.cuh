@@ -1,11 +1,11 @@
 // Two-float arithmetic for the set-up kernels: a value is the unevaluated sum h + l of two FP32
-// numbers, |l| <= ulp(h) / 2.  GB300 executes FP64 at a 64th of the FP32 rate, which made the domain
-// randomisation (some 380 FP64 warp instructions per 32 envs) a quarter of a 100-sub-step episode
-// of a 1,048,576-env fleet.  The sums and products below are exact or good to 2^-45, the elementary
-// functions to 2^-41 (every uniform draw checked against 64-bit mantissas: radius 2^-41.4, sine and
-// cosine 2^-41.8).  A result is rounded to FP32 from here only where both ends of its error bound
-// round alike (round_df); the few others are left to FP64, so what is stored is what FP64
-// arithmetic stores, bit for bit.
+// numbers, |l| <= ulp(h) / 2.  GB300 executes FP64 at a 64th of the FP32 rate, which made the
+// domain randomisation (some 380 FP64 warp instructions per 32 envs) a quarter of a 100-sub-step
+// episode of a 1,048,576-env fleet.  The sums and products below are exact or good to 2^-45, the
+// elementary functions to 2^-41 (every uniform draw checked against 64-bit mantissas: radius
+// 2^-41.4, sine and cosine 2^-41.8).  A result is rounded to FP32 from here only where both ends of
+// its error bound round alike (round_df); the few others are left to FP64, so what is stored is
+// what FP64 arithmetic stores, bit for bit.
 //
 // Published methods: Knuth's two-sum, Dekker's fast two-sum and the FMA two-product; the series of
 // atanh, sin and cos.  Every operation is an explicit round-to-nearest intrinsic, so the compiler
@@ -49,8 +49,8 @@ __device__ __forceinline__ constexpr df32 df_const(double c) {
   return {(float)c, (float)(c - (double)(float)c)};
 }
 
-// q + r, |r| << |q|, rounded to FP32.  open: some number within w rel of it rounds otherwise (or it is
-// not finite).
+// q + r, |r| << |q|, rounded to FP32.  open: some number within w rel of it rounds otherwise (or it
+// is not finite).
 __device__ __forceinline__ float round_df(float q, float r, float w, float rel, bool &open) {
   const float f = __fadd_rn(q, __fmaf_rn(w, rel, r));
   open = !(f == __fadd_rn(q, __fmaf_rn(-w, rel, r)));

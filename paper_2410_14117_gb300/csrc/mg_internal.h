@@ -171,8 +171,8 @@ bool vectored_layout(const Geo &g);
 // True for mirror images (MG_LAYOUT_MIRRORED in mg_device.cuh): six or eight thrusters whose rows
 // repeat one magnitude each with the signs given there.
 bool mirrored_layout(const Geo &g);
-// The fastest MG_LAYOUT_* of the diagonal-mass step that vehicle type v with geometry g has (mirrored asks for r_b on the
-// z axis too).
+// The fastest MG_LAYOUT_* of the diagonal-mass step that vehicle type v with geometry g has
+// (mirrored asks for r_b on the z axis too, or is the form for any r_b).
 int thruster_layout(const Geo &g, const mg_vehicle_params &v);
 
 // ---------------------------------------------------------------- launchers (mg_setup.cu)
@@ -187,8 +187,8 @@ struct SetupView {
   const float *xh;           // device [MG_NXPARAM][xh_stride] off-diagonal hydrodynamics, or null
   int64_t xh_stride;         // floats between xh's component planes (0: n)
   bool plain;                // plain_record() for every type's nominal record
-  bool diag_only;            // nominal mass matrices are diagonal and xh is null: a draw without r_g
-                             // keeps them so
+  bool diag_only;            // nominal mass matrices are diagonal and xh is null: a draw without
+                             // r_g keeps them so
 };
 
 // Whether a nominal record's magnitudes are ordinary (zero, or within [1e-25, 1e25]).

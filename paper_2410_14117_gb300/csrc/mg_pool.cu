@@ -42,9 +42,9 @@ struct ServeBlock {
 
 namespace {
 
-// Two warps per block: a tick's blocks come in any number, and the last ones leave SMs idle by whole
-// blocks (6 jobs of up to 4,000 envs served in 274-280 us with 64 threads, 289 with 128, 281 with
-// 32; 12 jobs of up to 32,768 in 909, 909, 897).
+// Two warps per block: a tick's blocks come in any number, and the last ones leave SMs idle by
+// whole blocks (6 jobs of up to 4,000 envs served in 274-280 us with 64 threads, 289 with 128, 281
+// with 32; 12 jobs of up to 32,768 in 909, 909, 897).
 constexpr int kServeThreads = 64;
 // Register cap of the tick kernel for ticks of many blocks: 144 (seven blocks per SM) served those
 // 12 jobs in 909 us against 960 at 128, where the vectored and dense allocations also spill.

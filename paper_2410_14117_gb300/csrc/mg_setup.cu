@@ -107,8 +107,8 @@ __device__ __forceinline__ void derive_diag(const SetupView &v, int64_t e, const
   pa.d7[e] = make_float4(mi[0], mi[1], mi[2], mi[3]);
   pa.d8[e] = make_float2(mi[4], mi[5]);
   if (open)
-    invert_diag_fp64(pa, e, m, p[MG_P_IG], p[MG_P_IG + 1], p[MG_P_IG + 2], ma[0], ma[1], ma[2], ma[3],
-                     ma[4], ma[5]);
+    invert_diag_fp64(pa, e, m, p[MG_P_IG], p[MG_P_IG + 1], p[MG_P_IG + 2], ma[0], ma[1], ma[2],
+                     ma[3], ma[4], ma[5]);
   const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
   pa.g0[e] = make_float4(__fmul_rn(m, rg[0]), __fmul_rn(m, rg[1]), __fmul_rn(m, rg[2]), 0.f);
   pa.g1[e] = z;
@@ -264,10 +264,10 @@ __device__ __forceinline__ uint32_t draw_word(const uint4 &x, int j) {
   return (j % 4 == 0) ? x.x : (j % 4 == 1) ? x.y : (j % 4 == 2) ? x.z : x.w;
 }
 
-// The draws whose bits are set in `open` again, in FP64, into the record `row`: the 27 scalars, then
-// the current.  One env in 3,000 comes here, mostly for one value.
-__device__ __noinline__ void redraw_fp64(uint32_t open, const float *__restrict__ nom, const Draw &d,
-                                         uint64_t gid, float *row) {
+// The draws whose bits are set in `open` again, in FP64, into the record `row`: the 27 scalars,
+// then the current.  One env in 3,000 comes here, mostly for one value.
+__device__ __noinline__ void redraw_fp64(uint32_t open, const float *__restrict__ nom,
+                                         const Draw &d, uint64_t gid, float *row) {
   for (; open; open &= open - 1u) {
     const int j = __ffs(open) - 1;
     if (j < 27) {
@@ -284,14 +284,14 @@ __device__ __noinline__ void redraw_fp64(uint32_t open, const float *__restrict_
   }
 }
 
-// Draw one tile of blockDim.x envs from e0 on (of the given vehicle type, or of v.types): each thread
-// draws and derives its env, the records are staged in rows [blockDim.x][MG_NPARAM] and leave as one
-// contiguous run (a thread's own row is 140 bytes, so direct stores would touch 32 sectors each).
-// FP32 pairs but where they leave a rounding open: the FP64 form of the same draws took 840 us for
-// 1,048,576 envs, FP64-pipe bound, against 55 us for the 360 bytes per env it stores; this takes
-// 71 us (63 without the test of each rounding, which left 7 of 3.5 million values off by an ulp).
-// DIAG: every mass matrix is diagonal (no r_g, no extension), so the FP64 Cholesky is not compiled
-// in (it doubles the registers).
+// Draw one tile of blockDim.x envs from e0 on (of the given vehicle type, or of v.types): each
+// thread draws and derives its env, the records are staged in rows [blockDim.x][MG_NPARAM] and
+// leave as one contiguous run (a thread's own row is 140 bytes, so direct stores would touch 32
+// sectors each). FP32 pairs but where they leave a rounding open: the FP64 form of the same draws
+// took 840 us for 1,048,576 envs, FP64-pipe bound, against 55 us for the 360 bytes per env it
+// stores; this takes 71 us (63 without the test of each rounding, which left 7 of 3.5 million
+// values off by an ulp). DIAG: every mass matrix is diagonal (no r_g, no extension), so the FP64
+// Cholesky is not compiled in (it doubles the registers).
 template <bool DIAG>
 __device__ __forceinline__ void randomize_tile(const SetupView &v,
                                                const float *__restrict__ nominal, const Draw &d,
@@ -362,9 +362,9 @@ __global__ void __launch_bounds__(kRandThreads)
   randomize_tile<DIAG>(v, nominal, d, (int64_t)blockIdx.x * kRandThreads, rows);
 }
 
-// Background form: up to 16 small blocks per SM stride over the fleet beside a step kernel on another
-// stream.  Beside the work queue four of them fit an SM at a time; a static grid lets them in at
-// its tail, which they then fill (one block per SM ran on alone after it: whole episodes of
+// Background form: up to 16 small blocks per SM stride over the fleet beside a step kernel on
+// another stream.  Beside the work queue four of them fit an SM at a time; a static grid lets them
+// in at its tail, which they then fill (one block per SM ran on alone after it: whole episodes of
 // 1,048,576 envs x 50 sub-steps 1,225 us against 1,054, of 65,536 x 10 55.6 against 42.7).  Same
 // per-env arithmetic.
 __global__ void __launch_bounds__(kRandBgThreads)
@@ -377,9 +377,10 @@ __global__ void __launch_bounds__(kRandBgThreads)
   }
 }
 
-// Admission of a serving job in one launch: its envs' type, parameters and start state (episode 0 of
-// the job's own seed).  As four operations (fill, draw, clear, reset), each bound by its own latency
-// and launch, it took 9 us longer a job: 12 jobs of 64 to 32,768 envs served in 1,015 us, 909 so.
+// Admission of a serving job in one launch: its envs' type, parameters and start state (episode 0
+// of the job's own seed).  As four operations (fill, draw, clear, reset), each bound by its own
+// latency and launch, it took 9 us longer a job: 12 jobs of 64 to 32,768 envs served in 1,015 us,
+// 909 so.
 template <bool DIAG>
 __global__ void __launch_bounds__(kRandThreads)
     k_admit(const SetupView v, const float *__restrict__ nominal, const Draw d, int32_t type,
@@ -454,8 +455,9 @@ __global__ void __launch_bounds__(kRowThreads)
   const int64_t e0 = (int64_t)blockIdx.x * kRowThreads;
   const int t = (int)threadIdx.x;
   const int64_t e = e0 + t;
-  // Programmatic dependent launch, both ways: this kernel's launch overlaps the step that writes the
-  // state, and the next step's launch overlaps this kernel (each waits here for the one before it).
+  // Programmatic dependent launch, both ways: this kernel's launch overlaps the step that writes
+  // the state, and the next step's launch overlaps this kernel (each waits here for the one before
+  // it).
   cudaTriggerProgrammaticLaunchCompletion();
   cudaGridDependencySynchronize();
   if (e < n) {
@@ -505,7 +507,8 @@ __global__ void __launch_bounds__(kRowThreads)
   st.s5[e] = r[20];
 }
 
-__global__ void k_rewind(unsigned long long *cursor, uint32_t *gen_word, uint32_t gen, bool always) {
+__global__ void k_rewind(unsigned long long *cursor, uint32_t *gen_word, uint32_t gen,
+                         bool always) {
   if (always || *gen_word != gen) {
     *cursor = 0;
     *gen_word = gen;
@@ -535,7 +538,8 @@ __global__ void k_philox(const uint32_t *__restrict__ ctr, const uint32_t *__res
 
 namespace {
 
-Draw make_draw(const SetupView &v, uint64_t seed, double lo, double hi, double current_sigma, double rg_halfwidth) {
+Draw make_draw(const SetupView &v, uint64_t seed, double lo, double hi, double current_sigma,
+               double rg_halfwidth) {
   Draw d{};
   d.seed = seed;
   d.lo = (float)lo;  // the bounds are FP32 numbers

@@ -196,12 +196,12 @@ cudaError_t launch_t(const FleetView &fv, const BlockDesc *blocks, int n_blocks,
   });
 }
 
-// Whether the static grid takes the 200-register kernel.  The mirrored allocation fits 128 registers
-// without spilling, which puts four 128-thread blocks on an SM against three: 65,536 envs x 200 in
-// 288 us against 373, 1,048,576 x 50 in 937 against 966; six thrusters gain nothing by more
-// registers at any size (1,000 envs x 200: 90 us both, 50,000: 223 against 233).  Eight, and mixed
-// fleets, do while all blocks are resident at once (1,000 envs: 95 against 102 us; 50,000: 241
-// against 246).  The other allocations spill at 128.
+// Whether the static grid takes the 200-register kernel.  The mirrored allocation fits 128
+// registers without spilling, which puts four 128-thread blocks on an SM against three: 65,536 envs
+// x 200 in 288 us against 373, 1,048,576 x 50 in 937 against 966; six thrusters gain nothing by
+// more registers at any size (1,000 envs x 200: 90 us both, 50,000: 223 against 233).  Eight, and
+// mixed fleets, do while all blocks are resident at once (1,000 envs: 95 against 102 us; 50,000:
+// 241 against 246).  The other allocations spill at 128.
 template <int NTV>
 bool wide_kernel(bool wide, int layout, int n_blocks, int threads) {
   if (!wide || !mirrored_sums(layout)) return wide;
@@ -326,8 +326,8 @@ void queue_launch(bool diag, bool wide, int layout, int grid, size_t smem, const
                   uint32_t *sched, cudaStream_t stream) {
   if (diag)
     with_layout<true>(layout, [&](auto l) {
-      queue_launch_w<NTV, true, decltype(l)::value>(wide, grid, smem, fv, slices, n_slices, k, chunk,
-                                                    sched, stream);
+      queue_launch_w<NTV, true, decltype(l)::value>(wide, grid, smem, fv, slices, n_slices, k,
+                                                    chunk, sched, stream);
     });
   else
     with_layout<false>(layout, [&](auto l) {

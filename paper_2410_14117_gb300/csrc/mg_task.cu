@@ -375,8 +375,8 @@ cudaError_t fleet_task_d(const FleetView &fv, const BlockDesc *blocks, int n_blo
     });
   return with_layout<false>(layout, [&](auto l) {
     constexpr int L = decltype(l)::value;
-    return fv.xh ? fleet_task_t<NTV, false, L, true>(fv, blocks, n_blocks, threads, k_launch, k_task,
-                                                     tv, to, smem, stream)
+    return fv.xh ? fleet_task_t<NTV, false, L, true>(fv, blocks, n_blocks, threads, k_launch,
+                                                     k_task, tv, to, smem, stream)
                  : fleet_task_t<NTV, false, L>(fv, blocks, n_blocks, threads, k_launch, k_task, tv,
                                                to, smem, stream);
   });
@@ -384,7 +384,8 @@ cudaError_t fleet_task_d(const FleetView &fv, const BlockDesc *blocks, int n_blo
 
 __global__ void k_clamp_actions(const float *__restrict__ in, float *__restrict__ out,
                                 int64_t count) {
-  // the task kernel that follows may launch now and wait for this copy at its dependency point
+  // k > steps_per_launch (else the task kernel clamps): the first of the step's launches may be
+  // placed now, and its blocks wait for this copy at their dependency point
   cudaTriggerProgrammaticLaunchCompletion();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= count) return;

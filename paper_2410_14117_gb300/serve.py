@@ -295,12 +295,12 @@ class NativeServer:
             self._servers[mode] = h
         return self._servers[mode]
 
-    def _buffer(self, *shape):
-        """Tensor of the caller's stream that the pool's stream writes."""
+    def _buffer(self, other, *shape):
+        """Tensor that the pool's stream writes; ``other``: the caller's stream, or None when it is
+        the pool's."""
         t = torch.empty(shape, dtype=torch.float32, device=self.pool.device)
-        current = torch.cuda.current_stream(self.pool.device)
-        if current != self.pool.stream:
-            self.pool.stream.wait_stream(current)  # the block's earlier use
+        if other is not None:
+            self.pool.stream.wait_stream(other)  # the block's earlier use
             t.record_stream(self.pool.stream)
         return t
 
@@ -320,6 +320,9 @@ class NativeServer:
                 raise ValueError(f"request of {r.n_envs} envs x {r.horizon} sub-steps can never "
                                  "be admitted (arena capacity or budget too small)")
         h = self._server(mode)
+        other = torch.cuda.current_stream(self.pool.device)  # asking costs as much as a launch
+        if other == self.pool.stream:
+            other = None
         d = [ctypes.c_double() for _ in range(3)]
 
         def clock():
@@ -344,7 +347,7 @@ class NativeServer:
                 if self.keep_results and self.record:
                     # the job records into the tensor its caller gets; the server keeps it alive
                     # while ticks may write it, also past an exception here
-                    traj = self._buffer(r.horizon, MG_NTRAJ, r.n_envs)
+                    traj = self._buffer(other, r.horizon, MG_NTRAJ, r.n_envs)
                     call("mg_server_submit_record", h, ctypes.byref(spec),
                          None if r.xh is None else _ptr(r.xh), _ptr(traj), ctypes.byref(tk))
                     self._records[mode, tk.value] = traj
@@ -371,7 +374,7 @@ class NativeServer:
             r.job_id = tk
             r.admitted_s, r.done_s = d[1].value - t_start, d[2].value - t_start
             if self.keep_results:
-                r.final_state = self._buffer(r.n_envs, MG_NSTATE)
+                r.final_state = self._buffer(other, r.n_envs, MG_NSTATE)
                 call("mg_server_job_result", h, tk, _ptr(r.final_state), None)
                 call("mg_server_release", h, tk)
                 r.traj = self._records.pop((mode, tk), None)
