@@ -8,13 +8,13 @@
 namespace mg {
 
 // Register caps: the narrow diagonal-mass step keeps 128 registers (16 resident warps per SM, for
-// the per-step form and large per-step grids; no spills with the mirrored allocation, 40-280 bytes
+// the per-step form and large per-step grids; no spills with the mirrored allocation, 70-440 bytes
 // with the others); the general step keeps 168.
 constexpr int kRegsDiag = 128;
 constexpr int kRegsGeneral = 168;
 // The wide diagonal-mass variants (mg_set_schedule's wide): the work-queue kernel runs at 8
 // warps/SM, where 256 registers per thread would fit; with the mirrored allocation ptxas uses
-// 164-178 (65,536 envs x 1,000 sub-steps: 1.29 ms; the static grid at 128 registers 1.38 ms).  The
+// 164-168 (65,536 envs x 1,000 sub-steps: 1.29 ms; the static grid at 128 registers 1.38 ms).  The
 // static grid takes it where that pays (wide_kernel in mg_step.cu).
 constexpr int kRegsWide = 200;
 // With the off-diagonal hydrodynamics the 45 extra coefficients stay in registers too (no
